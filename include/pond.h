@@ -75,9 +75,9 @@ typedef enum {
     POND_ETHETA = 5,    /* warning: the pressure floor was hit since the last
                            report (sticky flag; outputs are still written)         */
     POND_ENAN = 6,      /* a NaN/Inf appeared in the state (see pond_stats)        */
-    POND_ETIMEOUT = 7   /* a bounded wait of the D2Q9 step for a tile's staging
-                           copies (TMA) ran out: the tile was skipped, the state
-                           is incomplete (sticky, reported at the sync points)     */
+    POND_ETIMEOUT = 7   /* a bounded device wait ran out and the state is
+                           incomplete (sticky, reported at the sync points); no
+                           kernel of this version waits, so it is not returned     */
 } pond_status;
 
 enum { POND_PERIODIC = 0, POND_ZEROGRAD = 1 };     /* boundary per axis               */
@@ -121,11 +121,12 @@ typedef struct {
  * p_floor: pressure floor of the gauge temperature theta = max(p, p_floor)/(rho T_L).
  * stream: a cudaStream_t (NULL = default stream).
  * dalloc/dfree/alloc_ctx: optional device allocator (both or neither).
- * lanes_per_node: threads cooperating on one node in the step kernel, 8 or 16 (0 = 8).
- * tile_x: width of the step kernel's tile of 16 nodes, 1, 2, 4, 8 or 16 (tile height
- * 16 / tile_x; 0 = 16 for grids of fewer than 4 rows, else 4).  Both are performance
- * knobs (autotuning) of the D2Q9 kernel; results are the same to rounding.  The D2Q16
- * kernel (one thread per node) ignores them.
+ * lanes_per_node: work split of the D2Q9 step kernel: 8 = one thread per node (blocks of
+ * 128 nodes), 16 = nine lanes per node (blocks of 12 nodes, for small grids), 0 = by grid
+ * size.  tile_x: width of a block's tile of nodes, 1, 2, 4, 8 or 16 (its height is the
+ * block's nodes divided by it; with nine lanes per node 8 and 16 mean 6 and 12), 0 = by the
+ * grid's rows.  Both are performance knobs (autotuning); results are the same to rounding.
+ * The D2Q16 and D3Q27 kernels ignore them.
  * In the mixed form on D2Q16 the moments, e->T, EoS and frame-search residual are FP64;
  * the storage-rounding remainders of mass, momentum and energy are kept beside each
  * node as on D2Q9.
@@ -161,11 +162,11 @@ typedef struct {
     int64_t nonfinite;     /* node updates that produced NaN/Inf                */
     int64_t stalled;       /* mixed form: frame searches stopped at the FP32
                               rounding floor (residual no longer halving)      */
-    int64_t block_streams; /* streaming passes summed over kernel blocks (a block
-                              of 32 nodes streams until all its nodes stop)    */
-    int64_t max_streams;   /* largest streaming-pass count of any block        */
-    int64_t timeouts;      /* tiles skipped because a bounded wait for their
-                              staging copies ran out (reported as POND_ETIMEOUT) */
+    int64_t block_streams; /* D2Q9: streaming passes summed over warps (a warp
+                              streams until all its nodes stop)                */
+    int64_t max_streams;   /* largest streaming-pass count of any node         */
+    int64_t timeouts;      /* tiles skipped because a bounded device wait ran
+                              out (reported as POND_ETIMEOUT)                  */
     int64_t region_nodes;  /* stencil-region nodes carried into the arrival gauge,
                               summed over streams (the union of a node's 4x4
                               (4x4x4) departure stencils: 16..64 per stream on

@@ -1,14 +1,12 @@
 // pond.cu -- host side of libpond: the C ABI declared in include/pond.h.
 //
-// A context owns two state buffers of one 32-value record per node (ping-pong), a
-// 5-plane FP64 staging buffer
-// for host <-> device field copies, the block partials of the conservation sums and a
+// A context owns two state buffers of one 32-value record per node (ping-pong), a 6-plane
+// FP64 staging buffer for host <-> device field copies, the block partials of the conservation sums and a
 // small block of device counters.  Every call enqueues on the context stream; one time
 // step is one launch of the fused kernel k_pond_step (pond_step.cuh).
 #include "pond.h"
 
 #include <cuda_runtime.h>
-#include <cudaTypedefs.h>   // PFN_cuTensorMapEncodeTiled
 
 #include <algorithm>
 #include <cmath>
@@ -42,7 +40,7 @@ struct pond_ctx {
     DevStats *dstats = nullptr;
     cudaStream_t stream = nullptr;
     int64_t steps = 0;
-    int lanes = 8;                 // lanes per node of the step kernel (8 or 16)
+    int lanes = 8;                 // work split of the D2Q9 step: 8 = a thread, 16 = nine lanes per node
     bool initialised = false;
     pond_batch *batch = nullptr;   // batch that steps this context, if any
     int nonlocal = 0;              // 1: current-time non-local terms (two passes per step)
@@ -57,9 +55,6 @@ struct pond_ctx {
     // device counters already reported by a sync point's status (sticky flags: a
     // condition is reported once, by the first sync point after it occurred)
     unsigned long long rep_nonconv = 0, rep_clamped = 0, rep_timeouts = 0;
-    // D2Q9: tensor maps of the two state buffers for the TMA staging of interior tiles
-    CUtensorMap tmap[2];
-    int use_tma = 0;
 };
 
 namespace {
@@ -102,64 +97,25 @@ void dev_free(pond_ctx *c, void *p)
 
 inline unsigned blocks_for(size_t n, unsigned bs) { return (unsigned)((n + bs - 1) / bs); }
 
-// cuTensorMapEncodeTiled from the driver, looked up once (null if unavailable).
-PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder()
-{
-    static std::once_flag once;
-    static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
-    std::call_once(once, [] {
-        void *p = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) ==
-                cudaSuccess && q == cudaDriverEntryPointSuccess)
-            fn = (PFN_cuTensorMapEncodeTiled_v12000)p;
-        cudaGetLastError();
-    });
-    return fn;
-}
-
-// Tensor maps of a D2Q9 context's state buffers: the records as a 3-D tensor
-// [ny][nx][SL] of R, box = the staged slot values x the staged row pitch x the halo'd tile
-// height, so that a box lands in shared memory exactly as the step kernel's staged tile.
-// Leaves use_tma = 0 (every tile copied per chunk) if the maps cannot be made.
-void make_tensor_maps(pond_ctx *c)
-{
-    c->use_tma = 0;
-    PFN_cuTensorMapEncodeTiled_v12000 enc = tensor_map_encoder();
-    if (!enc || c->lattice != POND_D2Q9) return;
-    const bool f32 = c->opts.precision == POND_MIXED;
-    const int TS = f32 ? Slot<float>::stride : Slot<double>::stride;
-    const int PT = step_row_pitch(c->dp.tile_x, TS), HT = STEP_NB / c->dp.tile_x + 2 * HALO;
-    if (PT > c->grid.nx || HT > c->grid.ny) return;   // no interior tile
-    const cuuint64_t dims[3] = {(cuuint64_t)SL, (cuuint64_t)c->grid.nx, (cuuint64_t)c->grid.ny};
-    const cuuint64_t strides[2] = {(cuuint64_t)SL * c->esize, (cuuint64_t)SL * c->esize * c->grid.nx};
-    const cuuint32_t box[3] = {(cuuint32_t)TS, (cuuint32_t)PT, (cuuint32_t)HT};
-    const cuuint32_t estr[3] = {1, 1, 1};
-    for (int k = 0; k < 2; ++k)
-        if (enc(&c->tmap[k], f32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 3,
-                c->state[k], dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
-                CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-            return;
-    c->use_tma = 1;
-}
+// Largest grid (nodes) stepped with nine lanes per node.  One thread per node leaves most
+// of the GPU idle below about 150 blocks of 128 nodes and a step then costs one block's
+// serial time (mixed 21-25 us, FP64 390-450 us whatever the grid); nine lanes per node cut
+// that time but do more work in all.  Measured (us per step, thread / nine lanes), mixed:
+// 128 x 4 21.1 / 14.6, 64 x 64 23.8 / 18.0, 2048 x 4 22.8 / 26.8, 96 x 96 23.6 / 28.5; FP64:
+// 128 x 4 389 / 107, 64 x 64 449 / 232, 96 x 96 449 / 404, 128 x 128 449 / 661.
+size_t split_max_nodes(int precision) { return precision == POND_MIXED ? 4096 : 10000; }
 
 bool mixed(const pond_ctx *c) { return c->opts.precision == POND_MIXED; }
 
-// Tiles of 16 nodes of the D2Q9 step kernel over the grid.
-int step_tiles(const pond_ctx *c)
-{
-    const int ty = STEP_NB / c->dp.tile_x;
-    return c->dp.tiles_x * ((c->grid.ny + ty - 1) / ty);
-}
+// Tiles of the D2Q9 step kernel over the grid.
+int step_tiles(const pond_ctx *c) { return c->dp.tiles_x * ((c->grid.ny + c->dp.tile_y - 1) / c->dp.tile_y); }
 
-// Largest dynamic shared memory of a step block over the tile shapes, for lanes per node.
+bool split(const pond_ctx *c) { return c->lanes == 16; }
+
 template <typename R>
-size_t step_smem_max(int lanes)
+size_t step_smem(const pond_ctx *c)
 {
-    size_t m = 0;
-    for (int tx = 1; tx <= STEP_NB; tx *= 2)
-        m = std::max(m, step_smem_bytes(tx, Slot<R>::stride, (int)sizeof(R), lanes));
-    return m;
+    return step_smem_bytes(c->dp.tile_x, c->dp.tile_y, split(c), Slot<R>::stride, (int)sizeof(R));
 }
 
 // Lets the step kernels of type R use more than the default 48 KB of dynamic shared
@@ -167,18 +123,24 @@ size_t step_smem_max(int lanes)
 template <typename R>
 cudaError_t allow_step_smem()
 {
-    cudaError_t e = cudaFuncSetAttribute(k_pond_step<R, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)step_smem_max<R>(8));
+    size_t m = 0, ms = 0;
+    for (int tx = 1; tx <= STEP_NB; tx *= 2)
+        m = std::max(m, step_smem_bytes(tx, STEP_NB / tx, false, Slot<R>::stride, (int)sizeof(R)));
+    for (int tx = 1; tx <= SPLIT_NB; ++tx)
+        ms = std::max(ms, step_smem_bytes(tx, SPLIT_NB / tx, true, Slot<R>::stride, (int)sizeof(R)));
+    cudaError_t e = cudaFuncSetAttribute(k_pond_step<R, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)m);
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_pond_step<R, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)step_smem_max<R>(16));
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_pond_step_batch<R, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)step_smem_max<R>(8));
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_pond_step_batch<R, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)step_smem_max<R>(16));
+        e = cudaFuncSetAttribute(k_pond_step<R, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ms);
     return e;
+}
+
+// One launch of the D2Q9 step over `blocks` tiles (of `one`, or of a batch's work list).
+template <typename R>
+void launch_step_kernel(bool use_split, unsigned blocks, size_t smem, cudaStream_t s, const SimDesc<R> &one,
+                        const SimDesc<R> *descs, const int2 *work)
+{
+    if (use_split) k_pond_step<R, true><<<blocks, STEP_THREADS, smem, s>>>(one, descs, work);
+    else k_pond_step<R, false><<<blocks, STEP_THREADS, smem, s>>>(one, descs, work);
 }
 
 // D2Q16: the non-local terms of state `src` into nlbuf, then the node step in -> out.
@@ -251,20 +213,19 @@ pond_status launch_step(pond_ctx *c, cudaEvent_t *ev = nullptr)
     const R *in = (const R *)c->state[c->cur];
     R *out = (R *)c->state[1 - c->cur];
     const unsigned nb = (unsigned)step_tiles(c);
-    const size_t smem = step_smem_bytes(c->dp.tile_x, Slot<R>::stride, (int)sizeof(R), c->lanes);
-    const CUtensorMap &tm = c->tmap[c->cur];
+    const size_t smem = step_smem<R>(c);
     if (ev) cudaEventRecord(ev[0], c->stream);
     const R *nl = in;
     if (c->nonlocal) {
         // pass 1: the lagged step predicts rho, T at t (its counters kept apart); pass 2
         // redoes the step from the same state with the non-local terms of that prediction
         R *pred = (R *)c->pred;
-        if (c->lanes == 16) k_pond_step<R, 16><<<nb, STEP_NB * 16, smem, c->stream>>>(c->dp, in, pred, c->dstats_pred, in, tm, c->use_tma);
-        else k_pond_step<R, 8><<<nb, STEP_NB * 8, smem, c->stream>>>(c->dp, in, pred, c->dstats_pred, in, tm, c->use_tma);
+        const SimDesc<R> first{c->dp, in, pred, c->dstats_pred, in};
+        launch_step_kernel<R>(split(c), nb, smem, c->stream, first, nullptr, nullptr);
         nl = pred;
     }
-    if (c->lanes == 16) k_pond_step<R, 16><<<nb, STEP_NB * 16, smem, c->stream>>>(c->dp, in, out, c->dstats, nl, tm, c->use_tma);
-    else k_pond_step<R, 8><<<nb, STEP_NB * 8, smem, c->stream>>>(c->dp, in, out, c->dstats, nl, tm, c->use_tma);
+    const SimDesc<R> one{c->dp, in, out, c->dstats, nl};
+    launch_step_kernel<R>(split(c), nb, smem, c->stream, one, nullptr, nullptr);
     if (ev) cudaEventRecord(ev[1], c->stream);
     c->cur = 1 - c->cur;
     return POND_OK;
@@ -573,11 +534,21 @@ pond_status pond_create(const pond_grid *grid, const pond_lattice *lattice, cons
     c->N = (size_t)grid->nx * (size_t)grid->ny * (size_t)(grid->nz > 1 ? grid->nz : 1);
     if (c->lattice == POND_D3Q27) c->g3 = Grid3{grid->nz, grid->bc_z};
     c->esize = opts->precision == POND_MIXED ? sizeof(float) : sizeof(double);
-    // 8 lanes per node unless the caller picks 16 (measured faster on every grid tried so
-    // far; the choice is exposed for the autotuner).
-    c->lanes = opts->lanes_per_node ? opts->lanes_per_node : 8;
-    // tile of the step kernel: a 16 x 1 strip for grids of few rows, 4 x 4 otherwise
-    int tile_x = opts->tile_x ? opts->tile_x : (grid->ny < 4 ? 16 : 4);
+    // Work split of the D2Q9 step: one thread per node (8) or nine lanes per node (16).
+    c->lanes = opts->lanes_per_node ? opts->lanes_per_node : (c->N <= split_max_nodes(opts->precision) ? 16 : 8);
+    // Its tile: TX x TY nodes of STEP_NB (SPLIT_NB) nodes, by default no taller than the grid
+    // and otherwise 16 x 8 (4 x 3)
+    int tile_x = opts->tile_x, tile_y;
+    if (c->lanes == 16) {
+        if (!tile_x) tile_x = grid->ny == 1 ? 12 : (grid->ny == 2 || grid->ny == 4 ? 6 : 4);
+        else if (tile_x == 8) tile_x = 6;
+        else if (tile_x == 16) tile_x = 12;
+        tile_y = SPLIT_NB / tile_x;
+    } else {
+        if (!tile_x)
+            for (tile_x = 16; tile_x < STEP_NB && STEP_NB / (2 * tile_x) >= grid->ny; tile_x *= 2) {}
+        tile_y = STEP_NB / tile_x;
+    }
     cudaError_t e = cudaGetDevice(&c->device);
     if (e == cudaSuccess)
         e = opts->precision == POND_MIXED ? allow_step_smem<float>() : allow_step_smem<double>();
@@ -591,7 +562,7 @@ pond_status pond_create(const pond_grid *grid, const pond_lattice *lattice, cons
     d.a = c->eos.a; d.b = c->eos.b; d.R = c->eos.R; d.delta = c->eos.delta; d.cv = c->eos.R / c->eos.delta;
     d.kappa = kappa; d.tau = tau; d.omega = 1.0 / tau; d.dt = opts->dt; d.k_cond = opts->k_cond;
     d.p_floor = opts->p_floor; d.tol = opts->tol; d.max_iter = opts->max_iter;
-    d.tile_x = tile_x; d.tiles_x = (grid->nx + tile_x - 1) / tile_x;
+    d.tile_x = tile_x; d.tile_y = tile_y; d.tiles_x = (grid->nx + tile_x - 1) / tile_x;
     d.pd.a = d.a; d.pd.b = d.b; d.pd.R = d.R; d.pd.cv = d.cv; d.pd.inv_cv = 1.0 / d.cv;
     d.pd.kappa = d.kappa; d.pd.p_floor = d.p_floor; d.pd.dt = d.dt; d.pd.omega = d.omega;
     d.pd.mu_coef = (d.tau - 0.5) * d.dt; d.pd.cvR = d.cv + d.R; d.pd.k_cond = d.k_cond;
@@ -637,7 +608,6 @@ pond_status pond_create(const pond_grid *grid, const pond_lattice *lattice, cons
         pond_destroy(c);
         return POND_ECUDA;
     }
-    make_tensor_maps(c);
     *out = c;
     return POND_OK;
 }
@@ -894,14 +864,14 @@ pond_status pond_get_state(pond_ctx *c, double *state)
     for (int p = 0; p < NPL; ++p) {
         const int o = rec_off(p);
         for (size_t n = 0; n < N; ++n)
-            state[(size_t)p * N + n] = mixed(c) ? (double)f[n * SL + o] : d[n * SL + o];
+            state[(size_t)p * N + n] = mixed(c) ? (double)f[rec_at(f.data(), n, o, N)] : d[rec_at(d.data(), n, o, N)];
     }
     // the rest populations with their kept low parts (the momentum low parts, below one
     // ulp of the populations, are not part of the exchanged state)
     for (int k = 0; k < 2; ++k) {
         const int p = k == 0 ? P_F + 4 : P_G + 4, lo = k == 0 ? P_F4LO : P_G4LO;
         for (size_t n = 0; n < N; ++n)
-            state[(size_t)p * N + n] += mixed(c) ? (double)f[n * SL + lo] : d[n * SL + lo];
+            state[(size_t)p * N + n] += mixed(c) ? (double)f[rec_at(f.data(), n, lo, N)] : d[rec_at(d.data(), n, lo, N)];
     }
     return POND_OK;
 }
@@ -989,8 +959,8 @@ pond_status pond_set_state(pond_ctx *c, const double *state)
     for (int p = 0; p < NPL; ++p) {
         const int o = rec_off(p);
         for (size_t n = 0; n < N; ++n) {
-            if (mixed(c)) f[n * SL + o] = (float)state[(size_t)p * N + n];
-            else d[n * SL + o] = state[(size_t)p * N + n];
+            if (mixed(c)) f[rec_at(f.data(), n, o, N)] = (float)state[(size_t)p * N + n];
+            else d[rec_at(d.data(), n, o, N)] = state[(size_t)p * N + n];
         }
     }
     // FP32 form: the rest populations keep the part below their float as the low word
@@ -998,7 +968,7 @@ pond_status pond_set_state(pond_ctx *c, const double *state)
         for (int k = 0; k < 2; ++k) {
             const int p = k == 0 ? P_F + 4 : P_G + 4, lo = k == 0 ? P_F4LO : P_G4LO;
             for (size_t n = 0; n < N; ++n)
-                f[n * SL + lo] = (float)(state[(size_t)p * N + n] - (double)f[n * SL + p]);
+                f[rec_at(f.data(), n, lo, N)] = (float)(state[(size_t)p * N + n] - (double)f[rec_at(f.data(), n, p, N)]);
         }
     const void *src = mixed(c) ? (const void *)f.data() : (const void *)d.data();
     CK(cudaMemcpyAsync(c->state[c->cur], src, rec * c->esize, cudaMemcpyHostToDevice, c->stream),
@@ -1088,12 +1058,12 @@ cudaError_t build_group(pond_batch *b, pond_batch::Group &G)
     for (size_t k = 0; k < ns; ++k) {
         pond_ctx *c = G.sims[k];
         d0[k].p = c->dp; d0[k].in = (const R *)c->state[c->cur]; d0[k].out = (R *)c->state[1 - c->cur];
-        d0[k].stats = c->dstats;
+        d0[k].stats = c->dstats; d0[k].nlsrc = d0[k].in;
         d1[k] = d0[k]; d1[k].in = (const R *)c->state[1 - c->cur]; d1[k].out = (R *)c->state[c->cur];
-        const int ty = STEP_NB / c->dp.tile_x;
-        const int tiles = c->dp.tiles_x * ((c->grid.ny + ty - 1) / ty);
+        d1[k].nlsrc = d1[k].in;
+        const int tiles = step_tiles(c);
         for (int t = 0; t < tiles; ++t) work.push_back(make_int2((int)k, t));
-        G.smem = std::max(G.smem, step_smem_bytes(c->dp.tile_x, Slot<R>::stride, (int)sizeof(R), G.lanes));
+        G.smem = std::max(G.smem, step_smem<R>(c));
     }
     G.nwork = (int)work.size();
     cudaError_t e = cudaSuccess;
@@ -1125,10 +1095,7 @@ void launch_group(pond_batch *b, pond_batch::Group &G, int parity)
 {
     if (!G.nwork) return;
     const SimDesc<R> *d = (const SimDesc<R> *)G.desc[parity];
-    if (G.lanes == 16)
-        k_pond_step_batch<R, 16><<<G.nwork, STEP_NB * 16, G.smem, b->stream>>>(d, G.work);
-    else
-        k_pond_step_batch<R, 8><<<G.nwork, STEP_NB * 8, G.smem, b->stream>>>(d, G.work);
+    launch_step_kernel<R>(G.lanes == 16, (unsigned)G.nwork, G.smem, b->stream, SimDesc<R>{}, d, G.work);
 }
 
 template <typename R>

@@ -1,8 +1,9 @@
 // pond_kernels.cuh -- device code of the PonD van der Waals time step for sm_103a.
 //
-// Layout: a state buffer holds one record of SL = 32 values per node (node = y*nx + x),
-// 128 bytes in FP32 so that a node is one cache line and its 21 streamed values are read
-// with six 16-byte loads:
+// Layout: a state buffer holds one record of SL = 32 values per node (node = y*nx + x) in
+// 16-byte chunks (4 FP32 or 2 FP64 values), chunk c of all N nodes together (rec_at): one
+// thread per node then loads and stores whole 16-byte chunks on consecutive addresses.
+// The values of a record:
 //   [0..8] f_0..f_8, [9..17] g_0..g_8, [18] theta, [19] u_x, [20] u_y, [21] spare,
 //   [22] rho, [23] T, [24] uhat_x, [25] uhat_y, [26] f_4 lo, [27] g_4 lo, [28] j_x lo,
 //   [29] j_y lo, [30..31] unused
@@ -26,10 +27,17 @@ constexpr int NPL = 25;   // planes of the ABI state
 constexpr int SL = 32;    // values per node record on the device
 enum : int { P_F = 0, P_G = 9, P_TH = 18, P_UX = 19, P_UY = 20, P_SQ = 21, P_RHO = 22, P_T = 23,
              P_UHX = 24, P_UHY = 25, P_F4LO = 26, P_G4LO = 27, P_JXLO = 28, P_JYLO = 29 };
-// (P_SQ: sqrt(theta) in the staged copies)
+// (P_SQ: unused in the stored record; sqrt(theta) in a loaded copy)
 __host__ __device__ constexpr int rec_off(int plane) { return plane < 21 ? plane : plane + 1; }
-// value `off` of node n's record
-#define REC(buf, n, off) (buf)[(size_t)(n) * SL + (off)]
+// index of value `off` of node n's record in a state buffer of N nodes
+template <typename R>
+__host__ __device__ constexpr size_t rec_at(const R *, size_t n, int off, size_t N)
+{
+    constexpr int CW = 16 / (int)sizeof(R);
+    return ((size_t)(off / CW) * N + n) * CW + off % CW;
+}
+// value `off` of node n's record (in kernels whose parameters p hold the node count)
+#define REC(buf, n, off) (buf)[rec_at(buf, (size_t)(n), (off), (size_t)p.N)]
 
 // Model constants in the arithmetic type of a kernel (float copies keep FP64 work out of
 // the FP32 paths).
@@ -47,7 +55,7 @@ struct DevParams {
     double a, b, R, delta, cv;
     double kappa, tau, omega, dt, k_cond, p_floor, tol;
     int max_iter;
-    int tile_x, tiles_x;   // step kernel tile: tile_x by (16 / tile_x) nodes; tiles per row
+    int tile_x, tile_y, tiles_x;   // step kernel tile: tile_x by tile_y nodes; tiles per row
     TypedParams<float> pf;
     TypedParams<double> pd;
     // the FP32 form's frame-search EoS constants as (hi, lo) float pairs (hi + lo = the

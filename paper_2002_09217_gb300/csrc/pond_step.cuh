@@ -1,177 +1,89 @@
 // pond_step.cuh -- the fused time-step kernel of the PonD van der Waals model (sm_103a).
 //
-// One launch per time step.  A block owns NB = 16 nodes; each node is served by a group
-// of LPN = 8 or 16 lanes of one warp.  Per node:
-//   phase 0  non-local terms from the previous step's rho and T (radius 2): lane l of the
-//            group takes the l-th non-rest neighbour, builds the Korteweg stress K and the
-//            heat flux q there from the 8 differences around it, and the group sums
-//            W c . K and W c . q into F = -div K and M_0 = 2 div q (Eq. korteweg, Eq. gtilde).
-//   phase 1  frame search (block lockstep): the group streams all 9 directions x 16 stencil
-//            nodes (each lane 16/LPN stencil positions of every direction), keeps each
-//            lane's partial increments in shared memory and reduces only the four moment
-//            sums per stream; warp 0 (one lane per node) takes the moments, inverts
-//            e -> T, evaluates the EoS and the residual, in FP64 in the FP64 form and in
-//            float-float (pairs of FP32) in the mixed form.
+// One launch per time step, one thread per node, a block owns a tile of STEP_NB nodes
+// (tile_x columns).  Per block:
+//   staging  every record of the tile and a halo of HALO = 2 nodes is read once from
+//            global memory, its populations are carried into one gauge common to the tile
+//            (SM "Transfer matrix": G = M_lambda'^-1 M_lambda) and left in shared memory,
+//            one slot per unwrapped coordinate, so that periodic and zero-gradient
+//            boundaries need no special case.
+//   phase 0  non-local terms from the previous step's rho and T: the Korteweg stress K and
+//            the heat flux q once per node of the tile and its ring, then F = -div K and
+//            M_0 = 2 div q per node (Eq. korteweg, Eq. gtilde).
+//   phase 1  frame search: each thread streams its node's 18 populations, takes the
+//            moments, inverts e -> T, evaluates the EoS and the residual (FP64 in the FP64
+//            form, float-float in the mixed form) until its own gauge has converged.
 //   phase 2  BGK collision with the force source, heat-flux correction and forced g
-//            equilibrium, one population per lane; the rest population takes the exact
-//            remainder of mass and energy, and what storage rounding takes from the
-//            conserved sums is kept beside the record.
+//            equilibrium; the rest population takes the exact remainder of mass and
+//            energy, and what storage rounding takes from the conserved sums is kept
+//            beside the record.
 //
-// Staging.  Each block owns a tile of tile_x x (16 / tile_x) nodes and first copies the
-// records of the tile plus a halo of HALO = 3 nodes (their first 24 values) into shared
-// memory with 16-byte cp.async copies, one record slot per unwrapped coordinate, so that
-// periodic and zero-gradient boundaries need no special case.  All stencil reads of the
-// step come from there; a departure point farther than the halo (|v| dt >= 1) falls back
-// to a global load.
+// Streaming as one contraction.  The transfer map is linear, composes exactly
+// (G_(n->lambda) = G_(b->lambda) G_(n->b)) and is a product over the axes, and so are the
+// cubic Lagrange weights of a departure point.  With the stencil nodes already in the
+// tile's common gauge b, the streamed population of direction (k, l) is
+//   f~_(k,l) = sum_cy sum_n (wy[l][cy] Ly[l][n]) sum_cx sum_m (wx[k][cx] Lx[k][m]) f^b_(m,n)(cx, cy)
+// (L = row of G_(b->lambda) along one axis, w = Lagrange weights): an x pass of 5 rows x 3 n
+// x 3 k and a y pass, about 650 multiply-adds a population family, where carrying each of
+// the 25 stencil nodes into the arrival gauge and spreading it over nine directions took
+// about 2,700.  The tile is 128 nodes because the halo's share of the staging falls with its
+// size (1.9 staged nodes a node; 6.3 with 4 x 4 nodes and a halo of 3).
+// Measured (five steps of the 2048 x 1024 shock-droplet interaction with init and read-out,
+// mixed): 17.70 -> 4.50 ms; two FP64 steps of a 509 x 387 droplet 22.66 -> 5.27 ms.  Bound
+// by instruction issue (60 % active; FMA pipe 49 %, shared-memory pipe 41 %) in the mixed
+// form and by the FP64 pipe in the FP64 form; DRAM 6 % busy.
 //
-// Increment form.  With f~_i = sum_n A_n [G_n f(n)]_i and sum_n A_n = 1,
-//   f~_i = f_i(x) + sum_n A_n ( [G_n (f(n) - f(x))]_i + [(G_n - I) f(x)]_i ),
-// where G_n is the transfer map from the gauge of stencil node n into the arrival gauge
-// (SM "Transfer matrix", separable per axis) and (G_n - I) is evaluated from the gauge
-// differences directly, so equal gauges give exactly the identity and a uniform region
-// reproduces itself exactly.  The FP32 rounding error of a step is then proportional to
-// the local differences, not to the populations, and does not accumulate as a bias.
+// FP32 accuracy.  The slots hold differences f^b - (populations of the tile's base node),
+// computed in increment form (the map as I + E with E = 0 for equal gauges), and the
+// stream accumulates differences to the node's own slot, so that equal gauges and
+// populations give exactly zero, and rounding is proportional to local differences and
+// not to the populations, and does not accumulate as a bias.  The base is the staged node
+// of the largest theta: across an interface rho theta (the second moment) varies little,
+// so that in the hottest gauge only the rest population differs much between the phases,
+// and carrying it into a colder gauge does not amplify its rounding.
+// In FP64 the slots hold the moments about the velocity of one node of the tile.
 #pragma once
-
-#include <cuda.h>   // CUtensorMap (the tensor-map type of the TMA tile copies)
 
 #include "pond_kernels.cuh"
 
 namespace pond {
 
-constexpr int STEP_NB = 16;   // nodes per block (lanes per node LPN = 8 or 16 is a template
-                              // parameter: more lanes per node for grids too small to fill
-                              // the GPU with 8); 16 nodes per block keep small grids spread
-                              // evenly over the 152 SMs
-constexpr unsigned STEP_NB_MASK = STEP_NB == 32 ? 0xffffffffu : ((1u << STEP_NB) - 1u);
-constexpr int HALO = 3;       // staged halo width (stencil reach for |v| dt < 1)
+constexpr int STEP_THREADS = 128;   // threads per block
+constexpr int STEP_NB = 128;        // nodes per block, one thread per node
+constexpr int SPLIT_NB = 12;        // nodes per block, nine lanes per node (three nodes per warp)
+constexpr int HALO = 2;       // staged halo: stencil reach for |v| dt < 1, and of the non-local terms
 // Largest side of a node's stencil region (the union of its 9 directions' 4x4 stencils)
-// that the region stream handles: 4 + the spread of the departure points' floors, 5 for
-// |v| dt < 1; wider regions take the per-pair stream.
+// that the general stream handles as a region; wider ones take the per-pair stream.
 constexpr int REGION_MAX = 8;
 // Mixed form: a frame-search residual below this multiple of tol that no longer halves is
 // taken as the FP32 rounding floor (the EoS cancels up to ~200x inside interfaces).
 constexpr float STALL_TOL_FACTOR = 16.0f;
-// resident blocks per SM the register budget is sized for: in FP32 five blocks of 128
-// threads (8 lanes per node, about 96 registers) or two of 256 (16 lanes); in FP64 three
-// of 128 (168 registers, 2 % faster than two of 198) or one of 256, so that its wider
-// values stay in registers
-#define STEP_MIN_BLOCKS(R, LPN) (sizeof(R) == 8 ? ((LPN) == 8 ? 3 : 1) : ((LPN) == 8 ? 5 : 2))
+// resident blocks per SM the register budget is sized for
+#define STEP_MIN_BLOCKS(R) (sizeof(R) == 8 ? 2 : 3)
+#define SPLIT_MIN_BLOCKS(R) (sizeof(R) == 8 ? 2 : 3)
 
-// Shared-memory record slot: the first 24 values of a node record (f, g, theta, u, pad,
-// rho, T), padded to a 16-byte multiple that spreads consecutive slots over the banks.
-// slot words past the 24 staged values: p and p/rho of the staged node (shared memory only)
-constexpr int S_PR = 24, S_PRR = 25;
+// Values per staged slot: the 18 carried populations, padded so that slots start on
+// distinct banks (FP32: 16-byte loads, 20 words; FP64: 19 values).
 template <typename R> struct Slot;
-template <> struct Slot<float> { static constexpr int stride = 28, chunks = 6; };
-template <> struct Slot<double> { static constexpr int stride = 26, chunks = 12; };
+template <> struct Slot<float> { static constexpr int stride = 20; };
+template <> struct Slot<double> { static constexpr int stride = 19; };
+constexpr int AUXW = 4;   // rho, T, p, p/rho of a staged node
+constexpr int SPLIT_WORDS = SL + 9 * 18;   // nine lanes per node: the own record, the lanes' partials
+constexpr int KQW = 5;    // K_xx, K_xy, K_yy, q_x, q_y of a node of the tile and its ring
 
-// Slots per staged row: the tile width plus halos, rounded up (FP32 slots of 28 words) to
-// 4 mod 8 so that vertically adjacent slots start 16 banks apart and the two stencil rows
-// a lane group reads fall on disjoint banks.
-__host__ __device__ constexpr int step_row_pitch(int tile_x, int slot_words)
+__host__ __device__ constexpr int step_slots(int tx, int ty) { return (tx + 2 * HALO) * (ty + 2 * HALO); }
+
+// Dynamic shared memory of one step block: slots' rho, T, p, p/rho; populations; K and q;
+// with nine lanes per node also the partials of the general stream and the own records.
+__host__ __device__ constexpr size_t step_smem_bytes(int tx, int ty, bool split, int slot_values, int elem_bytes)
 {
-    return slot_words == 28 ? ((tile_x + 2 * HALO + 3) / 8) * 8 + 4 : tile_x + 2 * HALO;
+    return ((size_t)step_slots(tx, ty) * (AUXW + slot_values) + (size_t)(tx + 2) * (ty + 2) * KQW +
+            (split ? (size_t)SPLIT_NB * SPLIT_WORDS : 0)) * elem_bytes;
 }
 
-// Slots of the step kernel's staged tile (tile_x columns).
-__host__ __device__ constexpr int step_tile_slots(int tile_x, int slot_words)
-{
-    return step_row_pitch(tile_x, slot_words) * (STEP_NB / tile_x + 2 * HALO);
-}
-
-// Per-lane partial increments of the 18 streamed populations of every node, behind the
-// staged tile: node j's row d (0..8 f, 9..17 g) holds its lanes' partials at
-// [j * step_part_stride(LPN) + d * LPN + lane]; the extra LPN per node offsets
-// neighbouring groups of a warp onto other banks.
-__host__ __device__ constexpr int step_part_stride(int lpn) { return 19 * lpn; }
-
-// Dynamic shared memory of one step block: staged tile + halo, then the partials.
-__host__ __device__ constexpr size_t step_smem_bytes(int tile_x, int slot_words, int elem_bytes, int lpn)
-{
-    return ((size_t)step_tile_slots(tile_x, slot_words) * slot_words +
-            (size_t)STEP_NB * step_part_stride(lpn)) * elem_bytes;
-}
-
-__device__ __forceinline__ void cp_async16(void *smem, const void *gmem)
-{
-    const unsigned s = (unsigned)__cvta_generic_to_shared(smem);
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(s), "l"(gmem) : "memory");
-}
-__device__ __forceinline__ void cp_async_wait_all()
-{
-    asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;\n" ::: "memory");
-}
-
-// ---- TMA tile copies (cp.async.bulk.tensor) completed on an mbarrier ----------------
-__device__ __forceinline__ unsigned smem_u32(const void *p) { return (unsigned)__cvta_generic_to_shared(p); }
-
-__device__ __forceinline__ void mbar_init(unsigned long long *bar, unsigned count)
-{
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(smem_u32(bar)), "r"(count) : "memory");
-    // make the initialised barrier visible to the async (TMA) proxy
-    asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-}
-
-// One arrival that also expects `bytes` of asynchronous copies on the barrier.
-__device__ __forceinline__ void mbar_arrive_expect_tx(unsigned long long *bar, unsigned bytes)
-{
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(smem_u32(bar)), "r"(bytes)
-                 : "memory");
-}
-
-// Copy the box at coordinates (c0, c1, c2) of a 3-D tensor map into shared memory dst
-// (the box lands densely, innermost dimension first), completing on bar.
-__device__ __forceinline__ void tma_load_3d(void *dst, const CUtensorMap *map, int c0, int c1, int c2,
-                                            unsigned long long *bar)
-{
-    asm volatile(
-        "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
-        " [%0], [%1, {%2, %3, %4}], [%5];\n" ::"r"(smem_u32(dst)),
-        "l"(reinterpret_cast<unsigned long long>(map)), "r"(c0), "r"(c1), "r"(c2), "r"(smem_u32(bar))
-        : "memory");
-}
-
-// Wait for phase `parity` of bar to complete, for at most limit_ns nanoseconds of the
-// global timer; returns false if the limit ran out (the caller then gives up the tile
-// instead of hanging).
-__device__ __forceinline__ bool mbar_wait_bounded(unsigned long long *bar, unsigned parity,
-                                                  unsigned long long limit_ns)
-{
-    unsigned long long t0;
-    asm volatile("mov.u64 %0, %%globaltimer;\n" : "=l"(t0));
-    for (;;) {
-        unsigned done;
-        asm volatile(
-            "{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}\n"
-            : "=r"(done) : "r"(smem_u32(bar)), "r"(parity) : "memory");
-        if (done) return true;
-        unsigned long long t;
-        asm volatile("mov.u64 %0, %%globaltimer;\n" : "=l"(t));
-        if (t - t0 > limit_ns) return false;
-    }
-}
-constexpr unsigned long long TMA_WAIT_LIMIT_NS = 1000000000ull;   // one second
-
-template <typename R>
-struct StepShared {
-    R dsum[STEP_NB][4];        // sum dF, sum dF cx, sum dF cy, sum dG of the current stream
-    R lam[STEP_NB][3];         // current arrival gauge (theta, ux, uy)
-    R nl[STEP_NB][3];          // lagged F_x, F_y, rho E_lambda of the node
-    R mac[STEP_NB][10];        // rho, u*x, u*y, uhx, uhy, E, T, P, theta*, p
-    R dlam[STEP_NB][3];        // theta* - theta, u*x - ux, u*y - uy (from FP64)
-    R hilo[STEP_NB][4];        // rho and sum g~ as (hi, lo) pairs of R
-    R mom[STEP_NB][4];         // sum f~ c_x, sum f~ c_y (gauge units) as (hi, lo) pairs
-    R bhi[STEP_NB][4];         // sums of the node's stored f, f cx, f cy, g, error-free as
-    R blo[STEP_NB][4];         //   unevaluated (hi, lo) pairs of R
-    // Lagrange weights of the current stream per axis and region column (row) c, one per
-    // direction of that axis: wt[j][axis][c][k] = a_(c - o_k)(xi_k), zero outside the
-    // 4-node stencil of direction k (o_k its offset in the node's region)
-    R wt[STEP_NB][2][REGION_MAX][4];
-    int active[STEP_NB];
-    int any_active;
-    int nreg[STEP_NB];         // region nodes streamed by node j (summed over its streams)
-    int npair[STEP_NB];        // streams of node j that took the per-pair path
+// Counters of one block, summed into the context's by its last instructions.
+struct StepCounts {
+    unsigned streams, region_nodes, pair_streams, nonconv, stalled, clamped, nonfinite, warp_streams, max_streams;
 };
 
 // 1-D transfer-map increment E = l_k(c_a + e) - l_k(c_a) for target index k (c = k-1),
@@ -341,45 +253,48 @@ __device__ __forceinline__ ffv ff_rcp(ffv a)
     return ff_norm(r, r * res);
 }
 
-// The 21 streamed values of node nd's record (f[9], g[9], theta, u_x, u_y, plus rho and T
-// in [22..23]) with 16-byte loads through the read-only path.
-__device__ __forceinline__ void load_rec24(const float *__restrict__ b, float v[24])
+// Values 0..23 of node nd's record (f[9], g[9], theta, u_x, u_y, spare, rho, T).
+__device__ __forceinline__ void load_rec24(const float *__restrict__ b, size_t nd, size_t N, float v[24])
 {
-    const float4 *q = reinterpret_cast<const float4 *>(b);
+    const float4 *q = reinterpret_cast<const float4 *>(b) + nd;
 #pragma unroll
     for (int k = 0; k < 6; ++k) {
-        const float4 t = __ldg(q + k);
+        const float4 t = __ldg(q + k * N);
         v[4 * k] = t.x; v[4 * k + 1] = t.y; v[4 * k + 2] = t.z; v[4 * k + 3] = t.w;
     }
 }
-__device__ __forceinline__ void load_rec24(const double *__restrict__ b, double v[24])
+__device__ __forceinline__ void load_rec24(const double *__restrict__ b, size_t nd, size_t N, double v[24])
 {
-    const double2 *q = reinterpret_cast<const double2 *>(b);
+    const double2 *q = reinterpret_cast<const double2 *>(b) + nd;
 #pragma unroll
     for (int k = 0; k < 12; ++k) {
-        const double2 t = __ldg(q + k);
+        const double2 t = __ldg(q + k * N);
         v[2 * k] = t.x; v[2 * k + 1] = t.y;
     }
 }
-
-// The same 24 values from a shared-memory slot.
-__device__ __forceinline__ void load_slot24(const float *sl, float v[24])
+// Writes a whole record.
+__device__ __forceinline__ void store_rec(float *b, size_t nd, size_t N, const float (&v)[SL])
 {
-    const float4 *q = reinterpret_cast<const float4 *>(sl);
+    float4 *q = reinterpret_cast<float4 *>(b) + nd;
 #pragma unroll
-    for (int k = 0; k < 6; ++k) {
-        const float4 t = q[k];
-        v[4 * k] = t.x; v[4 * k + 1] = t.y; v[4 * k + 2] = t.z; v[4 * k + 3] = t.w;
-    }
+    for (int k = 0; k < SL / 4; ++k) q[k * N] = make_float4(v[4 * k], v[4 * k + 1], v[4 * k + 2], v[4 * k + 3]);
 }
-__device__ __forceinline__ void load_slot24(const double *sl, double v[24])
+__device__ __forceinline__ void store_rec(double *b, size_t nd, size_t N, const double (&v)[SL])
 {
-    const double2 *q = reinterpret_cast<const double2 *>(sl);
+    double2 *q = reinterpret_cast<double2 *>(b) + nd;
 #pragma unroll
-    for (int k = 0; k < 12; ++k) {
-        const double2 t = q[k];
-        v[2 * k] = t.x; v[2 * k + 1] = t.y;
-    }
+    for (int k = 0; k < SL / 2; ++k) q[k * N] = make_double2(v[2 * k], v[2 * k + 1]);
+}
+// Four staged values from a 16-byte boundary.
+__device__ __forceinline__ void lds4(const float *s, float (&o)[4])
+{
+    const float4 t = *reinterpret_cast<const float4 *>(s);
+    o[0] = t.x; o[1] = t.y; o[2] = t.z; o[3] = t.w;
+}
+__device__ __forceinline__ void lds4(const double *s, double (&o)[4])
+{
+    const double2 a = reinterpret_cast<const double2 *>(s)[0], b = reinterpret_cast<const double2 *>(s)[1];
+    o[0] = a.x; o[1] = a.y; o[2] = b.x; o[3] = b.y;
 }
 
 // Contribution of stencil node `nd` to direction (jx, jy) of the arrival node, in the
@@ -587,534 +502,1175 @@ __device__ __forceinline__ void eos_update(const DevParams &p, const float *bhi,
     o.dth = (ths.hi - lam[0]) + ths.lo;
     o.dux = dux.hi; o.duy = duy.hi;
 }
-
-// Issue (without waiting) the 16-byte cp.async copies of tile `tile_idx` and its halo of
-// HALO nodes (the first 24 values of each record) into the staged tile `tile`, one slot per
-// unwrapped coordinate (periodic wrap or zero-gradient clamp applied to the source), and
-// commit them as one group.
+// Transfer increments along one axis, E[k][a] = l_k((a - 1) + e_a) - delta_ka with
+// e_a = q (a - 1) + w (q = (s_src - s)/s, w = (u_src - u)/s), from h = e/2 and
+// p = h (2 c_a + e): E_0 = p - h, E_1 = -2 p, E_2 = p + h.
 template <typename R>
-__device__ __forceinline__ void stage_issue(const DevParams &p, const R *__restrict__ in, R *tile, int tile_idx)
+__device__ __forceinline__ void axis_map(R q, R w, R (&E)[3][3])
 {
-    constexpr int TS = Slot<R>::stride, CH = Slot<R>::chunks;
-    const int TX = p.tile_x, TY = STEP_NB / TX;
-    const int X0 = (tile_idx % p.tiles_x) * TX, Y0 = (tile_idx / p.tiles_x) * TY;
-    const int WT = TX + 2 * HALO, HT = TY + 2 * HALO;
-    const int PT = step_row_pitch(TX, TS);
-    const int total = WT * HT * CH;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        const R e = q * R(a - 1) + w;
+        const R h = R(0.5) * e, pp = h * (R(2 * (a - 1)) + e);
+        E[0][a] = pp - h; E[1][a] = R(-2) * pp; E[2][a] = pp + h;
+    }
+}
+
+// Increment of a separable map on nine values h (i = 3 b + a): [(I + Ey)(I + Ex) h]_i - h_i.
+template <typename R>
+__device__ __forceinline__ void map_inc(const R (&Ex)[3][3], const R (&Ey)[3][3], const R *h, R (&out)[9])
+{
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        R t[3], u[3];
+#pragma unroll
+        for (int b = 0; b < 3; ++b) {
+            t[b] = Ex[k][0] * h[3 * b] + Ex[k][1] * h[3 * b + 1] + Ex[k][2] * h[3 * b + 2];
+            u[b] = h[3 * b + k] + t[b];
+        }
+#pragma unroll
+        for (int l = 0; l < 3; ++l) out[3 * l + k] = t[l] + (Ey[l][0] * u[0] + Ey[l][1] * u[1] + Ey[l][2] * u[2]);
+    }
+}
+
+// Moments about (ux, uy) of nine populations at velocities s c + u_n along each axis
+// (wx, wy = u_n - u): M_mn at 3 n + m, m, n <= 2.
+__device__ __forceinline__ void moments9(const double *f, double s, double wx, double wy, double (&M)[9])
+{
+    const double s2 = s * s;
+    double r[9];
+#pragma unroll
+    for (int b = 0; b < 3; ++b) {
+        const double sum = f[3 * b] + f[3 * b + 2];
+        const double m0 = sum + f[3 * b + 1], A = s * (f[3 * b + 2] - f[3 * b]);
+        const double m1 = A + wx * m0;
+        r[3 * b] = m0; r[3 * b + 1] = m1; r[3 * b + 2] = s2 * sum + wx * (A + m1);
+    }
+#pragma unroll
+    for (int m = 0; m < 3; ++m) {
+        const double sum = r[m] + r[6 + m];
+        const double m0 = sum + r[3 + m], A = s * (r[6 + m] - r[m]);
+        const double m1 = A + wy * m0;
+        M[m] = m0; M[3 + m] = m1; M[6 + m] = s2 * sum + wy * (A + m1);
+    }
+}
+
+// Rows of the map from moments about u - t to populations of the gauge (s, u).
+__device__ __forceinline__ void moment_rows(double t, double inv_s, double (&L)[3][3])
+{
+    const double i2 = inv_s * inv_s, h2 = 0.5 * i2, ts = t * inv_s;
+    L[0][0] = 0.5 * ts * (ts + 1.0); L[0][1] = -(0.5 * inv_s + t * i2); L[0][2] = h2;
+    L[1][0] = 1.0 - ts * ts; L[1][1] = 2.0 * t * i2; L[1][2] = -i2;
+    L[2][0] = 0.5 * ts * (ts - 1.0); L[2][1] = 0.5 * inv_s - t * i2; L[2][2] = h2;
+}
+
+// Departure points of the three directions of an axis, x - (s (j - 1) + u) dt: their floors
+// and the cubic Lagrange weights of the four stencil nodes.  True when every floor is -1 or
+// 0 (|v| dt < 1 in general), so that the stencils lie within two nodes of the arrival node;
+// false also for NaN.
+template <typename R>
+__device__ __forceinline__ bool axis_weights(R s, R u, R dt, R (&a)[3][4], bool (&near0)[3])
+{
+    bool ok = true;
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+        const R d = -(s * R(j - 1) + u) * dt;
+        const R f = floor(d);
+        near0[j] = f == R(0);
+        ok = ok && (f == R(0) || f == R(-1));
+        const R t0 = d - f + R(1), t1 = t0 - R(1), t2 = t0 - R(2), t3 = t0 - R(3);
+        const R p12 = t1 * t2, p03 = t0 * t3;
+        a[j][0] = p12 * t3 * R(-1.0 / 6.0);
+        a[j][1] = p03 * t2 * R(0.5);
+        a[j][2] = p03 * t1 * R(-0.5);
+        a[j][3] = p12 * t0 * R(1.0 / 6.0);
+    }
+    return ok;
+}
+
+// General stream of node (X, Y) into the gauge (th, ux, uy), for departure points farther
+// than the staged halo (|v| dt >= 1) and non-finite gauges: reads the stencil nodes'
+// records from global memory.  Offsets are clamped to +-2^20 nodes first (a NaN offset
+// goes to the bound), so that the floors and their spread stay in int range.  Regions of
+// up to REGION_MAX nodes a side carry each node once for all nine directions; wider ones
+// take each direction's 16 stencil nodes in turn.  inc = the increments of the streamed
+// populations over the node's own (f, then g); of `lanes` callers, caller `lane` adds
+// every lanes-th stencil node only.
+template <typename R>
+__device__ __noinline__ void stream_general(const DevParams &p, const R *__restrict__ in, int X, int Y, R th, R ux,
+                                            R uy, bool first, int lane, int lanes, R *inc, unsigned &nreg,
+                                            unsigned &npair)
+{
+    const size_t N = (size_t)p.N;
+    const R dt = typed<R>(p).dt;
+    const R s = sqrt_(th), inv_s = R(1) / s;
+    R own[24];
+    load_rec24(in, (size_t)Y * p.nx + X, N, own);
+    int fl[2][3];
+    R xi[2][3];
+#pragma unroll
+    for (int ax = 0; ax < 2; ++ax)
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            const R d = clamp_offset(-(s * R(j - 1) + (ax == 0 ? ux : uy)) * dt);
+            const R f = floor(d);
+            fl[ax][j] = (int)f;
+            xi[ax][j] = d - f + R(1);
+        }
+    const int lo_x = min(fl[0][0], min(fl[0][1], fl[0][2])), lo_y = min(fl[1][0], min(fl[1][1], fl[1][2]));
+    const int ncols = 4 + max(fl[0][0], max(fl[0][1], fl[0][2])) - lo_x;
+    const int nrows = 4 + max(fl[1][0], max(fl[1][1], fl[1][2])) - lo_y;
+    R accf[9], accg[9];
+#pragma unroll
+    for (int i = 0; i < 9; ++i) accf[i] = accg[i] = R(0);
+    if (ncols <= REGION_MAX && nrows <= REGION_MAX) {
+        // in a first stream the node's own entry is carried by the identity: it is skipped
+        const bool skip = first && lo_x <= 1 && 1 - lo_x < ncols && lo_y <= 1 && 1 - lo_y < nrows;
+        const int own_r = skip ? (1 - lo_y) * ncols + (1 - lo_x) : -1;
+        nreg += (unsigned)(ncols * nrows - (skip ? 1 : 0));
+#pragma unroll 1
+        for (int r = lane; r < ncols * nrows; r += lanes) {
+            if (r == own_r) continue;
+            const int cy = r / ncols, cx = r - cy * ncols;
+            R wx[3], wy[3], v[24];
+#pragma unroll
+            for (int j = 0; j < 3; ++j) {
+                const int kx = cx - (fl[0][j] - lo_x), ky = cy - (fl[1][j] - lo_y);
+                wx[j] = (kx >= 0 && kx < 4) ? lag1_rt<R>(kx, xi[0][j]) : R(0);
+                wy[j] = (ky >= 0 && ky < 4) ? lag1_rt<R>(ky, xi[1][j]) : R(0);
+            }
+            load_rec24(in, (size_t)bc_wrap(Y + lo_y - 1 + cy, p.ny, p.bcy) * p.nx +
+                               bc_wrap(X + lo_x - 1 + cx, p.nx, p.bcx), N, v);
+            const R sn = sqrt_(v[P_TH]);
+            const R q = sizeof(R) == 8 ? sn * inv_s - R(1) : fdiv_(v[P_TH] - th, (sn + s) * s);
+            R Ex[3][3], Ey[3][3];
+            axis_map<R>(q, (v[P_UX] - ux) * inv_s, Ex);
+            axis_map<R>(q, (v[P_UY] - uy) * inv_s, Ey);
+            region_family<R>(v + P_F, own + P_F, Ex, Ey, wx, wy, accf);
+            region_family<R>(v + P_G, own + P_G, Ex, Ey, wx, wy, accg);
+        }
+    } else {
+        npair += 1;
+#pragma unroll
+        for (int jy = 0; jy < 3; ++jy)
+#pragma unroll
+            for (int jx = 0; jx < 3; ++jx) {
+                const int i = 3 * jy + jx;
+#pragma unroll 1
+                for (int q = lane; q < 16; q += lanes) {
+                    const int kx = q & 3, ky = q >> 2;
+                    const size_t nd = (size_t)bc_wrap(Y + fl[1][jy] - 1 + ky, p.ny, p.bcy) * p.nx +
+                                      bc_wrap(X + fl[0][jx] - 1 + kx, p.nx, p.bcx);
+                    R v[24], tf, tg;
+                    load_rec24(in, nd, N, v);
+                    v[P_SQ] = sqrt_(v[P_TH]);
+                    pair_inc<R>(v, jx, jy, th, s, inv_s, ux, uy, own[P_F + i], own[P_G + i], tf, tg);
+                    const R w = lag1_rt<R>(kx, xi[0][jx]) * lag1_rt<R>(ky, xi[1][jy]);
+                    accf[i] += w * tf;
+                    accg[i] += w * tg;
+                }
+            }
+    }
+#pragma unroll
+    for (int i = 0; i < 9; ++i) {
+        inc[i] = accf[i];
+        inc[9 + i] = accg[i];
+    }
+}
+
+// The stream as a contraction over the staged slots (see the head of this file), FP32:
+// own = the node's own slot, pitch = slots per staged row.  Five columns and rows with
+// zero weights outside a direction's four nodes, so that every offset is a constant.
+// acc = increments over the node's own populations (f, then g).
+__device__ __forceinline__ void contract(const float *own, int pitch, const float (&ax)[3][4],
+                                         const bool (&nx0)[3], const float (&ay)[3][4], const bool (&ny0)[3],
+                                         const float (&Lx)[3][3], const float (&Ly)[3][3], float (&acc)[2][9])
+{
+    constexpr int DS = Slot<float>::stride;
+    float wl[3][5][3], wy[3][5], dx[DS];
+#pragma unroll
+    for (int k = 0; k < 3; ++k)
+#pragma unroll
+        for (int c = 0; c < 5; ++c) {
+            const float w = nx0[k] ? (c == 0 ? 0.0f : ax[k][c - 1 < 0 ? 0 : c - 1]) : (c == 4 ? 0.0f : ax[k][c > 3 ? 3 : c]);
+            wy[k][c] = ny0[k] ? (c == 0 ? 0.0f : ay[k][c - 1 < 0 ? 0 : c - 1]) : (c == 4 ? 0.0f : ay[k][c > 3 ? 3 : c]);
+#pragma unroll
+            for (int m = 0; m < 3; ++m) wl[k][c][m] = w * Lx[k][m];
+        }
+#pragma unroll
+    for (int q = 0; q < DS / 4; ++q) {
+        float t[4];
+        lds4(own + 4 * q, t);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) dx[4 * q + e] = t[e];
+    }
+#pragma unroll
+    for (int fam = 0; fam < 2; ++fam)
+#pragma unroll
+        for (int i = 0; i < 9; ++i) acc[fam][i] = 0.0f;
+    const float *row = own - (2 * pitch + 2) * DS;
+#pragma unroll 1
+    for (int cy = 0; cy < 5; ++cy, row += pitch * DS) {
+        float t[2][3][3];   // family, n, k
+#pragma unroll
+        for (int fam = 0; fam < 2; ++fam)
+#pragma unroll
+            for (int n = 0; n < 3; ++n)
+#pragma unroll
+                for (int k = 0; k < 3; ++k) t[fam][n][k] = 0.0f;
+#pragma unroll
+        for (int cx = 0; cx < 5; ++cx) {
+            float v[DS];
+#pragma unroll
+            for (int q = 0; q < DS / 4; ++q) {
+                float x[4];
+                lds4(row + cx * DS + 4 * q, x);
+#pragma unroll
+                for (int e = 0; e < 4; ++e) v[4 * q + e] = x[e] - dx[4 * q + e];
+            }
+#pragma unroll
+            for (int fam = 0; fam < 2; ++fam)
+#pragma unroll
+                for (int n = 0; n < 3; ++n)
+#pragma unroll
+                    for (int m = 0; m < 3; ++m)
+#pragma unroll
+                        for (int k = 0; k < 3; ++k)
+                            t[fam][n][k] = fmaf(wl[k][cx][m], v[9 * fam + 3 * n + m], t[fam][n][k]);
+        }
+#pragma unroll
+        for (int l = 0; l < 3; ++l) {
+            const float w = wy[l][0];
+#pragma unroll
+            for (int c = 0; c < 4; ++c) wy[l][c] = wy[l][c + 1];   // the next row's weight moves to the front
+#pragma unroll
+            for (int n = 0; n < 3; ++n) {
+                const float wn = w * Ly[l][n];
+#pragma unroll
+                for (int fam = 0; fam < 2; ++fam)
+#pragma unroll
+                    for (int k = 0; k < 3; ++k) acc[fam][3 * l + k] = fmaf(wn, t[fam][n][k], acc[fam][3 * l + k]);
+            }
+        }
+    }
+}
+
+// The same over the FP64 slots (moments): the x pass reads each direction's own four
+// columns (shared-memory reads are cheap beside the FP64 pipe, which runs at 1/64 of the
+// FP32 rate), and a row pass costs 36 multiply-adds instead of 45.  acc = the streamed
+// populations.
+__device__ __forceinline__ void contract(const double *own, int pitch, const double (&ax)[3][4],
+                                         const bool (&nx0)[3], const double (&ay)[3][4], const bool (&ny0)[3],
+                                         const double (&Lx)[3][3], const double (&Ly)[3][3], double (&acc)[2][9])
+{
+    constexpr int DS = Slot<double>::stride;
+    double wl[3][4][3], wy[3][5];
+    int off[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        off[k] = nx0[k] ? DS : 0;
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+#pragma unroll
+            for (int m = 0; m < 3; ++m) wl[k][c][m] = ax[k][c] * Lx[k][m];
+#pragma unroll
+        for (int c = 0; c < 5; ++c)
+            wy[k][c] = ny0[k] ? (c == 0 ? 0.0 : ay[k][c - 1 < 0 ? 0 : c - 1]) : (c == 4 ? 0.0 : ay[k][c > 3 ? 3 : c]);
+    }
+#pragma unroll
+    for (int fam = 0; fam < 2; ++fam)
+#pragma unroll
+        for (int i = 0; i < 9; ++i) acc[fam][i] = 0.0;
+    const double *row = own - (2 * pitch + 2) * DS;
+#pragma unroll 1
+    for (int cy = 0; cy < 5; ++cy, row += pitch * DS) {
+        double wn[3][3];
+#pragma unroll
+        for (int l = 0; l < 3; ++l) {
+            const double w = wy[l][0];
+#pragma unroll
+            for (int c = 0; c < 4; ++c) wy[l][c] = wy[l][c + 1];
+#pragma unroll
+            for (int n = 0; n < 3; ++n) wn[l][n] = w * Ly[l][n];
+        }
+#pragma unroll
+        for (int fam = 0; fam < 2; ++fam)
+#pragma unroll
+            for (int n = 0; n < 3; ++n) {
+#pragma unroll
+                for (int k = 0; k < 3; ++k) {
+                    const double *r = row + off[k] + 9 * fam + 3 * n;
+                    double t = 0.0;
+#pragma unroll
+                    for (int c = 0; c < 4; ++c)
+#pragma unroll
+                        for (int m = 0; m < 3; ++m) t = fma(wl[k][c][m], r[c * DS + m], t);
+#pragma unroll
+                    for (int l = 0; l < 3; ++l) acc[fam][3 * l + k] = fma(wn[l][n], t, acc[fam][3 * l + k]);
+                }
+            }
+    }
+}
+
+// Streams node (X, Y) into the gauge (th, ux, uy): inc = the increments of the streamed
+// populations over the node's own (f, then g).  gauge_b: the tile's common gauge
+// (sqrt theta, u_x, u_y).
+template <typename R>
+__device__ __forceinline__ void stream_node(const DevParams &p, const R *__restrict__ in, int X, int Y, const R *slot,
+                                            int pitch, const R (&gauge_b)[3], R th, R ux, R uy, bool first,
+                                            R (&inc)[2][9], unsigned &nreg, unsigned &npair)
+{
+    const R dt = typed<R>(p).dt;
+    const R s = sqrt_(th), inv_s = R(1) / s;
+    R ax[3][4], ay[3][4];
+    bool nx0[3], ny0[3];
+    const bool okx = axis_weights<R>(s, ux, dt, ax, nx0), oky = axis_weights<R>(s, uy, dt, ay, ny0);
+    if (!(okx && oky)) {
+        R buf[18];
+        stream_general<R>(p, in, X, Y, th, ux, uy, first, 0, 1, buf, nreg, npair);
+#pragma unroll
+        for (int i = 0; i < 9; ++i) {
+            inc[0][i] = buf[i];
+            inc[1][i] = buf[9 + i];
+        }
+        return;
+    }
+    const int sx = (nx0[0] == nx0[1] && nx0[1] == nx0[2]) ? 4 : 5, sy = (ny0[0] == ny0[1] && ny0[1] == ny0[2]) ? 4 : 5;
+    nreg += (unsigned)(sx * sy - (first ? 1 : 0));
+    R Lx[3][3], Ly[3][3];
+    if constexpr (sizeof(R) == 8) {
+        moment_rows(ux - gauge_b[1], inv_s, Lx);
+        moment_rows(uy - gauge_b[2], inv_s, Ly);
+        contract(slot, pitch, ax, nx0, ay, ny0, Lx, Ly, inc);
+        R v[24];
+        load_rec24(in, (size_t)Y * p.nx + X, (size_t)p.N, v);
+#pragma unroll
+        for (int i = 0; i < 9; ++i) {
+            inc[0][i] -= v[P_F + i];
+            inc[1][i] -= v[P_G + i];
+        }
+    } else {
+        const R q = (gauge_b[0] - s) * inv_s;
+        axis_map<R>(q, (gauge_b[1] - ux) * inv_s, Lx);
+        axis_map<R>(q, (gauge_b[2] - uy) * inv_s, Ly);
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            Lx[k][k] += R(1);
+            Ly[k][k] += R(1);
+        }
+        contract(slot, pitch, ax, nx0, ay, ny0, Lx, Ly, inc);
+        if (!first) {
+            // the node's own populations carried from their stored gauge into this one
+            R v[24], Ex[3][3], Ey[3][3], o[9];
+            load_rec24(in, (size_t)Y * p.nx + X, (size_t)p.N, v);
+            const R qx = fdiv_(v[P_TH] - th, (sqrt_(v[P_TH]) + s) * s);
+            axis_map<R>(qx, (v[P_UX] - ux) * inv_s, Ex);
+            axis_map<R>(qx, (v[P_UY] - uy) * inv_s, Ey);
+#pragma unroll
+            for (int fam = 0; fam < 2; ++fam) {
+                map_inc<R>(Ex, Ey, v + 9 * fam, o);
+#pragma unroll
+                for (int i = 0; i < 9; ++i) inc[fam][i] += o[i];
+            }
+        }
+    }
+}
+
+// Korteweg stress and heat flux of the staged node at slot s0 (K = -kappa (rho lap rho +
+// |grad rho|^2/2) I + kappa grad rho (x) grad rho, q = -mu grad h + k grad T), from
+// differences to the centre value (sum_i W_i c_i = 0), which keeps their FP32 rounding
+// proportional to the differences.
+template <typename R>
+__device__ __forceinline__ void stress_and_flux(const TypedParams<R> &q, const R *aux, int s0, int pitch, R (&o)[KQW])
+{
+    R c[4];
+    lds4(aux + (size_t)s0 * AUXW, c);
+    R grx = 0, gry = 0, lap = 0, ghx = 0, ghy = 0, gTx = 0, gTy = 0;
+#pragma unroll
+    for (int i = 0; i < 9; ++i) {
+        const int ex = i % 3 - 1, ey = i / 3 - 1;
+        if (ex == 0 && ey == 0) continue;
+        R v[4];
+        lds4(aux + (s0 + ey * pitch + ex) * AUXW, v);
+        const R w = wst<R>(ex, ey);
+        const R dr = v[0] - c[0], dT = v[1] - c[1];
+        const R dh = q.cv * dT - q.a * dr + (v[3] - c[3]);
+        grx += w * R(ex) * dr;
+        gry += w * R(ey) * dr;
+        lap += w * dr;
+        ghx += w * R(ex) * dh;
+        ghy += w * R(ey) * dh;
+        gTx += w * R(ex) * dT;
+        gTy += w * R(ey) * dT;
+    }
+    grx *= R(3); gry *= R(3); lap *= R(6);
+    ghx *= R(3); ghy *= R(3); gTx *= R(3); gTy *= R(3);
+    const R kap = q.kappa;
+    const R iso = -kap * (c[0] * lap + R(0.5) * (grx * grx + gry * gry));
+    const R P0 = c[2] > q.p_floor ? c[2] : q.p_floor;
+    const R mu = q.mu_coef * P0;
+    const R kc = q.k_cond >= R(0) ? q.k_cond : mu * q.cvR;
+    o[0] = iso + kap * grx * grx;
+    o[1] = kap * grx * gry;
+    o[2] = iso + kap * gry * gry;
+    o[3] = -mu * ghx + kc * gTx;
+    o[4] = -mu * ghy + kc * gTy;
+}
+
+// Collision of one node: ft, gt = its streamed populations (f~ = own + inc), o = the last
+// corrector's results, (th, ux, uy) the streaming gauge.  Fills the record.
+template <typename R>
+__device__ __forceinline__ void collide(const TypedParams<R> &q, const EosOut<R> &o, R th, R ux, R uy, R Fx, R Fy,
+                                        R M0, const R (&ft)[9], const R (&gt)[9], R (&rec)[SL])
+{
+    const R s = sqrt_(th), inv_s = R(1) / s;
+    const R rr = o.rho_hi, uxr = o.uxs, uyr = o.uys, uhxr = o.uhx, uhyr = o.uhy, Er = o.E;
+    const R Pr = o.P, sst = sqrt_(o.ths);
+    const R qm1 = sizeof(R) == 8 ? sst * inv_s - R(1) : fdiv_(o.dth, (sst + s) * s);
+    const R wsx = o.dux * inv_s, wsy = o.duy * inv_s;
+    const R dtr = q.dt, om = q.omega;
+    const R irr = frcp_(rr), iP2 = frcp_(R(2) * Pr);
+    const R dvx = Fx * dtr * irr * inv_s, dvy = Fy * dtr * irr * inv_s;
+    const R W1[3] = {wlat<R>(0), wlat<R>(1), wlat<R>(2)};
+    // transfer increments from lambda* = (ths, u*) into the streaming gauge and from the
+    // force-shifted frame (ths, u* + F dt/rho) (Eq. S-i): E[k][a] = l_k increments at the
+    // source velocities, Ws[k] = sum_a E[k][a] W_a, Wh[k] = the shifted frame's extra weight
+    R Ex[3][3], Ey[3][3], Wsx[3], Wsy[3], Whx[3], Why[3];
+    auto rows = [&](R w, R dv, R (&E)[3][3], R (&Ws)[3], R (&Wh)[3]) {
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            Ws[k] = 0;
+            Wh[k] = 0;
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                const R e = qm1 * R(a - 1) + w;
+                E[k][a] = ell_inc<R>(k, a, e);
+                Ws[k] += E[k][a] * W1[a];
+                Wh[k] += (ell_inc<R>(k, a, e + dv) - E[k][a]) * W1[a];
+            }
+        }
+    };
+    rows(wsx, dvx, Ex, Wsx, Whx);
+    rows(wsy, dvy, Ey, Wsy, Why);
+    // g: forced equilibrium (Eq. new geq), heat-flux correction (Eq. gtilde) and the
+    // force-work source 2 W_i uhat.F, all in lambda*
+    const R H = Er + Pr * irr;
+    const R Ixx = R(2) * uhxr * Fx + dtr * Fx * Fx * Er * iP2;
+    const R Ixy = uhxr * Fy + Fx * uhyr + dtr * Fx * Fy * Er * iP2;
+    const R Iyy = R(2) * uhyr * Fy + dtr * Fy * Fy * Er * iP2;
+    const R cM = R(2) * dtr * rr * iP2;
+    const R Mx = cM * (Fx * H - (Ixx * uxr + Ixy * uyr));
+    const R My = cM * (Fy * H - (Ixy * uxr + Iyy * uyr));
+    const R cN = dtr * rr * iP2;
+    const R Nxx = rr + cN * Ixx, Nxy = cN * Ixy, Nyy = rr + cN * Iyy;
+    // P/rho in the g equilibrium as sqrt(theta*)^2 times the lattice temperature of
+    // the weights in use (sum_i W_i c_ix^2 = 2 W_+-1), so that the equilibrium's zeroth
+    // moment is 2 rho E to rounding also in FP32 (sum_i W_i (v_x^2 - P/rho - u_x^2) = 0)
+    const R Pd = sst * sst * (R(2) * W1[0]);
+    const R work = R(2) * (uhxr * Fx + uhyr * Fy);
+    R Xs[9], ginc[9];
+#pragma unroll
+    for (int i = 0; i < 9; ++i) {
+        const int ix = i % 3, iy = i / 3;
+        const R cx = R(ix - 1), cy = R(iy - 1);
+        const R w = W1[ix] * W1[iy];
+        const R ccx = sst * cx, ccy = sst * cy;                  // v - u* in lambda*
+        const R Axx = ccx * ccx + R(2) * ccx * uxr - Pd;          // v v - P/rho I - u u
+        const R Axy = ccx * ccy + ccx * uyr + ccy * uxr;
+        const R Ayy = ccy * ccy + R(2) * ccy * uyr - Pd;
+        const R geq = w * (R(2) * rr * Er + Mx * ccx + My * ccy + Nxx * Axx + R(2) * Nxy * Axy + Nyy * Ayy);
+        const R vx = ccx + uxr, vy = ccy + uyr;
+        const R uc = uxr * cx + uyr * cy;
+        const R gc = M0 * w * (R(1) + rr * uc * uc * iP2 * R(3) - rr * (vx * vx + vy * vy) * iP2 + R(1));
+        Xs[i] = om * geq + dtr * (gc + w * work);
+    }
+    map_inc<R>(Ex, Ey, Xs, ginc);
+    // The collision conserves mass exactly and changes the energy by dt (M_0 + 2 uhat.F);
+    // the rest population (i = 4) takes the remainder, summed error-free as (hi, lo)
+    // pairs, so that the stored populations keep these sums up to one rounding.
+    // The stored momentum (exact pair sums of the stored populations) falls short of the
+    // exact post-collision momentum sum f~ c + F dt / s by its storage rounding; that
+    // difference is kept beside the populations too.
+    R fh = 0, fl = 0, gh = 0, gl = 0, xh = 0, xl = 0, yh = 0, yl = 0;
+    auto add = [](R &h, R &l, R v) {
+        R e;
+        two_sum_(h, v, h, e);
+        l += e;
+    };
+#pragma unroll
+    for (int i = 0; i < 9; ++i) {
+        if (i == 4) continue;
+        const int kx = i % 3, ky = i / 3;
+        const R Wx = W1[kx] + Wsx[kx], Wy = W1[ky] + Wsy[ky];
+        // f^eq - f~ with the frame-offset increments kept apart from the O(1) weights:
+        // W + Ws rounded in FP32 would keep only the increment's leading bits (Ws ~ the gauge
+        // change of one step, a few ulps of W), and always the same way, since W is a constant
+        const R dfeq = (rr * W1[kx] * W1[ky] - ft[i]) + rr * (Wsx[kx] * W1[ky] + W1[kx] * Wsy[ky] + Wsx[kx] * Wsy[ky]);
+        const R S = rr * (Whx[kx] * (Wy + Why[ky]) + Wx * Why[ky]);
+        const R fo = ft[i] + om * dfeq + S;
+        // X* carried into the streaming gauge
+        const R go = (R(1) - om) * gt[i] + (Xs[i] + ginc[i]);
+        rec[P_F + i] = fo;
+        rec[P_G + i] = go;
+        add(fh, fl, fo);
+        add(gh, gl, go);
+        if (kx != 1) add(xh, xl, R(kx - 1) * fo);
+        if (ky != 1) add(yh, yl, R(ky - 1) * fo);
+    }
+    // target sums: rho (hi, lo) and sum g~ + dt (M_0 + work); the remainders as (hi, lo)
+    // pairs: hi is stored as the population, lo beside it for the next step's sums
+    R th_, tl_, s1, e1;
+    two_sum_(o.gs_hi, dtr * (M0 + work), th_, tl_);
+    tl_ += o.gs_lo;
+    two_sum_(o.rho_hi, -fh, s1, e1);
+    two_sum_(s1, e1 + (o.rho_lo - fl), rec[P_F + 4], rec[P_F4LO]);
+    two_sum_(th_, -gh, s1, e1);
+    two_sum_(s1, e1 + (tl_ - gl), rec[P_G + 4], rec[P_G4LO]);
+    rec[P_JXLO] = ((o.mx_hi - xh) + (o.mx_lo - xl)) + Fx * dtr * inv_s;
+    rec[P_JYLO] = ((o.my_hi - yh) + (o.my_lo - yl)) + Fy * dtr * inv_s;
+    rec[P_TH] = th; rec[P_UX] = ux; rec[P_UY] = uy; rec[P_SQ] = 0;
+    rec[P_RHO] = rr; rec[P_T] = o.T; rec[P_UHX] = uhxr; rec[P_UHY] = uhyr;
+    rec[30] = rec[31] = 0;
+}
+
+// A tile of a step kernel's block: NB = TX x TY nodes from (X0, Y0), WT staged slots and RW
+// ring nodes per row, and its shared memory.
+template <typename R>
+struct Tile {
+    int X0, Y0, TX, TY, WT, RW, nslots;
+    R *aux, *slots, *kq;
+};
+
+template <typename R>
+__device__ __forceinline__ Tile<R> make_tile(const DevParams &p, int idx, R *smem)
+{
+    Tile<R> t;
+    t.TX = p.tile_x;
+    t.TY = p.tile_y;
+    t.X0 = (idx % p.tiles_x) * t.TX;
+    t.Y0 = (idx / p.tiles_x) * t.TY;
+    t.WT = t.TX + 2 * HALO;
+    t.RW = t.TX + 2;
+    t.nslots = t.WT * (t.TY + 2 * HALO);
+    t.aux = smem;
+    t.slots = t.aux + (size_t)t.nslots * AUXW;
+    t.kq = t.slots + (size_t)t.nslots * Slot<R>::stride;
+    return t;
+}
+
+// Stages a tile and its halo (see the head of this file) and computes K and q on the tile
+// and its ring; gb = the tile's common gauge: sqrt(theta), u_x, u_y.  Every thread of the
+// block calls it; it ends with a barrier.
+template <typename R>
+__device__ __forceinline__ void stage_tile(const DevParams &p, const R *__restrict__ in, const R *nlsrc,
+                                           const Tile<R> &tl, StepCounts &counts, R (&gb)[3])
+{
+    constexpr int DS = Slot<R>::stride, ST_NT = STEP_THREADS;
+    const TypedParams<R> &q = typed<R>(p);
+    const size_t N = (size_t)p.N;
+    const int tid = threadIdx.x;
+    const int X0 = tl.X0, Y0 = tl.Y0, TX = tl.TX, TY = tl.TY, WT = tl.WT, nslots = tl.nslots;
+    R *aux = tl.aux, *slots = tl.slots, *kq = tl.kq;
+    __shared__ uint2 best[ST_NT / 32];   // per warp: largest theta (bits), its slot
+    if (tid == 0) counts = StepCounts{};
     // k / WT through the float reciprocal: exact for k < 2^20 (the quotient's fraction
     // stays >= 0.5 / WT away from an integer)
     const float iwt = 1.0f / (float)WT;
-    for (int idx = threadIdx.x; idx < total; idx += blockDim.x) {
-        const int k = idx / CH, ch = idx - k * CH;
+    auto node_of = [&](int k) -> size_t {
         const int cv = (int)(((float)k + 0.5f) * iwt), cu = k - cv * WT;
-        const int gxw = bc_wrap(X0 - HALO + cu, p.nx, p.bcx);
-        const int gyw = bc_wrap(Y0 - HALO + cv, p.ny, p.bcy);
-        const R *src = in + ((size_t)gyw * p.nx + gxw) * SL + ch * (16 / sizeof(R));
-        cp_async16(tile + (cv * PT + cu) * TS + ch * (16 / sizeof(R)), src);
-    }
-    asm volatile("cp.async.commit_group;\n" ::: "memory");
-}
-
-// One time step of one tile (block) of a simulation: the body of both step kernels.
-// tile: the block's staged tile (`staged`: its copies were issued and waited for by the
-// caller, else they are issued here); part: the per-lane partials.
-template <typename R, int LPN>
-__device__ __forceinline__ void step_tile(const DevParams &p, const R *__restrict__ in,
-                                          R *__restrict__ out, DevStats *stats, int tile_idx,
-                                          const R *nlsrc, R *tile, R *part_base, bool staged,
-                                          const CUtensorMap *tmap = nullptr)
-{
-    static_assert(LPN == 8 || LPN == 16, "8 or 16 lanes per node");
-    constexpr int PPL = 16 / LPN;   // stencil positions per lane and direction
-    __shared__ StepShared<R> sh;
-    constexpr int TS = Slot<R>::stride;
-    const TypedParams<R> &q = typed<R>(p);
-    const int grp = threadIdx.x / LPN, lane = threadIdx.x % LPN;
-    const unsigned gmask = (LPN == 8 ? 0xffu : 0xffffu) << (LPN * (grp % (32 / LPN)));
-    // tile of TX x TY nodes; node grp at (tx, ty) of the tile
-    const int TX = p.tile_x, TY = STEP_NB / TX;
-    const int X0 = (tile_idx % p.tiles_x) * TX, Y0 = (tile_idx / p.tiles_x) * TY;
-    const int WT = TX + 2 * HALO, HT = TY + 2 * HALO;
-    const int PT = step_row_pitch(TX, TS);   // slots per staged row (>= WT)
-    const int tx = grp % TX, ty = grp / TX;
-    const bool valid = X0 + tx < p.nx && Y0 + ty < p.ny;
-    const int X = min(X0 + tx, p.nx - 1), Y = min(Y0 + ty, p.ny - 1);
-    const long long n = (long long)Y * p.nx + X;
-    // slot of the unwrapped coordinate (u, v) in the staged tile, or -1 outside it
-    auto slot_of = [&](int u, int v) -> int {
-        const int cu = u - (X0 - HALO), cv = v - (Y0 - HALO);
-        return (cu >= 0 && cu < WT && cv >= 0 && cv < HT) ? cv * PT + cu : -1;
+        return (size_t)bc_wrap(Y0 - HALO + cv, p.ny, p.bcy) * p.nx + bc_wrap(X0 - HALO + cu, p.nx, p.bcx);
+    };
+    auto put_aux = [&](int k, size_t nd, R r, R t) {
+        if (nlsrc != in) {   // current-time non-local terms: rho, T of the first pass's prediction
+            r = nlsrc[rec_at(nlsrc, nd, P_RHO, N)];
+            t = nlsrc[rec_at(nlsrc, nd, P_T, N)];
+        }
+        const R pr = eos_pressure<R>(p.eos_kind, q.a, q.b, q.R, r, t, typed_sp<R>(p));
+        R *a = aux + (size_t)k * AUXW;
+        a[0] = r; a[1] = t; a[2] = pr; a[3] = fdiv_(pr, r);
     };
 
-    // ---------------- staging: tile + halo records into shared memory --------------
-    {
-        const float iwt = 1.0f / (float)WT;
-        // A tile whose halo'd box (PT x HT slots) lies inside the grid is one TMA copy of a
-        // box of the record tensor [ny][nx][SL] (first TS values of each record); tiles at
-        // the grid edges need the periodic wrap or zero-gradient clamp and take the
-        // per-chunk cp.async copies.
-        const bool tma = tmap != nullptr && X0 - HALO >= 0 && X0 - HALO + PT <= p.nx &&
-                         Y0 - HALO >= 0 && Y0 - HALO + HT <= p.ny && (smem_u32(tile) & 127u) == 0;
-        if (tma) {
-            __shared__ __align__(8) unsigned long long tma_bar;
-            __shared__ int tma_ok;
-            if (threadIdx.x == 0) {
-                mbar_init(&tma_bar, 1);
-                mbar_arrive_expect_tx(&tma_bar, (unsigned)(PT * HT * TS * sizeof(R)));
-                tma_load_3d(tile, tmap, 0, X0 - HALO, Y0 - HALO, &tma_bar);
-                tma_ok = mbar_wait_bounded(&tma_bar, 0, TMA_WAIT_LIMIT_NS) ? 1 : 0;
-                if (!tma_ok) atomicAdd(&stats->timeouts, 1ull);
-            }
-            __syncthreads();
-            if (!tma_ok) return;     // the tile is skipped; the sync points report POND_ETIMEOUT
-            // every thread observes the completed phase (returns at once), which orders the
-            // copied data before its reads
-            if (threadIdx.x != 0) mbar_wait_bounded(&tma_bar, 0, TMA_WAIT_LIMIT_NS);
-        } else if (!staged) {
-            stage_issue<R>(p, in, tile, tile_idx);
-            cp_async_wait_all();
-            __syncthreads();
-        }
-        // per staged node, once per step: sqrt(theta) into the slot's spare value, and the
-        // vdW pressure and p/rho of the stored rho, T (for the non-local terms) into the
-        // slot words past the staged values
-        for (int k = threadIdx.x; k < WT * HT; k += blockDim.x) {
-            const int cv = (int)(((float)k + 0.5f) * iwt), cu = k - cv * WT;
-            R *sl = tile + (cv * PT + cu) * TS;
-            sl[P_SQ] = sqrt_(sl[P_TH]);
-            R r = sl[P_RHO], t = sl[P_T];
-            if (nlsrc != in) {
-                // current-time non-local terms: rho, T of the first pass's prediction
-                const size_t g = ((size_t)bc_wrap(Y0 - HALO + cv, p.ny, p.bcy) * p.nx +
-                                  bc_wrap(X0 - HALO + cu, p.nx, p.bcx)) * SL;
-                r = nlsrc[g + P_RHO];
-                t = nlsrc[g + P_T];
-                sl[P_RHO] = r;
-                sl[P_T] = t;
-            }
-            const R pr = eos_pressure<R>(p.eos_kind, q.a, q.b, q.R, r, t, typed_sp<R>(p));
-            sl[S_PR] = pr;
-            sl[S_PRR] = fdiv_(pr, r);
+    // ---------------- staging ------------------------------------------------------
+    if constexpr (sizeof(R) == 4) {
+        R va[24], vb[24];
+        const int ka = tid, kb = tid + ST_NT;
+        size_t na = 0, nb = 0;
+        unsigned top = 0, at = 0;
+        auto offer = [&](R th, int k) {   // finite positive values only
+            const unsigned b = (th > R(0) && th < R(3.0e38)) ? __float_as_uint(th) : 0u;
+            if (b > top) { top = b; at = (unsigned)k; }
+        };
+        if (ka < nslots) { na = node_of(ka); load_rec24(in, na, N, va); }
+        if (kb < nslots) { nb = node_of(kb); load_rec24(in, nb, N, vb); }
+        if (ka < nslots) offer(va[P_TH], ka);
+        if (kb < nslots) offer(vb[P_TH], kb);
+        for (int k = tid + 2 * ST_NT; k < nslots; k += ST_NT) offer(__ldg(in + rec_at(in, node_of(k), P_TH, N)), k);
+        {
+            const unsigned m = __reduce_max_sync(0xffffffffu, top);
+            const unsigned w = __reduce_min_sync(0xffffffffu, top == m ? at : 0xffffffffu);
+            if ((tid & 31) == 0) best[tid >> 5] = make_uint2(m, w);
         }
         __syncthreads();
-    }
-
-    // ---------------- phase 0: non-local terms, own populations --------------------
-    R Fx = 0, Fy = 0, M0 = 0, rEl = 0;
-    {
-        // lane -> non-rest neighbour (cx, cy); index skips the rest direction 4, so the
-        // opposite neighbour (-cx, -cy) sits on lane 7 - l
-        const int l8 = lane & 7;
-        const int dir = l8 < 4 ? l8 : l8 + 1;
-        const int cx = dir % 3 - 1, cy = dir / 3 - 1;
-        // the neighbour in unwrapped tile coordinates; a zero-gradient edge clamps it onto
-        // the grid first (its stencil is that of the boundary node itself)
-        const int mx = p.bcx == 0 ? X0 + tx + cx : bc_wrap(X0 + tx + cx, p.nx, 1);
-        const int my = p.bcy == 0 ? Y0 + ty + cy : bc_wrap(Y0 + ty + cy, p.ny, 1);
-        // mx + ex, my + ey (|e| <= 1) lie within 2 nodes of the tile, inside the staged
-        // halo: slots by direct offsets from the neighbour's own slot
-        const int s0 = (my - (Y0 - HALO)) * PT + (mx - (X0 - HALO));
-        const R *c0 = tile + s0 * TS;
-        const R r0 = c0[P_RHO], t0 = c0[P_T];
-        const R pr0 = c0[S_PR], prr0 = c0[S_PRR];
-        // gradients from differences to the centre value (sum_i W_i c_i = 0), which keeps
-        // their FP32 rounding proportional to the differences
-        R grx = 0, gry = 0, lap = 0, ghx = 0, ghy = 0, gTx = 0, gTy = 0;
+        uint2 b = best[0];
 #pragma unroll
-        for (int i = 0; i < 9; ++i) {
-            const int ex = i % 3 - 1, ey = i / 3 - 1;
-            if (ex == 0 && ey == 0) continue;
-            const R *cm = c0 + (ey * PT + ex) * TS;
-            const R w = wst<R>(ex, ey);
-            const R r = cm[P_RHO], t = cm[P_T];
-            const R dr = r - r0, dT = t - t0;
-            const R dh = q.cv * dT - q.a * dr + (cm[S_PRR] - prr0);
-            grx += w * R(ex) * dr;
-            gry += w * R(ey) * dr;
-            lap += w * dr;
-            ghx += w * R(ex) * dh;
-            ghy += w * R(ey) * dh;
-            gTx += w * R(ex) * dT;
-            gTy += w * R(ey) * dT;
-        }
-        grx *= R(3); gry *= R(3); lap *= R(6);
-        ghx *= R(3); ghy *= R(3); gTx *= R(3); gTy *= R(3);
-        const R kap = q.kappa;
-        const R iso = -kap * (r0 * lap + R(0.5) * (grx * grx + gry * gry));
-        const R Kxx = iso + kap * grx * grx, Kxy = kap * grx * gry, Kyy = iso + kap * gry * gry;
-        const R P0 = pr0 > q.p_floor ? pr0 : q.p_floor;
-        const R mu = q.mu_coef * P0;
-        const R kc = q.k_cond >= R(0) ? q.k_cond : mu * q.cvR;
-        const R qx = -mu * ghx + kc * gTx, qy = -mu * ghy + kc * gTy;
-        const R w = lane < 8 ? wst<R>(cx, cy) : R(0);
-        // divergences from the difference to the opposite neighbour (lane 7 - l); each
-        // opposite pair is counted by both of its lanes, hence the halved factors
-        const int opp = 7 - l8;
-        const R Kxx_o = __shfl_sync(gmask, Kxx, opp, LPN), Kxy_o = __shfl_sync(gmask, Kxy, opp, LPN);
-        const R Kyy_o = __shfl_sync(gmask, Kyy, opp, LPN);
-        const R qx_o = __shfl_sync(gmask, qx, opp, LPN), qy_o = __shfl_sync(gmask, qy, opp, LPN);
-        const R r_o = __shfl_sync(gmask, r0, opp, LPN);
-        Fx = -R(1.5) * w * (R(cx) * (Kxx - Kxx_o) + R(cy) * (Kxy - Kxy_o));
-        Fy = -R(1.5) * w * (R(cx) * (Kxy - Kxy_o) + R(cy) * (Kyy - Kyy_o));
-        M0 = R(3) * w * (R(cx) * (qx - qx_o) + R(cy) * (qy - qy_o));
-        R gxn = R(1.5) * w * R(cx) * (r0 - r_o), gyn = R(1.5) * w * R(cy) * (r0 - r_o);
+        for (int w = 1; w < ST_NT / 32; ++w)
+            if (best[w].x > b.x || (best[w].x == b.x && best[w].y < b.y)) b = best[w];
+        R base[24];
+        load_rec24(in, node_of((int)min(b.y, (unsigned)(nslots - 1))), N, base);
+        const R thb = base[P_TH];
+        gb[0] = sqrt_(thb); gb[1] = base[P_UX]; gb[2] = base[P_UY];
+        const R inv_sb = R(1) / gb[0];
+        auto carry = [&](int k, size_t nd, const R (&v)[24]) {
+            const R sn = sqrt_(v[P_TH]);
+            const R e = fdiv_(v[P_TH] - thb, (sn + gb[0]) * gb[0]);
+            R Ex[3][3], Ey[3][3], o[9];
+            axis_map<R>(e, (v[P_UX] - gb[1]) * inv_sb, Ex);
+            axis_map<R>(e, (v[P_UY] - gb[2]) * inv_sb, Ey);
+            R d[DS];
 #pragma unroll
-        for (int o = LPN / 2; o > 0; o >>= 1) {
-            Fx += __shfl_xor_sync(gmask, Fx, o, LPN);
-            Fy += __shfl_xor_sync(gmask, Fy, o, LPN);
-            M0 += __shfl_xor_sync(gmask, M0, o, LPN);
-            gxn += __shfl_xor_sync(gmask, gxn, o, LPN);
-            gyn += __shfl_xor_sync(gmask, gyn, o, LPN);
-        }
-        rEl = R(0.5) * kap * (gxn * gxn + gyn * gyn);
-    }
-    const R *own = tile + slot_of(X0 + tx, Y0 + ty) * TS;
-    // the node's own populations are read from its staged slot where needed (holding
-    // them in 18 registers through the stream loop cost more than the shared loads)
-    if (lane == 0) {
-        sh.lam[grp][0] = own[P_TH];
-        sh.lam[grp][1] = own[P_UX];
-        sh.lam[grp][2] = own[P_UY];
-        sh.nl[grp][0] = Fx;
-        sh.nl[grp][1] = Fy;
-        sh.nl[grp][2] = rEl;
-        sh.active[grp] = valid ? 1 : 0;
-        sh.nreg[grp] = 0;
-        sh.npair[grp] = 0;
-    }
-    if (threadIdx.x < STEP_NB) {
-        // exact FP64 sums of node j's stored populations, one node per lane of warp 0
-        // (error-free in R: TwoSum cascades, each sum kept as an unevaluated (hi, lo) pair
-        // and rounded once to FP64, which keeps the FP64 pipe free in the FP32 form)
-        const R *rj = tile + slot_of(X0 + threadIdx.x % TX, Y0 + threadIdx.x / TX) * TS;
-        // the stored low parts of mass, momentum and energy (not staged) start the error terms
-        const R *gj = in + ((size_t)min(Y0 + (int)threadIdx.x / TX, p.ny - 1) * p.nx +
-                            min(X0 + (int)threadIdx.x % TX, p.nx - 1)) * SL;
-        R hi[4] = {R(0), R(0), R(0), R(0)}, lo[4] = {gj[P_F4LO], gj[P_JXLO], gj[P_JYLO], gj[P_G4LO]};
+            for (int fam = 0; fam < 2; ++fam) {
+                map_inc<R>(Ex, Ey, v + 9 * fam, o);
 #pragma unroll
-        for (int i = 0; i < 9; ++i) {
-            const R f = rj[P_F + i], gv = rj[P_G + i];
-            const R terms[4] = {f, R(i % 3 - 1) * f, R(i / 3 - 1) * f, gv};
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                if (k == 1 && i % 3 == 1) continue;
-                if (k == 2 && i / 3 == 1) continue;
-                R e;
-                two_sum_(hi[k], terms[k], hi[k], e);
-                lo[k] += e;
+                for (int i = 0; i < 9; ++i) d[9 * fam + i] = (v[9 * fam + i] - base[9 * fam + i]) + o[i];
             }
-        }
+            d[18] = d[19] = R(0);
+            float4 *dst = reinterpret_cast<float4 *>(slots + (size_t)k * DS);
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            sh.bhi[threadIdx.x][k] = hi[k];
-            sh.blo[threadIdx.x][k] = lo[k];
+            for (int c = 0; c < DS / 4; ++c) dst[c] = make_float4(d[4 * c], d[4 * c + 1], d[4 * c + 2], d[4 * c + 3]);
+            put_aux(k, nd, v[P_RHO], v[P_T]);
+        };
+        if (ka < nslots) carry(ka, na, va);
+        if (kb < nslots) carry(kb, nb, vb);
+        for (int k = tid + 2 * ST_NT; k < nslots; k += ST_NT) {
+            const size_t nd = node_of(k);
+            load_rec24(in, nd, N, va);
+            carry(k, nd, va);
+        }
+    } else {
+        // moments about the velocity of the tile's middle node
+        const size_t nc = (size_t)min(Y0 + TY / 2, p.ny - 1) * p.nx + min(X0 + TX / 2, p.nx - 1);
+        gb[0] = R(1);
+        gb[1] = __ldg(in + rec_at(in, nc, P_UX, N));
+        gb[2] = __ldg(in + rec_at(in, nc, P_UY, N));
+        for (int k = tid; k < nslots; k += ST_NT) {
+            const size_t nd = node_of(k);
+            R v[24], m[9];
+            load_rec24(in, nd, N, v);
+            const R sn = sqrt_(v[P_TH]), wx = v[P_UX] - gb[1], wy = v[P_UY] - gb[2];
+            R *dst = slots + (size_t)k * DS;
+#pragma unroll
+            for (int fam = 0; fam < 2; ++fam) {
+                moments9(v + 9 * fam, sn, wx, wy, m);
+#pragma unroll
+                for (int i = 0; i < 9; ++i) dst[9 * fam + i] = m[i];
+            }
+            put_aux(k, nd, v[P_RHO], v[P_T]);
         }
     }
-    if (threadIdx.x == 0) sh.any_active = 1;
     __syncthreads();
 
-    // ---------------- phase 1: frame search (block lockstep) -----------------------
-    // part: this lane's partial increments of the node's 18 populations in the latest stream
-    R *part = part_base + grp * step_part_stride(LPN) + lane;
-    int it = 0;                                   // iterations of this block
-    int my_it = 0, my_conv = 0, my_stall = 0;     // warp-0 lane bookkeeping for node threadIdx.x
-    float my_res = 3.0e38f;                       // previous residual of that node
-    const int kk = lane & 3, m1 = (lane >> 2) & 3, m2 = m1 + 2;
-    while (sh.any_active && it < p.max_iter) {
-        ++it;
-        if (sh.active[grp]) {
-            const R th = sh.lam[grp][0], ux = sh.lam[grp][1], uy = sh.lam[grp][2];
-            const R s = sqrt_(th), inv_s = R(1) / s;
-            R a0 = 0, a1 = 0, a2 = 0, a3 = 0;
-            // Departure points x - v_i dt of the directions of each axis (the x part depends
-            // on jx only, the y part on jy only): stencil start floor(.) - 1 and the
-            // Lagrange coordinate xi in [1, 2).  The node's region is the union of its
-            // directions' 4x4 stencils: (4 + spread of the floors) per axis.
-            // Offsets are clamped to +-2^20 nodes first (a NaN offset goes to the bound):
-            // with a non-finite or runaway gauge the floors and their spread stay in int
-            // range, so the region is always 4..8 wide when taken and its indices stay
-            // inside the weight tables.
-            int fl[2][3];
-            R xi[2][3];
+    // ---------------- phase 0: non-local terms --------------------------------------
+    const int RW = tl.RW;
+    {
+        const float irw = 1.0f / (float)RW;
+        for (int k = tid; k < RW * (TY + 2); k += ST_NT) {
+            const int j = (int)(((float)k + 0.5f) * irw), i = k - j * RW;
+            // a zero-gradient edge clamps the node onto the grid first (its stencil is that
+            // of the boundary node itself)
+            const int mx = p.bcx == 0 ? X0 + i - 1 : bc_wrap(X0 + i - 1, p.nx, 1);
+            const int my = p.bcy == 0 ? Y0 + j - 1 : bc_wrap(Y0 + j - 1, p.ny, 1);
+            R o[KQW];
+            stress_and_flux<R>(q, aux, (my - (Y0 - HALO)) * WT + (mx - (X0 - HALO)), WT, o);
 #pragma unroll
-            for (int ax = 0; ax < 2; ++ax)
+            for (int c = 0; c < KQW; ++c) kq[k * KQW + c] = o[c];
+        }
+    }
+    __syncthreads();
+}
+
+// Adds a block's counters (its warps' values) to the context's.  Every thread calls it.
+__device__ __forceinline__ void add_counts(StepCounts &counts, DevStats *stats, unsigned its, unsigned nreg,
+                                           unsigned npair, bool nonconv, bool stall, bool floored, bool bad)
+{
+    const int tid = threadIdx.x;
+    // ---------------- statistics: warp sums, then one set of atomics per block --------
+    {
+        const unsigned m = 0xffffffffu;
+        const unsigned w_its = __reduce_add_sync(m, its), w_reg = __reduce_add_sync(m, nreg);
+        const unsigned w_pair = __reduce_add_sync(m, npair), w_max = __reduce_max_sync(m, its);
+        const unsigned nc = __popc(__ballot_sync(m, nonconv)), st = __popc(__ballot_sync(m, stall));
+        const unsigned cl = __popc(__ballot_sync(m, floored)), nf = __popc(__ballot_sync(m, bad));
+        if ((tid & 31) == 0) {
+            atomicAdd(&counts.streams, w_its);
+            atomicAdd(&counts.region_nodes, w_reg);
+            atomicAdd(&counts.warp_streams, w_max);
+            atomicMax(&counts.max_streams, w_max);
+            if (w_pair) atomicAdd(&counts.pair_streams, w_pair);
+            if (nc) atomicAdd(&counts.nonconv, nc);
+            if (st) atomicAdd(&counts.stalled, st);
+            if (cl) atomicAdd(&counts.clamped, cl);
+            if (nf) atomicAdd(&counts.nonfinite, nf);
+        }
+    }
+    __syncthreads();
+    if (tid == 0) {
+        atomicAdd(&stats->streams, (unsigned long long)counts.streams);
+        atomicAdd(&stats->region_nodes, (unsigned long long)counts.region_nodes);
+        atomicAdd(&stats->block_streams, (unsigned long long)counts.warp_streams);
+        atomicMax(&stats->max_streams, (unsigned long long)counts.max_streams);
+        if (counts.pair_streams) atomicAdd(&stats->pair_streams, (unsigned long long)counts.pair_streams);
+        if (counts.nonconv) atomicAdd(&stats->nonconv, (unsigned long long)counts.nonconv);
+        if (counts.stalled) atomicAdd(&stats->stalled, (unsigned long long)counts.stalled);
+        if (counts.clamped) atomicAdd(&stats->clamped, (unsigned long long)counts.clamped);
+        if (counts.nonfinite) atomicAdd(&stats->nonfinite, (unsigned long long)counts.nonfinite);
+    }
+}
+
+// Divergences of K and q at a node from the differences of opposite neighbours:
+// F = -div K, M_0 = 2 div q, and grad rho (for rho E_lambda); c0, a0 = the node's entries
+// of kq and aux.  Pair i < 4 of the neighbours alone (add the four).
+template <typename R>
+__device__ __forceinline__ void divergence_pair(const Tile<R> &tl, const R *c0, const R *a0, int i, R &Fx, R &Fy,
+                                                R &M0, R &gx, R &gy)
+{
+    const int ex = i % 3 - 1, ey = i / 3 - 1;
+    const R *a = c0 + (ey * tl.RW + ex) * KQW, *b = c0 - (ey * tl.RW + ex) * KQW;
+    const R w = (ex != 0 && ey != 0) ? wst<R>(1, 1) : wst<R>(1, 0);
+    const R dxy = a[1] - b[1];
+    Fx -= R(3) * w * (R(ex) * (a[0] - b[0]) + R(ey) * dxy);
+    Fy -= R(3) * w * (R(ex) * dxy + R(ey) * (a[2] - b[2]));
+    M0 += R(6) * w * (R(ex) * (a[3] - b[3]) + R(ey) * (a[4] - b[4]));
+    const R dr = a0[(ey * tl.WT + ex) * AUXW] - a0[-(ey * tl.WT + ex) * AUXW];
+    gx += R(3) * w * R(ex) * dr;
+    gy += R(3) * w * R(ey) * dr;
+}
+
+// Relative change of the gauge by a corrector's results o, in the gauge (th, sr = sqrt th).
+template <typename R>
+__device__ __forceinline__ float gauge_change(const EosOut<R> &o, R th, R sr)
+{
+    const float rth = fabsf((float)o.dth) / (float)th;
+    const float rux = fabsf((float)o.dux) / (float)sr, ruy = fabsf((float)o.duy) / (float)sr;
+    return fmaxf(rth, fmaxf(rux, ruy));
+}
+
+// Stop rules of the frame search: converged, and (FP32 form only) stalled: the streamed
+// moments carry FP32 rounding that the EoS cancellation inside interfaces can lift above
+// tol; once a corrector no longer halves the residual the iteration has reached that floor
+// and stops.  Only a residual within STALL_TOL_FACTOR x tol counts as that floor: a larger
+// one that fails to halve once (the pressure floor's kink in theta* = max(p, p_floor)/(rho
+// T_L) can do that) keeps iterating, since stopping there left the gauge up to 8 % off and
+// single steps 3.6e-3 off the converged result inside a compressed sub-spinodal droplet.
+template <typename R>
+__device__ __forceinline__ void stop_rules(const DevParams &p, float res, float last, unsigned its, bool &conv,
+                                           bool &stall)
+{
+    conv = sizeof(R) == 4 ? res <= p.tol_f : (double)res <= p.tol;
+    stall = sizeof(R) == 4 && its >= 2 && !conv && res > 0.5f * last && res < STALL_TOL_FACTOR * p.tol_f;
+}
+
+// One time step of one tile, one thread per node.
+template <typename R>
+__device__ __forceinline__ void step_tile(const DevParams &p, const R *__restrict__ in, R *__restrict__ out,
+                                          DevStats *stats, int tile_idx, const R *nlsrc, R *smem)
+{
+    constexpr int DS = Slot<R>::stride;
+    const TypedParams<R> &q = typed<R>(p);
+    const size_t N = (size_t)p.N;
+    const int tid = threadIdx.x;
+    __shared__ StepCounts counts;
+    const Tile<R> tl = make_tile<R>(p, tile_idx, smem);
+    R gb[3];
+    stage_tile<R>(p, in, nlsrc, tl, counts, gb);
+    const int tx = tid % tl.TX, ty = tid / tl.TX;
+    const int X = tl.X0 + tx, Y = tl.Y0 + ty;
+    const bool valid = X < p.nx && Y < p.ny;
+    const int slot = (ty + HALO) * tl.WT + tx + HALO;
+    unsigned its = 0, nreg = 0, npair = 0;
+    bool conv = true, stall = false, floored = false, bad = false;
+    if (valid) {
+        R Fx = 0, Fy = 0, M0 = 0, gxn = 0, gyn = 0;
 #pragma unroll
-                for (int j = 0; j < 3; ++j) {
-                    const R d = clamp_offset(-(s * R(j - 1) + (ax == 0 ? ux : uy)) * q.dt);
-                    const R f = floor(d);
-                    fl[ax][j] = (int)f;
-                    xi[ax][j] = d - f + R(1);
+        for (int i = 0; i < 4; ++i)
+            divergence_pair<R>(tl, tl.kq + ((ty + 1) * tl.RW + tx + 1) * KQW, tl.aux + slot * AUXW, i, Fx, Fy, M0, gxn, gyn);
+        const R nl[3] = {Fx, Fy, R(0.5) * q.kappa * (gxn * gxn + gyn * gyn)};
+        // exact sums of the node's stored populations (error-free in R: TwoSum cascades,
+        // each sum an unevaluated (hi, lo) pair); the stored low parts start the error terms
+        const size_t n = (size_t)Y * p.nx + X;
+        R hi[4] = {R(0), R(0), R(0), R(0)}, lo[4];
+        R th, ux, uy;
+        {
+            R v[24];
+            load_rec24(in, n, N, v);
+            lo[0] = __ldg(in + rec_at(in, n, P_F4LO, N));
+            lo[1] = __ldg(in + rec_at(in, n, P_JXLO, N));
+            lo[2] = __ldg(in + rec_at(in, n, P_JYLO, N));
+            lo[3] = __ldg(in + rec_at(in, n, P_G4LO, N));
+            th = v[P_TH]; ux = v[P_UX]; uy = v[P_UY];
+#pragma unroll
+            for (int i = 0; i < 9; ++i) {
+                const R f = v[P_F + i];
+                const R terms[4] = {f, R(i % 3 - 1) * f, R(i / 3 - 1) * f, v[P_G + i]};
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    if (k == 1 && i % 3 == 1) continue;
+                    if (k == 2 && i / 3 == 1) continue;
+                    R e;
+                    two_sum_(hi[k], terms[k], hi[k], e);
+                    lo[k] += e;
                 }
-            const int lo_x = min(fl[0][0], min(fl[0][1], fl[0][2]));
-            const int lo_y = min(fl[1][0], min(fl[1][1], fl[1][2]));
-            const int ncols = 4 + max(fl[0][0], max(fl[0][1], fl[0][2])) - lo_x;
-            const int nrows = 4 + max(fl[1][0], max(fl[1][1], fl[1][2])) - lo_y;
-            if (ncols <= REGION_MAX && nrows <= REGION_MAX) {
-                // weight tables: lane c < 8 fills region column c and region row c
-                if (lane < REGION_MAX) {
-#pragma unroll
-                    for (int ax = 0; ax < 2; ++ax) {
-                        const int n_ax = ax == 0 ? ncols : nrows, lo = ax == 0 ? lo_x : lo_y;
-                        if (lane < n_ax) {
-                            R w4[4];
-#pragma unroll
-                            for (int j = 0; j < 3; ++j) {
-                                const int kk2 = lane - (fl[ax][j] - lo);
-                                w4[j] = (kk2 >= 0 && kk2 < 4) ? lag1_rt<R>(kk2, xi[ax][j]) : R(0);
-                            }
-                            w4[3] = R(0);
-                            R *dst = sh.wt[grp][ax][lane];
-#pragma unroll
-                            for (int j = 0; j < 4; ++j) dst[j] = w4[j];
-                        }
-                    }
-                }
-                __syncwarp(gmask);
-                if (lane == 0) sh.nreg[grp] += ncols * nrows - ((it == 1 && lo_x <= 1 && 1 - lo_x < ncols &&
-                                                                   lo_y <= 1 && 1 - lo_y < nrows) ? 1 : 0);
-                R accf[9], accg[9];
-#pragma unroll
-                for (int i = 0; i < 9; ++i) accf[i] = accg[i] = R(0);
-                const int x_lo = X + lo_x - 1, y_lo = Y + lo_y - 1;
-                // In the first stream the arrival gauge is the node's own stored gauge, so
-                // its own region entry is carried by the identity and adds exactly nothing
-                // in the FP32 increment form (about 1e-16 in FP64): it is skipped, which
-                // makes the usual 5 x 5 region 24 entries, three full passes of 8 lanes.
-                const int own_r = (1 - lo_y) * ncols + (1 - lo_x);
-                const bool skip_own = it == 1 && lo_x <= 1 && 1 - lo_x < ncols && lo_y <= 1 && 1 - lo_y < nrows;
-                const int nreg = ncols * nrows - (skip_own ? 1 : 0);
-                const float inc = 1.0f / (float)ncols;
-                // the whole region inside the staged tile (always for |v| dt < 1): slots by
-                // direct indexing from its corner, else per node with a global fallback
-                const int cu0 = x_lo - (X0 - HALO), cv0 = y_lo - (Y0 - HALO);
-                const bool staged_region = cu0 >= 0 && cu0 + ncols <= WT && cv0 >= 0 && cv0 + nrows <= HT;
-                const R *corner = staged_region ? tile + (cv0 * PT + cu0) * TS : tile;
-                // region nodes round-robin over the group's lanes
-#pragma unroll 1
-                for (int rr = lane; rr < nreg; rr += LPN) {
-                    const int r = rr + (skip_own && rr >= own_r ? 1 : 0);
-                    const int cy = (int)(((float)r + 0.5f) * inc), cx = r - cy * ncols;
-                    R v[24];
-                    if (staged_region) {
-                        load_slot24(corner + (cy * PT + cx) * TS, v);
-                    } else {
-                        const int sl = slot_of(x_lo + cx, y_lo + cy);
-                        if (sl >= 0) {
-                            load_slot24(tile + sl * TS, v);
-                        } else {
-                            const size_t nd = (size_t)bc_wrap(y_lo + cy, p.ny, p.bcy) * p.nx +
-                                              bc_wrap(x_lo + cx, p.nx, p.bcx);
-                            load_rec24(in + nd * SL, v);
-                            v[P_SQ] = sqrt_(v[P_TH]);
-                        }
-                    }
-                    const R thn = v[P_TH], sn = v[P_SQ];
-                    const R qm1 = sizeof(R) == 8 ? sn * inv_s - R(1) : fdiv_(thn - th, (sn + s) * s);
-                    const R wxg = (v[P_UX] - ux) * inv_s, wyg = (v[P_UY] - uy) * inv_s;
-                    // transfer increments per axis from h = e/2 and p = h (2 c_a + e):
-                    // E_0 = p - h, E_1 = -2 p, E_2 = p + h (the three l_k increments)
-                    R Ex[3][3], Ey[3][3];
-#pragma unroll
-                    for (int a = 0; a < 3; ++a) {
-                        const R ex = qm1 * R(a - 1) + wxg, ey = qm1 * R(a - 1) + wyg;
-                        const R hx = R(0.5) * ex, hy = R(0.5) * ey;
-                        const R px = hx * (R(2 * (a - 1)) + ex), py = hy * (R(2 * (a - 1)) + ey);
-                        Ex[0][a] = px - hx; Ex[1][a] = R(-2) * px; Ex[2][a] = px + hx;
-                        Ey[0][a] = py - hy; Ey[1][a] = R(-2) * py; Ey[2][a] = py + hy;
-                    }
-                    R wx[3], wy[3];
-                    {
-                        const R *px = sh.wt[grp][0][cx], *py = sh.wt[grp][1][cy];
-#pragma unroll
-                        for (int j = 0; j < 3; ++j) {
-                            wx[j] = px[j];
-                            wy[j] = py[j];
-                        }
-                    }
-                    // the node's own populations from its staged slot (16-byte loads)
-                    R ov[24];
-                    load_slot24(own, ov);
-                    region_family<R>(v + P_F, ov + P_F, Ex, Ey, wx, wy, accf);
-                    region_family<R>(v + P_G, ov + P_G, Ex, Ey, wx, wy, accg);
-                }
-#pragma unroll
-                for (int i = 0; i < 9; ++i) {
-                    part[i * LPN] = accf[i];
-                    part[(9 + i) * LPN] = accg[i];
-                    a0 += accf[i];
-                    if (i % 3 == 0) a1 -= accf[i];
-                    if (i % 3 == 2) a1 += accf[i];
-                    a2 += accf[i] * R(i / 3 - 1);
-                    a3 += accg[i];
-                }
-            } else {
-            if (lane == 0) sh.npair[grp] += 1;
-            // per-pair stream for wide regions (|v| dt of 2 nodes or more): rows of
-            // directions (jy) in a rolled loop, the three directions of a row unrolled so
-            // that their transfer coefficients are compile-time selections
-#pragma unroll 1
-            for (int jy = 0; jy < 3; ++jy) {
-                R fxr[3], gxr[3];   // own populations of this row of directions
-#pragma unroll
-                for (int a = 0; a < 3; ++a) {
-                    fxr[a] = own[P_F + 3 * jy + a];
-                    gxr[a] = own[P_G + 3 * jy + a];
-                }
-                const R dy = clamp_offset(-(s * R(jy - 1) + uy) * q.dt);
-                const R fly = floor(dy);
-                const int y0 = Y + (int)fly - 1;
-                const R eta = dy - fly + R(1);
-#pragma unroll
-                for (int jx = 0; jx < 3; ++jx) {
-                    const int i = 3 * jy + jx;
-                    const R dx = clamp_offset(-(s * R(jx - 1) + ux) * q.dt);
-                    const R flx = floor(dx);
-                    const int x0 = X + (int)flx - 1;
-                    const R ax = lag1<R>(kk, dx - flx + R(1));
-                    R vf = 0, vg = 0;
-#pragma unroll
-                    for (int pp = 0; pp < PPL; ++pp) {
-                        const int mm = pp == 0 ? m1 : m2;
-                        const int sl = slot_of(x0 + kk, y0 + mm);
-                        R v[24];
-                        if (sl >= 0) {
-                            load_slot24(tile + sl * TS, v);
-                        } else {
-                            const size_t nd = (size_t)bc_wrap(y0 + mm, p.ny, p.bcy) * p.nx +
-                                              bc_wrap(x0 + kk, p.nx, p.bcx);
-                            load_rec24(in + nd * SL, v);
-                            v[P_SQ] = sqrt_(v[P_TH]);
-                        }
-                        R tf, tg;
-                        pair_inc<R>(v, jx, jy, th, s, inv_s, ux, uy, fxr[jx], gxr[jx], tf, tg);
-                        const R ay = lag1<R>(mm, eta);
-                        vf += ay * tf;
-                        vg += ay * tg;
-                    }
-                    vf *= ax;
-                    vg *= ax;
-                    // this lane's partials: kept for the collision (the node's last stream
-                    // leaves them in place) and summed into the moments right away
-                    part[i * LPN] = vf;
-                    part[(9 + i) * LPN] = vg;
-                    a0 += vf;
-                    if (jx == 0) a1 -= vf;
-                    if (jx == 2) a1 += vf;
-                    a2 += vf * R(jy - 1);
-                    a3 += vg;
-                }
-            }
-            }
-#pragma unroll
-            for (int o = LPN / 2; o > 0; o >>= 1) {
-                a0 += __shfl_xor_sync(gmask, a0, o, LPN);
-                a1 += __shfl_xor_sync(gmask, a1, o, LPN);
-                a2 += __shfl_xor_sync(gmask, a2, o, LPN);
-                a3 += __shfl_xor_sync(gmask, a3, o, LPN);
-            }
-            if (lane == 0) {
-                sh.dsum[grp][0] = a0; sh.dsum[grp][1] = a1; sh.dsum[grp][2] = a2; sh.dsum[grp][3] = a3;
             }
         }
-        __syncthreads();
-        // warp 0: moments, e -> T, EoS, residual for node j = threadIdx.x, in FP64 (FP64
-        // form) or float-float (FP32 form)
-        if (threadIdx.x < STEP_NB) {
-            const int j = threadIdx.x;
-            if (sh.active[j]) {
-                const R thr = sh.lam[j][0];
-                const R sr = sqrt_(thr);
-                EosOut<R> o;
-                eos_update(p, sh.bhi[j], sh.blo[j], sh.dsum[j], sh.nl[j], sh.lam[j], sr, o);
-                // relative change of the gauge
-                const float rth = fabsf((float)o.dth) / (float)thr;
-                const float rux = fabsf((float)o.dux) / (float)sr, ruy = fabsf((float)o.duy) / (float)sr;
-                const float res = fmaxf(rth, fmaxf(rux, ruy));
-                const bool conv = sizeof(R) == 4 ? res <= p.tol_f : (double)res <= p.tol;
-                const bool bad = !(res == res);
-                // FP32 form only: the streamed moments carry FP32 rounding that the EoS
-                // cancellation inside interfaces can lift above tol; once a corrector no
-                // longer halves the residual the iteration has reached that floor and stops.
-                // Only a residual within STALL_TOL_FACTOR x tol counts as that floor: a larger
-                // one that fails to halve once (the pressure floor's kink in
-                // theta* = max(p, p_floor)/(rho T_L) can do that) keeps iterating, since
-                // stopping there left the gauge up to 8 % off and single steps 3.6e-3 off the
-                // converged result inside a compressed sub-spinodal droplet.
-                const bool stall = sizeof(R) == 4 && it >= 2 && !conv && res > 0.5f * my_res &&
-                                   res < STALL_TOL_FACTOR * p.tol_f;
-                my_res = res;
-                my_it = it;
-                if (conv || bad || stall || it >= p.max_iter) {
-                    sh.active[j] = 0;
-                    my_conv = conv || stall;
-                    my_stall = stall;
-                    R *m = sh.mac[j];
-                    m[0] = o.rho_hi; m[1] = o.uxs; m[2] = o.uys; m[3] = o.uhx; m[4] = o.uhy;
-                    m[5] = o.E; m[6] = o.T; m[7] = o.P; m[8] = o.ths; m[9] = o.pr;
-                    sh.dlam[j][0] = o.dth; sh.dlam[j][1] = o.dux; sh.dlam[j][2] = o.duy;
-                    sh.hilo[j][0] = o.rho_hi; sh.hilo[j][1] = o.rho_lo;
-                    sh.hilo[j][2] = o.gs_hi; sh.hilo[j][3] = o.gs_lo;
-                    sh.mom[j][0] = o.mx_hi; sh.mom[j][1] = o.mx_lo;
-                    sh.mom[j][2] = o.my_hi; sh.mom[j][3] = o.my_lo;
-                } else {
-                    sh.lam[j][0] = o.ths;
-                    sh.lam[j][1] = o.uxs;
-                    sh.lam[j][2] = o.uys;
-                }
+
+        // ---------------- phase 1: frame search -------------------------------------
+        R inc[2][9];
+        EosOut<R> o;
+        float last = 3.0e38f;   // previous residual
+        for (;;) {
+            ++its;
+            stream_node<R>(p, in, X, Y, tl.slots + (size_t)slot * DS, tl.WT, gb, th, ux, uy, its == 1, inc, nreg, npair);
+            R sum[4] = {R(0), R(0), R(0), R(0)};
+#pragma unroll
+            for (int i = 0; i < 9; ++i) {
+                sum[0] += inc[0][i];
+                if (i % 3 == 0) sum[1] -= inc[0][i];
+                if (i % 3 == 2) sum[1] += inc[0][i];
+                if (i / 3 == 0) sum[2] -= inc[0][i];
+                if (i / 3 == 2) sum[2] += inc[0][i];
+                sum[3] += inc[1][i];
             }
-            const int any = __any_sync(STEP_NB_MASK, sh.active[j]);
-            if (j == 0) sh.any_active = any;
+            const R lam[3] = {th, ux, uy};
+            const R sr = sqrt_(th);
+            eos_update(p, hi, lo, sum, nl, lam, sr, o);
+            const float res = gauge_change<R>(o, th, sr);
+            stop_rules<R>(p, res, last, its, conv, stall);
+            last = res;
+            if (conv || stall || !(res == res) || its >= (unsigned)p.max_iter) break;
+            th = o.ths; ux = o.uxs; uy = o.uys;
         }
-        __syncthreads();
+        conv = conv || stall;
+
+        // ---------------- phase 2: collision ----------------------------------------
+        R rec[SL];
+        {
+            R v[24], ft[9], gt[9];
+            load_rec24(in, n, N, v);
+#pragma unroll
+            for (int i = 0; i < 9; ++i) {
+                ft[i] = v[P_F + i] + inc[0][i];
+                gt[i] = v[P_G + i] + inc[1][i];
+            }
+            collide<R>(q, o, th, ux, uy, Fx, Fy, M0, ft, gt, rec);
+        }
+        store_rec(out, n, N, rec);
+        floored = o.pr < q.p_floor;
+        bad = !(o.rho_hi == o.rho_hi) || !(o.T == o.T) || isinf(o.rho_hi) || isinf(o.T);
+    }
+    add_counts(counts, stats, its, nreg, npair, !conv, stall, floored, bad);
+}
+
+// ---------------------------------------------------------------------------
+// Nine lanes per node, for grids too small to fill the GPU with one thread per node.
+// Lane e = 3 n + k of a node first sums the stream's partial of direction component k over
+// the source index n (an x pass of 20 slots x 3 values and a y pass onto l = 0..2), three
+// lanes exchange so that lane e = 3 l + k holds the increments of population e, and the
+// collision then runs one population per lane.  Three nodes per warp; lanes 27..31 repeat
+// lanes 18..22.  All lanes of a node compute the moments and the EoS from the same values
+// in the same order, so they agree bitwise.
+template <typename R>
+__device__ __forceinline__ R grp(R v, int base, int e) { return __shfl_sync(0xffffffffu, v, base + e); }
+
+// Error-free sums over a node's nine lanes of (f, f c_x, f c_y, g) as (hi, lo) pairs, the
+// same bits in every lane: rows first, then the three rows.
+template <typename R>
+__device__ __forceinline__ void lane_sums(R f, R g, int base, int l, R (&hi)[4], R (&lo)[4])
+{
+    const int r = base + 3 * l;
+    const R f0 = grp(f, r, 0), f1 = grp(f, r, 1), f2 = grp(f, r, 2);
+    const R g0 = grp(g, r, 0), g1 = grp(g, r, 1), g2 = grp(g, r, 2);
+    R e, S, Sl, D, Dl, G, Gl;
+    two_sum_(f0, f1, S, e); Sl = e;
+    two_sum_(S, f2, S, e); Sl += e;
+    two_sum_(f2, -f0, D, Dl);
+    two_sum_(g0, g1, G, e); Gl = e;
+    two_sum_(G, g2, G, e); Gl += e;
+    auto fold = [&](R v, R vl, R &h, R &w) {
+        const R a = grp(v, base, 0), b = grp(v, base, 3), c = grp(v, base, 6);
+        const R al = grp(vl, base, 0), bl = grp(vl, base, 3), cl = grp(vl, base, 6);
+        R e1, e2;
+        two_sum_(a, b, h, e1);
+        two_sum_(h, c, h, e2);
+        w = (al + bl) + cl + (e1 + e2);
+    };
+    fold(S, Sl, hi[0], lo[0]);
+    fold(D, Dl, hi[1], lo[1]);
+    fold(G, Gl, hi[3], lo[3]);
+    const R s0 = grp(S, base, 0), s2 = grp(S, base, 6), s0l = grp(Sl, base, 0), s2l = grp(Sl, base, 6);
+    two_sum_(s2, -s0, hi[2], e);
+    lo[2] = e + (s2l - s0l);
+}
+
+template <typename R>
+__device__ __forceinline__ void step_tile_split(const DevParams &p, const R *__restrict__ in, R *__restrict__ out,
+                                                DevStats *stats, int tile_idx, const R *nlsrc, R *smem)
+{
+    constexpr int DS = Slot<R>::stride;
+    constexpr unsigned ALL = 0xffffffffu;
+    const TypedParams<R> &q = typed<R>(p);
+    const size_t N = (size_t)p.N;
+    __shared__ StepCounts counts;
+    const Tile<R> tl = make_tile<R>(p, tile_idx, smem);
+    R gb[3];
+    stage_tile<R>(p, in, nlsrc, tl, counts, gb);
+
+    const int ln = threadIdx.x & 31, lq = ln < 27 ? ln : ln - 9;
+    const int base = lq < 9 ? 0 : (lq < 18 ? 9 : 18);
+    const int e = lq - base, k = e % 3, l = e / 3;
+    const int j = (threadIdx.x >> 5) * 3 + base / 9;
+    const int tx = j % tl.TX, ty = j / tl.TX;
+    const bool valid = tl.X0 + tx < p.nx && tl.Y0 + ty < p.ny;
+    const int X = min(tl.X0 + tx, p.nx - 1), Y = min(tl.Y0 + ty, p.ny - 1);
+    const size_t n = (size_t)Y * p.nx + X;
+    const int slot = (ty + HALO) * tl.WT + tx + HALO;
+    const bool writer = ln < 27;
+    // the node's own record and the general stream's partials
+    R *own = tl.kq + (size_t)(tl.TX + 2) * (tl.TY + 2) * KQW + (size_t)j * SPLIT_WORDS, *part = own + SL;
+    for (int v = e; v < 30; v += 9)
+        if (writer) own[v] = __ldg(in + rec_at(in, n, v, N));
+    R Fx = 0, Fy = 0, M0 = 0, rEl;
+    {
+        R gx = 0, gy = 0;
+        if (e < 4)
+            divergence_pair<R>(tl, tl.kq + ((ty + 1) * tl.RW + tx + 1) * KQW, tl.aux + slot * AUXW, e, Fx, Fy, M0, gx, gy);
+        auto four = [&](R v) { return (grp(v, base, 0) + grp(v, base, 1)) + (grp(v, base, 2) + grp(v, base, 3)); };
+        Fx = four(Fx); Fy = four(Fy); M0 = four(M0); gx = four(gx); gy = four(gy);
+        rEl = R(0.5) * q.kappa * (gx * gx + gy * gy);
+    }
+    __syncwarp();
+    const R nl[3] = {Fx, Fy, rEl};
+    R th = own[P_TH], ux = own[P_UX], uy = own[P_UY];
+    const R fe = own[P_F + e], ge = own[P_G + e];
+    R hi[4], lo[4];
+    lane_sums<R>(fe, ge, base, l, hi, lo);
+    lo[0] += own[P_F4LO]; lo[1] += own[P_JXLO]; lo[2] += own[P_JYLO]; lo[3] += own[P_G4LO];
+    R dx[6];   // the own slot's values this lane differences against (FP32)
+    const R *sl = tl.slots + (size_t)slot * DS;
+#pragma unroll
+    for (int m = 0; m < 3; ++m) {
+        dx[m] = sizeof(R) == 4 ? sl[3 * l + m] : R(0);
+        dx[3 + m] = sizeof(R) == 4 ? sl[9 + 3 * l + m] : R(0);
     }
 
-    // ---------------- phase 2: collision (one population per lane) -----------------
-    if (valid) {
-        // Population `pop` of this lane.  The rest population (4) is stored as the exact
-        // remainder of mass and energy, so with 8 lanes per node lane 4 takes population 8
-        // instead; with 16, lanes 0..8 take their own index (lane 4's result is replaced).
-        const int pop = (LPN == 8 && lane == 4) ? 8 : (lane < 9 ? lane : 8);
-        const bool owner = lane < 9 && pop != 4;
-        // its increment from the node's final stream: the sum of the lanes' partials, read
-        // in a lane-rotated order so that the rows fall on different banks
-        R my_df = 0, my_dg = 0;
+    // ---------------- phase 1: frame search (warp lockstep) ---------------------------
+    unsigned its = 0, nreg = 0, npair = 0;
+    bool conv = true, stall = false, active = valid;
+    R df = 0, dg = 0;         // increments of population e
+    EosOut<R> o{};
+    float last = 3.0e38f;
+    for (unsigned it = 1; __any_sync(ALL, active); ++it) {
+        const R s = sqrt_(th), inv_s = R(1) / s, dt = q.dt;
+        // departure along x of component k, along y of all three
+        R wx[4], wy[3][5], Lx[3], Ly[3];
+        bool near_x, ok = true;
         {
-            const R *row = part - lane;
+            auto weights = [&](R v, R (&a)[4]) -> bool {   // true: floor 0, false: floor -1
+                const R d = -v * dt;
+                const R f = floor(d);
+                ok = ok && (f == R(0) || f == R(-1));
+                const R t0 = d - f + R(1), t1 = t0 - R(1), t2 = t0 - R(2), t3 = t0 - R(3);
+                const R p12 = t1 * t2, p03 = t0 * t3;
+                a[0] = p12 * t3 * R(-1.0 / 6.0);
+                a[1] = p03 * t2 * R(0.5);
+                a[2] = p03 * t1 * R(-0.5);
+                a[3] = p12 * t0 * R(1.0 / 6.0);
+                return f == R(0);
+            };
+            near_x = weights(s * R(k - 1) + ux, wx);
 #pragma unroll
-            for (int l = 0; l < LPN; ++l) {
-                const int ll = (l + lane) & (LPN - 1);
-                my_df += row[pop * LPN + ll];
-                my_dg += row[(9 + pop) * LPN + ll];
+            for (int c = 0; c < 3; ++c) {
+                R a[4];
+                const bool near = weights(s * R(c - 1) + uy, a);
+                wy[c][0] = near ? R(0) : a[0];
+                wy[c][1] = near ? a[0] : a[1];
+                wy[c][2] = near ? a[1] : a[2];
+                wy[c][3] = near ? a[2] : a[3];
+                wy[c][4] = near ? a[3] : R(0);
             }
         }
-        const R th = sh.lam[grp][0], ux = sh.lam[grp][1], uy = sh.lam[grp][2];
+        const unsigned okm = __ballot_sync(ALL, ok), nxm = __ballot_sync(ALL, near_x);
+        const unsigned gm = 0x1ffu << base;
+        const bool fast = (okm & gm) == gm;
+        R nf = 0, ng = 0;
+        {
+            // row k of the x map, column n (= l) of the y map
+            if constexpr (sizeof(R) == 8) {
+                const R i2 = inv_s * inv_s, c = R(k - 1);
+                const R t = ux - gb[1], ts = t * inv_s;
+                Lx[0] = k == 1 ? R(1) - ts * ts : R(0.5) * ts * (ts - c);
+                Lx[1] = k == 1 ? R(2) * t * i2 : R(0.5) * c * inv_s - t * i2;
+                Lx[2] = k == 1 ? -i2 : R(0.5) * i2;
+                const R ty_ = uy - gb[2], tsy = ty_ * inv_s;
+#pragma unroll
+                for (int c2 = 0; c2 < 3; ++c2) {
+                    const R cc = R(c2 - 1);
+                    const R a0 = c2 == 1 ? R(1) - tsy * tsy : R(0.5) * tsy * (tsy - cc);
+                    const R a1 = c2 == 1 ? R(2) * ty_ * i2 : R(0.5) * cc * inv_s - ty_ * i2;
+                    const R a2 = c2 == 1 ? -i2 : R(0.5) * i2;
+                    Ly[c2] = l == 0 ? a0 : (l == 1 ? a1 : a2);
+                }
+            } else {
+                const R qq = (gb[0] - s) * inv_s, w1 = (gb[1] - ux) * inv_s, w2 = (gb[2] - uy) * inv_s;
+#pragma unroll
+                for (int m = 0; m < 3; ++m) Lx[m] = ell_inc_rt<R>(k, m, qq * R(m - 1) + w1) + (m == k ? R(1) : R(0));
+                const R ey = qq * R(l - 1) + w2, h = R(0.5) * ey, pp = h * (R(2 * (l - 1)) + ey);
+                Ly[0] = (pp - h) + (l == 0 ? R(1) : R(0));
+                Ly[1] = R(-2) * pp + (l == 1 ? R(1) : R(0));
+                Ly[2] = (pp + h) + (l == 2 ? R(1) : R(0));
+            }
+            R wl[4][3];
+#pragma unroll
+            for (int c = 0; c < 4; ++c)
+#pragma unroll
+                for (int m = 0; m < 3; ++m) wl[c][m] = wx[c] * Lx[m];
+            R af[3] = {R(0), R(0), R(0)}, ag[3] = {R(0), R(0), R(0)};
+            const R *row = sl - (2 * tl.WT + (near_x ? 1 : 2)) * DS + 3 * l;
+#pragma unroll
+            for (int cy = 0; cy < 5; ++cy, row += tl.WT * DS) {
+                R tf = 0, tg = 0;
+#pragma unroll
+                for (int c = 0; c < 4; ++c)
+#pragma unroll
+                    for (int m = 0; m < 3; ++m) {
+                        tf += wl[c][m] * (sizeof(R) == 4 ? row[c * DS + m] - dx[m] : row[c * DS + m]);
+                        tg += wl[c][m] * (sizeof(R) == 4 ? row[c * DS + 9 + m] - dx[3 + m] : row[c * DS + 9 + m]);
+                    }
+#pragma unroll
+                for (int c = 0; c < 3; ++c) {
+                    const R w = wy[c][cy] * Ly[c];
+                    af[c] += w * tf;
+                    ag[c] += w * tg;
+                }
+            }
+            // lane (k, n) keeps its share of l = n and sends the others to their lanes
+            nf = sel3(l, af[0], af[1], af[2]);
+            ng = sel3(l, ag[0], ag[1], ag[2]);
+#pragma unroll
+            for (int r = 1; r < 3; ++r) {
+                const int to = (l + 3 - r) % 3, from = (l + r) % 3;
+                nf += grp(sel3(to, af[0], af[1], af[2]), base, 3 * from + k);
+                ng += grp(sel3(to, ag[0], ag[1], ag[2]), base, 3 * from + k);
+            }
+        }
+        if (sizeof(R) == 8) {
+            nf -= fe;
+            ng -= ge;
+        } else if (it > 1) {
+            // the node's own populations carried from their stored gauge into this one
+            const R tho = own[P_TH];
+            const R qx = fdiv_(tho - th, (sqrt_(tho) + s) * s);
+            const R w1 = (own[P_UX] - ux) * inv_s, w2 = (own[P_UY] - uy) * inv_s;
+            R Er[3], Ec[3];
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                Er[a] = ell_inc_rt<R>(k, a, qx * R(a - 1) + w1);
+                Ec[a] = ell_inc_rt<R>(l, a, qx * R(a - 1) + w2);
+            }
+#pragma unroll
+            for (int fam = 0; fam < 2; ++fam) {
+                const R *h = own + 9 * fam;
+                R acc = 0;
+#pragma unroll
+                for (int b = 0; b < 3; ++b) {
+                    const R t = Er[0] * h[3 * b] + Er[1] * h[3 * b + 1] + Er[2] * h[3 * b + 2];
+                    acc += Ec[b] * (h[3 * b + k] + t) + (b == l ? t : R(0));
+                }
+                if (fam == 0) nf += acc;
+                else ng += acc;
+            }
+        }
+        unsigned add_reg = 0, add_pair = 0;
+        if (fast) {
+            const unsigned nx3 = (nxm >> base) & 7u;   // the row l = 0 holds all three components
+            const int sx = (nx3 == 0u || nx3 == 7u) ? 4 : 5;
+            const R dy0 = floor(-(s * R(-1) + uy) * dt), dy2 = floor(-(s + uy) * dt);
+            add_reg = (unsigned)(sx * (dy0 == dy2 ? 4 : 5) - (it == 1 ? 1 : 0));
+        }
+        if (__any_sync(ALL, active && !fast)) {
+            // departure points beyond the halo: the node's lanes share its stencil nodes
+            if (!fast) {
+                R buf[18];
+                stream_general<R>(p, in, X, Y, th, ux, uy, it == 1, e, 9, buf, add_reg, add_pair);
+                if (writer)
+#pragma unroll
+                    for (int i = 0; i < 18; ++i) part[i * 9 + e] = buf[i];
+            }
+            __syncwarp();
+            if (!fast) {
+                nf = ng = R(0);
+#pragma unroll
+                for (int i = 0; i < 9; ++i) {
+                    nf += part[e * 9 + i];
+                    ng += part[(9 + e) * 9 + i];
+                }
+            }
+            __syncwarp();
+        }
+        // sums of the increments, the same in every lane
+        R sum[4];
+        {
+            const int r = base + 3 * l;
+            const R f0 = grp(nf, r, 0), f1 = grp(nf, r, 1), f2 = grp(nf, r, 2);
+            const R S = f0 + f1 + f2, D = f2 - f0, G = grp(ng, r, 0) + grp(ng, r, 1) + grp(ng, r, 2);
+            const R s0 = grp(S, base, 0), s1 = grp(S, base, 3), s2 = grp(S, base, 6);
+            sum[0] = s0 + s1 + s2;
+            sum[1] = grp(D, base, 0) + grp(D, base, 3) + grp(D, base, 6);
+            sum[2] = s2 - s0;
+            sum[3] = grp(G, base, 0) + grp(G, base, 3) + grp(G, base, 6);
+        }
+        if (active) {
+            its = it;
+            nreg += add_reg;
+            npair += add_pair;
+            df = nf;
+            dg = ng;
+            const R lam[3] = {th, ux, uy};
+            const R sr = sqrt_(th);
+            eos_update(p, hi, lo, sum, nl, lam, sr, o);
+            const float res = gauge_change<R>(o, th, sr);
+            stop_rules<R>(p, res, last, it, conv, stall);
+            last = res;
+            if (conv || stall || !(res == res) || it >= (unsigned)p.max_iter) active = false;
+            else { th = o.ths; ux = o.uxs; uy = o.uys; }
+        }
+    }
+    conv = conv || stall;
+
+    // ---------------- phase 2: collision, population e of the node per lane ------------
+    // (the formulas of collide(), one population at a time)
+    {
         const R s = sqrt_(th), inv_s = R(1) / s;
-        const R *m = sh.mac[grp];
-        const R rr = m[0], uxr = m[1], uyr = m[2], uhxr = m[3], uhyr = m[4], Er = m[5];
-        const R Pr = m[7], thsr = m[8];
-        const R sst = sqrt_(thsr);
-        const R qm1 = sizeof(R) == 8 ? sst * inv_s - R(1) : fdiv_(sh.dlam[grp][0], (sst + s) * s);
-        const R wsx = sh.dlam[grp][1] * inv_s, wsy = sh.dlam[grp][2] * inv_s;
+        const R rr = o.rho_hi, uxr = o.uxs, uyr = o.uys, uhxr = o.uhx, uhyr = o.uhy, Er = o.E;
+        const R Pr = o.P, sst = sqrt_(o.ths);
+        const R qm1 = sizeof(R) == 8 ? sst * inv_s - R(1) : fdiv_(o.dth, (sst + s) * s);
+        const R wsx = o.dux * inv_s, wsy = o.duy * inv_s;
         const R dtr = q.dt, om = q.omega;
         const R irr = frcp_(rr), iP2 = frcp_(R(2) * Pr);
         const R dvx = Fx * dtr * irr * inv_s, dvy = Fy * dtr * irr * inv_s;
         const R W1[3] = {wlat<R>(0), wlat<R>(1), wlat<R>(2)};
-        // transfer increments from lambda* = (ths, u*) into the streaming gauge, and from the
-        // force-shifted frame (ths, u* + F dt/rho) (Eq. S-i), for the row k of one axis:
-        // E[a] = l_k increments at the source velocities, Ws = sum_a E[a] W_a, Wh = the
-        // force-shifted frame's extra weight
-        auto row = [&](int k, R w, R dv, R (&E)[3], R &Ws, R &Wh) {
+        auto row = [&](int kk, R w, R dv, R (&E)[3], R &Ws, R &Wh) {
             Ws = 0;
             Wh = 0;
 #pragma unroll
             for (int a = 0; a < 3; ++a) {
-                E[a] = ell_inc_rt<R>(k, a, qm1 * R(a - 1) + w);
+                const R ea = qm1 * R(a - 1) + w;
+                E[a] = ell_inc_rt<R>(kk, a, ea);
                 Ws += E[a] * W1[a];
-                Wh += (ell_inc_rt<R>(k, a, qm1 * R(a - 1) + w + dv) - E[a]) * W1[a];
+                Wh += (ell_inc_rt<R>(kk, a, ea + dv) - E[a]) * W1[a];
             }
         };
-        // g: forced equilibrium (Eq. new geq), heat-flux correction (Eq. gtilde) and the
-        // force-work source 2 W_i uhat.F, all in lambda*, in every lane (9 values)
+        R exk[3], eyl[3], Wsk, Wsl, Whk, Whl;
+        row(k, wsx, dvx, exk, Wsk, Whk);
+        row(l, wsy, dvy, eyl, Wsl, Whl);
         const R H = Er + Pr * irr;
         const R Ixx = R(2) * uhxr * Fx + dtr * Fx * Fx * Er * iP2;
         const R Ixy = uhxr * Fy + Fx * uhyr + dtr * Fx * Fy * Er * iP2;
@@ -1124,208 +1680,102 @@ __device__ __forceinline__ void step_tile(const DevParams &p, const R *__restric
         const R My = cM * (Fy * H - (Ixy * uxr + Iyy * uyr));
         const R cN = dtr * rr * iP2;
         const R Nxx = rr + cN * Ixx, Nxy = cN * Ixy, Nyy = rr + cN * Iyy;
-        // P/rho in the g equilibrium as sqrt(theta*)^2 times the lattice temperature of
-        // the weights in use (sum_i W_i c_ix^2 = 2 W_+-1), so that the equilibrium's zeroth
-        // moment is 2 rho E to rounding also in FP32 (sum_i W_i (v_x^2 - P/rho - u_x^2) = 0)
         const R Pd = sst * sst * (R(2) * W1[0]);
         const R work = R(2) * (uhxr * Fx + uhyr * Fy);
-        // X*_i for this lane's population(s) only, then gathered across the group
-        auto xstar = [&](int i) -> R {
-            const int ix = i % 3, iy = i / 3;
-            const R cx = R(ix - 1), cy = R(iy - 1);
-            const R w = pick(W1, ix) * pick(W1, iy);
-            const R ccx = sst * cx, ccy = sst * cy;                  // v - u* in lambda*
-            const R Axx = ccx * ccx + R(2) * ccx * uxr - Pd;          // v v - P/rho I - u u
-            const R Axy = ccx * ccy + ccx * uyr + ccy * uxr;
-            const R Ayy = ccy * ccy + R(2) * ccy * uyr - Pd;
-            const R geq = w * (R(2) * rr * Er + Mx * ccx + My * ccy + Nxx * Axx + R(2) * Nxy * Axy + Nyy * Ayy);
-            const R vx = ccx + uxr, vy = ccy + uyr;
-            const R uc = uxr * cx + uyr * cy;
-            const R gc = M0 * w * (R(1) + rr * uc * uc * iP2 * R(3)
-                                   - rr * (vx * vx + vy * vy) * iP2 + R(1));
-            return om * geq + dtr * (gc + w * work);
-        };
-        const R my_x = xstar(pop);
-        const R x4 = LPN == 8 ? xstar(4) : R(0);   // no lane holds population 4 then
-        R Xs[9];
+        const R cx = R(k - 1), cy = R(l - 1);
+        const R W1k = pick(W1, k), W1l = pick(W1, l), w = W1k * W1l;
+        const R ccx = sst * cx, ccy = sst * cy;
+        const R Axx = ccx * ccx + R(2) * ccx * uxr - Pd;
+        const R Axy = ccx * ccy + ccx * uyr + ccy * uxr;
+        const R Ayy = ccy * ccy + R(2) * ccy * uyr - Pd;
+        const R geq = w * (R(2) * rr * Er + Mx * ccx + My * ccy + Nxx * Axx + R(2) * Nxy * Axy + Nyy * Ayy);
+        const R vx = ccx + uxr, vy = ccy + uyr;
+        const R uc = uxr * cx + uyr * cy;
+        const R gc = M0 * w * (R(1) + rr * uc * uc * iP2 * R(3) - rr * (vx * vx + vy * vy) * iP2 + R(1));
+        const R X_e = om * geq + dtr * (gc + w * work);
+        R acc = X_e;
 #pragma unroll
-        for (int k = 0; k < 9; ++k) {
-            if (LPN == 8) Xs[k] = k == 4 ? x4 : __shfl_sync(gmask, my_x, k == 8 ? 4 : k, LPN);
-            else Xs[k] = __shfl_sync(gmask, my_x, k, LPN);
+        for (int b = 0; b < 3; ++b) {
+            const R x0 = grp(X_e, base, 3 * b), x1 = grp(X_e, base, 3 * b + 1), x2 = grp(X_e, base, 3 * b + 2);
+            const R t = exk[0] * x0 + exk[1] * x1 + exk[2] * x2;
+            acc += eyl[b] * (sel3(k, x0, x1, x2) + t) + (b == l ? t : R(0));
         }
-        R fo, go;
-        {
-            {
-                const int i = pop;
-                const int kx = i % 3, ky = i / 3;
-                const R ft = own[P_F + i] + my_df, gt = own[P_G + i] + my_dg;
-                R exk[3], eyl[3], Wsk, Wsl, Whk, Whl;
-                row(kx, wsx, dvx, exk, Wsk, Whk);
-                row(ky, wsy, dvy, eyl, Wsl, Whl);
-                const R W1k = pick(W1, kx), W1l = pick(W1, ky);
-                const R Wx = W1k + Wsk, Wy = W1l + Wsl;
-                // f^eq - f~ with the frame-offset increments kept apart from the O(1)
-                // weights: W + Ws rounded in FP32 would keep only the increment's leading
-                // bits (Ws ~ the gauge change of one step, a few ulps of W), and always the
-                // same way, since W is a constant
-                const R dfeq = (rr * W1k * W1l - ft) + rr * (Wsk * W1l + W1k * Wsl + Wsk * Wsl);
-                const R S = rr * (Whk * (Wy + Whl) + Wx * Whl);
-                fo = ft + om * dfeq + S;
-                // carry X* into the streaming gauge: X = X* + (G* - I) X*
-                R acc = pick(Xs, i);
-#pragma unroll
-                for (int a = 0; a < 3; ++a) {
-                    R gyc = 0;
-#pragma unroll
-                    for (int b = 0; b < 3; ++b) gyc += (eyl[b] + (b == ky ? R(1) : R(0))) * Xs[a + 3 * b];
-                    acc += exk[a] * gyc;
-                }
-                R xcol[3];
-#pragma unroll
-                for (int b = 0; b < 3; ++b)
-                    xcol[b] = kx == 0 ? Xs[3 * b] : (kx == 1 ? Xs[3 * b + 1] : Xs[3 * b + 2]);
-#pragma unroll
-                for (int b = 0; b < 3; ++b) acc += eyl[b] * xcol[b];
-                go = (R(1) - om) * gt + acc;
+        const R ft = fe + df, gt = ge + dg;
+        const R Wx = W1k + Wsk, Wy = W1l + Wsl;
+        const R dfeq = (rr * W1k * W1l - ft) + rr * (Wsk * W1l + W1k * Wsl + Wsk * Wsl);
+        const R S = rr * (Whk * (Wy + Whl) + Wx * Whl);
+        R fo = ft + om * dfeq + S, go = (R(1) - om) * gt + acc;
+        R sh[4], sl4[4];
+        lane_sums<R>(e == 4 ? R(0) : fo, e == 4 ? R(0) : go, base, l, sh, sl4);
+        if (valid && writer) {
+            if (e == 4) {
+                R t_h, t_l, s1, e1, f4lo, g4lo;
+                two_sum_(o.gs_hi, dtr * (M0 + work), t_h, t_l);
+                t_l += o.gs_lo;
+                two_sum_(o.rho_hi, -sh[0], s1, e1);
+                two_sum_(s1, e1 + (o.rho_lo - sl4[0]), fo, f4lo);
+                two_sum_(t_h, -sh[3], s1, e1);
+                two_sum_(s1, e1 + (t_l - sl4[3]), go, g4lo);
+                REC(out, n, P_F4LO) = f4lo;
+                REC(out, n, P_G4LO) = g4lo;
+                REC(out, n, P_JXLO) = ((o.mx_hi - sh[1]) + (o.mx_lo - sl4[1])) + Fx * dtr * inv_s;
+                REC(out, n, P_JYLO) = ((o.my_hi - sh[2]) + (o.my_lo - sl4[2])) + Fy * dtr * inv_s;
             }
-        }
-        // The collision conserves mass exactly and changes the energy by dt (M_0 + 2 uhat.F);
-        // the rest population (i = 4) takes the remainder, summed error-free as (hi, lo)
-        // pairs, so that the stored populations keep these sums up to one rounding.
-        // The stored momentum (exact pair sums of the stored populations) falls short of the
-        // exact post-collision momentum sum f~ c + F dt / s by its storage rounding; that
-        // difference is kept beside the populations too.
-        R f4 = 0, g4 = 0, f4lo = 0, g4lo = 0, jxlo = 0, jylo = 0;
-        {
-            R fh = owner ? fo : R(0), fl = 0;
-            R gh = owner ? go : R(0), gl = 0;
-            R xh = owner ? R(pop % 3 - 1) * fo : R(0), xl = 0;
-            R yh = owner ? R(pop / 3 - 1) * fo : R(0), yl = 0;
-#pragma unroll
-            for (int o = LPN / 2; o > 0; o >>= 1) {
-                const R fh2 = __shfl_xor_sync(gmask, fh, o, LPN), fl2 = __shfl_xor_sync(gmask, fl, o, LPN);
-                const R gh2 = __shfl_xor_sync(gmask, gh, o, LPN), gl2 = __shfl_xor_sync(gmask, gl, o, LPN);
-                const R xh2 = __shfl_xor_sync(gmask, xh, o, LPN), xl2 = __shfl_xor_sync(gmask, xl, o, LPN);
-                const R yh2 = __shfl_xor_sync(gmask, yh, o, LPN), yl2 = __shfl_xor_sync(gmask, yl, o, LPN);
-                R e;
-                two_sum_(fh, fh2, fh, e);
-                fl = fl + fl2 + e;
-                two_sum_(gh, gh2, gh, e);
-                gl = gl + gl2 + e;
-                two_sum_(xh, xh2, xh, e);
-                xl = xl + xl2 + e;
-                two_sum_(yh, yh2, yh, e);
-                yl = yl + yl2 + e;
+            if (e == 0) {
+                REC(out, n, P_TH) = th;
+                REC(out, n, P_UX) = ux;
+                REC(out, n, P_UY) = uy;
+                REC(out, n, P_RHO) = rr;
+                REC(out, n, P_T) = o.T;
+                REC(out, n, P_UHX) = uhxr;
+                REC(out, n, P_UHY) = uhyr;
             }
-            if (lane == 4) {
-                // target sums: rho (hi, lo) and sum g~ + dt (M_0 + work)
-                R th_, tl_;
-                two_sum_(sh.hilo[grp][2], dtr * (M0 + work), th_, tl_);
-                tl_ += sh.hilo[grp][3];
-                // the remainders as (hi, lo) pairs: hi is stored as the population, lo
-                // beside it for the next step's sums
-                R s1, e1;
-                two_sum_(sh.hilo[grp][0], -fh, s1, e1);
-                two_sum_(s1, e1 + (sh.hilo[grp][1] - fl), f4, f4lo);
-                two_sum_(th_, -gh, s1, e1);
-                two_sum_(s1, e1 + (tl_ - gl), g4, g4lo);
-                jxlo = ((sh.mom[grp][0] - xh) + (sh.mom[grp][1] - xl)) + Fx * dtr * inv_s;
-                jylo = ((sh.mom[grp][2] - yh) + (sh.mom[grp][3] - yl)) + Fy * dtr * inv_s;
-            }
-        }
-        if (owner) {
-            REC(out, n, P_F + pop) = fo;
-            REC(out, n, P_G + pop) = go;
-        }
-        if (lane == 4) {
-            REC(out, n, P_F + 4) = f4;
-            REC(out, n, P_G + 4) = g4;
-            REC(out, n, P_F4LO) = f4lo;
-            REC(out, n, P_G4LO) = g4lo;
-            REC(out, n, P_JXLO) = jxlo;
-            REC(out, n, P_JYLO) = jylo;
-        }
-        if (lane == 0) {
-            REC(out, n, P_TH) = th;
-            REC(out, n, P_UX) = ux;
-            REC(out, n, P_UY) = uy;
-            REC(out, n, P_RHO) = rr;
-            REC(out, n, P_T) = m[6];
-            REC(out, n, P_UHX) = uhxr;
-            REC(out, n, P_UHY) = uhyr;
+            REC(out, n, P_F + e) = fo;
+            REC(out, n, P_G + e) = go;
         }
     }
-    // ---------------- statistics (warp 0, one lane per node) -----------------------
-    if (threadIdx.x < STEP_NB) {
-        const int j = threadIdx.x;
-        const bool v = X0 + j % TX < p.nx && Y0 + j / TX < p.ny;
-        const R T = sh.mac[j][6], rr = sh.mac[j][0], pr = sh.mac[j][9];
-        warp_add(&stats->streams, v ? my_it : 0);
-        warp_add(&stats->region_nodes, v ? sh.nreg[j] : 0);
-        warp_add(&stats->pair_streams, v ? sh.npair[j] : 0);
-        warp_add(&stats->nonconv, (v && !my_conv) ? 1 : 0);
-        warp_add(&stats->stalled, (v && my_stall) ? 1 : 0);
-        warp_add(&stats->clamped, (v && pr < q.p_floor) ? 1 : 0);
-        const bool bad = v && (!(rr == rr) || !(T == T) || isinf(rr) || isinf(T));
-        warp_add(&stats->nonfinite, bad ? 1 : 0);
-        if (j == 0) {
-            atomicAdd(&stats->block_streams, (unsigned long long)it);
-            atomicMax(&stats->max_streams, (unsigned long long)it);
-        }
-    }
+    const bool one = valid && writer && e == 0;   // one lane reports for the node
+    const bool bad = !(o.rho_hi == o.rho_hi) || !(o.T == o.T) || isinf(o.rho_hi) || isinf(o.T);
+    add_counts(counts, stats, one ? its : 0, one ? nreg : 0, one ? npair : 0, one && !conv, one && stall,
+               one && o.pr < q.p_floor, one && bad);
 }
 
-// One time step of one simulation: one block per tile.  (A persistent variant that
-// prefetched its next tile into a second staging buffer was slower on GB300: 2.64 against
-// 2.41 ms on the 2048 x 1024 droplet-shock; the block scheduler already overlaps one
-// block's staging with the others' work, and the second buffer takes L1 capacity.)
-// tmap: tensor map of `in` for the TMA staging of interior tiles (use_tma = 0: every tile
-// takes the per-chunk copies).
-template <typename R, int LPN>
-__global__ void __launch_bounds__(STEP_NB *LPN, STEP_MIN_BLOCKS(R, LPN)) k_pond_step(DevParams p, const R *__restrict__ in,
-                                                             R *__restrict__ out, DevStats *stats,
-                                                             const R *nlsrc, const __grid_constant__ CUtensorMap tmap,
-                                                             int use_tma)
-{
-    extern __shared__ __align__(128) unsigned char step_dyn_smem[];
-    R *tile = reinterpret_cast<R *>(step_dyn_smem);
-    step_tile<R, LPN>(p, in, out, stats, blockIdx.x, nlsrc, tile,
-                      tile + (size_t)step_tile_slots(p.tile_x, Slot<R>::stride) * Slot<R>::stride, false,
-                      use_tma ? &tmap : nullptr);
-}
-
-// A simulation of a batch as one launch sees it: parameters, the buffers this step reads
-// and writes, and its counters.
+// A simulation as one launch sees it: parameters, the buffers this step reads and writes
+// (nlsrc: the state the non-local terms come from) and its counters.
 template <typename R>
 struct SimDesc {
     DevParams p;
     const R *in;
     R *out;
     DevStats *stats;
+    const R *nlsrc;
 };
 
-// One time step of every simulation of a batch in one launch: block b steps tile
-// work[b].y of simulation work[b].x (a device work-list of (simulation, tile) pairs).
-template <typename R, int LPN>
-__global__ void __launch_bounds__(STEP_NB *LPN, STEP_MIN_BLOCKS(R, LPN)) k_pond_step_batch(const SimDesc<R> *__restrict__ descs,
-                                                                   const int2 *__restrict__ work)
+// One time step.  A simulation stepped alone is one block per tile of `one` (work = null);
+// a batch's blocks step tile work[b].y of simulation work[b].x of `descs` (a device
+// work-list of (simulation, tile) pairs).  Both are this one kernel with the parameters
+// in shared memory, so that a context gives bitwise the same result alone and in a batch.
+template <typename R, bool SPLIT>
+__global__ void __launch_bounds__(STEP_THREADS, SPLIT ? SPLIT_MIN_BLOCKS(R) : STEP_MIN_BLOCKS(R))
+    k_pond_step(const __grid_constant__ SimDesc<R> one, const SimDesc<R> *__restrict__ descs,
+                const int2 *__restrict__ work)
 {
-    __shared__ DevParams sp;
-    __shared__ const R *s_in;
-    __shared__ R *s_out;
-    __shared__ DevStats *s_stats;
-    const int2 w = work[blockIdx.x];
-    if (threadIdx.x == 0) {
-        sp = descs[w.x].p;
-        s_in = descs[w.x].in;
-        s_out = descs[w.x].out;
-        s_stats = descs[w.x].stats;
+    static_assert(sizeof(SimDesc<R>) % 8 == 0, "copied by 8-byte words");
+    __shared__ SimDesc<R> d;
+    int tile = blockIdx.x;
+    const unsigned long long *src = reinterpret_cast<const unsigned long long *>(&one);
+    if (work) {
+        const int2 w = work[blockIdx.x];
+        tile = w.y;
+        src = reinterpret_cast<const unsigned long long *>(descs + w.x);
     }
+    for (int k = threadIdx.x; k < (int)(sizeof(SimDesc<R>) / 8); k += STEP_THREADS)
+        reinterpret_cast<unsigned long long *>(&d)[k] = src[k];
     __syncthreads();
     extern __shared__ __align__(128) unsigned char step_dyn_smem[];
-    R *tile = reinterpret_cast<R *>(step_dyn_smem);
-    step_tile<R, LPN>(sp, s_in, s_out, s_stats, w.y, s_in, tile,
-                      tile + (size_t)step_tile_slots(sp.tile_x, Slot<R>::stride) * Slot<R>::stride, false);
+    R *smem = reinterpret_cast<R *>(step_dyn_smem);
+    if constexpr (SPLIT) step_tile_split<R>(d.p, d.in, d.out, d.stats, tile, d.nlsrc, smem);
+    else step_tile<R>(d.p, d.in, d.out, d.stats, tile, d.nlsrc, smem);
 }
 
 }  // namespace pond
