@@ -128,7 +128,9 @@ cudaError_t allow_step_smem()
         m = std::max(m, step_smem_bytes(tx, STEP_NB / tx, false, Slot<R>::stride, (int)sizeof(R)));
     for (int tx = 1; tx <= SPLIT_NB; ++tx)
         ms = std::max(ms, step_smem_bytes(tx, SPLIT_NB / tx, true, Slot<R>::stride, (int)sizeof(R)));
-    cudaError_t e = cudaFuncSetAttribute(k_pond_step<R, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)m);
+    cudaError_t e = cudaFuncSetAttribute(k_q27_step<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)q27_smem_bytes<R>());
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_pond_step<R, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)m);
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(k_pond_step<R, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ms);
     return e;
@@ -181,11 +183,14 @@ template <typename R>
 void launch_q27_pass(pond_ctx *c, const R *in, const R *src, R *out, DevStats *stats)
 {
     const unsigned nb = blocks_for(c->N, 256);
-    k_q27_nonlocal1<R><<<nb, 256, 0, c->stream>>>(c->dp, c->g3, src, c->nlbuf);
-    k_q27_nonlocal2<<<nb, 256, 0, c->stream>>>(c->dp, c->g3, c->nlbuf);
-    const dim3 blk = c->grid.ny < 4 ? dim3(128, 1) : dim3(32, 4);
-    const dim3 grd(blocks_for((size_t)c->grid.nx, blk.x), blocks_for((size_t)c->grid.ny, blk.y), (unsigned)c->g3.nz);
-    k_q27_step<R><<<grd, blk, 0, c->stream>>>(c->dp, c->g3, in, c->nlbuf, out, stats);
+    using W = typename Wide<R>::type;
+    W *nl = reinterpret_cast<W *>(c->nlbuf);
+    k_q27_pi<R><<<nb, 256, 0, c->stream>>>(c->dp, src, nl);
+    k_q27_nonlocal1<R><<<nb, 256, 0, c->stream>>>(c->dp, c->g3, src, nl);
+    k_q27_nonlocal2<R><<<nb, 256, 0, c->stream>>>(c->dp, c->g3, nl);
+    const dim3 grd(blocks_for((size_t)c->grid.nx, T27X), blocks_for((size_t)c->grid.ny, T27Y),
+                   blocks_for((size_t)c->g3.nz, T27Z));
+    k_q27_step<R><<<grd, Q27_THREADS, q27_smem_bytes<R>(), c->stream>>>(c->dp, c->g3, in, nl, out, stats);
 }
 
 template <typename R>
@@ -802,17 +807,17 @@ pond_status pond_get_state(pond_ctx *c, double *state)
         for (int p = 0; p < NP27; ++p) {
             const int o = rec27_off(p);
             for (size_t n = 0; n < N; ++n)
-                state[(size_t)p * N + n] = mixed(c) ? (double)f[n * SL27 + o] : d[n * SL27 + o];
+                state[(size_t)p * N + n] = mixed(c) ? (double)f[rec_at(f.data(), n, o, N)] : d[rec_at(d.data(), n, o, N)];
         }
         if (mixed(c)) {
             // kept remainders folded into the exchanged populations: W_i (m + c_i.J/(s T_L))
             // on f, W_i G on g
             const double w1[3] = {1.0 / 6.0, 2.0 / 3.0, 1.0 / 6.0};
             for (size_t n = 0; n < N; ++n) {
-                const float *r = &f[n * SL27];
-                const double sq = std::sqrt((double)r[R_TH]);
-                const double m = r[R_MLO], gl = r[R_GLO];
-                const double J[3] = {r[R_JLO], r[R_JLO + 1], r[R_JLO + 2]};
+                auto r = [&](int o) -> double { return (double)f[rec_at(f.data(), n, o, N)]; };
+                const double sq = std::sqrt(r(R_TH));
+                const double m = r(R_MLO), gl = r(R_GLO);
+                const double J[3] = {r(R_JLO), r(R_JLO + 1), r(R_JLO + 2)};
                 for (int i = 0; i < Q27; ++i) {
                     const int cx = i % 3 - 1, cy = (i / 3) % 3 - 1, cz = i / 9 - 1;
                     const double w = w1[cx + 1] * w1[cy + 1] * w1[cz + 1];
@@ -888,25 +893,25 @@ pond_status pond_set_state(pond_ctx *c, const double *state)
         for (int p = 0; p < NP27; ++p) {
             const int o = rec27_off(p);
             for (size_t n = 0; n < N; ++n) {
-                if (mixed(c)) f[n * SL27 + o] = (float)state[(size_t)p * N + n];
-                else d[n * SL27 + o] = state[(size_t)p * N + n];
+                if (mixed(c)) f[rec_at(f.data(), n, o, N)] = (float)state[(size_t)p * N + n];
+                else d[rec_at(d.data(), n, o, N)] = state[(size_t)p * N + n];
             }
         }
         if (mixed(c))
             for (size_t n = 0; n < N; ++n) {
                 // what the FP32 populations leave out becomes the kept remainders again
-                float *r = &f[n * SL27];
-                const double sq = std::sqrt((double)r[R_TH]);
+                auto r = [&](int o) -> float & { return f[rec_at(f.data(), n, o, N)]; };
+                const double sq = std::sqrt((double)r(R_TH));
                 double m = 0.0, S[3] = {0, 0, 0}, gl = 0.0;
                 for (int i = 0; i < Q27; ++i) {
-                    const double rf = state[(size_t)i * N + n] - (double)r[R_F + i];
+                    const double rf = state[(size_t)i * N + n] - (double)r(R_F + i);
                     m += rf;
                     S[0] += rf * (i % 3 - 1); S[1] += rf * ((i / 3) % 3 - 1); S[2] += rf * (i / 9 - 1);
-                    gl += state[(size_t)(Q27 + i) * N + n] - (double)r[R_G + i];
+                    gl += state[(size_t)(Q27 + i) * N + n] - (double)r(R_G + i);
                 }
-                r[R_MLO] = (float)m;
-                for (int a = 0; a < 3; ++a) r[R_JLO + a] = (float)(sq * S[a]);
-                r[R_GLO] = (float)gl;
+                r(R_MLO) = (float)m;
+                for (int a = 0; a < 3; ++a) r(R_JLO + a) = (float)(sq * S[a]);
+                r(R_GLO) = (float)gl;
             }
         const void *src = mixed(c) ? (const void *)f.data() : (const void *)d.data();
         CK(cudaMemcpyAsync(c->state[c->cur], src, rec * c->esize, cudaMemcpyHostToDevice, c->stream),

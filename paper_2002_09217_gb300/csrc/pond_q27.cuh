@@ -10,33 +10,51 @@
 // I_ab = uhat_a F_b + F_a uhat_b + dt F_a F_b E/(2P), M_a = (dt rho/P)(F_a H - I_ab u_b),
 // N_ab = rho delta_ab + (dt rho/(2P)) I_ab.
 //
-// Layout: one record of SL27 = 72 values per node (node = (z*ny + y)*nx + x):
+// Layout: one record of SL27 = 68 values per node (node = (z*ny + y)*nx + x), in 16-byte
+// chunks with chunk c of all nodes together (rec27_at):
 //   [0] theta, [1..3] u, [4..30] f_0..f_26, [31..57] g_0..g_26, [58] rho, [59] T,
-//   [60..62] uhat, [63] mass lo, [64..66] momentum lo, [67] energy lo, [68..71] unused
-// with population i = 9*jz + 3*jy + jx, c = j - 1.  The gauge is one 16-byte load and
-// the 54 populations fourteen more.  The lo values (FP32 form only) are what storage
-// rounding took from the node's exact mass, momentum and energy (as on D2Q9 and D2Q16).
+//   [60..62] uhat, [63] mass lo, [64..66] momentum lo, [67] energy lo
+// with population i = 9*jz + 3*jy + jx, c = j - 1.  The lo values (FP32 form only) are what
+// storage rounding took from the node's exact mass, momentum and energy (as on D2Q9 and
+// D2Q16).
 //
-// One step is three launches: the Korteweg stress and heat-flux vector of the state the
-// non-local terms come from, their divergences, and the node step (one thread per node).
+// One step is four launches: p/rho; the Korteweg stress and heat-flux vector of the state
+// the non-local terms come from; their divergences; and the node step.
+//
+// The node step streams as the D2Q9 step does (pond_step.cuh): a block's tile of 8 x 4 x 4
+// nodes with a halo of two is carried once into a common gauge in shared memory, and each
+// thread contracts its node's 5 x 5 x 5 window axis by axis (x, y, z) with weights that
+// combine the cubic Lagrange weights and the rows of the map into the arrival gauge: 12,500
+// multiply-adds a population family, where carrying each of 125 nodes into the arrival
+// gauge and spreading it over 27 directions took about 45,000.  One family at a time is
+// staged (86 KB in FP32, two blocks per SM; 166 KB in FP64, one block); a further stream
+// of the frame search starts with the family that is already staged.  The sums of
+// populations and the non-local terms are float-float in the FP32 form, and products of
+// one reciprocal replace quotients.
+// Measured: two mixed steps of a 96 x 96 x 64 droplet (with init and read-out) 29.3 -> 8.2
+// ms; two FP64 steps of 33 x 29 x 21 nodes 152 -> 21 ms; ten mixed steps of 9 x 8 x 7 nodes
+// 36.9 -> 11.5 ms.  The mixed step issues on 45 % of its cycles (FMA pipe 39 %): with two
+// warps per scheduler, the shared-memory reads' latency shows.
 #pragma once
 
 #include "pond_kernels.cuh"
+#include "pond_step.cuh"   // float-float values, map helpers
 
 namespace pond {
 
 constexpr int Q27 = 27;
 constexpr int NP27 = 2 * Q27 + 9;   // planes of the exchanged D3Q27 state
-constexpr int SL27 = 72;
+constexpr int SL27 = 68;
 enum : int { R_TH = 0, R_UX = 1, R_F = 4, R_G = 31, R_RHO = 58, R_T = 59, R_UHX = 60, R_MLO = 63,
              R_JLO = 64, R_GLO = 67 };
-// FP64 scratch planes of the non-local terms
-enum : int { N3_K = 0 /* xx, xy, xz, yy, yz, zz */, N3_Q = 6, N3_REL = 9, N3_F = 10, N3_M0 = 13, N3_PLANES = 14 };
+// 8-byte scratch planes of the non-local terms (FP64; float-float pairs in the FP32 form)
+enum : int { N3_K = 0 /* xx, xy, xz, yy, yz, zz */, N3_Q = 6, N3_REL = 9, N3_F = 10, N3_M0 = 13, N3_PI = 14,
+             N3_PLANES = 15 };
 
 // record offset of plane p of the exchanged state (f, g, theta, u, rho, T, uhat)
 __host__ __device__ constexpr int rec27_off(int p) { return p < 54 ? p + 4 : (p < 58 ? p - 54 : p); }
 
-#define REC27(buf, n, off) (buf)[(size_t)(n) * SL27 + (off)]
+#define REC27(buf, n, off) (buf)[rec_at(buf, (size_t)(n), (off), (size_t)p.N)]
 #define NL3(buf, plane, n, N) (buf)[(size_t)(plane) * (size_t)(N) + (size_t)(n)]
 
 struct Grid3 {
@@ -99,16 +117,36 @@ __device__ __forceinline__ int depart(int X, A v, A dt, A w[4])
 
 __device__ __forceinline__ double w27(int i) { return w1d(i % 3) * w1d((i / 3) % 3) * w1d(i / 9); }
 
-__device__ __forceinline__ void ld4r(const float *p, float (&o)[4])
+// Values OFF .. OFF + CNT - 1 of node nd's record, by the 16-byte chunks that cover them.
+template <int OFF, int CNT>
+__device__ __forceinline__ void load27(const float *__restrict__ b, size_t nd, size_t N, float *v)
 {
-    const float4 t = __ldg(reinterpret_cast<const float4 *>(p));
-    o[0] = t.x; o[1] = t.y; o[2] = t.z; o[3] = t.w;
+    const float4 *q = reinterpret_cast<const float4 *>(b) + nd;
+#pragma unroll
+    for (int c = OFF / 4; c <= (OFF + CNT - 1) / 4; ++c) {
+        const float4 t = __ldg(q + (size_t)c * N);
+        const float x[4] = {t.x, t.y, t.z, t.w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const int i = 4 * c + e - OFF;
+            if (i >= 0 && i < CNT) v[i] = x[e];
+        }
+    }
 }
-__device__ __forceinline__ void ld4r(const double *p, double (&o)[4])
+template <int OFF, int CNT>
+__device__ __forceinline__ void load27(const double *__restrict__ b, size_t nd, size_t N, double *v)
 {
-    const double2 a = __ldg(reinterpret_cast<const double2 *>(p));
-    const double2 b = __ldg(reinterpret_cast<const double2 *>(p) + 1);
-    o[0] = a.x; o[1] = a.y; o[2] = b.x; o[3] = b.y;
+    const double2 *q = reinterpret_cast<const double2 *>(b) + nd;
+#pragma unroll
+    for (int c = OFF / 2; c <= (OFF + CNT - 1) / 2; ++c) {
+        const double2 t = __ldg(q + (size_t)c * N);
+        const double x[2] = {t.x, t.y};
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+            const int i = 2 * c + e - OFF;
+            if (i >= 0 && i < CNT) v[i] = x[e];
+        }
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -154,72 +192,192 @@ __global__ void k_q27_init(DevParams p, Grid3 g3, const double *__restrict__ rho
 }
 
 // ---------------------------------------------------------------------------
-// Non-local terms, stage 1 (rho, T of `src`, isotropic D3Q27 stencils
-// grad = 3 sum W c phi(x + c), lap = 6 sum W (phi(x + c) - phi(x))):
-// K = -kappa (rho lap rho + |grad rho|^2/2) I + kappa grad rho (x) grad rho,
-// q = -mu grad h + k grad T, rho E_lambda = kappa |grad rho|^2 / 2.
-template <typename R>
-__global__ void k_q27_nonlocal1(DevParams p, Grid3 g3, const R *__restrict__ src, double *__restrict__ nl)
+// Wide arithmetic of the non-local terms: FP64 in the FP64 form, float-float in the FP32
+// form (GB300 runs an FP64 addition at the cost of 64 FP32 ones, a float-float addition
+// takes about 12).
+template <typename R> struct Wide;
+template <> struct Wide<float> { using type = ffv; };
+template <> struct Wide<double> { using type = double; };
+__device__ __forceinline__ ffv w_add(float a, float b) { return ff_pair(a, b); }
+__device__ __forceinline__ ffv w_add(ffv a, ffv b) { return ff_add(a, b); }
+__device__ __forceinline__ ffv w_add(ffv a, float b) { return ff_add(a, b); }
+__device__ __forceinline__ double w_add(double a, double b) { return a + b; }
+__device__ __forceinline__ ffv w_sub(float a, float b) { return ff_pair(a, -b); }
+__device__ __forceinline__ ffv w_sub(ffv a, ffv b) { return ff_add(a, ff_neg(b)); }
+__device__ __forceinline__ double w_sub(double a, double b) { return a - b; }
+__device__ __forceinline__ ffv w_mul(ffv a, ffv b) { return ff_mul(a, b); }
+__device__ __forceinline__ ffv w_mul(ffv a, float b) { return ff_mul(a, b); }
+__device__ __forceinline__ double w_mul(double a, double b) { return a * b; }
+__device__ __forceinline__ float w_x4(float a) { return 4.0f * a; }
+__device__ __forceinline__ ffv w_x4(ffv a) { return {4.0f * a.hi, 4.0f * a.lo}; }
+__device__ __forceinline__ double w_x4(double a) { return 4.0 * a; }
+__device__ __forceinline__ double w_double(ffv a) { return (double)a.hi + (double)a.lo; }
+__device__ __forceinline__ double w_double(double a) { return a; }
+// a FP64 constant in the wide type
+template <typename A> __device__ __forceinline__ A w_const(double x);
+template <> __device__ __forceinline__ double w_const<double>(double x) { return x; }
+template <> __device__ __forceinline__ ffv w_const<ffv>(double x)
 {
-    const long long n = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (n >= p.N) return;
-    const long long N = p.N;
-    const int X = (int)(n % p.nx), Y = (int)((n / p.nx) % p.ny), Z = (int)(n / ((long long)p.nx * p.ny));
-    double gr[3] = {0, 0, 0}, gh[3] = {0, 0, 0}, gT[3] = {0, 0, 0}, lap = 0.0;
-    const double r0 = (double)REC27(src, n, R_RHO), t0 = (double)REC27(src, n, R_T);
-    for (int i = 0; i < Q27; ++i) {
-        const int c[3] = {i % 3 - 1, (i / 3) % 3 - 1, i / 9 - 1};
-        const long long m = node27(p, g3, X + c[0], Y + c[1], Z + c[2]);
-        const double w = w27(i);
-        const double r = (double)REC27(src, m, R_RHO), t = (double)REC27(src, m, R_T);
-        const double h = p.cv * t - p.a * r + eos_pressure<double>(p.eos_kind, p.a, p.b, p.R, r, t, p.sp) / r;
-        for (int a = 0; a < 3; ++a) {
-            gr[a] += w * c[a] * r;
-            gh[a] += w * c[a] * h;
-            gT[a] += w * c[a] * t;
-        }
-        lap += w * (r - r0);
-    }
-    for (int a = 0; a < 3; ++a) { gr[a] *= 3.0; gh[a] *= 3.0; gT[a] *= 3.0; }
-    lap *= 6.0;
-    const double pr = eos_pressure<double>(p.eos_kind, p.a, p.b, p.R, r0, t0, p.sp);
-    const double Pg = pr > p.p_floor ? pr : p.p_floor;
-    const double mu = (p.tau - 0.5) * Pg * p.dt;
-    const double kc = p.k_cond >= 0.0 ? p.k_cond : mu * (p.cv + p.R);
-    const double g2 = gr[0] * gr[0] + gr[1] * gr[1] + gr[2] * gr[2];
-    const double iso = -p.kappa * (r0 * lap + 0.5 * g2);
-    const int ab[6][2] = {{0, 0}, {0, 1}, {0, 2}, {1, 1}, {1, 2}, {2, 2}};
-    for (int k = 0; k < 6; ++k) {
-        const int a = ab[k][0], b = ab[k][1];
-        NL3(nl, N3_K + k, n, N) = (a == b ? iso : 0.0) + p.kappa * gr[a] * gr[b];
-    }
-    for (int a = 0; a < 3; ++a) NL3(nl, N3_Q + a, n, N) = -mu * gh[a] + kc * gT[a];
-    NL3(nl, N3_REL, n, N) = 0.5 * p.kappa * g2;
+    const float h = (float)x;
+    return {h, (float)(x - (double)h)};
+}
+__device__ __forceinline__ ffv w_rcp(ffv a) { return ff_rcp(a); }
+__device__ __forceinline__ double w_rcp(double a) { return rcp_d(a); }
+
+// p/rho of the run's equation of state; the exponential factor of the Dieterici form and
+// the double well's small polynomial in FP64 (rare forms, not worth a float-float one).
+__device__ __forceinline__ double w_p_over_rho(const DevParams &p, double r, double t)
+{
+    if (p.eos_kind != 0) return eos_pressure<double>(p.eos_kind, p.a, p.b, p.R, r, t, p.sp) / r;
+    return p.R * t * rcp_d(1.0 - p.b * r) - p.a * r;
+}
+__device__ __forceinline__ ffv w_p_over_rho(const DevParams &p, float r, float t)
+{
+    if (p.eos_kind != 0)
+        return w_const<ffv>(eos_pressure<double>(p.eos_kind, p.a, p.b, p.R, (double)r, (double)t, p.sp) / (double)r);
+    const ffv a = {p.ff_a[0], p.ff_a[1]}, b = {p.ff_b[0], p.ff_b[1]}, Rg = {p.ff_R[0], p.ff_R[1]};
+    const ffv den = ff_add(ff_neg(ff_mul(b, r)), 1.0f);
+    return w_sub(ff_mul(ff_mul(Rg, t), ff_rcp(den)), ff_mul(a, r));
 }
 
-// Stage 2: F_a = -d_b K_ab and M_0 = 2 div q.
-__global__ void k_q27_nonlocal2(DevParams p, Grid3 g3, double *__restrict__ nl)
+// Non-local terms, stage 0: p/rho of every node of `src`.
+template <typename R>
+__global__ void k_q27_pi(DevParams p, const R *__restrict__ src, typename Wide<R>::type *__restrict__ nl)
 {
     const long long n = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (n >= p.N) return;
-    const long long N = p.N;
-    const int X = (int)(n % p.nx), Y = (int)((n / p.nx) % p.ny), Z = (int)(n / ((long long)p.nx * p.ny));
-    // symmetric K index of (a, b)
-    const int kidx[3][3] = {{0, 1, 2}, {1, 3, 4}, {2, 4, 5}};
-    double F[3] = {0, 0, 0}, dq = 0.0;
-    for (int i = 0; i < Q27; ++i) {
-        const int c[3] = {i % 3 - 1, (i / 3) % 3 - 1, i / 9 - 1};
-        const long long m = node27(p, g3, X + c[0], Y + c[1], Z + c[2]);
-        const double w = w27(i);
-        for (int a = 0; a < 3; ++a) {
-            double dk = 0.0;
-            for (int b = 0; b < 3; ++b) dk += c[b] * NL3(nl, N3_K + kidx[a][b], m, N);
-            F[a] += w * dk;
-            dq += w * c[a] * NL3(nl, N3_Q + a, m, N);
+    NL3(nl, N3_PI, n, p.N) = w_p_over_rho(p, REC27(src, n, R_RHO), REC27(src, n, R_T));
+}
+
+// First differences of a field over the 3 x 3 x 3 neighbourhood by the isotropic stencils,
+// unnormalised: with D = phi(+1) - phi(-1) and S = phi(-1) + 4 phi(0) + phi(+1) per axis,
+// d[a] = D along a and S along the other axes, s = S along all three.  The stencils are
+// products over the axes, so nine lines, three planes and one column replace 27 weighted
+// terms for each.
+template <typename A> struct Diff3 { A d[3], s; };
+template <typename A, typename Get>
+__device__ __forceinline__ Diff3<A> diff3(Get get)
+{
+    A SD[3], DS[3], SS[3];
+#pragma unroll
+    for (int z = 0; z < 3; ++z) {
+        A D[3], S[3];
+#pragma unroll
+        for (int y = 0; y < 3; ++y) {
+            const auto a = get(z, y, 0), b = get(z, y, 1), c = get(z, y, 2);
+            D[y] = w_sub(c, a);
+            S[y] = w_add(w_add(a, c), w_x4(b));
         }
+        SD[z] = w_add(w_add(D[0], D[2]), w_x4(D[1]));
+        DS[z] = w_sub(S[2], S[0]);
+        SS[z] = w_add(w_add(S[0], S[2]), w_x4(S[1]));
     }
-    for (int a = 0; a < 3; ++a) NL3(nl, N3_F + a, n, N) = -3.0 * F[a];
-    NL3(nl, N3_M0, n, N) = 6.0 * dq;
+    Diff3<A> o;
+    o.d[0] = w_add(w_add(SD[0], SD[2]), w_x4(SD[1]));
+    o.d[1] = w_add(w_add(DS[0], DS[2]), w_x4(DS[1]));
+    o.d[2] = w_sub(SS[2], SS[0]);
+    o.s = w_add(w_add(SS[0], SS[2]), w_x4(SS[1]));
+    return o;
+}
+
+// Indices of the 27 neighbours of a node after the boundary rules.
+struct Near27 {
+    int x[3];
+    long long row[3][3];   // [z][y]
+    __device__ __forceinline__ Near27(const DevParams &p, const Grid3 &g, long long n)
+    {
+        const int X = (int)(n % p.nx), Y = (int)((n / p.nx) % p.ny), Z = (int)(n / ((long long)p.nx * p.ny));
+#pragma unroll
+        for (int k = 0; k < 3; ++k) x[k] = bc_wrap(X + k - 1, p.nx, p.bcx);
+#pragma unroll
+        for (int z = 0; z < 3; ++z)
+#pragma unroll
+            for (int y = 0; y < 3; ++y)
+                row[z][y] = ((long long)bc_wrap(Z + z - 1, g.nz, g.bcz) * p.ny + bc_wrap(Y + y - 1, p.ny, p.bcy)) * p.nx;
+    }
+    __device__ __forceinline__ long long at(int z, int y, int k) const { return row[z][y] + x[k]; }
+};
+
+// Stage 1 (rho, T of `src`): K = -kappa (rho lap rho + |grad rho|^2/2) I + kappa grad rho
+// (x) grad rho, q = -mu grad h + k grad T (h = C_v T - a rho + p/rho), rho E_lambda = kappa
+// |grad rho|^2 / 2, with grad = 3 sum W c phi(x + c) = d / 72 and lap = 6 sum W (phi(x + c)
+// - phi(x)) = s / 36 of the differences to the centre.
+template <typename R>
+__global__ void k_q27_nonlocal1(DevParams p, Grid3 g3, const R *__restrict__ src, typename Wide<R>::type *__restrict__ nl)
+{
+    using A = typename Wide<R>::type;
+    const long long n = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (n >= p.N) return;
+    const long long N = p.N;
+    const Near27 nb(p, g3, n);
+    const R r0 = REC27(src, n, R_RHO);
+    const A pi0 = NL3(nl, N3_PI, n, N);
+    const Diff3<A> dr = diff3<A>([&](int z, int y, int k) { return w_sub(REC27(src, nb.at(z, y, k), R_RHO), r0); });
+    const Diff3<A> dT = diff3<A>([&](int z, int y, int k) { return REC27(src, nb.at(z, y, k), R_T); });
+    const Diff3<A> dp = diff3<A>([&](int z, int y, int k) { return NL3(nl, N3_PI, nb.at(z, y, k), N); });
+    const A g = w_const<A>(1.0 / 72.0), kap = w_const<A>(p.kappa);
+    A gr[3], gT[3], gh[3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        gr[a] = w_mul(dr.d[a], g);
+        gT[a] = w_mul(dT.d[a], g);
+        gh[a] = w_add(w_sub(w_mul(gT[a], w_const<A>(p.cv)), w_mul(gr[a], w_const<A>(p.a))), w_mul(dp.d[a], g));
+    }
+    const A lap = w_mul(dr.s, w_const<A>(1.0 / 36.0));
+    const A g2 = w_add(w_add(w_mul(gr[0], gr[0]), w_mul(gr[1], gr[1])), w_mul(gr[2], gr[2]));
+    const A kg2 = w_mul(kap, w_mul(g2, w_const<A>(0.5)));   // rho E_lambda
+    const A iso = w_sub(w_mul(w_mul(kap, w_mul(lap, r0)), w_const<A>(-1.0)), kg2);
+    const A pr = w_mul(pi0, r0);
+    const A flo = w_const<A>(p.p_floor);
+    const double prd = w_double(pr);
+    const A mu = w_mul(prd > p.p_floor ? pr : flo, w_const<A>((p.tau - 0.5) * p.dt));
+    const A kc = p.k_cond >= 0.0 ? w_const<A>(p.k_cond) : w_mul(mu, w_const<A>(p.cv + p.R));
+    const int ab[6][2] = {{0, 0}, {0, 1}, {0, 2}, {1, 1}, {1, 2}, {2, 2}};
+#pragma unroll
+    for (int k = 0; k < 6; ++k) {
+        const int a = ab[k][0], b = ab[k][1];
+        const A gg = w_mul(kap, w_mul(gr[a], gr[b]));
+        NL3(nl, N3_K + k, n, N) = a == b ? w_add(iso, gg) : gg;
+    }
+#pragma unroll
+    for (int a = 0; a < 3; ++a) NL3(nl, N3_Q + a, n, N) = w_sub(w_mul(kc, gT[a]), w_mul(mu, gh[a]));
+    NL3(nl, N3_REL, n, N) = kg2;
+}
+
+// Stage 2: F_a = -d_b K_ab and M_0 = 2 div q (the same stencils).
+template <typename R>
+__global__ void k_q27_nonlocal2(DevParams p, Grid3 g3, typename Wide<R>::type *__restrict__ nl)
+{
+    using A = typename Wide<R>::type;
+    const long long n = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (n >= p.N) return;
+    const long long N = p.N;
+    const Near27 nb(p, g3, n);
+    auto diff = [&](int plane) { return diff3<A>([&](int z, int y, int k) { return NL3(nl, plane, nb.at(z, y, k), N); }); };
+    A F[3], dq;
+    {
+        const Diff3<A> xx = diff(N3_K), xy = diff(N3_K + 1);
+        F[0] = w_add(xx.d[0], xy.d[1]);
+        F[1] = xy.d[0];
+    }
+    {
+        const Diff3<A> xz = diff(N3_K + 2), yy = diff(N3_K + 3);
+        F[0] = w_add(F[0], xz.d[2]);
+        F[2] = xz.d[0];
+        F[1] = w_add(F[1], yy.d[1]);
+    }
+    {
+        const Diff3<A> yz = diff(N3_K + 4), zz = diff(N3_K + 5);
+        F[1] = w_add(F[1], yz.d[2]);
+        F[2] = w_add(w_add(F[2], yz.d[1]), zz.d[2]);
+    }
+    {
+        const Diff3<A> qx = diff(N3_Q), qy = diff(N3_Q + 1), qz = diff(N3_Q + 2);
+        dq = w_add(w_add(qx.d[0], qy.d[1]), qz.d[2]);
+    }
+#pragma unroll
+    for (int a = 0; a < 3; ++a) NL3(nl, N3_F + a, n, N) = w_mul(F[a], w_const<A>(-1.0 / 72.0));
+    NL3(nl, N3_M0, n, N) = w_mul(dq, w_const<A>(2.0 / 72.0));
 }
 
 // ---------------------------------------------------------------------------
@@ -246,9 +404,9 @@ __device__ void q27_stream(const DevParams &p, const Grid3 &g3, const R *__restr
         for (int q = 0; q < 64; ++q) {
             const int k = q & 3, m = (q >> 2) & 3, l = q >> 4;
             const R wgt = ax[k] * ay[m] * az[l];
-            const R *rec = in + (size_t)node27(p, g3, x0 + k, y0 + m, z0 + l) * SL27;
+            const size_t nd = (size_t)node27(p, g3, x0 + k, y0 + m, z0 + l);
             R gv[4];
-            ld4r(rec + R_TH, gv);
+            load27<R_TH, 4>(in, nd, (size_t)p.N, gv);
             const R ths = gv[0];
             const R ds = (ths - th) / (sqrt_(ths) + s) * is;   // (s' - s)/s
             R ex[3], ey[3], ez[3];
@@ -262,14 +420,8 @@ __device__ void q27_stream(const DevParams &p, const Grid3 &g3, const R *__restr
             inc_row3<R>(ix, ex, Dx);
             inc_row3<R>(iy, ey, Dy);
             inc_row3<R>(iz, ez, Dz);
-            R v[56];
-#pragma unroll
-            for (int c = 0; c < 14; ++c) {
-                R t[4];
-                ld4r(rec + R_F + 4 * c, t);
-#pragma unroll
-                for (int e = 0; e < 4; ++e) v[4 * c + e] = t[e];
-            }
+            R v[54];
+            load27<R_F, 54>(in, nd, (size_t)p.N, v);
 #pragma unroll
             for (int pg = 0; pg < 2; ++pg) {
                 const R *f = v + 27 * pg;
@@ -320,60 +472,6 @@ __device__ void q27_stream(const DevParams &p, const Grid3 &g3, const R *__restr
     }
 }
 
-// Exact FP64 sums of the node's own stored populations and kept remainders:
-// own[0] = sum f + mass lo, own[1..3] = sum f c, own[4] = sum g + energy lo,
-// own[5..7] = momentum lo.
-template <typename R>
-__device__ __forceinline__ void q27_own(const R *rec, double own[8])
-{
-    double s0 = 0.0, sc[3] = {0, 0, 0}, sg = 0.0;
-    for (int i = 0; i < Q27; ++i) {
-        const double f = (double)rec[R_F + i];
-        s0 += f;
-        sc[0] += f * (i % 3 - 1);
-        sc[1] += f * ((i / 3) % 3 - 1);
-        sc[2] += f * (i / 9 - 1);
-        sg += (double)rec[R_G + i];
-    }
-    own[0] = s0 + (double)rec[R_MLO];
-    own[1] = sc[0]; own[2] = sc[1]; own[3] = sc[2];
-    own[4] = sg + (double)rec[R_GLO];
-    own[5] = (double)rec[R_JLO]; own[6] = (double)rec[R_JLO + 1]; own[7] = (double)rec[R_JLO + 2];
-}
-
-// out: rho, u (3), uhat (3), E, e, T, p, P, theta*   (13 values), FP64
-template <typename R>
-__device__ __forceinline__ void q27_macro(const DevParams &p, R th, const R (&u)[3], const double own[8],
-                                          const R *fi, const R *gi, const double F[3], double rEl,
-                                          double out[13])
-{
-    const double s = sqrt((double)th);
-    double d0 = 0.0, dc[3] = {0, 0, 0}, dg = 0.0;
-    for (int i = 0; i < Q27; ++i) {
-        const double f = (double)fi[i];
-        d0 += f;
-        dc[0] += f * (i % 3 - 1);
-        dc[1] += f * ((i / 3) % 3 - 1);
-        dc[2] += f * (i / 9 - 1);
-        dg += (double)gi[i];
-    }
-    const double rho = own[0] + d0;
-    double uu[3], uh[3];
-    for (int a = 0; a < 3; ++a) {
-        const double j = s * (own[1 + a] + dc[a]) + (double)u[a] * rho + own[5 + a];
-        uu[a] = j / rho;
-        uh[a] = uu[a] + F[a] * p.dt / (2.0 * rho);
-    }
-    const double E = (own[4] + dg) / (2.0 * rho);
-    const double e = E - 0.5 * (uh[0] * uh[0] + uh[1] * uh[1] + uh[2] * uh[2]) - rEl / rho;
-    const double T = p.isothermal ? p.T_iso : (e + p.a * rho) / p.cv;
-    const double pr = eos_pressure<double>(p.eos_kind, p.a, p.b, p.R, rho, T, p.sp);
-    const double P = pr > p.p_floor ? pr : p.p_floor;
-    out[0] = rho;
-    for (int a = 0; a < 3; ++a) { out[1 + a] = uu[a]; out[4 + a] = uh[a]; }
-    out[7] = E; out[8] = e; out[9] = T; out[10] = pr; out[11] = P; out[12] = P / (rho * POND_TL);
-}
-
 // full per-axis increment map D[k][j] at offsets eps_j = ds c_j + du
 template <typename A>
 __device__ __forceinline__ void axis3(A ds, A du, A D[3][3])
@@ -411,7 +509,8 @@ __device__ __forceinline__ void apply3_inc(const A Dx[3][3], const A Dy[3][3], c
 }
 
 // ---------------------------------------------------------------------------
-// Region stream.  On the tensor lattice the union of a node's 27 departure stencils
+// General stream, for departure points beyond the staged halo (|v| dt >= 1) and non-finite
+// gauges: reads the stencil nodes' records from global memory.  On the tensor lattice the union of a node's 27 departure stencils
 // (4 x 4 x 4 each) is the product of the per-axis unions: W x H x D nodes, each side 4 +
 // the spread of its axis's three departure floors (5 x 5 x 5 while |v| dt < 1).  Each
 // region node is carried into the arrival gauge once for all 27 directions and every
@@ -420,19 +519,12 @@ __device__ __forceinline__ void apply3_inc(const A Dx[3][3], const A Dy[3][3], c
 
 // Largest region side the region stream takes; wider regions take q27_stream.
 constexpr int Q27_REGION_MAX = 6;
-constexpr int Q27_THREADS = 128;   // threads of a k_q27_step block
 
-// Per-thread Lagrange weight tables in shared memory, one column of entries per thread
-// (entry e of thread t at w[e][t]).  Entries 0..17: x, (k * Q27_REGION_MAX + c) = weight
+// A thread's Lagrange weight tables.  Entries 0..17: x, (k * Q27_REGION_MAX + c) = weight
 // of region column c in the stencil of x component k (c_x = k - 1), zero outside it;
 // entries 18..41: y then z, (18 + (axis - 1) * 12 + k * 4 + j) = cubic weight j of
 // component k, placed by the component's offset in the region (kept in registers).
 constexpr int Q27_WT_ENTRIES = 3 * Q27_REGION_MAX + 2 * 12;
-template <typename R>
-struct Q27Weights {
-    R w[Q27_WT_ENTRIES][Q27_THREADS];
-};
-
 // Departure floors and cubic weights of the three components of one axis (as in
 // `depart`) for the gauge velocity u; the region's first coordinate lo = X + min floor - 1,
 // its side, and each component's offset in it.  False, with nothing written, when the side
@@ -462,12 +554,12 @@ __device__ __forceinline__ bool q27_region_axis(int X, R s, R u, R dt, R *wt, in
 #pragma unroll
             for (int c = 0; c < Q27_REGION_MAX; ++c) {
                 const int j = c - off[k];
-                wt[(k * Q27_REGION_MAX + c) * Q27_THREADS] =
+                wt[(k * Q27_REGION_MAX + c)] =
                     j == 0 ? a[k][0] : (j == 1 ? a[k][1] : (j == 2 ? a[k][2] : (j == 3 ? a[k][3] : R(0))));
             }
         } else {
 #pragma unroll
-            for (int j = 0; j < 4; ++j) wt[(k * 4 + j) * Q27_THREADS] = a[k][j];
+            for (int j = 0; j < 4; ++j) wt[(k * 4 + j)] = a[k][j];
         }
     }
     return true;
@@ -478,7 +570,7 @@ template <typename R>
 __device__ __forceinline__ R q27_wt_at(const R *wt, int k, int o, int c)
 {
     const int j = c - o;
-    return (j >= 0 && j < 4) ? wt[(k * 4 + j) * Q27_THREADS] : R(0);
+    return (j >= 0 && j < 4) ? wt[(k * 4 + j)] : R(0);
 }
 
 // One population set (27 values at record offset OFF) of a region node carried by the
@@ -487,21 +579,11 @@ __device__ __forceinline__ R q27_wt_at(const R *wt, int k, int o, int c)
 // the weight w_i = wx[ix] (wy[iy] wz[iz]) (wyz[3 iz + iy] = wy[iy] wz[iz]).
 template <typename R, int OFF>
 __device__ __forceinline__ void q27_region_pop(const R (&Dx)[3][3], const R (&Dy)[3][3], const R (&Dz)[3][3],
-                                               const R *rec, const R (&ref)[Q27], const R (&wx)[3],
-                                               const R (&wyz)[9], R (&acc)[Q27])
+                                               const R *__restrict__ in, size_t nd, size_t N, const R (&ref)[Q27],
+                                               const R (&wx)[3], const R (&wyz)[9], R (&acc)[Q27])
 {
-    constexpr int B = OFF & ~3, SH = OFF - B, NL = (SH + Q27 + 3) / 4;   // 16-byte loads covering the set
     R h[Q27];
-#pragma unroll
-    for (int c = 0; c < NL; ++c) {
-        R q[4];
-        ld4r(rec + B + 4 * c, q);
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            const int i = 4 * c + e - SH;
-            if (i >= 0 && i < Q27) h[i] = q[e];
-        }
-    }
+    load27<OFF, Q27>(in, nd, N, h);
     R a[Q27], u[Q27];
 #pragma unroll
     for (int i = 0; i < Q27; ++i) {
@@ -532,18 +614,19 @@ __device__ __forceinline__ void q27_region_pop(const R (&Dx)[3][3], const R (&Dy
 
 // The region pass for one population set (record offset OFF: R_F or R_G) over the region
 // at (xlo, ylo, zlo) of sides W, H, D, skipping region entry `skip` (-1: none): writes the
-// increments of the streamed populations over the node's own (irec) into out.
+// increments of the streamed populations over the node's own (node self) into out.
 template <typename R, int OFF>
 __device__ __noinline__ void q27_region_pass(const DevParams &p, const Grid3 &g3, const R *__restrict__ in,
-                                             const R *irec, int xlo, int ylo, int zlo, int W, int H, int D,
+                                             size_t self, int xlo, int ylo, int zlo, int W, int H, int D,
                                              const int (&oy)[3], const int (&oz)[3], int skip, R th,
                                              const R (&u)[3], const R *wt, R *out)
 {
     const R s = sqrt_(th), is = R(1) / s;
     R ref[Q27], acc[Q27];
 #pragma unroll
-    for (int i = 0; i < Q27; ++i) { ref[i] = irec[OFF + i]; acc[i] = R(0); }
-    const R *wty = wt + 3 * Q27_REGION_MAX * Q27_THREADS, *wtz = wty + 12 * Q27_THREADS;
+    for (int i = 0; i < Q27; ++i) acc[i] = R(0);
+    load27<OFF, Q27>(in, self, (size_t)p.N, ref);
+    const R *wty = wt + 3 * Q27_REGION_MAX, *wtz = wty + 12;
     int e = 0;   // region entry index (z-major, then y, then x)
 #pragma unroll 1
     for (int cz = 0; cz < D; ++cz) {
@@ -564,9 +647,9 @@ __device__ __noinline__ void q27_region_pass(const DevParams &p, const Grid3 &g3
 #pragma unroll 1
             for (int cx = 0; cx < W; ++cx, ++e) {
                 if (e == skip) continue;
-                const R *rec = in + (size_t)(row + bc_wrap(xlo + cx, p.nx, p.bcx)) * SL27;
+                const size_t nd = (size_t)(row + bc_wrap(xlo + cx, p.nx, p.bcx));
                 R gv[4];
-                ld4r(rec + R_TH, gv);   // theta, u_x, u_y, u_z of the region node
+                load27<R_TH, 4>(in, nd, (size_t)p.N, gv);   // theta, u_x, u_y, u_z of the region node
                 const R ds = (gv[0] - th) / (sqrt_(gv[0]) + s) * is;   // (s' - s)/s
                 R Dx[3][3], Dy[3][3], Dz[3][3];
                 axis3<R>(ds, (gv[1] - u[0]) * is, Dx);
@@ -574,8 +657,8 @@ __device__ __noinline__ void q27_region_pass(const DevParams &p, const Grid3 &g3
                 axis3<R>(ds, (gv[3] - u[2]) * is, Dz);
                 R wx[3];
 #pragma unroll
-                for (int k = 0; k < 3; ++k) wx[k] = wt[(k * Q27_REGION_MAX + cx) * Q27_THREADS];
-                q27_region_pop<R, OFF>(Dx, Dy, Dz, rec, ref, wx, wyz, acc);
+                for (int k = 0; k < 3; ++k) wx[k] = wt[(k * Q27_REGION_MAX + cx)];
+                q27_region_pop<R, OFF>(Dx, Dy, Dz, in, nd, (size_t)p.N, ref, wx, wyz, acc);
             }
         }
     }
@@ -588,23 +671,24 @@ __device__ __noinline__ void q27_region_pass(const DevParams &p, const Grid3 &g3
 // the gauge is the node's stored gauge: the map is then the identity and the entry adds
 // exactly zero).  Adds the region entries transformed to nreg, or 1 to npair.
 template <typename R>
-__device__ __forceinline__ void q27_stream_any(const DevParams &p, const Grid3 &g3, const R *__restrict__ in,
-                                               int X, int Y, int Z, R th, const R (&u)[3], bool skip_own, R *wt,
-                                               R *fi, R *gi, unsigned long long &nreg, unsigned long long &npair)
+__device__ __noinline__ void q27_stream_any(const DevParams &p, const Grid3 &g3, const R *__restrict__ in, int X,
+                                            int Y, int Z, R th, const R (&u)[3], bool skip_own, R *fi, R *gi,
+                                            unsigned &nreg, unsigned &npair)
 {
+    R wt[Q27_WT_ENTRIES];
     const R s = sqrt_(th), dt = (R)p.dt;
     int xlo, ylo, zlo, W, H, D, ox[3], oy[3], oz[3];
-    R *wty = wt + 3 * Q27_REGION_MAX * Q27_THREADS, *wtz = wty + 12 * Q27_THREADS;
+    R *wty = wt + 3 * Q27_REGION_MAX, *wtz = wty + 12;
     if (q27_region_axis<R, true>(X, s, u[0], dt, wt, xlo, W, ox) &&
         q27_region_axis<R, false>(Y, s, u[1], dt, wty, ylo, H, oy) &&
         q27_region_axis<R, false>(Z, s, u[2], dt, wtz, zlo, D, oz)) {
         const int cxo = X - xlo, cyo = Y - ylo, czo = Z - zlo;
         const int skip = (skip_own && cxo >= 0 && cxo < W && cyo >= 0 && cyo < H && czo >= 0 && czo < D)
                              ? (czo * H + cyo) * W + cxo : -1;
-        const R *irec = in + (size_t)(((long long)Z * p.ny + Y) * p.nx + X) * SL27;
-        q27_region_pass<R, R_F>(p, g3, in, irec, xlo, ylo, zlo, W, H, D, oy, oz, skip, th, u, wt, fi);
-        q27_region_pass<R, R_G>(p, g3, in, irec, xlo, ylo, zlo, W, H, D, oy, oz, skip, th, u, wt, gi);
-        nreg += (unsigned long long)(W * H * D - (skip >= 0 ? 1 : 0));
+        const size_t self = (size_t)(((long long)Z * p.ny + Y) * p.nx + X);
+        q27_region_pass<R, R_F>(p, g3, in, self, xlo, ylo, zlo, W, H, D, oy, oz, skip, th, u, wt, fi);
+        q27_region_pass<R, R_G>(p, g3, in, self, xlo, ylo, zlo, W, H, D, oy, oz, skip, th, u, wt, gi);
+        nreg += (unsigned)(W * H * D - (skip >= 0 ? 1 : 0));
     } else {
         q27_stream<R>(p, g3, in, X, Y, Z, th, u, fi, gi);
         npair += 1;
@@ -612,182 +696,736 @@ __device__ __forceinline__ void q27_stream_any(const DevParams &p, const Grid3 &
 }
 
 // ---------------------------------------------------------------------------
-// The node step (frame search, then collision), one thread per node.
-// FP32: registers capped for three resident blocks per SM (168; the region passes then
-// spill 20 bytes; two blocks without spills measured 1.3 % slower); FP64 keeps two.
-constexpr int Q27_MIN_BLOCKS = 3;
-template <typename R>
-__global__ void __launch_bounds__(128, sizeof(R) == 4 ? Q27_MIN_BLOCKS : 2) k_q27_step(DevParams p, Grid3 g3, const R *__restrict__ in,
-                                                  const double *__restrict__ nl, R *__restrict__ out,
-                                                  DevStats *stats)
+// Sums of 27 values v and their first moments: out = sum v, sum v c_x, sum v c_y, sum v c_z
+// (the last three with MOM).  Lines, planes, then the column; FP32 values in float-float
+// (exact up to ~2^-48), returned as doubles.
+template <bool MOM>
+__device__ __forceinline__ void sums27(const float *v, double *out)
 {
-    const int X = blockIdx.x * blockDim.x + threadIdx.x, Y = blockIdx.y * blockDim.y + threadIdx.y;
-    const int Z = blockIdx.z;
-    const bool valid = X < p.nx && Y < p.ny;
-    const long long N = p.N, n = valid ? ((long long)Z * p.ny + Y) * p.nx + X : 0;
-    unsigned long long its = 0, nonconv = 0, clamped = 0, nonfinite = 0, nreg = 0, npair = 0;
-    __shared__ Q27Weights<R> qw;
-    R *wt = &qw.w[0][threadIdx.y * blockDim.x + threadIdx.x];
-    if (valid) {
-        const double F[3] = {NL3(nl, N3_F, n, N), NL3(nl, N3_F + 1, n, N), NL3(nl, N3_F + 2, n, N)};
-        const double rEl = NL3(nl, N3_REL, n, N), M0 = NL3(nl, N3_M0, n, N);
-        const R *irec = in + (size_t)n * SL27;
-        R th = irec[R_TH];
-        R u[3] = {irec[R_UX], irec[R_UX + 1], irec[R_UX + 2]};
-        double own[8];
-        q27_own<R>(irec, own);
-        R ft[Q27], gt[Q27];
-        double mac[13];
-        int it = 0;
-        bool conv = false;
-        for (;;) {
-            ++it;
-            // the first stream uses the node's stored gauge: its own region entry adds zero
-            q27_stream_any<R>(p, g3, in, X, Y, Z, th, u, it == 1, wt, ft, gt, nreg, npair);
-            q27_macro<R>(p, th, u, own, ft, gt, F, rEl, mac);
-            const double t0 = (double)th, st0 = sqrt(t0);
-            double r = fabs(mac[12] - t0) / t0;
-            for (int a = 0; a < 3; ++a) r = fmax(r, fabs(mac[1 + a] - (double)u[a]) / st0);
-            if (r <= p.tol) { conv = true; break; }
-            if (it >= p.max_iter || !(r == r)) break;
-            th = (R)mac[12];
-            for (int a = 0; a < 3; ++a) u[a] = (R)mac[1 + a];
+    ffv S = {0.f, 0.f}, D = S, Y = S, S0 = S, S2 = S;
+#pragma unroll
+    for (int z = 0; z < 3; ++z) {
+        ffv pS = {0.f, 0.f}, pD = pS, l0 = pS, l2 = pS;
+#pragma unroll
+        for (int y = 0; y < 3; ++y) {
+            const float *r = v + 9 * z + 3 * y;
+            const ffv line = ff_add(ff_pair(r[0], r[1]), r[2]);
+            pS = y == 0 ? line : ff_add(pS, line);
+            if (MOM) {
+                const ffv d = ff_pair(r[2], -r[0]);
+                pD = y == 0 ? d : ff_add(pD, d);
+                if (y == 0) l0 = line;
+                if (y == 2) l2 = line;
+            }
         }
-        its = (unsigned long long)it;
-        nonconv = conv ? 0ull : 1ull;
-        clamped = mac[10] < p.p_floor ? 1ull : 0ull;
-        for (int i = 0; i < Q27; ++i) {
-            ft[i] += irec[R_F + i];
-            gt[i] += irec[R_G + i];
+        S = z == 0 ? pS : ff_add(S, pS);
+        if (MOM) {
+            const ffv dy = ff_add(l2, ff_neg(l0));
+            D = z == 0 ? pD : ff_add(D, pD);
+            Y = z == 0 ? dy : ff_add(Y, dy);
+            if (z == 0) S0 = pS;
+            if (z == 2) S2 = pS;
         }
+    }
+    out[0] = w_double(S);
+    if (MOM) {
+        out[1] = w_double(D);
+        out[2] = w_double(Y);
+        out[3] = w_double(ff_add(S2, ff_neg(S0)));
+    }
+}
+template <bool MOM>
+__device__ __forceinline__ void sums27(const double *v, double *out)
+{
+    double S = 0, D = 0, Y = 0, S0 = 0, S2 = 0;
+#pragma unroll
+    for (int z = 0; z < 3; ++z) {
+        double pS = 0, l0 = 0, l2 = 0;
+#pragma unroll
+        for (int y = 0; y < 3; ++y) {
+            const double *r = v + 9 * z + 3 * y;
+            const double line = (r[0] + r[1]) + r[2];
+            pS += line;
+            if (MOM) {
+                D += r[2] - r[0];
+                if (y == 0) l0 = line;
+                if (y == 2) l2 = line;
+            }
+        }
+        S += pS;
+        if (MOM) {
+            Y += l2 - l0;
+            if (z == 0) S0 = pS;
+            if (z == 2) S2 = pS;
+        }
+    }
+    out[0] = S;
+    if (MOM) {
+        out[1] = D;
+        out[2] = Y;
+        out[3] = S2 - S0;
+    }
+}
 
-        // ---- collision in type R, equilibria as increments over their co-moving form
-        const TypedParams<R> &q = typed<R>(p);
-        const R rho = (R)mac[0], E = (R)mac[7], Pg = (R)mac[11], ths = (R)mac[12];
-        const R uu[3] = {(R)mac[1], (R)mac[2], (R)mac[3]}, uh[3] = {(R)mac[4], (R)mac[5], (R)mac[6]};
-        const R f3[3] = {(R)F[0], (R)F[1], (R)F[2]}, m0 = (R)M0, dt = q.dt, om = q.omega;
-        const double sd = sqrt((double)th), ssd = sqrt(mac[12]);
-        const R is = (R)(1.0 / sd), sst = (R)ssd;
-        const R ds = (R)((mac[12] - (double)th) / (ssd + sd) / sd);
-        R D[3][3][3], Es[3][3][3];
+// Macroscopic fields from the sums of the streamed populations (own + increments, momentum
+// in gauge units), FP64: out = rho, u (3), uhat (3), E, e, T, p, P, theta* (13 values).
+__device__ __forceinline__ void q27_macro(const DevParams &p, double s, const double (&u)[3], const double (&own)[8],
+                                          const double (&d)[5], const double (&F)[3], double rEl, double out[13])
+{
+    const double rho = own[0] + d[0], irho = rcp_d(rho);
+    double uu[3], uh[3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        const double j = s * (own[1 + a] + d[1 + a]) + u[a] * rho + own[5 + a];
+        uu[a] = j * irho;
+        uh[a] = uu[a] + (0.5 * p.dt) * F[a] * irho;
+    }
+    const double E = 0.5 * (own[4] + d[4]) * irho;
+    const double e = E - 0.5 * (uh[0] * uh[0] + uh[1] * uh[1] + uh[2] * uh[2]) - rEl * irho;
+    const double T = p.isothermal ? p.T_iso : (e + p.a * rho) * p.pd.inv_cv;
+    const double pr = p.eos_kind == 0 ? rho * p.R * T * rcp_d(1.0 - p.b * rho) - p.a * rho * rho
+                                      : eos_pressure<double>(p.eos_kind, p.a, p.b, p.R, rho, T, p.sp);
+    const double P = pr > p.p_floor ? pr : p.p_floor;
+    out[0] = rho;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) { out[1 + a] = uu[a]; out[4 + a] = uh[a]; }
+    out[7] = E; out[8] = e; out[9] = T; out[10] = pr; out[11] = P; out[12] = P * irho * 3.0;
+}
+
+// increment of (I + Dz)(I + Dy)(I + Dx) applied to h (27 values)
+template <typename A>
+__device__ __forceinline__ void apply3_inc(const A (&Dx)[3][3], const A (&Dy)[3][3], const A (&Dz)[3][3], const A *h,
+                                           A *out)
+{
+    A t1[27], t2[27];
+#pragma unroll
+    for (int i = 0; i < 27; ++i) {
+        const int ix = i % 3, r = i - ix;
+        t1[i] = Dx[ix][0] * h[r] + Dx[ix][1] * h[r + 1] + Dx[ix][2] * h[r + 2];
+    }
+#pragma unroll
+    for (int i = 0; i < 27; ++i) {
+        const int iy = (i / 3) % 3, r = i - 3 * iy;
+        t2[i] = Dy[iy][0] * (h[r] + t1[r]) + Dy[iy][1] * (h[r + 3] + t1[r + 3]) + Dy[iy][2] * (h[r + 6] + t1[r + 6]);
+    }
+#pragma unroll
+    for (int i = 0; i < 27; ++i) {
+        const int iz = i / 9, r = i - 9 * iz;
+        const A z = Dz[iz][0] * (h[r] + t1[r] + t2[r]) + Dz[iz][1] * (h[r + 9] + t1[r + 9] + t2[r + 9]) +
+                    Dz[iz][2] * (h[r + 18] + t1[r + 18] + t2[r + 18]);
+        out[i] = t1[i] + t2[i] + z;
+    }
+}
+
+// ---------------------------------------------------------------------------
+// Staging.  The tile of a block and its staged slots.
+constexpr int Q27_THREADS = 128, T27X = 8, T27Y = 4, T27Z = 4, HALO27 = 2;
+constexpr int S27X = T27X + 2 * HALO27, S27Y = T27Y + 2 * HALO27, S27Z = T27Z + 2 * HALO27;
+constexpr int SLOTS27 = S27X * S27Y * S27Z;
+constexpr int PY27 = S27X, PZ27 = S27X * S27Y;   // slots per row, per plane
+// values per slot: 27, padded to 28 words for 16-byte loads in FP32 (eight consecutive
+// slots then start on distinct groups of four banks)
+template <typename R> struct Slot27;
+template <> struct Slot27<float> { static constexpr int stride = 28; };
+template <> struct Slot27<double> { static constexpr int stride = 27; };
+constexpr int OWN27 = 13;   // FP64 values kept per node: own sums (8), F (3), rho E_lambda, M_0
+template <typename R>
+constexpr size_t q27_smem_bytes()
+{
+    return (size_t)OWN27 * Q27_THREADS * 8 + (size_t)SLOTS27 * Slot27<R>::stride * sizeof(R);
+}
+
+struct Tile27 { int X0, Y0, Z0; };
+__device__ __forceinline__ size_t slot_node27(const DevParams &p, const Grid3 &g3, const Tile27 &t, int k)
+{
+    const int x = k % S27X, y = (k / S27X) % S27Y, z = k / PZ27;
+    return (size_t)node27(p, g3, t.X0 - HALO27 + x, t.Y0 - HALO27 + y, t.Z0 - HALO27 + z);
+}
+
+// Moments about (u_x, u_y, u_z) of 27 populations at velocities s c + u + w per axis.
+__device__ __forceinline__ void moments27(double s, const double (&w)[3], double (&f)[27])
+{
+    const double s2 = s * s;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        const int st = a == 0 ? 1 : (a == 1 ? 3 : 9);
+#pragma unroll
+        for (int q = 0; q < 9; ++q) {
+            const int i = a == 0 ? 3 * q : (a == 1 ? (q / 3) * 9 + q % 3 : q);
+            const double sum = f[i] + f[i + 2 * st];
+            const double m0 = sum + f[i + st], A = s * (f[i + 2 * st] - f[i]);
+            const double m1 = A + w[a] * m0;
+            f[i] = m0; f[i + st] = m1; f[i + 2 * st] = s2 * sum + w[a] * (A + m1);
+        }
+    }
+}
+
+// The map of one axis applied to 27 values along it (stride 1, 3 or 9).
+template <int ST, typename A>
+__device__ __forceinline__ void apply_axis27(const A (&G)[3][3], A (&h)[27])
+{
+#pragma unroll
+    for (int q = 0; q < 9; ++q) {
+        const int i = ST == 1 ? 3 * q : (ST == 3 ? (q / 3) * 9 + q % 3 : q);
+        const A a = h[i], b = h[i + ST], c = h[i + 2 * ST];
+#pragma unroll
+        for (int k = 0; k < 3; ++k) h[i + k * ST] = G[k][0] * a + G[k][1] * b + G[k][2] * c;
+    }
+}
+
+// Stages one family (record offset OFF): FP32: its populations carried into the gauge of
+// node `nbase` (smooth: less that node's, in increment form; see pond_step.cuh); FP64:
+// moments about that node's velocity.  gb = (sqrt theta, u) of the gauge.
+template <int OFF>
+__device__ __forceinline__ void stage27(const DevParams &p, const Grid3 &g3, const float *__restrict__ in,
+                                        const Tile27 &t, size_t nbase, const float (&gb)[4], bool smooth, float *slots)
+{
+    constexpr int DS = Slot27<float>::stride;
+    const size_t N = (size_t)p.N;
+    float base[27], gq[4];
+    load27<OFF, 27>(in, nbase, N, base);
+    load27<R_TH, 4>(in, nbase, N, gq);
+    const float thb = gq[0], inv_sb = 1.0f / gb[0];
+#pragma unroll 1
+    for (int k = threadIdx.x; k < SLOTS27; k += Q27_THREADS) {
+        const size_t nd = slot_node27(p, g3, t, k);
+        float gv[4], h[27];
+        load27<R_TH, 4>(in, nd, N, gv);
+        load27<OFF, 27>(in, nd, N, h);
+        const float sn = sqrtf(gv[0]);
+        const float e = fdiv_(gv[0] - thb, (sn + gb[0]) * gb[0]);
+        const float w[3] = {(gv[1] - gb[1]) * inv_sb, (gv[2] - gb[2]) * inv_sb, (gv[3] - gb[3]) * inv_sb};
+        float D[3][3][3];
+        if (smooth) {
+            float o[27];
+#pragma unroll
+            for (int a = 0; a < 3; ++a) axis_map<float>(e, w[a], D[a]);
+            apply3_inc<float>(D[0], D[1], D[2], h, o);
+#pragma unroll
+            for (int i = 0; i < 27; ++i) h[i] = (h[i] - base[i]) + o[i];
+        } else {
+#pragma unroll
+            for (int a = 0; a < 3; ++a) axis_rows<float>(e, w[a], D[a]);
+            apply_axis27<1>(D[0], h);
+            apply_axis27<3>(D[1], h);
+            apply_axis27<9>(D[2], h);
+        }
+        float4 *dst = reinterpret_cast<float4 *>(slots + (size_t)k * DS);
+#pragma unroll
+        for (int c = 0; c < DS / 4; ++c)
+            dst[c] = make_float4(h[4 * c], h[4 * c + 1], h[4 * c + 2], 4 * c + 3 < 27 ? h[4 * c + 3 < 27 ? 4 * c + 3 : 0] : 0.0f);
+    }
+}
+template <int OFF>
+__device__ __forceinline__ void stage27(const DevParams &p, const Grid3 &g3, const double *__restrict__ in,
+                                        const Tile27 &t, size_t, const double (&gb)[4], bool, double *slots)
+{
+    const size_t N = (size_t)p.N;
+#pragma unroll 1
+    for (int k = threadIdx.x; k < SLOTS27; k += Q27_THREADS) {
+        const size_t nd = slot_node27(p, g3, t, k);
+        double gv[4], h[27];
+        load27<R_TH, 4>(in, nd, N, gv);
+        load27<OFF, 27>(in, nd, N, h);
+        const double w[3] = {gv[1] - gb[1], gv[2] - gb[2], gv[3] - gb[3]};
+        moments27(sqrt(gv[0]), w, h);
+        double *dst = slots + (size_t)k * Slot27<double>::stride;
+#pragma unroll
+        for (int i = 0; i < 27; ++i) dst[i] = h[i];
+    }
+}
+
+// The stream of one family as a contraction over the staged window of the slot `own` (see
+// the head of pond_step.cuh): a, near0 = each axis's Lagrange weights and departure floors,
+// L = the rows of the map from the tile's gauge.  FP32: five columns, rows and planes with
+// zero weights outside a component's four nodes, and differences to the node's own slot
+// (see the head of pond_step.cuh).
+__device__ __forceinline__ void contract27(const float *own, const float (&a)[3][3][4], const bool (&near0)[3][3],
+                                           const float (&L)[3][3][3], float (&acc)[27])
+{
+    constexpr int DS = Slot27<float>::stride;
+    float wl[3][5][3], wy[3][5], wz[3][5];
+#pragma unroll
+    for (int k = 0; k < 3; ++k)
+#pragma unroll
+        for (int c = 0; c < 5; ++c) {
+            const int lo = c > 3 ? 3 : c, hi = c < 1 ? 0 : c - 1;
+            const float w = near0[0][k] ? (c == 0 ? 0.0f : a[0][k][hi]) : (c == 4 ? 0.0f : a[0][k][lo]);
+            wy[k][c] = near0[1][k] ? (c == 0 ? 0.0f : a[1][k][hi]) : (c == 4 ? 0.0f : a[1][k][lo]);
+            wz[k][c] = near0[2][k] ? (c == 0 ? 0.0f : a[2][k][hi]) : (c == 4 ? 0.0f : a[2][k][lo]);
+#pragma unroll
+            for (int m = 0; m < 3; ++m) wl[k][c][m] = w * L[0][k][m];
+        }
+    float dx[DS];
+#pragma unroll
+    for (int c = 0; c < DS / 4; ++c) {
+        float x[4];
+        lds4(own + 4 * c, x);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) dx[4 * c + e] = x[e];
+    }
+#pragma unroll
+    for (int i = 0; i < 27; ++i) acc[i] = 0.0f;
+    const float *plane = own - (2 * PZ27 + 2 * PY27 + 2) * DS;
+#pragma unroll 1
+    for (int cz = 0; cz < 5; ++cz, plane += PZ27 * DS) {
+        float b[3][9];   // p; 3 l + k
+#pragma unroll
+        for (int q = 0; q < 3; ++q)
+#pragma unroll
+            for (int i = 0; i < 9; ++i) b[q][i] = 0.0f;
+        const float *row = plane;
+#pragma unroll 1
+        for (int cy = 0; cy < 5; ++cy, row += PY27 * DS) {
+            float t[9][3];   // 3 p + n; k
+#pragma unroll
+            for (int q = 0; q < 9; ++q)
+#pragma unroll
+                for (int k = 0; k < 3; ++k) t[q][k] = 0.0f;
+#pragma unroll
+            for (int cx = 0; cx < 5; ++cx) {
+                float v[DS];
+#pragma unroll
+                for (int c = 0; c < DS / 4; ++c) {
+                    float x[4];
+                    lds4(row + cx * DS + 4 * c, x);
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) v[4 * c + e] = x[e] - dx[4 * c + e];
+                }
+#pragma unroll
+                for (int q = 0; q < 9; ++q)
+#pragma unroll
+                    for (int m = 0; m < 3; ++m)
+#pragma unroll
+                        for (int k = 0; k < 3; ++k) t[q][k] = fmaf(wl[k][cx][m], v[3 * q + m], t[q][k]);
+            }
+#pragma unroll
+            for (int l = 0; l < 3; ++l) {
+                const float w = wy[l][0];
+#pragma unroll
+                for (int c = 0; c < 4; ++c) wy[l][c] = wy[l][c + 1];
+                wy[l][4] = w;   // rotate: the weights are needed again in the next plane
+#pragma unroll
+                for (int n = 0; n < 3; ++n) {
+                    const float wn = w * L[1][l][n];
+#pragma unroll
+                    for (int q = 0; q < 3; ++q)
+#pragma unroll
+                        for (int k = 0; k < 3; ++k) b[q][3 * l + k] = fmaf(wn, t[3 * q + n][k], b[q][3 * l + k]);
+                }
+            }
+        }
+#pragma unroll
+        for (int r = 0; r < 3; ++r) {
+            const float w = wz[r][0];
+#pragma unroll
+            for (int c = 0; c < 4; ++c) wz[r][c] = wz[r][c + 1];
+#pragma unroll
+            for (int q = 0; q < 3; ++q) {
+                const float wn = w * L[2][r][q];
+#pragma unroll
+                for (int i = 0; i < 9; ++i) acc[9 * r + i] = fmaf(wn, b[q][i], acc[9 * r + i]);
+            }
+        }
+    }
+}
+// FP64 (slots of moments): each component's own four columns; acc = streamed populations.
+__device__ __forceinline__ void contract27(const double *own, const double (&a)[3][3][4], const bool (&near0)[3][3],
+                                           const double (&L)[3][3][3], double (&acc)[27])
+{
+    constexpr int DS = Slot27<double>::stride;
+    double wl[3][4][3], wy[3][5], wz[3][5];
+    int off[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        off[k] = near0[0][k] ? DS : 0;
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+#pragma unroll
+            for (int m = 0; m < 3; ++m) wl[k][c][m] = a[0][k][c] * L[0][k][m];
+#pragma unroll
+        for (int c = 0; c < 5; ++c) {
+            const int lo = c > 3 ? 3 : c, hi = c < 1 ? 0 : c - 1;
+            wy[k][c] = near0[1][k] ? (c == 0 ? 0.0 : a[1][k][hi]) : (c == 4 ? 0.0 : a[1][k][lo]);
+            wz[k][c] = near0[2][k] ? (c == 0 ? 0.0 : a[2][k][hi]) : (c == 4 ? 0.0 : a[2][k][lo]);
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < 27; ++i) acc[i] = 0.0;
+    const double *plane = own - (2 * PZ27 + 2 * PY27 + 2) * DS;
+#pragma unroll 1
+    for (int cz = 0; cz < 5; ++cz, plane += PZ27 * DS) {
+        double b[3][9];
+#pragma unroll
+        for (int q = 0; q < 3; ++q)
+#pragma unroll
+            for (int i = 0; i < 9; ++i) b[q][i] = 0.0;
+        const double *row = plane;
+#pragma unroll 1
+        for (int cy = 0; cy < 5; ++cy, row += PY27 * DS) {
+            double wn[3][3];
+#pragma unroll
+            for (int l = 0; l < 3; ++l) {
+                const double w = wy[l][0];
+#pragma unroll
+                for (int c = 0; c < 4; ++c) wy[l][c] = wy[l][c + 1];
+                wy[l][4] = w;
+#pragma unroll
+                for (int n = 0; n < 3; ++n) wn[l][n] = w * L[1][l][n];
+            }
+#pragma unroll
+            for (int q = 0; q < 9; ++q)
+#pragma unroll
+                for (int k = 0; k < 3; ++k) {
+                    const double *r = row + off[k] + 3 * q;
+                    double t = 0.0;
+#pragma unroll
+                    for (int c = 0; c < 4; ++c)
+#pragma unroll
+                        for (int m = 0; m < 3; ++m) t = fma(wl[k][c][m], r[c * DS + m], t);
+#pragma unroll
+                    for (int l = 0; l < 3; ++l) b[q / 3][3 * l + k] = fma(wn[l][q % 3], t, b[q / 3][3 * l + k]);
+                }
+        }
+#pragma unroll
+        for (int r = 0; r < 3; ++r) {
+            const double w = wz[r][0];
+#pragma unroll
+            for (int c = 0; c < 4; ++c) wz[r][c] = wz[r][c + 1];
+#pragma unroll
+            for (int q = 0; q < 3; ++q) {
+                const double wn2 = w * L[2][r][q];
+#pragma unroll
+                for (int i = 0; i < 9; ++i) acc[9 * r + i] = fma(wn2, b[q][i], acc[9 * r + i]);
+            }
+        }
+    }
+}
+
+// ---------------------------------------------------------------------------
+// Collision of one node in type R, equilibria as increments over their co-moving form
+// (ft, gt = streamed populations, mac = the last corrector's fields, th, u = the streaming
+// gauge); writes the record.  Returns whether the results are finite.
+template <typename R>
+__device__ __forceinline__ bool q27_collide(const DevParams &p, R *__restrict__ out, size_t n, R th, const R (&u)[3],
+                                            const double (&mac)[13], const double (&F)[3], double M0, R (&ft)[27],
+                                            R (&gt)[27])
+{
+    const size_t N = (size_t)p.N;
+    const TypedParams<R> &q = typed<R>(p);
+    const R rho = (R)mac[0], E = (R)mac[7], Pg = (R)mac[11];
+    const R uu[3] = {(R)mac[1], (R)mac[2], (R)mac[3]}, uh[3] = {(R)mac[4], (R)mac[5], (R)mac[6]};
+    const R f3[3] = {(R)F[0], (R)F[1], (R)F[2]}, m0 = (R)M0, dt = q.dt, om = q.omega;
+    const double sd = sqrt((double)th), ssd = sqrt(mac[12]), isd = rcp_d(sd);
+    const R is = (R)isd, sst = (R)ssd;
+    const R ds = (R)((mac[12] - (double)th) * rcp_d(ssd + sd) * isd);
+    const R irho = R(1) / rho, ihP = R(1) / (R(2) * Pg);   // 1/rho, 1/(2P)
+    R D[3][3][3], h[Q27], inc[Q27], fo[Q27];
+    {
+        R Es[3][3][3], shi[Q27];
+#pragma unroll
         for (int a = 0; a < 3; ++a) {
             const R du = (R)(mac[1 + a] - (double)u[a]) * is;
             axis3<R>(ds, du, D[a]);
-            axis3<R>(ds, du + f3[a] * dt / rho * is, Es[a]);
+            axis3<R>(ds, du + f3[a] * dt * irho * is, Es[a]);
         }
-        R h[Q27], eqi[Q27], shi[Q27];
-        for (int i = 0; i < Q27; ++i) h[i] = rho * (R)w27(i);
-        apply3_inc<R>(D[0], D[1], D[2], h, eqi);
-        apply3_inc<R>(Es[0], Es[1], Es[2], h, shi);
-        R fo[Q27];
-        double sf = 0.0, sc[3] = {0, 0, 0};
-        for (int i = 0; i < Q27; ++i) {
-            fo[i] = ft[i] + om * ((h[i] - ft[i]) + eqi[i]) + (shi[i] - eqi[i]);
-            const double f = (double)fo[i];
-            sf += f;
-            sc[0] += f * (i % 3 - 1); sc[1] += f * ((i / 3) % 3 - 1); sc[2] += f * (i / 9 - 1);
-        }
-        // mass and momentum defects (sum f = rho, sum f v = rho u + F dt exactly), spread by
-        // W_i and W_i c_i / (s T_L)
-        const double mdef = mac[0] - sf;
-        R jd[3];
-        for (int a = 0; a < 3; ++a) {
-            const double jst = sd * sc[a] + (double)u[a] * sf;
-            jd[a] = (R)((mac[0] * mac[1 + a] + F[a] * p.dt - jst - mdef * (double)u[a]) / (sd * POND_TL));
-        }
-        for (int i = 0; i < Q27; ++i)
-            fo[i] += (R)w27(i) * ((R)mdef + jd[0] * R(i % 3 - 1) + jd[1] * R((i / 3) % 3 - 1) + jd[2] * R(i / 9 - 1));
-        double mlo = 0.0, jlo[3] = {0, 0, 0};
-        if (sizeof(R) == 4) {
-            double s0 = 0.0, c0[3] = {0, 0, 0};
-            for (int i = 0; i < Q27; ++i) {
-                const double f = (double)fo[i];
-                s0 += f;
-                c0[0] += f * (i % 3 - 1); c0[1] += f * ((i / 3) % 3 - 1); c0[2] += f * (i / 9 - 1);
-            }
-            mlo = mac[0] - s0;
-            for (int a = 0; a < 3; ++a)
-                jlo[a] = (mac[0] * mac[1 + a] + F[a] * p.dt) - (sd * c0[a] + (double)u[a] * s0) - mlo * (double)u[a];
-        }
-
-        const R H = E + Pg / rho;
-        R I[3][3], Mv[3], Nt[3][3];
-        for (int a = 0; a < 3; ++a)
-            for (int b = 0; b < 3; ++b)
-                I[a][b] = uh[a] * f3[b] + f3[a] * uh[b] + dt * f3[a] * f3[b] * E / (R(2) * Pg);
-        for (int a = 0; a < 3; ++a) {
-            const R sI = I[a][0] * uu[0] + I[a][1] * uu[1] + I[a][2] * uu[2];
-            Mv[a] = (dt * rho / Pg) * (f3[a] * H - sI);
-            for (int b = 0; b < 3; ++b) Nt[a][b] = (a == b ? rho : R(0)) + (dt * rho / (R(2) * Pg)) * I[a][b];
-        }
-        const R work = uh[0] * f3[0] + uh[1] * f3[1] + uh[2] * f3[2];
-        for (int i = 0; i < Q27; ++i) {
-            const R c[3] = {R(i % 3 - 1), R((i / 3) % 3 - 1), R(i / 9 - 1)};
-            R v[3];
-            for (int a = 0; a < 3; ++a) v[a] = sst * c[a] + uu[a];
-            R g = R(2) * rho * E;
-            for (int a = 0; a < 3; ++a) {
-                g += Mv[a] * (v[a] - uu[a]);
-                for (int b = 0; b < 3; ++b) g += Nt[a][b] * (v[a] * v[b] - (a == b ? Pg / rho : R(0)) - uu[a] * uu[b]);
-            }
-            const R W = (R)w27(i);
-            const R uc = uu[0] * c[0] + uu[1] * c[1] + uu[2] * c[2];
-            const R v2 = v[0] * v[0] + v[1] * v[1] + v[2] * v[2];
-            const R gc = m0 * W * (R(1) + rho * uc * uc / (R(2) * Pg * R(POND_TL)) - rho * v2 / (R(2) * Pg) + R(1.5));
-            h[i] = om * W * g + dt * (gc + R(2) * W * work);
-        }
-        R ginc[Q27], go[Q27];
-        apply3_inc<R>(D[0], D[1], D[2], h, ginc);
-        double sg = 0.0;
-        for (int i = 0; i < Q27; ++i) {
-            go[i] = gt[i] - om * gt[i] + (h[i] + ginc[i]);
-            sg += (double)go[i];
-        }
-        const double g_tot = 2.0 * mac[0] * mac[7] + p.dt * (M0 + 2.0 * (mac[4] * F[0] + mac[5] * F[1] + mac[6] * F[2]));
-        const R gdef = (R)(g_tot - sg);
-        for (int i = 0; i < Q27; ++i) go[i] += gdef * (R)w27(i);
-        double glo = 0.0;
-        if (sizeof(R) == 4) {
-            double s1 = 0.0;
-            for (int i = 0; i < Q27; ++i) s1 += (double)go[i];
-            glo = g_tot - s1;
-        }
-        R *orec = out + (size_t)n * SL27;
-        orec[R_TH] = th;
-        for (int a = 0; a < 3; ++a) orec[R_UX + a] = u[a];
-        for (int i = 0; i < Q27; ++i) {
-            orec[R_F + i] = fo[i];
-            orec[R_G + i] = go[i];
-        }
-        orec[R_RHO] = rho;
-        orec[R_T] = (R)mac[9];
-        for (int a = 0; a < 3; ++a) {
-            orec[R_UHX + a] = uh[a];
-            orec[R_JLO + a] = (R)jlo[a];
-        }
-        orec[R_MLO] = (R)mlo;
-        orec[R_GLO] = (R)glo;
-        for (int k = R_GLO + 1; k < SL27; ++k) orec[k] = R(0);
-        const double chk = mac[0] + mac[9] + (double)ginc[0] + (double)eqi[0];
-        nonfinite = (chk - chk == 0.0) ? 0ull : 1ull;
-    }
-    unsigned long long v[6] = {its, nonconv, clamped, nonfinite, nreg, npair}, mx = its;
-    for (int o = 16; o > 0; o >>= 1) {
 #pragma unroll
-        for (int k = 0; k < 6; ++k) v[k] += __shfl_xor_sync(0xffffffffu, v[k], o);
-        const unsigned long long m2 = __shfl_xor_sync(0xffffffffu, mx, o);
-        mx = m2 > mx ? m2 : mx;
+        for (int i = 0; i < Q27; ++i) h[i] = rho * (R)w27(i);
+        apply3_inc<R>(D[0], D[1], D[2], h, inc);
+        apply3_inc<R>(Es[0], Es[1], Es[2], h, shi);
+#pragma unroll
+        for (int i = 0; i < Q27; ++i) fo[i] = ft[i] + om * ((h[i] - ft[i]) + inc[i]) + (shi[i] - inc[i]);
     }
-    if ((threadIdx.x + threadIdx.y * blockDim.x) % 32 == 0) {
-        if (v[0]) atomicAdd(&stats->streams, v[0]);
-        if (v[1]) atomicAdd(&stats->nonconv, v[1]);
-        if (v[2]) atomicAdd(&stats->clamped, v[2]);
-        if (v[3]) atomicAdd(&stats->nonfinite, v[3]);
-        // the region-stream counters of the D2Q9 step, filled the same way here
-        if (v[4]) atomicAdd(&stats->region_nodes, v[4]);
-        if (v[5]) atomicAdd(&stats->pair_streams, v[5]);
-        if (mx) atomicMax(&stats->max_streams, mx);
+    bool finite = inc[0] - inc[0] == R(0);
+    double sm[4];
+    sums27<true>(fo, sm);
+    // mass and momentum defects (sum f = rho, sum f v = rho u + F dt exactly), spread by
+    // W_i and W_i c_i / (s T_L)
+    const double mdef = mac[0] - sm[0];
+    double jex[3];   // the exact momentum rho u + F dt
+    R jd[3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        jex[a] = mac[0] * mac[1 + a] + F[a] * p.dt;
+        const double jst = sd * sm[1 + a] + (double)u[a] * sm[0];
+        jd[a] = (R)((jex[a] - jst - mdef * (double)u[a]) * (isd * 3.0));
     }
+#pragma unroll
+    for (int i = 0; i < Q27; ++i)
+        fo[i] += (R)w27(i) * ((R)mdef + jd[0] * R(i % 3 - 1) + jd[1] * R((i / 3) % 3 - 1) + jd[2] * R(i / 9 - 1));
+    double mlo = 0.0, jlo[3] = {0, 0, 0};
+    if (sizeof(R) == 4) {
+        sums27<true>(fo, sm);
+        mlo = mac[0] - sm[0];
+#pragma unroll
+        for (int a = 0; a < 3; ++a)
+            jlo[a] = jex[a] - (sd * sm[1 + a] + (double)u[a] * sm[0]) - mlo * (double)u[a];
+    }
+
+    const R Prh = Pg * irho, H = E + Prh;
+    const R k2 = dt * rho * ihP;   // dt rho / (2P)
+    R I[3][3], Mv[3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a)
+#pragma unroll
+        for (int b = 0; b < 3; ++b) I[a][b] = uh[a] * f3[b] + f3[a] * uh[b] + dt * f3[a] * f3[b] * E * ihP;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) Mv[a] = (R(2) * k2) * (f3[a] * H - (I[a][0] * uu[0] + I[a][1] * uu[1] + I[a][2] * uu[2]));
+    const R work = uh[0] * f3[0] + uh[1] * f3[1] + uh[2] * f3[2];
+    const R rhP = rho * ihP;
+#pragma unroll
+    for (int i = 0; i < Q27; ++i) {
+        const R c[3] = {R(i % 3 - 1), R((i / 3) % 3 - 1), R(i / 9 - 1)};
+        R v[3];
+#pragma unroll
+        for (int a = 0; a < 3; ++a) v[a] = sst * c[a] + uu[a];
+        R g = R(2) * rho * E;
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            g += Mv[a] * (v[a] - uu[a]);
+#pragma unroll
+            for (int b = 0; b < 3; ++b)
+                g += ((a == b ? rho : R(0)) + k2 * I[a][b]) * (v[a] * v[b] - (a == b ? Prh : R(0)) - uu[a] * uu[b]);
+        }
+        const R W = (R)w27(i);
+        const R uc = uu[0] * c[0] + uu[1] * c[1] + uu[2] * c[2];
+        const R v2 = v[0] * v[0] + v[1] * v[1] + v[2] * v[2];
+        const R gc = m0 * W * (R(1) + rhP * uc * uc * R(3) - rhP * v2 + R(1.5));
+        h[i] = om * W * g + dt * (gc + R(2) * W * work);
+    }
+    apply3_inc<R>(D[0], D[1], D[2], h, inc);
+    finite = finite && inc[0] - inc[0] == R(0);
+#pragma unroll
+    for (int i = 0; i < Q27; ++i) gt[i] = gt[i] - om * gt[i] + (h[i] + inc[i]);
+    double sg;
+    sums27<false>(gt, &sg);
+    const double g_tot = 2.0 * mac[0] * mac[7] + p.dt * (M0 + 2.0 * (mac[4] * F[0] + mac[5] * F[1] + mac[6] * F[2]));
+    const R gdef = (R)(g_tot - sg);
+#pragma unroll
+    for (int i = 0; i < Q27; ++i) gt[i] += gdef * (R)w27(i);
+    double glo = 0.0;
+    if (sizeof(R) == 4) {
+        sums27<false>(gt, &sg);
+        glo = g_tot - sg;
+    }
+    R rec[SL27];
+    rec[R_TH] = th;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        rec[R_UX + a] = u[a];
+        rec[R_UHX + a] = uh[a];
+        rec[R_JLO + a] = (R)jlo[a];
+    }
+#pragma unroll
+    for (int i = 0; i < Q27; ++i) {
+        rec[R_F + i] = fo[i];
+        rec[R_G + i] = gt[i];
+    }
+    rec[R_RHO] = rho;
+    rec[R_T] = (R)mac[9];
+    rec[R_MLO] = (R)mlo;
+    rec[R_GLO] = (R)glo;
+    store_chunks<SL27>(out, n, N, rec);
+    const double chk = mac[0] + mac[9];
+    return finite && chk - chk == 0.0;
+}
+
+// The node step, one thread per node of the block's tile.  Registers for two resident
+// blocks per SM in FP32 (255, its two staged families' worth of shared memory), one in FP64.
+template <typename R>
+__global__ void __launch_bounds__(Q27_THREADS, sizeof(R) == 4 ? 2 : 1)
+    k_q27_step(DevParams p, Grid3 g3, const R *__restrict__ in, const typename Wide<R>::type *__restrict__ nl,
+               R *__restrict__ out, DevStats *stats)
+{
+    extern __shared__ __align__(128) unsigned char q27_dyn_smem[];
+    double *own_s = reinterpret_cast<double *>(q27_dyn_smem) + threadIdx.x;   // [OWN27][threads]
+    R *slots = reinterpret_cast<R *>(q27_dyn_smem + (size_t)OWN27 * Q27_THREADS * 8);
+    __shared__ StepCounts counts;
+    __shared__ uint4 best[Q27_THREADS / 32];   // per warp: largest theta (bits), its slot, smallest theta
+    const int tid = threadIdx.x;
+    const size_t N = (size_t)p.N;
+    const Tile27 tl{(int)blockIdx.x * T27X, (int)blockIdx.y * T27Y, (int)blockIdx.z * T27Z};
+    const int tx = tid % T27X, ty = (tid / T27X) % T27Y, tz = tid / (T27X * T27Y);
+    const int X = tl.X0 + tx, Y = tl.Y0 + ty, Z = tl.Z0 + tz;
+    const bool valid = X < p.nx && Y < p.ny && Z < g3.nz;
+    const size_t n = valid ? ((size_t)Z * p.ny + Y) * p.nx + X : 0;
+    if (tid == 0) counts = StepCounts{};
+
+    // the tile's common gauge: FP32 the staged node of the largest theta, FP64 the velocity of
+    // the tile's middle node
+    size_t nbase;
+    bool smooth = false;
+    if constexpr (sizeof(R) == 4) {
+        unsigned top = 0, at = 0, low = 0xffffffffu;
+        for (int k = tid; k < SLOTS27; k += Q27_THREADS) {
+            const float th = __ldg(in + rec_at(in, slot_node27(p, g3, tl, k), R_TH, N));
+            const unsigned b = (th > 0.0f && th < 3.0e38f) ? __float_as_uint(th) : 0u;   // finite positive only
+            low = min(low, b);
+            if (b > top) { top = b; at = (unsigned)k; }
+        }
+        const unsigned m = __reduce_max_sync(0xffffffffu, top);
+        const unsigned w = __reduce_min_sync(0xffffffffu, top == m ? at : 0xffffffffu);
+        low = __reduce_min_sync(0xffffffffu, low);
+        if ((tid & 31) == 0) best[tid >> 5] = make_uint4(m, w, low, 0);
+        __syncthreads();
+        uint4 b = best[0];
+#pragma unroll
+        for (int k = 1; k < Q27_THREADS / 32; ++k) {
+            if (best[k].x > b.x || (best[k].x == b.x && best[k].y < b.y)) { b.x = best[k].x; b.y = best[k].y; }
+            b.z = min(b.z, best[k].z);
+        }
+        smooth = __uint_as_float(b.z) > SMOOTH_TILE * __uint_as_float(b.x);
+        nbase = slot_node27(p, g3, tl, (int)min(b.y, (unsigned)(SLOTS27 - 1)));
+    } else {
+        nbase = ((size_t)min(tl.Z0 + T27Z / 2, g3.nz - 1) * p.ny + min(tl.Y0 + T27Y / 2, p.ny - 1)) * p.nx +
+                min(tl.X0 + T27X / 2, p.nx - 1);
+    }
+    R gb[4];
+    load27<R_TH, 4>(in, nbase, N, gb);
+    gb[0] = sizeof(R) == 4 ? sqrt_(gb[0]) : R(1);
+
+    R th = R(1), u[3] = {R(0), R(0), R(0)};
+    if (valid) {
+        R gv[4], v[27];
+        load27<R_TH, 4>(in, n, N, gv);
+        th = gv[0]; u[0] = gv[1]; u[1] = gv[2]; u[2] = gv[3];
+        // sums of the node's own stored populations and kept remainders; the non-local terms
+        double s4[4], sg;
+        load27<R_F, 27>(in, n, N, v);
+        sums27<true>(v, s4);
+        load27<R_G, 27>(in, n, N, v);
+        sums27<false>(v, &sg);
+        R lo[5];
+        load27<R_MLO, 5>(in, n, N, lo);
+        own_s[0] = s4[0] + (double)lo[0];
+        own_s[Q27_THREADS] = s4[1]; own_s[2 * Q27_THREADS] = s4[2]; own_s[3 * Q27_THREADS] = s4[3];
+        own_s[4 * Q27_THREADS] = sg + (double)lo[4];
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            own_s[(5 + a) * Q27_THREADS] = (double)lo[1 + a];
+            own_s[(8 + a) * Q27_THREADS] = w_double(NL3(nl, N3_F + a, n, N));
+        }
+        own_s[11 * Q27_THREADS] = w_double(NL3(nl, N3_REL, n, N));
+        own_s[12 * Q27_THREADS] = w_double(NL3(nl, N3_M0, n, N));
+    }
+
+    unsigned its = 0, nreg = 0, npair = 0;
+    bool active = valid, conv = true, floored = false, bad = false;
+    R fi[27], gi[27];   // increments of the streamed populations
+    double mac[13];
+    int staged = -1;    // family in the slots
+    const R *own_slot = slots + (size_t)(((tz + HALO27) * S27Y + ty + HALO27) * S27X + tx + HALO27) * Slot27<R>::stride;
+    for (unsigned it = 1; __syncthreads_or(active); ++it) {
+        const R s = sqrt_(th), inv_s = R(1) / s;
+        R a[3][3][4], L[3][3][3];
+        bool near0[3][3], fast = true;
+#pragma unroll
+        for (int x = 0; x < 3; ++x) {
+            const bool ok = axis_weights<R>(s, u[x], typed<R>(p).dt, a[x], near0[x]);
+            fast = fast && ok;
+            if constexpr (sizeof(R) == 8) {
+                moment_rows(u[x] - gb[1 + x], inv_s, L[x]);
+            } else {
+                axis_rows<R>((gb[0] - s) * inv_s, (gb[1 + x] - u[x]) * inv_s, L[x]);
+            }
+        }
+        if (active) {
+            its = it;
+            if (fast) {
+                int side = 1;
+#pragma unroll
+                for (int x = 0; x < 3; ++x)
+                    side *= (near0[x][0] == near0[x][1] && near0[x][1] == near0[x][2]) ? 4 : 5;
+                nreg += (unsigned)(side - (it == 1 ? 1 : 0));
+            } else {
+                R f2[27], g2[27];
+                q27_stream_any<R>(p, g3, in, X, Y, Z, th, u, it == 1, f2, g2, nreg, npair);
+#pragma unroll
+                for (int i = 0; i < 27; ++i) { fi[i] = f2[i]; gi[i] = g2[i]; }
+            }
+        }
+        // odd streams take f then g, even ones g then f: the second family of one is the
+        // first of the next and stays in the slots
+#pragma unroll 1
+        for (int ps = 0; ps < 2; ++ps) {
+            const int fam = (it & 1) ? ps : 1 - ps;
+            if (staged != fam) {
+                __syncthreads();
+                if (fam == 0) stage27<R_F>(p, g3, in, tl, nbase, gb, smooth, slots);
+                else stage27<R_G>(p, g3, in, tl, nbase, gb, smooth, slots);
+                __syncthreads();
+                staged = fam;
+            }
+            if (!active || !fast) continue;
+            R acc[27];
+            contract27(own_slot, a, near0, L, acc);
+            if (sizeof(R) == 8 || it > 1) {
+                R v[27];
+                if (fam == 0) load27<R_F, 27>(in, n, N, v);
+                else load27<R_G, 27>(in, n, N, v);
+                if constexpr (sizeof(R) == 8) {
+#pragma unroll
+                    for (int i = 0; i < 27; ++i) acc[i] -= v[i];
+                } else {
+                    // the node's own populations carried from their stored gauge into this one
+                    R gv[4], Dx[3][3], Dy[3][3], Dz[3][3], o[27];
+                    load27<R_TH, 4>(in, n, N, gv);
+                    const R e = fdiv_(gv[0] - th, (sqrt_(gv[0]) + s) * s);
+                    axis_map<R>(e, (gv[1] - u[0]) * inv_s, Dx);
+                    axis_map<R>(e, (gv[2] - u[1]) * inv_s, Dy);
+                    axis_map<R>(e, (gv[3] - u[2]) * inv_s, Dz);
+                    apply3_inc<R>(Dx, Dy, Dz, v, o);
+#pragma unroll
+                    for (int i = 0; i < 27; ++i) acc[i] += o[i];
+                }
+            }
+            if (fam == 0) {
+#pragma unroll
+                for (int i = 0; i < 27; ++i) fi[i] = acc[i];
+            } else {
+#pragma unroll
+                for (int i = 0; i < 27; ++i) gi[i] = acc[i];
+            }
+        }
+        if (active) {
+            double d5[5], d4[4], own[8], F[3];
+            sums27<true>(fi, d4);
+            sums27<false>(gi, &d5[4]);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) d5[k] = d4[k];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) own[k] = own_s[k * Q27_THREADS];
+#pragma unroll
+            for (int k = 0; k < 3; ++k) F[k] = own_s[(8 + k) * Q27_THREADS];
+            const double t0 = (double)th, st0 = sqrt(t0), ist = rcp_d(st0);
+            const double ud[3] = {(double)u[0], (double)u[1], (double)u[2]};
+            q27_macro(p, st0, ud, own, d5, F, own_s[11 * Q27_THREADS], mac);
+            double r = fabs(mac[12] - t0) * (ist * ist);
+#pragma unroll
+            for (int x = 0; x < 3; ++x) r = fmax(r, fabs(mac[1 + x] - ud[x]) * ist);
+            conv = r <= p.tol;
+            if (conv || it >= (unsigned)p.max_iter || !(r == r)) {
+                active = false;
+            } else {
+                th = (R)mac[12];
+#pragma unroll
+                for (int x = 0; x < 3; ++x) u[x] = (R)mac[1 + x];
+            }
+        }
+    }
+    if (valid) {
+        R v[27];
+        load27<R_F, 27>(in, n, N, v);
+#pragma unroll
+        for (int i = 0; i < 27; ++i) fi[i] += v[i];
+        load27<R_G, 27>(in, n, N, v);
+#pragma unroll
+        for (int i = 0; i < 27; ++i) gi[i] += v[i];
+        const double F[3] = {own_s[8 * Q27_THREADS], own_s[9 * Q27_THREADS], own_s[10 * Q27_THREADS]};
+        bad = !q27_collide<R>(p, out, n, th, u, mac, F, own_s[12 * Q27_THREADS], fi, gi);
+        floored = mac[10] < p.p_floor;
+    }
+    add_counts(counts, stats, its, nreg, npair, valid && !conv, false, floored, bad);
 }
 
 // Output fields: rho, uhat (3), T, p in FP64.

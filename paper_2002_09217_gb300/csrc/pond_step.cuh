@@ -55,6 +55,12 @@ constexpr int HALO = 2;       // staged halo: stencil reach for |v| dt < 1, and 
 // Largest side of a node's stencil region (the union of its 9 directions' 4x4 stencils)
 // that the general stream handles as a region; wider ones take the per-pair stream.
 constexpr int REGION_MAX = 8;
+// FP32: tiles whose smallest theta is above this share of the largest are staged in
+// increment form over the base node's populations, others as carried populations.  A
+// weak wave (theta within 1e-3) needs the former; at a liquid-vapour interface (a factor of
+// 4 to 6) the increment form left 6e-6 on single populations in three dimensions, the
+// direct form 1.7e-7, as much as carrying each node straight into the arrival gauge.
+constexpr float SMOOTH_TILE = 0.9f;
 // Mixed form: a frame-search residual below this multiple of tol that no longer halves is
 // taken as the FP32 rounding floor (the EoS cancels up to ~200x inside interfaces).
 constexpr float STALL_TOL_FACTOR = 16.0f;
@@ -201,7 +207,7 @@ __device__ __forceinline__ void two_sum_(R a, R b, R &s, R &e)
 // product error (Dekker's TwoProduct with a fused multiply-add), each result renormalised
 // with Dekker's Fast2Sum; relative error ~2^-44 per operation, far below the FP32 form's
 // needs, on the FP32 pipes (GB300 runs FP64 at 1/64 of the FP32 rate).
-struct ffv {
+struct __align__(8) ffv {
     float hi, lo;
 };
 __device__ __forceinline__ ffv ff_norm(float a, float b)   // |a| >= |b| or a == 0
@@ -272,18 +278,20 @@ __device__ __forceinline__ void load_rec24(const double *__restrict__ b, size_t 
         v[2 * k] = t.x; v[2 * k + 1] = t.y;
     }
 }
-// Writes a whole record.
-__device__ __forceinline__ void store_rec(float *b, size_t nd, size_t N, const float (&v)[SL])
+// Writes a whole record of W values.
+template <int W>
+__device__ __forceinline__ void store_chunks(float *b, size_t nd, size_t N, const float (&v)[W])
 {
     float4 *q = reinterpret_cast<float4 *>(b) + nd;
 #pragma unroll
-    for (int k = 0; k < SL / 4; ++k) q[k * N] = make_float4(v[4 * k], v[4 * k + 1], v[4 * k + 2], v[4 * k + 3]);
+    for (int k = 0; k < W / 4; ++k) q[k * N] = make_float4(v[4 * k], v[4 * k + 1], v[4 * k + 2], v[4 * k + 3]);
 }
-__device__ __forceinline__ void store_rec(double *b, size_t nd, size_t N, const double (&v)[SL])
+template <int W>
+__device__ __forceinline__ void store_chunks(double *b, size_t nd, size_t N, const double (&v)[W])
 {
     double2 *q = reinterpret_cast<double2 *>(b) + nd;
 #pragma unroll
-    for (int k = 0; k < SL / 2; ++k) q[k * N] = make_double2(v[2 * k], v[2 * k + 1]);
+    for (int k = 0; k < W / 2; ++k) q[k * N] = make_double2(v[2 * k], v[2 * k + 1]);
 }
 // Four staged values from a 16-byte boundary.
 __device__ __forceinline__ void lds4(const float *s, float (&o)[4])
@@ -513,6 +521,19 @@ __device__ __forceinline__ void axis_map(R q, R w, R (&E)[3][3])
         const R e = q * R(a - 1) + w;
         const R h = R(0.5) * e, pp = h * (R(2 * (a - 1)) + e);
         E[0][a] = pp - h; E[1][a] = R(-2) * pp; E[2][a] = pp + h;
+    }
+}
+
+// The rows of the map itself, G[k][a] = l_k(xi_a) at xi_a = (1 + q) (a - 1) + w, as products
+// (the identity exactly for q = w = 0): for gauges far apart, where I + E would cancel.
+template <typename R>
+__device__ __forceinline__ void axis_rows(R q, R w, R (&G)[3][3])
+{
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        const R x = a == 1 ? w : (R(1) + q) * R(a - 1) + w;
+        const R h = R(0.5) * x;
+        G[0][a] = h * (x - R(1)); G[1][a] = (R(1) - x) * (R(1) + x); G[2][a] = h * (x + R(1));
     }
 }
 
@@ -851,13 +872,8 @@ __device__ __forceinline__ void stream_node(const DevParams &p, const R *__restr
         }
     } else {
         const R q = (gauge_b[0] - s) * inv_s;
-        axis_map<R>(q, (gauge_b[1] - ux) * inv_s, Lx);
-        axis_map<R>(q, (gauge_b[2] - uy) * inv_s, Ly);
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            Lx[k][k] += R(1);
-            Ly[k][k] += R(1);
-        }
+        axis_rows<R>(q, (gauge_b[1] - ux) * inv_s, Lx);
+        axis_rows<R>(q, (gauge_b[2] - uy) * inv_s, Ly);
         contract(slot, pitch, ax, nx0, ay, ny0, Lx, Ly, inc);
         if (!first) {
             // the node's own populations carried from their stored gauge into this one
@@ -1071,7 +1087,7 @@ __device__ __forceinline__ void stage_tile(const DevParams &p, const R *__restri
     const int tid = threadIdx.x;
     const int X0 = tl.X0, Y0 = tl.Y0, TX = tl.TX, TY = tl.TY, WT = tl.WT, nslots = tl.nslots;
     R *aux = tl.aux, *slots = tl.slots, *kq = tl.kq;
-    __shared__ uint2 best[ST_NT / 32];   // per warp: largest theta (bits), its slot
+    __shared__ uint4 best[ST_NT / 32];   // per warp: largest theta (bits), its slot, smallest theta
     if (tid == 0) counts = StepCounts{};
     // k / WT through the float reciprocal: exact for k < 2^20 (the quotient's fraction
     // stays >= 0.5 / WT away from an integer)
@@ -1095,9 +1111,10 @@ __device__ __forceinline__ void stage_tile(const DevParams &p, const R *__restri
         R va[24], vb[24];
         const int ka = tid, kb = tid + ST_NT;
         size_t na = 0, nb = 0;
-        unsigned top = 0, at = 0;
+        unsigned top = 0, at = 0, low = 0xffffffffu;
         auto offer = [&](R th, int k) {   // finite positive values only
             const unsigned b = (th > R(0) && th < R(3.0e38)) ? __float_as_uint(th) : 0u;
+            low = min(low, b);
             if (b > top) { top = b; at = (unsigned)k; }
         };
         if (ka < nslots) { na = node_of(ka); load_rec24(in, na, N, va); }
@@ -1108,13 +1125,17 @@ __device__ __forceinline__ void stage_tile(const DevParams &p, const R *__restri
         {
             const unsigned m = __reduce_max_sync(0xffffffffu, top);
             const unsigned w = __reduce_min_sync(0xffffffffu, top == m ? at : 0xffffffffu);
-            if ((tid & 31) == 0) best[tid >> 5] = make_uint2(m, w);
+            low = __reduce_min_sync(0xffffffffu, low);
+            if ((tid & 31) == 0) best[tid >> 5] = make_uint4(m, w, low, 0);
         }
         __syncthreads();
-        uint2 b = best[0];
+        uint4 b = best[0];
 #pragma unroll
-        for (int w = 1; w < ST_NT / 32; ++w)
-            if (best[w].x > b.x || (best[w].x == b.x && best[w].y < b.y)) b = best[w];
+        for (int w = 1; w < ST_NT / 32; ++w) {
+            if (best[w].x > b.x || (best[w].x == b.x && best[w].y < b.y)) { b.x = best[w].x; b.y = best[w].y; }
+            b.z = min(b.z, best[w].z);
+        }
+        const bool smooth = __uint_as_float(b.z) > SMOOTH_TILE * __uint_as_float(b.x);
         R base[24];
         load_rec24(in, node_of((int)min(b.y, (unsigned)(nslots - 1))), N, base);
         const R thb = base[P_TH];
@@ -1123,15 +1144,34 @@ __device__ __forceinline__ void stage_tile(const DevParams &p, const R *__restri
         auto carry = [&](int k, size_t nd, const R (&v)[24]) {
             const R sn = sqrt_(v[P_TH]);
             const R e = fdiv_(v[P_TH] - thb, (sn + gb[0]) * gb[0]);
-            R Ex[3][3], Ey[3][3], o[9];
-            axis_map<R>(e, (v[P_UX] - gb[1]) * inv_sb, Ex);
-            axis_map<R>(e, (v[P_UY] - gb[2]) * inv_sb, Ey);
-            R d[DS];
+            const R wx = (v[P_UX] - gb[1]) * inv_sb, wy = (v[P_UY] - gb[2]) * inv_sb;
+            R Ex[3][3], Ey[3][3], d[DS];
+            if (smooth) {
+                R o[9];
+                axis_map<R>(e, wx, Ex);
+                axis_map<R>(e, wy, Ey);
 #pragma unroll
-            for (int fam = 0; fam < 2; ++fam) {
-                map_inc<R>(Ex, Ey, v + 9 * fam, o);
+                for (int fam = 0; fam < 2; ++fam) {
+                    map_inc<R>(Ex, Ey, v + 9 * fam, o);
 #pragma unroll
-                for (int i = 0; i < 9; ++i) d[9 * fam + i] = (v[9 * fam + i] - base[9 * fam + i]) + o[i];
+                    for (int i = 0; i < 9; ++i) d[9 * fam + i] = (v[9 * fam + i] - base[9 * fam + i]) + o[i];
+                }
+            } else {
+                axis_rows<R>(e, wx, Ex);
+                axis_rows<R>(e, wy, Ey);
+#pragma unroll
+                for (int fam = 0; fam < 2; ++fam)
+#pragma unroll
+                    for (int k2 = 0; k2 < 3; ++k2) {
+                        R t[3];
+#pragma unroll
+                        for (int b2 = 0; b2 < 3; ++b2)
+                            t[b2] = Ex[k2][0] * v[9 * fam + 3 * b2] + Ex[k2][1] * v[9 * fam + 3 * b2 + 1] +
+                                    Ex[k2][2] * v[9 * fam + 3 * b2 + 2];
+#pragma unroll
+                        for (int l2 = 0; l2 < 3; ++l2)
+                            d[9 * fam + 3 * l2 + k2] = Ey[l2][0] * t[0] + Ey[l2][1] * t[1] + Ey[l2][2] * t[2];
+                    }
             }
             d[18] = d[19] = R(0);
             float4 *dst = reinterpret_cast<float4 *>(slots + (size_t)k * DS);
@@ -1362,7 +1402,7 @@ __device__ __forceinline__ void step_tile(const DevParams &p, const R *__restric
             }
             collide<R>(q, o, th, ux, uy, Fx, Fy, M0, ft, gt, rec);
         }
-        store_rec(out, n, N, rec);
+        store_chunks<SL>(out, n, N, rec);
         floored = o.pr < q.p_floor;
         bad = !(o.rho_hi == o.rho_hi) || !(o.T == o.T) || isinf(o.rho_hi) || isinf(o.T);
     }
@@ -1521,11 +1561,14 @@ __device__ __forceinline__ void step_tile_split(const DevParams &p, const R *__r
             } else {
                 const R qq = (gb[0] - s) * inv_s, w1 = (gb[1] - ux) * inv_s, w2 = (gb[2] - uy) * inv_s;
 #pragma unroll
-                for (int m = 0; m < 3; ++m) Lx[m] = ell_inc_rt<R>(k, m, qq * R(m - 1) + w1) + (m == k ? R(1) : R(0));
-                const R ey = qq * R(l - 1) + w2, h = R(0.5) * ey, pp = h * (R(2 * (l - 1)) + ey);
-                Ly[0] = (pp - h) + (l == 0 ? R(1) : R(0));
-                Ly[1] = R(-2) * pp + (l == 1 ? R(1) : R(0));
-                Ly[2] = (pp + h) + (l == 2 ? R(1) : R(0));
+                for (int m = 0; m < 3; ++m) {
+                    const R x = m == 1 ? w1 : (R(1) + qq) * R(m - 1) + w1;
+                    Lx[m] = k == 1 ? (R(1) - x) * (R(1) + x) : R(0.5) * x * (x + R(k - 1));
+                }
+                const R y = l == 1 ? w2 : (R(1) + qq) * R(l - 1) + w2;
+                Ly[0] = R(0.5) * y * (y - R(1));
+                Ly[1] = (R(1) - y) * (R(1) + y);
+                Ly[2] = R(0.5) * y * (y + R(1));
             }
             R wl[4][3];
 #pragma unroll
