@@ -121,18 +121,31 @@ size_t step_smem(const pond_ctx *c)
 // Lets the step kernels of type R use more than the default 48 KB of dynamic shared
 // memory on the current device (idempotent; not a stream operation).
 template <typename R>
-cudaError_t allow_step_smem()
+cudaError_t allow_step_smem(int device)
 {
+    // set once per device (a context's creation need not pay for it again)
+    static std::mutex mutex;
+    static std::vector<bool> done;
+    std::lock_guard<std::mutex> lock(mutex);
+    if (device < (int)done.size() && done[device]) return cudaSuccess;
     size_t m = 0, ms = 0;
     for (int tx = 1; tx <= STEP_NB; tx *= 2)
         m = std::max(m, step_smem_bytes(tx, STEP_NB / tx, false, Slot<R>::stride, (int)sizeof(R)));
     for (int tx = 1; tx <= SPLIT_NB; ++tx)
         ms = std::max(ms, step_smem_bytes(tx, SPLIT_NB / tx, true, Slot<R>::stride, (int)sizeof(R)));
-    cudaError_t e = cudaFuncSetAttribute(k_q27_step<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)q27_smem_bytes<R>());
+    size_t mq = 0;
+    for (int tx = 1; tx <= STEP_NB; tx *= 2) mq = std::max(mq, q16_smem_bytes<R>(tx, STEP_NB / tx));
+    cudaError_t e = cudaFuncSetAttribute(k_q16_step<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mq);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_q27_step<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)q27_smem_bytes<R>());
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(k_pond_step<R, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)m);
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(k_pond_step<R, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ms);
+    if (e == cudaSuccess) {
+        if (device >= (int)done.size()) done.resize(device + 1, false);
+        done[device] = true;
+    }
     return e;
 }
 
@@ -151,12 +164,12 @@ void launch_q16_pass(pond_ctx *c, const R *in, const R *src, R *out, DevStats *s
                      cudaStream_t strm)
 {
     const unsigned nb = blocks_for(c->N, 256);
-    k_q16_nonlocal1<R><<<nb, 256, 0, strm>>>(c->dp, src, c->nlbuf);
-    k_q16_nonlocal2<<<nb, 256, 0, strm>>>(c->dp, c->nlbuf);
-    // 32 x 4 node patches (128 x 1 strips on grids of fewer than 4 rows)
-    const dim3 blk = c->grid.ny < 4 ? dim3(128, 1) : dim3(32, 4);
-    const dim3 grd(blocks_for((size_t)c->grid.nx, blk.x), blocks_for((size_t)c->grid.ny, blk.y));
-    k_q16_step<R><<<grd, blk, 0, strm>>>(c->dp, in, c->nlbuf, out, stats);
+    using W = typename Wide<R>::type;
+    W *nl = reinterpret_cast<W *>(c->nlbuf);
+    k_q16_nonlocal1<R><<<nb, 256, 0, strm>>>(c->dp, src, nl);
+    k_q16_nonlocal2<R><<<nb, 256, 0, strm>>>(c->dp, nl);
+    k_q16_step<R><<<(unsigned)step_tiles(c), STEP_THREADS, q16_smem_bytes<R>(c->dp.tile_x, c->dp.tile_y), strm>>>(
+        c->dp, in, nl, out, stats);
 }
 
 template <typename R>
@@ -540,7 +553,9 @@ pond_status pond_create(const pond_grid *grid, const pond_lattice *lattice, cons
     if (c->lattice == POND_D3Q27) c->g3 = Grid3{grid->nz, grid->bc_z};
     c->esize = opts->precision == POND_MIXED ? sizeof(float) : sizeof(double);
     // Work split of the D2Q9 step: one thread per node (8) or nine lanes per node (16).
+    // (The other lattices' kernels have one split and share the tile rule.)
     c->lanes = opts->lanes_per_node ? opts->lanes_per_node : (c->N <= split_max_nodes(opts->precision) ? 16 : 8);
+    if (c->lattice != POND_D2Q9) c->lanes = 8;
     // Its tile: TX x TY nodes of STEP_NB (SPLIT_NB) nodes, by default no taller than the grid
     // and otherwise 16 x 8 (4 x 3)
     int tile_x = opts->tile_x, tile_y;
@@ -556,7 +571,7 @@ pond_status pond_create(const pond_grid *grid, const pond_lattice *lattice, cons
     }
     cudaError_t e = cudaGetDevice(&c->device);
     if (e == cudaSuccess)
-        e = opts->precision == POND_MIXED ? allow_step_smem<float>() : allow_step_smem<double>();
+        e = opts->precision == POND_MIXED ? allow_step_smem<float>(c->device) : allow_step_smem<double>(c->device);
     if (e != cudaSuccess) {
         delete c;
         return POND_ECUDA;
@@ -580,7 +595,7 @@ pond_status pond_create(const pond_grid *grid, const pond_lattice *lattice, cons
         out[1] = (float)(x - (double)out[0]);
     };
     split(d.a, d.ff_a); split(d.b, d.ff_b); split(d.R, d.ff_R); split(d.pd.inv_cv, d.ff_icv);
-    split(d.p_floor, d.ff_pfl);
+    split(d.p_floor, d.ff_pfl); split(d.dt, d.ff_dt);
     d.tol_f = (float)d.tol;
     d.eos_kind = c->eos.kind == POND_DIETERICI ? 2 : (c->eos.kind == POND_SIMPLIFIED ? 3 : 0);
     d.sp[0] = c->eos.beta; d.sp[1] = c->eos.rho_l; d.sp[2] = c->eos.rho_v; d.sp[3] = c->eos.p0;
@@ -839,7 +854,7 @@ pond_status pond_get_state(pond_ctx *c, double *state)
         CK(cudaStreamSynchronize(c->stream), "cudaStreamSynchronize");
         for (int p = 0; p < NP16; ++p)
             for (size_t n = 0; n < N; ++n)
-                state[(size_t)p * N + n] = mixed(c) ? (double)f[n * SLQ + p] : d[n * SLQ + p];
+                state[(size_t)p * N + n] = mixed(c) ? (double)f[rec_at(f.data(), n, p, N)] : d[rec_at(d.data(), n, p, N)];
         if (mixed(c)) {
             // the kept remainders go into the exchanged populations: mass and momentum as
             // W_i (m + (c_ix J_x + c_iy J_y)/s) on f (its sum is m, its momentum m u + J),
@@ -847,9 +862,9 @@ pond_status pond_get_state(pond_ctx *c, double *state)
             double cq[4], wq[4];
             lattice16(cq, wq);
             for (size_t n = 0; n < N; ++n) {
-                const float *r = &f[n * SLQ];
-                const double sq = std::sqrt((double)r[Q_TH]);
-                const double m = r[Q_MLO], jx = r[Q_JXLO], jy = r[Q_JYLO], gl = r[Q_GLO];
+                auto r = [&](int o) -> double { return (double)f[rec_at(f.data(), n, o, N)]; };
+                const double sq = std::sqrt(r(Q_TH));
+                const double m = r(Q_MLO), jx = r(Q_JXLO), jy = r(Q_JYLO), gl = r(Q_GLO);
                 for (int i = 0; i < Q16; ++i) {
                     const double w = wq[i & 3] * wq[i >> 2];
                     state[(size_t)(Q_F + i) * N + n] += w * (m + (cq[i & 3] * jx + cq[i >> 2] * jy) / sq);
@@ -926,8 +941,8 @@ pond_status pond_set_state(pond_ctx *c, const double *state)
         std::vector<float> f(mixed(c) ? rec : 0, 0.0f);
         for (int p = 0; p < NP16; ++p)
             for (size_t n = 0; n < N; ++n) {
-                if (mixed(c)) f[n * SLQ + p] = (float)state[(size_t)p * N + n];
-                else d[n * SLQ + p] = state[(size_t)p * N + n];
+                if (mixed(c)) f[rec_at(f.data(), n, p, N)] = (float)state[(size_t)p * N + n];
+                else d[rec_at(d.data(), n, p, N)] = state[(size_t)p * N + n];
             }
         if (mixed(c)) {
             // what the FP32 populations leave out becomes the kept remainders again: mass
@@ -935,20 +950,20 @@ pond_status pond_set_state(pond_ctx *c, const double *state)
             double cq[4], wq[4];
             lattice16(cq, wq);
             for (size_t n = 0; n < N; ++n) {
-                float *r = &f[n * SLQ];
-                const double sq = std::sqrt((double)r[Q_TH]);
+                auto r = [&](int o) -> float & { return f[rec_at(f.data(), n, o, N)]; };
+                const double sq = std::sqrt((double)r(Q_TH));
                 double m = 0.0, sx = 0.0, sy = 0.0, gl = 0.0;
                 for (int i = 0; i < Q16; ++i) {
-                    const double rf = state[(size_t)(Q_F + i) * N + n] - (double)r[Q_F + i];
+                    const double rf = state[(size_t)(Q_F + i) * N + n] - (double)r(Q_F + i);
                     m += rf;
                     sx += rf * cq[i & 3];
                     sy += rf * cq[i >> 2];
-                    gl += state[(size_t)(Q_G + i) * N + n] - (double)r[Q_G + i];
+                    gl += state[(size_t)(Q_G + i) * N + n] - (double)r(Q_G + i);
                 }
-                r[Q_MLO] = (float)m;
-                r[Q_JXLO] = (float)(sq * sx);
-                r[Q_JYLO] = (float)(sq * sy);
-                r[Q_GLO] = (float)gl;
+                r(Q_MLO) = (float)m;
+                r(Q_JXLO) = (float)(sq * sx);
+                r(Q_JYLO) = (float)(sq * sy);
+                r(Q_GLO) = (float)gl;
             }
         }
         const void *src = mixed(c) ? (const void *)f.data() : (const void *)d.data();

@@ -60,7 +60,7 @@ struct DevParams {
     TypedParams<double> pd;
     // the FP32 form's frame-search EoS constants as (hi, lo) float pairs (hi + lo = the
     // FP64 value to ~2^-48), and its tolerance
-    float ff_a[2], ff_b[2], ff_R[2], ff_icv[2], ff_pfl[2];
+    float ff_a[2], ff_b[2], ff_R[2], ff_icv[2], ff_pfl[2], ff_dt[2];
     float tol_f;
     // equation of state: 0 van der Waals, 2 Dieterici (isothermal only); isothermal runs
     // hold T at T_iso (and ff_Tiso, its float pair)

@@ -7,29 +7,36 @@
 // G = M_lambda'^-1 M_lambda (SM "Transfer matrix") is then the product of two 4-node
 // Lagrange maps, one per axis, and keeps the sixteen moments M_mn, m, n <= 3.
 //
-// Layout: one record of SLQ = 40 values per node (node = y*nx + x), in the ABI state's
-// plane order:
+// Layout: one record of SLQ = 44 values per node (node = y*nx + x), in 16-byte chunks with
+// chunk c of all nodes together (rec_at), in the ABI state's plane order:
 //   [0..15] f_0..f_15, [16..31] g_0..g_15, [32] theta, [33] u_x, [34] u_y, [35] rho,
 //   [36] T, [37] uhat_x, [38] uhat_y, [39] mass lo, [40] momentum_x lo,
 //   [41] momentum_y lo, [42] energy lo, [43] unused
-// with population i = 4*jy + jx, c_i = (C1[jx], C1[jy]).  Each row of four populations
-// and the gauge (theta, u_x, u_y, rho) start on 16-byte boundaries (176-byte records in
-// FP32, 352 in FP64), so a stencil node is read with nine 16-byte loads (FP32) at fixed
-// offsets from one address.  The lo values (FP32 form only; zero in FP64) are what the
-// storage rounding of the populations took from the node's exact post-collision mass,
-// momentum (sum f v) and energy (sum g); the next step's moments add them back, so that
-// changes below half an ulp of the populations (the weak edge of an acoustic pulse) are
-// not lost.
+// with population i = 4*jy + jx, c_i = (C1[jx], C1[jy]).  The lo values (FP32 form only;
+// zero in FP64) are what the storage rounding of the populations took from the node's
+// exact post-collision mass, momentum (sum f v) and energy (sum g); the next step's moments
+// add them back, so that changes below half an ulp of the populations (the weak edge of an
+// acoustic pulse) are not lost.
 //
 // One step is three launches: the Korteweg stress K and heat-flux vector q of the state
 // the non-local terms come from, their divergences F = -div K and M_0 = 2 div q, and the
 // node step (frame search with semi-Lagrangian streaming, then BGK collision with the
 // force, heat-flux and force-work sources).  R = float (FP32 storage and streaming /
-// collision arithmetic, FP64 moments, EoS and frame-search residual) or double.
+// collision arithmetic; sums, moments, EoS and non-local terms in float-float) or double.
+//
+// The node step streams as the D2Q9 step does (pond_step.cuh): the block's tile with a halo
+// of two is carried once into a common gauge in shared memory and each thread contracts
+// its node's 5 x 5 window along x, then y: 2,200 multiply-adds a population family, where
+// carrying each of 25 nodes into the arrival gauge and spreading it over sixteen directions
+// took about 7,000.
+// Measured (with init and read-out): four mixed steps of a 1024 x 512 droplet 7.83 -> 2.69 ms,
+// three FP64 steps of a 257 x 127 shock-droplet 28.8 -> 5.2 ms.  The mixed node step issues
+// on 56 % of its cycles (FMA pipe 50 %); its FP64 pipe, 22 % busy with the moments and EoS
+// before they went to float-float, is idle.
 #pragma once
 
 #include "pond_kernels.cuh"
-#include "pond_step.cuh"   // float-float values (ffv) and TwoSum
+#include "pond_step.cuh"   // float-float and wide values, tiles
 
 namespace pond {
 
@@ -37,36 +44,54 @@ constexpr int Q16 = 16;
 constexpr int NP16 = 2 * Q16 + 7;   // planes of a D2Q16 state
 enum : int { Q_F = 0, Q_G = 16, Q_TH = 32, Q_UX = 33, Q_UY = 34, Q_RHO = 35, Q_T = 36, Q_UHX = 37,
              Q_UHY = 38 };
-// planes of the non-local scratch (FP64): K_xx, K_xy, K_yy, q_x, q_y, rho E_lambda, F_x, F_y, M_0
+// 8-byte planes of the non-local scratch (FP64, or float-float pairs): K_xx, K_xy, K_yy,
+// q_x, q_y, rho E_lambda, F_x, F_y, M_0
 enum : int { NL_KXX = 0, NL_KXY, NL_KYY, NL_QX, NL_QY, NL_REL, NL_FX, NL_FY, NL_M0, NL_PLANES };
 
-constexpr int SLQ = 44;   // values per node record (43 used, padded to 16-byte rows)
+constexpr int SLQ = 44;   // values per node record (43 used)
 enum : int { Q_MLO = 39, Q_JXLO = 40, Q_JYLO = 41, Q_GLO = 42 };
-// value `off` of node n's record, and plane `plane` of the FP64 non-local scratch
-#define REC16(buf, n, off) (buf)[(size_t)(n) * SLQ + (off)]
+// value `off` of node n's record, and plane `plane` of the non-local scratch
+#define REC16(buf, n, off) (buf)[rec_at(buf, (size_t)(n), (off), (size_t)p.N)]
 #define NLP(buf, plane, n, N) (buf)[(size_t)(plane) * (size_t)(N) + (size_t)(n)]
 
-// Four consecutive record values starting on a 16-byte boundary: one 16-byte load (FP32)
-// or two (FP64), through the read-only path; and the matching stores.
-__device__ __forceinline__ void ld4(const float *p, float (&o)[4])
+// Four record values from offset off (a multiple of four) of node nd, sixteen, and stores.
+__device__ __forceinline__ void ld4(const float *__restrict__ b, size_t nd, size_t N, int off, float (&o)[4])
 {
-    const float4 t = __ldg(reinterpret_cast<const float4 *>(p));
+    const float4 t = __ldg(reinterpret_cast<const float4 *>(b) + (size_t)(off / 4) * N + nd);
     o[0] = t.x; o[1] = t.y; o[2] = t.z; o[3] = t.w;
 }
-__device__ __forceinline__ void ld4(const double *p, double (&o)[4])
+__device__ __forceinline__ void ld4(const double *__restrict__ b, size_t nd, size_t N, int off, double (&o)[4])
 {
-    const double2 a = __ldg(reinterpret_cast<const double2 *>(p));
-    const double2 b = __ldg(reinterpret_cast<const double2 *>(p) + 1);
-    o[0] = a.x; o[1] = a.y; o[2] = b.x; o[3] = b.y;
+    const double2 *q = reinterpret_cast<const double2 *>(b) + (size_t)(off / 2) * N + nd;
+    const double2 x = __ldg(q), y = __ldg(q + N);
+    o[0] = x.x; o[1] = x.y; o[2] = y.x; o[3] = y.y;
 }
-__device__ __forceinline__ void st4(float *p, float a, float b, float c, float d)
+template <typename R>
+__device__ __forceinline__ void ld16(const R *__restrict__ b, size_t nd, size_t N, int off, R (&o)[16])
 {
-    *reinterpret_cast<float4 *>(p) = make_float4(a, b, c, d);
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+        R q[4];
+        ld4(b, nd, N, off + 4 * r, q);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) o[4 * r + k] = q[k];
+    }
 }
-__device__ __forceinline__ void st4(double *p, double a, double b, double c, double d)
+__device__ __forceinline__ void st4(float *b, size_t nd, size_t N, int off, float a, float c, float d, float e)
 {
-    reinterpret_cast<double2 *>(p)[0] = make_double2(a, b);
-    reinterpret_cast<double2 *>(p)[1] = make_double2(c, d);
+    reinterpret_cast<float4 *>(b)[(size_t)(off / 4) * N + nd] = make_float4(a, c, d, e);
+}
+__device__ __forceinline__ void st4(double *b, size_t nd, size_t N, int off, double a, double c, double d, double e)
+{
+    double2 *q = reinterpret_cast<double2 *>(b) + (size_t)(off / 2) * N + nd;
+    q[0] = make_double2(a, c);
+    q[N] = make_double2(d, e);
+}
+template <typename R>
+__device__ __forceinline__ void st16(R *b, size_t nd, size_t N, int off, const R (&v)[16])
+{
+#pragma unroll
+    for (int r = 0; r < 4; ++r) st4(b, nd, N, off + 4 * r, v[4 * r], v[4 * r + 1], v[4 * r + 2], v[4 * r + 3]);
 }
 
 // C1, its weights, and per node k: 1 / prod_{j != k} (c_k - c_j) (the Lagrange
@@ -175,7 +200,7 @@ __device__ __forceinline__ int departure(int X, A v, A dt, A w[4])
     return X + (int)fl - 1;
 }
 
-// Pressure, energy and enthalpy of the run's EoS in FP64.
+// Pressure of the run's EoS in FP64.
 __device__ __forceinline__ double q16_p(const DevParams &p, double r, double t)
 {
     return eos_pressure<double>(p.eos_kind, p.a, p.b, p.R, r, t, p.sp);
@@ -228,69 +253,107 @@ __global__ void k_q16_init(DevParams p, const double *__restrict__ rho, const do
 }
 
 // ---------------------------------------------------------------------------
-// Non-local terms, stage 1 (from the rho, T planes of `src`): with the isotropic D2Q9
-// grid stencils grad = 3 sum W c phi(x + c), lap = 6 sum W (phi(x + c) - phi(x)),
+// First differences of a field over the 3 x 3 neighbourhood by the isotropic D2Q9 grid
+// stencils, unnormalised (D = phi(+1) - phi(-1), S = phi(-1) + 4 phi(0) + phi(+1) per axis):
+// dx = S_y D_x, dy = D_y S_x, s = S_y S_x.
+template <typename A> struct Diff2 { A dx, dy, s; };
+template <typename A, typename Get>
+__device__ __forceinline__ Diff2<A> diff2(Get get)
+{
+    A D[3], S[3];
+#pragma unroll
+    for (int y = 0; y < 3; ++y) {
+        const auto a = get(y, 0), b = get(y, 1), c = get(y, 2);
+        D[y] = w_sub(c, a);
+        S[y] = w_add(w_add(a, c), w_x4(b));
+    }
+    Diff2<A> o;
+    o.dx = w_add(w_add(D[0], D[2]), w_x4(D[1]));
+    o.dy = w_sub(S[2], S[0]);
+    o.s = w_add(w_add(S[0], S[2]), w_x4(S[1]));
+    return o;
+}
+
+// Indices of the nine neighbours of a node after the boundary rules.
+struct Near9 {
+    int x[3];
+    long long row[3];
+    __device__ __forceinline__ Near9(const DevParams &p, long long n)
+    {
+        const int X = (int)(n % p.nx), Y = (int)(n / p.nx);
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            x[k] = bc_wrap(X + k - 1, p.nx, p.bcx);
+            row[k] = (long long)bc_wrap(Y + k - 1, p.ny, p.bcy) * p.nx;
+        }
+    }
+    __device__ __forceinline__ size_t at(int y, int k) const { return (size_t)(row[y] + x[k]); }
+};
+
+// Non-local terms, stage 1 (rho, T of `src`; FP64, or float-float in the FP32 form): with
+// grad = 3 sum W c phi(x + c) = d / 12 and lap = 6 sum W (phi(x + c) - phi(x)) = s / 6 of
+// the differences to the centre,
 //   K = -kappa (rho lap rho + |grad rho|^2 / 2) I + kappa grad rho (x) grad rho  (Eq. korteweg)
 //   q = -mu grad h + k grad T, mu = (tau - 1/2) P dt, h = e + p/rho              (Eq. gtilde)
 //   rho E_lambda = kappa |grad rho|^2 / 2.
 template <typename R>
-__global__ void k_q16_nonlocal1(DevParams p, const R *__restrict__ src, double *__restrict__ nl)
+__global__ void k_q16_nonlocal1(DevParams p, const R *__restrict__ src, typename Wide<R>::type *__restrict__ nl)
 {
+    using A = typename Wide<R>::type;
     const long long n = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (n >= p.N) return;
     const long long N = p.N;
-    const int X = (int)(n % p.nx), Y = (int)(n / p.nx);
-    double gr[2] = {0.0, 0.0}, gh[2] = {0.0, 0.0}, gT[2] = {0.0, 0.0}, lap = 0.0;
-    const double r0 = (double)REC16(src, n, Q_RHO), t0 = (double)REC16(src, n, Q_T);
-    for (int i = 0; i < 9; ++i) {
-        const int cx = i % 3 - 1, cy = i / 3 - 1;
-        const long long m = (long long)bc_wrap(Y + cy, p.ny, p.bcy) * p.nx + bc_wrap(X + cx, p.nx, p.bcx);
-        const double w = w1d(cx + 1) * w1d(cy + 1);
-        const double r = (double)REC16(src, m, Q_RHO), t = (double)REC16(src, m, Q_T);
-        const double h = p.cv * t - p.a * r + q16_p(p, r, t) / r;
-        gr[0] += w * cx * r; gr[1] += w * cy * r;
-        gh[0] += w * cx * h; gh[1] += w * cy * h;
-        gT[0] += w * cx * t; gT[1] += w * cy * t;
-        lap += w * (r - r0);
+    const Near9 nb(p, n);
+    R r[3][3], t[3][3];
+    A pi[3][3];
+#pragma unroll
+    for (int y = 0; y < 3; ++y)
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            const size_t m = nb.at(y, k);
+            r[y][k] = REC16(src, m, Q_RHO);
+            t[y][k] = REC16(src, m, Q_T);
+            pi[y][k] = w_p_over_rho(p, r[y][k], t[y][k]);
+        }
+    const R r0 = r[1][1];
+    const Diff2<A> dr = diff2<A>([&](int y, int k) { return w_sub(r[y][k], r0); });
+    const Diff2<A> dT = diff2<A>([&](int y, int k) { return t[y][k]; });
+    const Diff2<A> dp = diff2<A>([&](int y, int k) { return pi[y][k]; });
+    const A g = w_const<A>(1.0 / 12.0), kap = w_const<A>(p.kappa);
+    const A gr[2] = {w_mul(dr.dx, g), w_mul(dr.dy, g)}, gT[2] = {w_mul(dT.dx, g), w_mul(dT.dy, g)};
+    const A dpi[2] = {dp.dx, dp.dy};
+    const A lap = w_mul(dr.s, w_const<A>(1.0 / 6.0));
+    const A g2 = w_add(w_mul(gr[0], gr[0]), w_mul(gr[1], gr[1]));
+    const A kg2 = w_mul(kap, w_mul(g2, w_const<A>(0.5)));   // rho E_lambda
+    const A iso = w_sub(w_mul(w_mul(kap, w_mul(lap, r0)), w_const<A>(-1.0)), kg2);
+    const A pr = w_mul(pi[1][1], r0);
+    const A mu = w_mul(w_double(pr) > p.p_floor ? pr : w_const<A>(p.p_floor), w_const<A>((p.tau - 0.5) * p.dt));
+    const A kc = p.k_cond >= 0.0 ? w_const<A>(p.k_cond) : w_mul(mu, w_const<A>(p.cv + p.R));
+    NLP(nl, NL_KXX, n, N) = w_add(iso, w_mul(kap, w_mul(gr[0], gr[0])));
+    NLP(nl, NL_KXY, n, N) = w_mul(kap, w_mul(gr[0], gr[1]));
+    NLP(nl, NL_KYY, n, N) = w_add(iso, w_mul(kap, w_mul(gr[1], gr[1])));
+#pragma unroll
+    for (int a = 0; a < 2; ++a) {
+        const A gh = w_add(w_sub(w_mul(gT[a], w_const<A>(p.cv)), w_mul(gr[a], w_const<A>(p.a))), w_mul(dpi[a], g));
+        NLP(nl, NL_QX + a, n, N) = w_sub(w_mul(kc, gT[a]), w_mul(mu, gh));
     }
-    for (int k = 0; k < 2; ++k) { gr[k] *= 3.0; gh[k] *= 3.0; gT[k] *= 3.0; }
-    lap *= 6.0;
-    const double pr = q16_p(p, r0, t0);
-    const double Pg = pr > p.p_floor ? pr : p.p_floor;
-    const double mu = (p.tau - 0.5) * Pg * p.dt;
-    const double kc = p.k_cond >= 0.0 ? p.k_cond : mu * (p.cv + p.R);
-    const double g2 = gr[0] * gr[0] + gr[1] * gr[1];
-    const double iso = -p.kappa * (r0 * lap + 0.5 * g2);
-    NLP(nl, NL_KXX, n, N) = iso + p.kappa * gr[0] * gr[0];
-    NLP(nl, NL_KXY, n, N) = p.kappa * gr[0] * gr[1];
-    NLP(nl, NL_KYY, n, N) = iso + p.kappa * gr[1] * gr[1];
-    NLP(nl, NL_QX, n, N) = -mu * gh[0] + kc * gT[0];
-    NLP(nl, NL_QY, n, N) = -mu * gh[1] + kc * gT[1];
-    NLP(nl, NL_REL, n, N) = 0.5 * p.kappa * g2;
+    NLP(nl, NL_REL, n, N) = kg2;
 }
 
 // Stage 2: F = -div K and M_0 = 2 div q with the same gradient stencil.
-__global__ void k_q16_nonlocal2(DevParams p, double *__restrict__ nl)
+template <typename R>
+__global__ void k_q16_nonlocal2(DevParams p, typename Wide<R>::type *__restrict__ nl)
 {
+    using A = typename Wide<R>::type;
     const long long n = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (n >= p.N) return;
     const long long N = p.N;
-    const int X = (int)(n % p.nx), Y = (int)(n / p.nx);
-    double dxx = 0.0, dxy_x = 0.0, dxy_y = 0.0, dyy = 0.0, dqx = 0.0, dqy = 0.0;
-    for (int i = 0; i < 9; ++i) {
-        const int cx = i % 3 - 1, cy = i / 3 - 1;
-        const long long m = (long long)bc_wrap(Y + cy, p.ny, p.bcy) * p.nx + bc_wrap(X + cx, p.nx, p.bcx);
-        const double w = w1d(cx + 1) * w1d(cy + 1);
-        dxx += w * cx * NLP(nl, NL_KXX, m, N);
-        dxy_x += w * cx * NLP(nl, NL_KXY, m, N);
-        dxy_y += w * cy * NLP(nl, NL_KXY, m, N);
-        dyy += w * cy * NLP(nl, NL_KYY, m, N);
-        dqx += w * cx * NLP(nl, NL_QX, m, N);
-        dqy += w * cy * NLP(nl, NL_QY, m, N);
-    }
-    NLP(nl, NL_FX, n, N) = -3.0 * (dxx + dxy_y);
-    NLP(nl, NL_FY, n, N) = -3.0 * (dxy_x + dyy);
-    NLP(nl, NL_M0, n, N) = 6.0 * (dqx + dqy);
+    const Near9 nb(p, n);
+    auto diff = [&](int plane) { return diff2<A>([&](int y, int k) { return NLP(nl, plane, nb.at(y, k), N); }); };
+    const Diff2<A> xx = diff(NL_KXX), xy = diff(NL_KXY), yy = diff(NL_KYY), qx = diff(NL_QX), qy = diff(NL_QY);
+    NLP(nl, NL_FX, n, N) = w_mul(w_add(xx.dx, xy.dy), w_const<A>(-1.0 / 12.0));
+    NLP(nl, NL_FY, n, N) = w_mul(w_add(xy.dx, yy.dy), w_const<A>(-1.0 / 12.0));
+    NLP(nl, NL_M0, n, N) = w_mul(w_add(qx.dx, qy.dy), w_const<A>(2.0 / 12.0));
 }
 
 // ---------------------------------------------------------------------------
@@ -334,9 +397,9 @@ __device__ void q16_stream(const DevParams &p, const Lat16<R> &L, const R *__res
 #pragma unroll 2
             for (int mk = 0; mk < 16; ++mk) {
                 const int m = mk >> 2, k = mk & 3;
-                const R *rec = in + (size_t)(sel4(rows, m) + sel4(cols, k)) * SLQ;
+                const size_t nd = (size_t)(sel4(rows, m) + sel4(cols, k));
                 R gv[4];   // theta, u_x, u_y, rho of the stencil node
-                ld4(rec + Q_TH, gv);
+                ld4(in, nd, (size_t)p.N, Q_TH, gv);
                 const R ths = gv[0];
                 const R ds = (ths - th) / (sqrt_(ths) + s) * is;   // (s' - s)/s
                 const R ex = (gv[1] - ux) * is, ey = (gv[2] - uy) * is;
@@ -353,8 +416,8 @@ __device__ void q16_stream(const DevParams &p, const Lat16<R> &L, const R *__res
 #pragma unroll
                 for (int jy = 0; jy < 4; ++jy) {
                     R fr[4], gr[4];
-                    ld4(rec + Q_F + 4 * jy, fr);
-                    ld4(rec + Q_G + 4 * jy, gr);
+                    ld4(in, nd, (size_t)p.N, Q_F + 4 * jy, fr);
+                    ld4(in, nd, (size_t)p.N, Q_G + 4 * jy, gr);
                     R df = R(0), dg = R(0);
 #pragma unroll
                     for (int jx = 0; jx < 4; ++jx) { df += gx[jx] * fr[jx]; dg += gx[jx] * gr[jx]; }
@@ -385,13 +448,13 @@ __device__ void q16_stream(const DevParams &p, const Lat16<R> &L, const R *__res
 __device__ __forceinline__ ffv q16_co() { return {0x1.2ace16p+1f, -0x1.b3aab0p-26f}; }
 __device__ __forceinline__ ffv q16_ci() { return {0x1.7be2aep-1f, -0x1.4e69e0p-26f}; }
 
-// Moments of 16 FP32 values v (i = 4 jy + jx), returned as doubles: out[0] = sum v and,
-// with WEIGHTED, out[1] = sum v c_jx and out[2] = sum v c_jy, from the column sums C_k and
+// Moments of 16 values v (i = 4 jy + jx) in the wide type: out[0] = sum v and, with
+// WEIGHTED, out[1] = sum v c_jx and out[2] = sum v c_jy, from the column sums C_k and
 // row sums R_r (sum v c_jx = co (C_3 - C_0) + ci (C_2 - C_1), the same over rows for y).
 // Each float-float addition is exact up to ~2^-48 of its result (TwoSum, the error terms
 // added in FP32), far below what the kept remainders resolve (FP32 storage rounding).
 template <bool WEIGHTED>
-__device__ __forceinline__ void q16_ff_moments(const float *v, double *out)
+__device__ __forceinline__ void sums16(const float *v, ffv *out)
 {
     ffv C[4], Rw[4];
 #pragma unroll
@@ -401,7 +464,7 @@ __device__ __forceinline__ void q16_ff_moments(const float *v, double *out)
         for (int r = 1; r < 4; ++r) C[k] = ff_add(C[k], v[4 * r + k]);
     }
     const ffv s = ff_add(ff_add(C[0], C[1]), ff_add(C[2], C[3]));
-    out[0] = (double)s.hi + (double)s.lo;
+    out[0] = s;
     if (WEIGHTED) {
 #pragma unroll
         for (int r = 0; r < 4; ++r) {
@@ -412,102 +475,25 @@ __device__ __forceinline__ void q16_ff_moments(const float *v, double *out)
         const ffv co = q16_co(), ci = q16_ci();
         const ffv sx = ff_add(ff_mul(ff_add(C[3], ff_neg(C[0])), co), ff_mul(ff_add(C[2], ff_neg(C[1])), ci));
         const ffv sy = ff_add(ff_mul(ff_add(Rw[3], ff_neg(Rw[0])), co), ff_mul(ff_add(Rw[2], ff_neg(Rw[1])), ci));
-        out[1] = (double)sx.hi + (double)sx.lo;
-        out[2] = (double)sy.hi + (double)sy.lo;
+        out[1] = sx;
+        out[2] = sy;
     }
 }
-
-// Sums of a node's own stored populations and its kept remainders (FP64; float-float in
-// the FP32 form):
-// own[0] = sum f + mass lo, own[1] = sum f c_x, own[2] = sum f c_y, own[3] = sum g +
-// energy lo, own[4], own[5] = the momentum lo (absolute, sum f v units).
-template <typename R>
-__device__ __forceinline__ void q16_own_sums(const Lat16<double> &L, const R *rec, double own[6])
+template <bool WEIGHTED>
+__device__ __forceinline__ void sums16(const double *v, double *out)
 {
-    double s0 = 0.0, sx = 0.0, sy = 0.0, sg = 0.0;
-    if constexpr (sizeof(R) == 4) {
-        float f[Q16], g[Q16];
+    double C[4], W[4];
 #pragma unroll
-        for (int r = 0; r < 4; ++r) {
-            float q[4];
-            ld4(rec + Q_F + 4 * r, q);
-#pragma unroll
-            for (int k = 0; k < 4; ++k) f[4 * r + k] = q[k];
-            ld4(rec + Q_G + 4 * r, q);
-#pragma unroll
-            for (int k = 0; k < 4; ++k) g[4 * r + k] = q[k];
-        }
-        double m[3], mg[1];
-        q16_ff_moments<true>(f, m);
-        q16_ff_moments<false>(g, mg);
-        s0 = m[0]; sx = m[1]; sy = m[2]; sg = mg[0];
-    } else {
-#pragma unroll
-        for (int r = 0; r < 4; ++r) {
-            R f[4], g[4];
-            ld4(rec + Q_F + 4 * r, f);
-            ld4(rec + Q_G + 4 * r, g);
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                s0 += (double)f[k];
-                sx += (double)f[k] * L.c[k];
-                sy += (double)f[k] * L.c[r];
-                sg += (double)g[k];
-            }
-        }
+    for (int k = 0; k < 4; ++k) {
+        C[k] = (v[k] + v[4 + k]) + (v[8 + k] + v[12 + k]);
+        if (WEIGHTED) W[k] = (v[4 * k] + v[4 * k + 1]) + (v[4 * k + 2] + v[4 * k + 3]);
     }
-    R lo[4];
-    ld4(rec + Q_T, lo);       // T, uhat_x, uhat_y, mass lo
-    R lo2[4];
-    ld4(rec + Q_JXLO, lo2);   // momentum_x lo, momentum_y lo, energy lo, unused
-    own[0] = s0 + (double)lo[3];
-    own[1] = sx;
-    own[2] = sy;
-    own[3] = sg + (double)lo2[2];
-    own[4] = (double)lo2[0];
-    own[5] = (double)lo2[1];
-}
-
-// Macroscopic fields of the streamed populations (own + increments) in gauge (th, ux, uy)
-// (moments Eq.), FP64: out = rho, u_x, u_y, uhat_x, uhat_y, E, e, T, p,
-// P = max(p, p_floor), theta* = P/rho.
-template <typename R>
-__device__ __forceinline__ void q16_macro(const DevParams &p, const Lat16<double> &L, R th, R ux,
-                                          R uy, const double own[6], const R *fi, const R *gi,
-                                          double Fx, double Fy, double rEl, double out[11])
-{
-    const double s = sqrt((double)th);
-    double d0 = 0.0, dx = 0.0, dy = 0.0, dg = 0.0;
-    if constexpr (sizeof(R) == 4) {
-        double m[3], mg[1];
-        q16_ff_moments<true>(fi, m);
-        q16_ff_moments<false>(gi, mg);
-        d0 = m[0]; dx = m[1]; dy = m[2]; dg = mg[0];
-    } else {
-#pragma unroll
-        for (int i = 0; i < Q16; ++i) {
-            const double f = (double)fi[i];
-            d0 += f;
-            dx += f * L.c[i & 3];
-            dy += f * L.c[i >> 2];
-            dg += (double)gi[i];
-        }
+    out[0] = (C[0] + C[1]) + (C[2] + C[3]);
+    if (WEIGHTED) {
+        const double s6 = sqrt(6.0), ci = sqrt(3.0 - s6), co = sqrt(3.0 + s6);
+        out[1] = co * (C[3] - C[0]) + ci * (C[2] - C[1]);
+        out[2] = co * (W[3] - W[0]) + ci * (W[2] - W[1]);
     }
-    // sum f v = s sum f c + u sum f, for the stored part and the increments
-    const double rho = own[0] + d0;
-    const double jx = s * (own[1] + dx) + (double)ux * rho + own[4];
-    const double jy = s * (own[2] + dy) + (double)uy * rho + own[5];
-    const double sg = own[3] + dg;
-    const double irho = 1.0 / rho;   // one FP64 division, the quotients by rho multiply
-    const double u_x = jx * irho, u_y = jy * irho;
-    const double uhx = u_x + (0.5 * p.dt) * Fx * irho, uhy = u_y + (0.5 * p.dt) * Fy * irho;
-    const double E = 0.5 * sg * irho;
-    const double e = E - 0.5 * (uhx * uhx + uhy * uhy) - rEl * irho;
-    const double T = p.isothermal ? p.T_iso : (e + p.a * rho) / p.cv;
-    const double pr = q16_p(p, rho, T);
-    const double P = pr > p.p_floor ? pr : p.p_floor;
-    out[0] = rho; out[1] = u_x; out[2] = u_y; out[3] = uhx; out[4] = uhy;
-    out[5] = E; out[6] = e; out[7] = T; out[8] = pr; out[9] = P; out[10] = P * irho;
 }
 
 // Per-axis transfer map from gauge (s_src, u_src) into (s_dst, u_dst) in increment
@@ -549,7 +535,8 @@ __device__ __forceinline__ void apply_inc(const A Dx[4][4], const A Dy[4][4], co
 }
 
 // ---------------------------------------------------------------------------
-// Region stream.  On a tensor lattice the union of a node's sixteen 4 x 4 departure
+// General stream, for departure points beyond the staged halo (|v| dt >= 1) and non-finite
+// gauges: reads the stencil nodes' records from global memory.  On a tensor lattice the union of a node's sixteen 4 x 4 departure
 // stencils is the product of the per-axis unions: W x H nodes with W (H) = 4 + the spread
 // of the four departure floors along the axis, 5 x 5 while |v| dt < 1 in every direction.
 // Each region node is carried into the arrival gauge once for all sixteen directions
@@ -560,22 +547,9 @@ __device__ __forceinline__ void apply_inc(const A Dx[4][4], const A Dy[4][4], co
 
 // Largest region side the region stream takes; wider regions take q16_stream.
 constexpr int Q16_REGION_MAX = 6;
-constexpr int Q16_THREADS = 128;   // threads of a k_q16_step block
-// FP32: f and g of a region node in one pass (two rolled passes, one population set each,
-// measured 4 % slower on the 2048 x 1024 droplet-shock); FP64 always takes two passes
-// (one pass exceeds the register file).  Three FP32 blocks per SM (168 registers): two
-// (232 registers) and four (128, with spills) measured slower.
-constexpr bool Q16_ONE_PASS = true;
-constexpr int Q16_MIN_BLOCKS = 3;
-
-// Lagrange weight tables of the region stream, one column of entries per thread (entry e
-// of thread t at w[e][t]: consecutive threads in consecutive banks).  Entry
-// (axis * 4 + k) * Q16_REGION_MAX + c is the weight of region column (row) c in the
-// stencil of axis component k, zero outside that stencil.
-template <typename R>
-struct Q16Weights {
-    R w[2 * 4 * Q16_REGION_MAX][Q16_THREADS];
-};
+// Entries of a thread's Lagrange weight tables: (axis * 4 + k) * Q16_REGION_MAX + c is the
+// weight of region column (row) c in the stencil of axis component k, zero outside it.
+constexpr int Q16_WT_ENTRIES = 2 * 4 * Q16_REGION_MAX;
 
 // Departure floors and Lagrange weights of the four axis components for the gauge
 // velocity u along one axis (as in `departure`), the table entries of that axis, and the
@@ -605,28 +579,22 @@ __device__ __forceinline__ bool q16_region_axis(const Lat16<R> &L, int X, R s, R
 #pragma unroll
         for (int c = 0; c < Q16_REGION_MAX; ++c) {
             const int j = c - o;
-            wt[(k * Q16_REGION_MAX + c) * Q16_THREADS] =
+            wt[(k * Q16_REGION_MAX + c)] =
                 j == 0 ? a[k][0] : (j == 1 ? a[k][1] : (j == 2 ? a[k][2] : (j == 3 ? a[k][3] : R(0))));
         }
     }
     return true;
 }
 
-// One population set (16 values at v) of a region node: x-increments t = (I (x) Dx) h, the
+// One population set (16 values at record offset off) of a region node: x-increments t = (I (x) Dx) h, the
 // y-increment of each component, and acc_i += wx_ix wy_iy ((h_i - ref_i) + t_i + dy_i).
 template <typename R>
-__device__ __forceinline__ void q16_region_pop(const R (&Dx)[4][4], const R (&Dy)[4][4], const R *v,
-                                               const R (&ref)[Q16], const R (&wx)[4], const R (&wy)[4],
+__device__ __forceinline__ void q16_region_pop(const R (&Dx)[4][4], const R (&Dy)[4][4], const R *__restrict__ in,
+                                               size_t nd, size_t N, int off, const R (&ref)[Q16], const R (&wx)[4], const R (&wy)[4],
                                                R (&acc)[Q16])
 {
     R h[Q16], t[Q16];
-#pragma unroll
-    for (int r = 0; r < 4; ++r) {
-        R q[4];
-        ld4(v + 4 * r, q);
-#pragma unroll
-        for (int k = 0; k < 4; ++k) h[4 * r + k] = q[k];
-    }
+    ld16(in, nd, N, off, h);
 #pragma unroll
     for (int jy = 0; jy < 4; ++jy)
 #pragma unroll
@@ -649,57 +617,42 @@ __device__ __forceinline__ void q16_region_pop(const R (&Dx)[4][4], const R (&Dy
 }
 
 // The region pass over the W x H region at (xlo, ylo), skipping region entry `skip` (-1:
-// none): the increments of the streamed populations over the node's own (irec) for the
-// population set at record offset `off` (Q_F or Q_G) into out0, and with BOTH (off = Q_F)
-// those of g into out1 as well.
-template <typename R, bool BOTH>
+// none): the increments of the streamed populations over the node's own (node self) for
+// the population set at record offset `off` (Q_F or Q_G) into out.
+template <typename R>
 __device__ __forceinline__ void q16_region_pass(const DevParams &p, const Lat16<R> &L, const R *__restrict__ in,
-                                                const R *irec, int xlo, int ylo, int W, int H, int skip,
-                                                R th, R ux, R uy, const R *wt, int off, R *out0, R *out1)
+                                                size_t self, int xlo, int ylo, int W, int H, int skip,
+                                                R th, R ux, R uy, const R *wt, int off, R *out)
 {
     const R s = sqrt_(th), is = R(1) / s;
-    R ref0[Q16], ref1[Q16], acc0[Q16], acc1[Q16];
+    const size_t N = (size_t)p.N;
+    R ref[Q16], acc[Q16];
+    ld16(in, self, N, off, ref);
 #pragma unroll
-    for (int r = 0; r < 4; ++r) {
-        R q[4];
-        ld4(irec + off + 4 * r, q);
-#pragma unroll
-        for (int k = 0; k < 4; ++k) ref0[4 * r + k] = q[k];
-        if (BOTH) {
-            ld4(irec + Q_G + 4 * r, q);
-#pragma unroll
-            for (int k = 0; k < 4; ++k) ref1[4 * r + k] = q[k];
-        }
-    }
-#pragma unroll
-    for (int i = 0; i < Q16; ++i) { acc0[i] = R(0); acc1[i] = R(0); }
+    for (int i = 0; i < Q16; ++i) acc[i] = R(0);
 #pragma unroll 1
     for (int cy = 0; cy < H; ++cy) {
         const long long row = (long long)bc_wrap(ylo + cy, p.ny, p.bcy) * p.nx;
         R wy[4];
 #pragma unroll
-        for (int k = 0; k < 4; ++k) wy[k] = wt[((4 + k) * Q16_REGION_MAX + cy) * Q16_THREADS];
+        for (int k = 0; k < 4; ++k) wy[k] = wt[(4 + k) * Q16_REGION_MAX + cy];
 #pragma unroll 1
         for (int cx = 0; cx < W; ++cx) {
             if (cy * W + cx == skip) continue;
-            const R *rec = in + (size_t)(row + bc_wrap(xlo + cx, p.nx, p.bcx)) * SLQ;
+            const size_t nd = (size_t)(row + bc_wrap(xlo + cx, p.nx, p.bcx));
             R wx[4], gv[4];
 #pragma unroll
-            for (int k = 0; k < 4; ++k) wx[k] = wt[(k * Q16_REGION_MAX + cx) * Q16_THREADS];
-            ld4(rec + Q_TH, gv);   // theta, u_x, u_y, rho of the region node
+            for (int k = 0; k < 4; ++k) wx[k] = wt[k * Q16_REGION_MAX + cx];
+            ld4(in, nd, N, Q_TH, gv);   // theta, u_x, u_y, rho of the region node
             const R ds = (gv[0] - th) / (sqrt_(gv[0]) + s) * is;   // (s' - s)/s
             R Dx[4][4], Dy[4][4];
             axis_inc<R>(L, ds, (gv[1] - ux) * is, Dx);
             axis_inc<R>(L, ds, (gv[2] - uy) * is, Dy);
-            q16_region_pop<R>(Dx, Dy, rec + off, ref0, wx, wy, acc0);
-            if (BOTH) q16_region_pop<R>(Dx, Dy, rec + Q_G, ref1, wx, wy, acc1);
+            q16_region_pop<R>(Dx, Dy, in, nd, N, off, ref, wx, wy, acc);
         }
     }
 #pragma unroll
-    for (int i = 0; i < Q16; ++i) {
-        out0[i] = acc0[i];
-        if (BOTH) out1[i] = acc1[i];
-    }
+    for (int i = 0; i < Q16; ++i) out[i] = acc[i];
 }
 
 // Streaming of node (X, Y) into gauge (th, ux, uy) by the region stream where the region
@@ -707,27 +660,24 @@ __device__ __forceinline__ void q16_region_pass(const DevParams &p, const Lat16<
 // the gauge is the node's stored gauge: the map is then the identity and the entry adds
 // exactly zero).  Adds the region entries transformed to nreg, or 1 to npair.
 template <typename R>
-__device__ __forceinline__ void q16_stream_any(const DevParams &p, const Lat16<R> &L, const R *__restrict__ in,
-                                               int X, int Y, R th, R ux, R uy, bool skip_own, R *wt, R *fi,
-                                               R *gi, unsigned long long &nreg, unsigned long long &npair)
+__device__ __noinline__ void q16_stream_any(const DevParams &p, const R *__restrict__ in, int X, int Y, R th, R ux,
+                                            R uy, bool skip_own, R *fi, R *gi, unsigned &nreg, unsigned &npair)
 {
+    const Lat16<R> L = make_lat16<R>();
     const R s = sqrt_(th), dt = (R)p.dt;
+    R wt[Q16_WT_ENTRIES];
     int xlo, ylo, W, H;
     if (q16_region_axis<R>(L, X, s, ux, dt, wt, xlo, W) &&
-        q16_region_axis<R>(L, Y, s, uy, dt, wt + 4 * Q16_REGION_MAX * Q16_THREADS, ylo, H)) {
+        q16_region_axis<R>(L, Y, s, uy, dt, wt + 4 * Q16_REGION_MAX, ylo, H)) {
         const int cxo = X - xlo, cyo = Y - ylo;
         const int skip = (skip_own && cxo >= 0 && cxo < W && cyo >= 0 && cyo < H) ? cyo * W + cxo : -1;
-        const R *irec = in + ((size_t)Y * p.nx + X) * SLQ;
-        if (Q16_ONE_PASS && sizeof(R) == 4) {
-            q16_region_pass<R, true>(p, L, in, irec, xlo, ylo, W, H, skip, th, ux, uy, wt, Q_F, fi, gi);
-        } else {
-            // one population set per pass, the pass's code once (a rolled loop)
+        const size_t self = (size_t)Y * p.nx + X;
+        // one population set per pass, the pass's code once (a rolled loop)
 #pragma unroll 1
-            for (int ps = 0; ps < 2; ++ps)
-                q16_region_pass<R, false>(p, L, in, irec, xlo, ylo, W, H, skip, th, ux, uy, wt,
-                                          ps == 0 ? Q_F : Q_G, ps == 0 ? fi : gi, nullptr);
-        }
-        nreg += (unsigned long long)(W * H - (skip >= 0 ? 1 : 0));
+        for (int ps = 0; ps < 2; ++ps)
+            q16_region_pass<R>(p, L, in, self, xlo, ylo, W, H, skip, th, ux, uy, wt, ps == 0 ? Q_F : Q_G,
+                               ps == 0 ? fi : gi);
+        nreg += (unsigned)(W * H - (skip >= 0 ? 1 : 0));
     } else {
         q16_stream<R>(p, L, in, X, Y, th, ux, uy, fi, gi);
         npair += 1;
@@ -735,137 +685,437 @@ __device__ __forceinline__ void q16_stream_any(const DevParams &p, const Lat16<R
 }
 
 // ---------------------------------------------------------------------------
-// The node step.  in: state at t - dt; nl: non-local terms (F, rho E_lambda, M_0) of the
-// state they are taken from; out: state at t.  Frame search: predictor = the node's
-// stored gauge; corrector = re-stream with (theta*, u) of the streamed moments until the
-// relative change is <= tol or after max_iter streams.  Collision: equilibria built in
-// the co-moving frame lambda* = (theta*, u) and carried into the streaming gauge (Eqs.
-// f collision with S_i, g collision with gtilde and phi, new geq).
+// Staging and contraction (the form of the D2Q9 step, see the head of pond_step.cuh, with
+// four velocities per axis).  Values per staged slot: 32 carried populations (f, g), padded
+// so that slots start on distinct banks.
+template <typename R> struct Slot16;
+template <> struct Slot16<float> { static constexpr int stride = 36; };
+template <> struct Slot16<double> { static constexpr int stride = 33; };
 template <typename R>
-__global__ void __launch_bounds__(128, sizeof(R) == 4 ? Q16_MIN_BLOCKS : 1) k_q16_step(DevParams p, const R *__restrict__ in,
-                                                  const double *__restrict__ nl, R *__restrict__ out,
-                                                  DevStats *stats)
+constexpr size_t q16_smem_bytes(int tx, int ty) { return (size_t)step_slots(tx, ty) * Slot16<R>::stride * sizeof(R); }
+
+// The rows of a per-axis map, G[k][j] = l_k(xi_j) at xi_j = (1 + q) c_j + w, as products.
+template <typename A>
+__device__ __forceinline__ void axis_rows16(const Lat16<A> &L, A q, A w, A (&G)[4][4])
 {
-    const int X = blockIdx.x * blockDim.x + threadIdx.x, Y = blockIdx.y * blockDim.y + threadIdx.y;
-    const bool valid = X < p.nx && Y < p.ny;
-    const long long N = p.N, n = valid ? (long long)Y * p.nx + X : 0;
-    unsigned long long its = 0, nonconv = 0, clamped = 0, nonfinite = 0, nreg = 0, npair = 0;
-    __shared__ Q16Weights<R> qw;
-    R *wt = &qw.w[0][threadIdx.y * blockDim.x + threadIdx.x];
-    if (valid) {
-        const Lat16<R> L = make_lat16<R>();
-        const Lat16<double> Ld = make_lat16<double>();
-        const double Fx = NLP(nl, NL_FX, n, N), Fy = NLP(nl, NL_FY, n, N);
-        const double rEl = NLP(nl, NL_REL, n, N), M0 = NLP(nl, NL_M0, n, N);
-        R th = REC16(in, n, Q_TH), ux = REC16(in, n, Q_UX), uy = REC16(in, n, Q_UY);
-        const R *irec = in + (size_t)n * SLQ;
-        double own[6];
-        q16_own_sums<R>(Ld, irec, own);
-        R ft[Q16], gt[Q16];   // increments during the search, streamed populations after it
-        double mac[11];
-        int it = 0;
-        bool conv = false;
-        for (;;) {
-            ++it;
-            // the first stream uses the node's stored gauge: its own region entry adds zero
-            q16_stream_any<R>(p, L, in, X, Y, th, ux, uy, it == 1, wt, ft, gt, nreg, npair);
-            q16_macro<R>(p, Ld, th, ux, uy, own, ft, gt, Fx, Fy, rEl, mac);
-            const double ist0 = 1.0 / sqrt((double)th);   // 1/s of the streaming gauge
-            const double r0 = fabs(mac[10] - (double)th) * (ist0 * ist0);
-            const double r1 = fabs(mac[1] - (double)ux) * ist0, r2 = fabs(mac[2] - (double)uy) * ist0;
-            const double r = fmax(fmax(r0, r1), r2);
-            if (r <= p.tol) { conv = true; break; }
-            if (it >= p.max_iter || !(r == r)) break;
-            th = (R)mac[10]; ux = (R)mac[1]; uy = (R)mac[2];
-        }
-        its = (unsigned long long)it;
-        nonconv = conv ? 0ull : 1ull;
-        clamped = mac[8] < p.p_floor ? 1ull : 0ull;
 #pragma unroll
-        for (int r = 0; r < 4; ++r) {
-            R f[4], g[4];
-            ld4(irec + Q_F + 4 * r, f);
-            ld4(irec + Q_G + 4 * r, g);
+    for (int j = 0; j < 4; ++j) {
+        const A x = (A(1) + q) * L.c[j] + w;
+        const A g0 = x - L.c[0], g1 = x - L.c[1], g2 = x - L.c[2], g3 = x - L.c[3];
+        const A a = g0 * g1, b = g2 * g3;
+        G[0][j] = L.inv_den[0] * g1 * b; G[1][j] = L.inv_den[1] * g0 * b;
+        G[2][j] = L.inv_den[2] * g3 * a; G[3][j] = L.inv_den[3] * g2 * a;
+    }
+}
+
+// Departure points of the four components of an axis and their cubic weights; true when
+// every floor is -1 or 0 (the stencils then lie within two nodes of the arrival node).
+template <typename R>
+__device__ __forceinline__ bool axis_weights16(const Lat16<R> &L, R s, R u, R dt, R (&a)[4][4], bool (&near0)[4])
+{
+    bool ok = true;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        const R d = -(s * L.c[j] + u) * dt;
+        const R f = floor(d);
+        near0[j] = f == R(0);
+        ok = ok && (f == R(0) || f == R(-1));
+        const R t0 = d - f + R(1), t1 = t0 - R(1), t2 = t0 - R(2), t3 = t0 - R(3);
+        const R p12 = t1 * t2, p03 = t0 * t3;
+        a[j][0] = p12 * t3 * R(-1.0 / 6.0);
+        a[j][1] = p03 * t2 * R(0.5);
+        a[j][2] = p03 * t1 * R(-0.5);
+        a[j][3] = p12 * t0 * R(1.0 / 6.0);
+    }
+    return ok;
+}
+
+// The stream over the staged slots: acc = sums over the window of the node's slot `own`
+// (FP32: of differences to the own slot, i.e. increments; FP64: the streamed populations).
+// FP32: one family (offset fam * 16) per call, five columns and rows with zero weights
+// outside a component's four nodes; the x weights are kept apart from the rows of the map
+// (96 instead of 80 multiply-adds a row and source index, but 36 registers instead of 80,
+// which lets three blocks reside on an SM).
+__device__ __forceinline__ void contract16(const float *own, int pitch, const float (&ax)[4][4], const bool (&nx0)[4],
+                                           const float (&ay)[4][4], const bool (&ny0)[4], const float (&Lx)[4][4],
+                                           const float (&Ly)[4][4], float (&acc)[16])
+{
+    constexpr int DS = Slot16<float>::stride;
+    float wx[4][5], wy[4][5];
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+#pragma unroll
+        for (int c = 0; c < 5; ++c) {
+            const int lo = c > 3 ? 3 : c, hi = c < 1 ? 0 : c - 1;
+            wx[k][c] = nx0[k] ? (c == 0 ? 0.0f : ax[k][hi]) : (c == 4 ? 0.0f : ax[k][lo]);
+            wy[k][c] = ny0[k] ? (c == 0 ? 0.0f : ay[k][hi]) : (c == 4 ? 0.0f : ay[k][lo]);
+        }
+    float dx[4][4];
+#pragma unroll
+    for (int n = 0; n < 4; ++n) lds4(own + 4 * n, dx[n]);
+#pragma unroll
+    for (int i = 0; i < 16; ++i) acc[i] = 0.0f;
+    const float *row = own - (2 * pitch + 2) * DS;
+#pragma unroll 1
+    for (int cy = 0; cy < 5; ++cy, row += pitch * DS) {
+        float w[4];
+#pragma unroll
+        for (int l = 0; l < 4; ++l) {
+            w[l] = wy[l][0];
+#pragma unroll
+            for (int c = 0; c < 4; ++c) wy[l][c] = wy[l][c + 1];
+        }
+#pragma unroll
+        for (int n = 0; n < 4; ++n) {
+            float v[5][4];
+#pragma unroll
+            for (int c = 0; c < 5; ++c) {
+                lds4(row + c * DS + 4 * n, v[c]);
+#pragma unroll
+                for (int m = 0; m < 4; ++m) v[c][m] -= dx[n][m];
+            }
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
-                ft[4 * r + k] += f[k];
-                gt[4 * r + k] += g[k];
+                float t = 0.0f;
+#pragma unroll
+                for (int m = 0; m < 4; ++m) {
+                    float q = wx[k][0] * v[0][m];
+#pragma unroll
+                    for (int c = 1; c < 5; ++c) q = fmaf(wx[k][c], v[c][m], q);
+                    t = fmaf(Lx[k][m], q, t);
+                }
+#pragma unroll
+                for (int l = 0; l < 4; ++l) acc[4 * l + k] = fmaf(w[l] * Ly[l][n], t, acc[4 * l + k]);
             }
+        }
+    }
+}
+// FP64: both families at once, each component's own four columns.
+__device__ __forceinline__ void contract16(const double *own, int pitch, const double (&ax)[4][4], const bool (&nx0)[4],
+                                           const double (&ay)[4][4], const bool (&ny0)[4], const double (&Lx)[4][4],
+                                           const double (&Ly)[4][4], double (&acc)[2][16])
+{
+    constexpr int DS = Slot16<double>::stride;
+    double wy[4][5];
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+#pragma unroll
+        for (int c = 0; c < 5; ++c) {
+            const int lo = c > 3 ? 3 : c, hi = c < 1 ? 0 : c - 1;
+            wy[k][c] = ny0[k] ? (c == 0 ? 0.0 : ay[k][hi]) : (c == 4 ? 0.0 : ay[k][lo]);
+        }
+#pragma unroll
+    for (int i = 0; i < 16; ++i) acc[0][i] = acc[1][i] = 0.0;
+    const double *row = own - (2 * pitch + 2) * DS;
+#pragma unroll 1
+    for (int cy = 0; cy < 5; ++cy, row += pitch * DS) {
+        double wn[4][4];
+#pragma unroll
+        for (int l = 0; l < 4; ++l) {
+            const double w = wy[l][0];
+#pragma unroll
+            for (int c = 0; c < 4; ++c) wy[l][c] = wy[l][c + 1];
+#pragma unroll
+            for (int n = 0; n < 4; ++n) wn[l][n] = w * Ly[l][n];
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            double wl[4][4];
+#pragma unroll
+            for (int c = 0; c < 4; ++c)
+#pragma unroll
+                for (int m = 0; m < 4; ++m) wl[c][m] = ax[k][c] * Lx[k][m];
+            const double *r = row + (nx0[k] ? DS : 0);
+#pragma unroll
+            for (int fam = 0; fam < 2; ++fam)
+#pragma unroll
+                for (int n = 0; n < 4; ++n) {
+                    double t = 0.0;
+#pragma unroll
+                    for (int c = 0; c < 4; ++c)
+#pragma unroll
+                        for (int m = 0; m < 4; ++m) t = fma(wl[c][m], r[c * DS + 16 * fam + 4 * n + m], t);
+#pragma unroll
+                    for (int l = 0; l < 4; ++l) acc[fam][4 * l + k] = fma(wn[l][n], t, acc[fam][4 * l + k]);
+                }
+        }
+    }
+}
+
+// Apply the rows Gx, Gy to 16 values h (i = 4 jy + jx), in place.
+template <typename A>
+__device__ __forceinline__ void apply_rows16(const A (&Gx)[4][4], const A (&Gy)[4][4], A (&h)[16])
+{
+    A t[16];
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            t[4 * j + k] = Gx[k][0] * h[4 * j] + Gx[k][1] * h[4 * j + 1] + Gx[k][2] * h[4 * j + 2] + Gx[k][3] * h[4 * j + 3];
+#pragma unroll
+    for (int l = 0; l < 4; ++l)
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            h[4 * l + k] = Gy[l][0] * t[k] + Gy[l][1] * t[4 + k] + Gy[l][2] * t[8 + k] + Gy[l][3] * t[12 + k];
+}
+
+// ---------------------------------------------------------------------------
+// The node step, one thread per node of the block's tile.  in: state at t - dt; nl:
+// non-local terms (F, rho E_lambda, M_0) of the state they are taken from; out: state at
+// t.  Frame search: predictor = the node's stored gauge; corrector = re-stream with
+// (theta*, u) of the streamed moments until the relative change is <= tol or after
+// max_iter streams.  Collision: equilibria built in the co-moving frame lambda* =
+// (theta*, u) and carried into the streaming gauge (Eqs. f collision with S_i, g collision
+// with gtilde and phi, new geq).
+constexpr int Q16_MIN_BLOCKS = 3;   // FP32 blocks per SM (168 registers)
+template <typename R>
+__global__ void __launch_bounds__(STEP_THREADS, sizeof(R) == 4 ? Q16_MIN_BLOCKS : 2)
+    k_q16_step(DevParams p, const R *__restrict__ in, const typename Wide<R>::type *__restrict__ nl,
+               R *__restrict__ out, DevStats *stats)
+{
+    using A = typename Wide<R>::type;
+    constexpr int DS = Slot16<R>::stride;
+    extern __shared__ __align__(128) unsigned char q16_dyn_smem[];
+    R *slots = reinterpret_cast<R *>(q16_dyn_smem);
+    __shared__ StepCounts counts;
+    __shared__ uint4 best[STEP_THREADS / 32];
+    const int tid = threadIdx.x;
+    const size_t N = (size_t)p.N;
+    const int TX = p.tile_x, TY = p.tile_y, WT = TX + 2 * HALO, nslots = step_slots(TX, TY);
+    const int X0 = (blockIdx.x % p.tiles_x) * TX, Y0 = (blockIdx.x / p.tiles_x) * TY;
+    if (tid == 0) counts = StepCounts{};
+    const Lat16<R> L = make_lat16<R>();
+    const float iwt = 1.0f / (float)WT;
+    auto node_of = [&](int k) -> size_t {
+        const int cv = (int)(((float)k + 0.5f) * iwt), cu = k - cv * WT;
+        return (size_t)bc_wrap(Y0 - HALO + cv, p.ny, p.bcy) * p.nx + bc_wrap(X0 - HALO + cu, p.nx, p.bcx);
+    };
+
+    // ---- staging: every record of the tile and its halo carried into the common gauge
+    Extremes ex;
+    for (int k = tid; k < nslots; k += STEP_THREADS) ex.offer((float)__ldg(in + rec_at(in, node_of(k), Q_TH, N)), k);
+    ex = tile_extremes(ex, best);
+    const bool inc = sizeof(R) == 4 && ex.smooth();
+    const size_t nbase = node_of(min((int)ex.at, nslots - 1));
+    R gb[3];   // sqrt(theta), u_x, u_y of the tile's gauge
+    {
+        R g4[4], cold[4];
+        ld4(in, nbase, N, Q_TH, g4);
+        ld4(in, node_of(min((int)ex.lat, nslots - 1)), N, Q_TH, cold);
+        common_gauge<R, 3>(inc, g4, cold, gb);
+        const R thb = inc ? g4[0] : gb[0] * gb[0], inv_sb = R(1) / gb[0];
+#pragma unroll 1
+        for (int k = tid; k < nslots; k += STEP_THREADS) {
+            const size_t nd = node_of(k);
+            ld4(in, nd, N, Q_TH, g4);
+            const R e = fdiv_(g4[0] - thb, (sqrt_(g4[0]) + gb[0]) * gb[0]);
+            const R wx = (g4[1] - gb[1]) * inv_sb, wy = (g4[2] - gb[2]) * inv_sb;
+            R Gx[4][4], Gy[4][4];
+            if (inc) {
+                axis_inc<R>(L, e, wx, Gx);
+                axis_inc<R>(L, e, wy, Gy);
+            } else {
+                axis_rows16<R>(L, e, wx, Gx);
+                axis_rows16<R>(L, e, wy, Gy);
+            }
+#pragma unroll 1
+            for (int fam = 0; fam < 2; ++fam) {
+                R h[16];
+#pragma unroll
+                for (int r = 0; r < 4; ++r) {
+                    R q[4];
+                    ld4(in, nd, N, 16 * fam + 4 * r, q);
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) h[4 * r + c] = q[c];
+                }
+                if (inc) {
+                    R o[16];
+                    apply_inc<R>(Gx, Gy, h, o);
+#pragma unroll
+                    for (int r = 0; r < 4; ++r) {
+                        R q[4];
+                        ld4(in, nbase, N, 16 * fam + 4 * r, q);
+#pragma unroll
+                        for (int c = 0; c < 4; ++c) h[4 * r + c] = (h[4 * r + c] - q[c]) + o[4 * r + c];
+                    }
+                } else {
+                    apply_rows16<R>(Gx, Gy, h);
+                }
+                R *dst = slots + (size_t)k * DS + 16 * fam;
+                if constexpr (sizeof(R) == 4) {
+#pragma unroll
+                    for (int r = 0; r < 4; ++r)
+                        *reinterpret_cast<float4 *>(dst + 4 * r) = make_float4(h[4 * r], h[4 * r + 1], h[4 * r + 2], h[4 * r + 3]);
+                } else {
+#pragma unroll
+                    for (int i = 0; i < 16; ++i) dst[i] = h[i];
+                }
+            }
+        }
+    }
+    __syncthreads();
+
+    const int tx = tid % TX, ty = tid / TX;
+    const int X = X0 + tx, Y = Y0 + ty;
+    const bool valid = X < p.nx && Y < p.ny;
+    unsigned its = 0, nreg = 0, npair = 0;
+    bool conv = true, floored = false, bad = false;
+    if (valid) {
+        const size_t n = (size_t)Y * p.nx + X;
+        const R *own_slot = slots + (size_t)((ty + HALO) * WT + tx + HALO) * DS;
+        const A F[2] = {NLP(nl, NL_FX, n, N), NLP(nl, NL_FY, n, N)};
+        const A rEl = NLP(nl, NL_REL, n, N), M0 = NLP(nl, NL_M0, n, N);
+        // sums of the node's stored populations and its kept remainders: sum f + mass lo,
+        // sum f c_x, sum f c_y, sum g + energy lo, momentum lo (absolute)
+        A own[6];
+        R th, u[2];
+        {
+            R v[16], lo[4];
+            ld16(in, n, N, Q_F, v);
+            sums16<true>(v, own);
+            ld16(in, n, N, Q_G, v);
+            sums16<false>(v, own + 3);
+            ld4(in, n, N, Q_T, lo);
+            own[0] = w_add(own[0], lo[3]);
+            ld4(in, n, N, Q_JXLO, lo);
+            own[3] = w_add(own[3], lo[2]);
+            own[4] = w_wide(lo[0]);
+            own[5] = w_wide(lo[1]);
+            R g4[4];
+            ld4(in, n, N, Q_TH, g4);
+            th = g4[0]; u[0] = g4[1]; u[1] = g4[2];
+        }
+        R fi[16], gi[16];   // increments of the streamed populations
+        Macro<2, R> m;
+        for (;;) {
+            ++its;
+            const R s = sqrt_(th), inv_s = R(1) / s;
+            R ax[4][4], ay[4][4];
+            bool nx0[4], ny0[4];
+            const R dt = typed<R>(p).dt;
+            const bool okx = axis_weights16<R>(L, s, u[0], dt, ax, nx0), oky = axis_weights16<R>(L, s, u[1], dt, ay, ny0);
+            if (okx && oky) {
+                auto side = [](const bool (&z)[4]) { return (z[0] == z[1] && z[1] == z[2] && z[2] == z[3]) ? 4 : 5; };
+                nreg += (unsigned)(side(nx0) * side(ny0) - (its == 1 ? 1 : 0));
+                R Lx[4][4], Ly[4][4];
+                const R q = (gb[0] - s) * inv_s;
+                axis_rows16<R>(L, q, (gb[1] - u[0]) * inv_s, Lx);
+                axis_rows16<R>(L, q, (gb[2] - u[1]) * inv_s, Ly);
+                if constexpr (sizeof(R) == 8) {
+                    R acc[2][16], v[16];
+                    contract16(own_slot, WT, ax, nx0, ay, ny0, Lx, Ly, acc);
+                    ld16(in, n, N, Q_F, v);
+#pragma unroll
+                    for (int i = 0; i < 16; ++i) fi[i] = acc[0][i] - v[i];
+                    ld16(in, n, N, Q_G, v);
+#pragma unroll
+                    for (int i = 0; i < 16; ++i) gi[i] = acc[1][i] - v[i];
+                } else {
+#pragma unroll 1
+                    for (int fam = 0; fam < 2; ++fam) {
+                        R acc[16];
+                        contract16(own_slot + 16 * fam, WT, ax, nx0, ay, ny0, Lx, Ly, acc);
+                        if (its > 1) {
+                            // the node's own populations carried from their stored gauge
+                            R g4[4], v[16], o[16], Dx[4][4], Dy[4][4];
+                            ld4(in, n, N, Q_TH, g4);
+                            const R e = fdiv_(g4[0] - th, (sqrt_(g4[0]) + s) * s);
+                            axis_inc<R>(L, e, (g4[1] - u[0]) * inv_s, Dx);
+                            axis_inc<R>(L, e, (g4[2] - u[1]) * inv_s, Dy);
+                            ld16(in, n, N, 16 * fam, v);
+                            apply_inc<R>(Dx, Dy, v, o);
+#pragma unroll
+                            for (int i = 0; i < 16; ++i) acc[i] += o[i];
+                        }
+                        if (fam == 0) {
+#pragma unroll
+                            for (int i = 0; i < 16; ++i) fi[i] = acc[i];
+                        } else {
+#pragma unroll
+                            for (int i = 0; i < 16; ++i) gi[i] = acc[i];
+                        }
+                    }
+                }
+            } else {
+                R f2[16], g2[16];
+                q16_stream_any<R>(p, in, X, Y, th, u[0], u[1], its == 1, f2, g2, nreg, npair);
+#pragma unroll
+                for (int i = 0; i < 16; ++i) { fi[i] = f2[i]; gi[i] = g2[i]; }
+            }
+            A d[4];
+            sums16<true>(fi, d);
+            sums16<false>(gi, d + 3);
+            m.update(p, th, u, own, d, F, rEl, 1.0);
+            const float res = m.change(th);
+            conv = sizeof(R) == 4 ? res <= p.tol_f : (double)res <= p.tol;
+            if (conv || its >= (unsigned)p.max_iter || !(res == res)) break;
+            th = w_round(m.ths);
+            u[0] = w_round(m.uu[0]);
+            u[1] = w_round(m.uu[1]);
         }
 
         // ---- collision in type R, equilibria as increments over their co-moving form
         const TypedParams<R> &q = typed<R>(p);
-        const R rho = (R)mac[0], u_x = (R)mac[1], u_y = (R)mac[2], uhx = (R)mac[3], uhy = (R)mac[4];
-        const R E = (R)mac[5], Pg = (R)mac[9], ths = (R)mac[10];
-        const R fx = (R)Fx, fy = (R)Fy, m0 = (R)M0, dt = q.dt, om = q.omega;
-        const double sd = sqrt((double)th), ssd = sqrt(mac[10]);
-        const double isd = 1.0 / sd;
-        const R is = (R)isd, sst = (R)ssd;
-        const R ds = (R)((mac[10] - (double)th) / (ssd + sd) * isd);   // (s* - s)/s
-        const R dux = (R)(mac[1] - (double)ux) * is, duy = (R)(mac[2] - (double)uy) * is;
-        const R shx = fx * dt / rho * is, shy = fy * dt / rho * is;   // du of the force
-        R Dx[4][4], Dy[4][4], Ex[4][4], Ey[4][4];
+        {
+            R v[16];
+            ld16(in, n, N, Q_F, v);
+#pragma unroll
+            for (int i = 0; i < 16; ++i) fi[i] += v[i];
+            ld16(in, n, N, Q_G, v);
+#pragma unroll
+            for (int i = 0; i < 16; ++i) gi[i] += v[i];
+        }
+        const R rho = w_round(m.rho), u_x = w_round(m.uu[0]), u_y = w_round(m.uu[1]);
+        const R uhx = w_round(m.uh[0]), uhy = w_round(m.uh[1]), E = w_round(m.E), Pg = w_round(m.P);
+        const R fx = w_round(F[0]), fy = w_round(F[1]), m0 = w_round(M0), dt = q.dt, om = q.omega;
+        const A sA = w_sqrt(th);
+        const R s = w_round(sA), is = R(1) / s, sst = sqrt_(w_round(m.ths));
+        const R ds = fdiv_(m.dth, (sst + s) * s);                    // (s* - s)/s
+        const R dux = w_round(m.du[0]) * is, duy = w_round(m.du[1]) * is;
+        const R irh = R(1) / rho, ihP = R(1) / (R(2) * Pg);          // 1/rho, 1/(2P)
+        const R shx = fx * dt * irh * is, shy = fy * dt * irh * is;  // du of the force
+        R Dx[4][4], Dy[4][4], h[Q16], eqi[Q16], fo[Q16];
         axis_inc<R>(L, ds, dux, Dx);                                  // lambda* -> lambda
         axis_inc<R>(L, ds, duy, Dy);
-        axis_inc<R>(L, ds, dux + shx, Ex);                            // lambda* + du -> lambda
-        axis_inc<R>(L, ds, duy + shy, Ey);
-        R h[Q16], eqi[Q16], shi[Q16];
 #pragma unroll
         for (int i = 0; i < Q16; ++i) h[i] = rho * (L.w[i & 3] * L.w[i >> 2]);
         apply_inc<R>(Dx, Dy, h, eqi);
-        apply_inc<R>(Ex, Ey, h, shi);
-        // Collision keeps the mass and adds F dt to the momentum: sum_i f_out = rho and
-        // sum_i f_out v_i = rho u + F dt exactly.  The stored values are made to carry both
-        // (their FP64 sums are compared with the exact ones; the mass defect, which the
-        // rounded weights and products would otherwise add every step in the same
-        // direction, is spread by W_i, the momentum defect by W_i s c_i / theta, which has
-        // no mass).  Zero in exact arithmetic.
-        R fo[Q16];
-        double sf = 0.0, sjx = 0.0, sjy = 0.0;
+        {
+            R Ex[4][4], Ey[4][4], shi[Q16];
+            axis_inc<R>(L, ds, dux + shx, Ex);                        // lambda* + du -> lambda
+            axis_inc<R>(L, ds, duy + shy, Ey);
+            apply_inc<R>(Ex, Ey, h, shi);
 #pragma unroll
-        for (int i = 0; i < Q16; ++i) fo[i] = ft[i] + om * ((h[i] - ft[i]) + eqi[i]) + (shi[i] - eqi[i]);
-        if constexpr (sizeof(R) == 4) {
-            double m[3];
-            q16_ff_moments<true>(fo, m);
-            sf = m[0]; sjx = m[1]; sjy = m[2];
-        } else {
-#pragma unroll
-            for (int i = 0; i < Q16; ++i) {
-                const double f = (double)fo[i];
-                sf += f;
-                sjx += f * Ld.c[i & 3];
-                sjy += f * Ld.c[i >> 2];
-            }
+            for (int i = 0; i < Q16; ++i) fo[i] = fi[i] + om * ((h[i] - fi[i]) + eqi[i]) + (shi[i] - eqi[i]);
         }
-        // momentum of the stored values in the streaming gauge: sum f (s c + u)
-        sjx = sd * sjx + sf * (double)ux;
-        sjy = sd * sjy + sf * (double)uy;
-        const double mdef = mac[0] - sf;
-        const R fdef = (R)mdef;
-        // W_i s c_i J / theta = W_i c_i J / s (sum_i W_i c_i^2 = T_L = 1); the mass part
-        // W_i mdef already carries the momentum mdef u
-        const R jxdef = (R)((mac[0] * mac[1] + Fx * p.dt - sjx - mdef * (double)ux) * isd);
-        const R jydef = (R)((mac[0] * mac[2] + Fy * p.dt - sjy - mdef * (double)uy) * isd);
-        R *orec = out + (size_t)n * SLQ;
+        bad = !(eqi[0] - eqi[0] == R(0));
+        // Collision keeps the mass and adds F dt to the momentum: sum_i f_out = rho and
+        // sum_i f_out (v_i - u) = rho (u* - u) + F dt exactly.  The stored values are made to
+        // carry both (their sums are compared with the exact ones; the mass defect, which the
+        // rounded weights and products would otherwise add every step in the same direction,
+        // is spread by W_i, the momentum defect by W_i s c_i / theta, which has no mass).
+        // Zero in exact arithmetic.
+        A sm[3], jex[2];
+#pragma unroll
+        for (int a = 0; a < 2; ++a) jex[a] = w_add(w_mul(m.rho, m.du[a]), w_mul(F[a], wide_dt<A>(p)));
+        sums16<true>(fo, sm);
+        const R fdef = w_round(w_sub(m.rho, sm[0]));
+        // W_i s c_i J / theta = W_i c_i J / s (sum_i W_i c_i^2 = T_L = 1)
+        const R jxdef = w_round(w_sub(jex[0], w_mul(sA, sm[1]))) * is;
+        const R jydef = w_round(w_sub(jex[1], w_mul(sA, sm[2]))) * is;
 #pragma unroll
         for (int i = 0; i < Q16; ++i)
             fo[i] += (L.w[i & 3] * L.w[i >> 2]) * (fdef + jxdef * L.c[i & 3] + jydef * L.c[i >> 2]);
         // what the stored values still miss (below their rounding) is kept beside them
-        double mlo = 0.0, jxlo = 0.0, jylo = 0.0;
+        R mlo = R(0), jxlo = R(0), jylo = R(0);
         if constexpr (sizeof(R) == 4) {
-            double m[3];
-            q16_ff_moments<true>(fo, m);
-            const double s0 = m[0], cx = m[1], cy = m[2];
-            mlo = mac[0] - s0;
-            // the mass lo carries momentum u mlo in the next step's sums
-            jxlo = (mac[0] * mac[1] + Fx * p.dt) - (sd * cx + (double)ux * s0) - mlo * (double)ux;
-            jylo = (mac[0] * mac[2] + Fy * p.dt) - (sd * cy + (double)uy * s0) - mlo * (double)uy;
+            sums16<true>(fo, sm);
+            mlo = w_round(w_sub(m.rho, sm[0]));
+            jxlo = w_round(w_sub(jex[0], w_mul(sA, sm[1])));
+            jylo = w_round(w_sub(jex[1], w_mul(sA, sm[2])));
         }
-#pragma unroll
-        for (int r = 0; r < 4; ++r) st4(orec + Q_F + 4 * r, fo[4 * r], fo[4 * r + 1], fo[4 * r + 2], fo[4 * r + 3]);
+        st16(out, n, N, Q_F, fo);
 
-        // the quotients by P and rho as products with two reciprocals
-        const R irh = R(1) / rho, ihP = R(1) / (R(2) * Pg);   // 1/rho, 1/(2P)
         const R Prh = Pg * irh, k2 = dt * rho * ihP;            // P/rho, dt rho/(2P)
         const R H = E + Prh;
         const R Ixx = R(2) * uhx * fx + dt * fx * fx * E * ihP;
@@ -893,55 +1143,31 @@ __global__ void __launch_bounds__(128, sizeof(R) == 4 ? Q16_MIN_BLOCKS : 1) k_q1
         }
         R ginc[Q16];
         apply_inc<R>(Dx, Dy, h, ginc);
+        bad = bad || !(ginc[0] - ginc[0] == R(0));
         // energy: sum_i g_out = sum_i g~ + dt (M_0 + 2 uhat . F) exactly (the heat-flux
         // correction sums to M_0, the force work to 2 uhat . F); the same defect spreading
-        R go[Q16];
-        double sg = 0.0;
+        const A work = w_add(w_mul(m.uh[0], F[0]), w_mul(m.uh[1], F[1]));
+        const A g_tot = w_add(m.gs, w_mul(w_add(M0, w_mul(work, R(2))), wide_dt<A>(p)));
 #pragma unroll
-        for (int i = 0; i < Q16; ++i) go[i] = gt[i] - om * gt[i] + (h[i] + ginc[i]);
+        for (int i = 0; i < Q16; ++i) fo[i] = gi[i] - om * gi[i] + (h[i] + ginc[i]);
+        sums16<false>(fo, sm);
+        const R gdef = w_round(w_sub(g_tot, sm[0]));
+#pragma unroll
+        for (int i = 0; i < Q16; ++i) fo[i] += gdef * (L.w[i & 3] * L.w[i >> 2]);
+        R glo = R(0);
         if constexpr (sizeof(R) == 4) {
-            q16_ff_moments<false>(go, &sg);
-        } else {
-#pragma unroll
-            for (int i = 0; i < Q16; ++i) sg += (double)go[i];
+            sums16<false>(fo, sm);
+            glo = w_round(w_sub(g_tot, sm[0]));
         }
-        const double g_tot = 2.0 * mac[0] * mac[5] + p.dt * (M0 + 2.0 * (mac[3] * Fx + mac[4] * Fy));
-        const R gdef = (R)(g_tot - sg);
-#pragma unroll
-        for (int i = 0; i < Q16; ++i) go[i] += gdef * (L.w[i & 3] * L.w[i >> 2]);
-        double glo = 0.0;
-        if constexpr (sizeof(R) == 4) {
-            double s1;
-            q16_ff_moments<false>(go, &s1);
-            glo = g_tot - s1;
-        }
-#pragma unroll
-        for (int r = 0; r < 4; ++r) st4(orec + Q_G + 4 * r, go[4 * r], go[4 * r + 1], go[4 * r + 2], go[4 * r + 3]);
-        st4(orec + Q_TH, th, ux, uy, rho);
-        st4(orec + Q_T, (R)mac[7], uhx, uhy, (R)mlo);
-        st4(orec + Q_JXLO, (R)jxlo, (R)jylo, (R)glo, R(0));
-        const double chk = mac[0] + mac[7] + (double)ginc[0] + (double)eqi[0];
-        nonfinite = (chk - chk == 0.0) ? 0ull : 1ull;
+        st16(out, n, N, Q_G, fo);
+        const R T = w_round(m.T);
+        st4(out, n, N, Q_TH, th, u[0], u[1], rho);
+        st4(out, n, N, Q_T, T, uhx, uhy, mlo);
+        st4(out, n, N, Q_JXLO, jxlo, jylo, glo, R(0));
+        floored = w_double(m.pr) < p.p_floor;
+        bad = bad || !(rho - rho == R(0)) || !(T - T == R(0));
     }
-    // counters: warp sums (every thread of the block reaches here; the warp's lanes are
-    // its linear thread indices, whatever the block's x extent), one atomic per warp
-    unsigned long long v[6] = {its, nonconv, clamped, nonfinite, nreg, npair}, mx = its;
-    for (int o = 16; o > 0; o >>= 1) {
-#pragma unroll
-        for (int k = 0; k < 6; ++k) v[k] += __shfl_xor_sync(0xffffffffu, v[k], o);
-        const unsigned long long m2 = __shfl_xor_sync(0xffffffffu, mx, o);
-        mx = m2 > mx ? m2 : mx;
-    }
-    if ((threadIdx.x + threadIdx.y * blockDim.x) % 32 == 0) {
-        if (v[0]) atomicAdd(&stats->streams, v[0]);
-        if (v[1]) atomicAdd(&stats->nonconv, v[1]);
-        if (v[2]) atomicAdd(&stats->clamped, v[2]);
-        if (v[3]) atomicAdd(&stats->nonfinite, v[3]);
-        // the region-stream counters of the D2Q9 step, filled the same way here
-        if (v[4]) atomicAdd(&stats->region_nodes, v[4]);
-        if (v[5]) atomicAdd(&stats->pair_streams, v[5]);
-        if (mx) atomicMax(&stats->max_streams, mx);
-    }
+    add_counts(counts, stats, its, nreg, npair, !conv, false, floored, bad);
 }
 
 // Output fields: rho, uhat, T, p in FP64.

@@ -192,54 +192,6 @@ __global__ void k_q27_init(DevParams p, Grid3 g3, const double *__restrict__ rho
 }
 
 // ---------------------------------------------------------------------------
-// Wide arithmetic of the non-local terms: FP64 in the FP64 form, float-float in the FP32
-// form (GB300 runs an FP64 addition at the cost of 64 FP32 ones, a float-float addition
-// takes about 12).
-template <typename R> struct Wide;
-template <> struct Wide<float> { using type = ffv; };
-template <> struct Wide<double> { using type = double; };
-__device__ __forceinline__ ffv w_add(float a, float b) { return ff_pair(a, b); }
-__device__ __forceinline__ ffv w_add(ffv a, ffv b) { return ff_add(a, b); }
-__device__ __forceinline__ ffv w_add(ffv a, float b) { return ff_add(a, b); }
-__device__ __forceinline__ double w_add(double a, double b) { return a + b; }
-__device__ __forceinline__ ffv w_sub(float a, float b) { return ff_pair(a, -b); }
-__device__ __forceinline__ ffv w_sub(ffv a, ffv b) { return ff_add(a, ff_neg(b)); }
-__device__ __forceinline__ double w_sub(double a, double b) { return a - b; }
-__device__ __forceinline__ ffv w_mul(ffv a, ffv b) { return ff_mul(a, b); }
-__device__ __forceinline__ ffv w_mul(ffv a, float b) { return ff_mul(a, b); }
-__device__ __forceinline__ double w_mul(double a, double b) { return a * b; }
-__device__ __forceinline__ float w_x4(float a) { return 4.0f * a; }
-__device__ __forceinline__ ffv w_x4(ffv a) { return {4.0f * a.hi, 4.0f * a.lo}; }
-__device__ __forceinline__ double w_x4(double a) { return 4.0 * a; }
-__device__ __forceinline__ double w_double(ffv a) { return (double)a.hi + (double)a.lo; }
-__device__ __forceinline__ double w_double(double a) { return a; }
-// a FP64 constant in the wide type
-template <typename A> __device__ __forceinline__ A w_const(double x);
-template <> __device__ __forceinline__ double w_const<double>(double x) { return x; }
-template <> __device__ __forceinline__ ffv w_const<ffv>(double x)
-{
-    const float h = (float)x;
-    return {h, (float)(x - (double)h)};
-}
-__device__ __forceinline__ ffv w_rcp(ffv a) { return ff_rcp(a); }
-__device__ __forceinline__ double w_rcp(double a) { return rcp_d(a); }
-
-// p/rho of the run's equation of state; the exponential factor of the Dieterici form and
-// the double well's small polynomial in FP64 (rare forms, not worth a float-float one).
-__device__ __forceinline__ double w_p_over_rho(const DevParams &p, double r, double t)
-{
-    if (p.eos_kind != 0) return eos_pressure<double>(p.eos_kind, p.a, p.b, p.R, r, t, p.sp) / r;
-    return p.R * t * rcp_d(1.0 - p.b * r) - p.a * r;
-}
-__device__ __forceinline__ ffv w_p_over_rho(const DevParams &p, float r, float t)
-{
-    if (p.eos_kind != 0)
-        return w_const<ffv>(eos_pressure<double>(p.eos_kind, p.a, p.b, p.R, (double)r, (double)t, p.sp) / (double)r);
-    const ffv a = {p.ff_a[0], p.ff_a[1]}, b = {p.ff_b[0], p.ff_b[1]}, Rg = {p.ff_R[0], p.ff_R[1]};
-    const ffv den = ff_add(ff_neg(ff_mul(b, r)), 1.0f);
-    return w_sub(ff_mul(ff_mul(Rg, t), ff_rcp(den)), ff_mul(a, r));
-}
-
 // Non-local terms, stage 0: p/rho of every node of `src`.
 template <typename R>
 __global__ void k_q27_pi(DevParams p, const R *__restrict__ src, typename Wide<R>::type *__restrict__ nl)
@@ -819,7 +771,7 @@ __device__ __forceinline__ void apply3_inc(const A (&Dx)[3][3], const A (&Dy)[3]
 
 // ---------------------------------------------------------------------------
 // Staging.  The tile of a block and its staged slots.
-constexpr int Q27_THREADS = 128, T27X = 8, T27Y = 4, T27Z = 4, HALO27 = 2;
+constexpr int Q27_THREADS = STEP_THREADS, T27X = 8, T27Y = 4, T27Z = 4, HALO27 = 2;
 constexpr int S27X = T27X + 2 * HALO27, S27Y = T27Y + 2 * HALO27, S27Z = T27Z + 2 * HALO27;
 constexpr int SLOTS27 = S27X * S27Y * S27Z;
 constexpr int PY27 = S27X, PZ27 = S27X * S27Y;   // slots per row, per plane
@@ -842,24 +794,6 @@ __device__ __forceinline__ size_t slot_node27(const DevParams &p, const Grid3 &g
     return (size_t)node27(p, g3, t.X0 - HALO27 + x, t.Y0 - HALO27 + y, t.Z0 - HALO27 + z);
 }
 
-// Moments about (u_x, u_y, u_z) of 27 populations at velocities s c + u + w per axis.
-__device__ __forceinline__ void moments27(double s, const double (&w)[3], double (&f)[27])
-{
-    const double s2 = s * s;
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        const int st = a == 0 ? 1 : (a == 1 ? 3 : 9);
-#pragma unroll
-        for (int q = 0; q < 9; ++q) {
-            const int i = a == 0 ? 3 * q : (a == 1 ? (q / 3) * 9 + q % 3 : q);
-            const double sum = f[i] + f[i + 2 * st];
-            const double m0 = sum + f[i + st], A = s * (f[i + 2 * st] - f[i]);
-            const double m1 = A + w[a] * m0;
-            f[i] = m0; f[i + st] = m1; f[i + 2 * st] = s2 * sum + w[a] * (A + m1);
-        }
-    }
-}
-
 // The map of one axis applied to 27 values along it (stride 1, 3 or 9).
 template <int ST, typename A>
 __device__ __forceinline__ void apply_axis27(const A (&G)[3][3], A (&h)[27])
@@ -873,65 +807,50 @@ __device__ __forceinline__ void apply_axis27(const A (&G)[3][3], A (&h)[27])
     }
 }
 
-// Stages one family (record offset OFF): FP32: its populations carried into the gauge of
-// node `nbase` (smooth: less that node's, in increment form; see pond_step.cuh); FP64:
-// moments about that node's velocity.  gb = (sqrt theta, u) of the gauge.
-template <int OFF>
-__device__ __forceinline__ void stage27(const DevParams &p, const Grid3 &g3, const float *__restrict__ in,
-                                        const Tile27 &t, size_t nbase, const float (&gb)[4], bool smooth, float *slots)
+// Stages one family (record offset OFF): its populations carried into the tile's gauge gb
+// = (sqrt theta, u), theta = thb; inc (FP32): less those of node `nbase`, whose gauge gb
+// then is, in increment form (see the head of pond_step.cuh).
+template <int OFF, typename R>
+__device__ __forceinline__ void stage27(const DevParams &p, const Grid3 &g3, const R *__restrict__ in,
+                                        const Tile27 &t, size_t nbase, const R (&gb)[4], R thb, bool inc, R *slots)
 {
-    constexpr int DS = Slot27<float>::stride;
+    constexpr int DS = Slot27<R>::stride;
     const size_t N = (size_t)p.N;
-    float base[27], gq[4];
-    load27<OFF, 27>(in, nbase, N, base);
-    load27<R_TH, 4>(in, nbase, N, gq);
-    const float thb = gq[0], inv_sb = 1.0f / gb[0];
+    const R inv_sb = R(1) / gb[0];
 #pragma unroll 1
     for (int k = threadIdx.x; k < SLOTS27; k += Q27_THREADS) {
         const size_t nd = slot_node27(p, g3, t, k);
-        float gv[4], h[27];
+        R gv[4], h[27];
         load27<R_TH, 4>(in, nd, N, gv);
         load27<OFF, 27>(in, nd, N, h);
-        const float sn = sqrtf(gv[0]);
-        const float e = fdiv_(gv[0] - thb, (sn + gb[0]) * gb[0]);
-        const float w[3] = {(gv[1] - gb[1]) * inv_sb, (gv[2] - gb[2]) * inv_sb, (gv[3] - gb[3]) * inv_sb};
-        float D[3][3][3];
-        if (smooth) {
-            float o[27];
+        const R e = fdiv_(gv[0] - thb, (sqrt_(gv[0]) + gb[0]) * gb[0]);
+        const R w[3] = {(gv[1] - gb[1]) * inv_sb, (gv[2] - gb[2]) * inv_sb, (gv[3] - gb[3]) * inv_sb};
+        R D[3][3][3];
+        if (sizeof(R) == 4 && inc) {
+            R o[27], base[27];
 #pragma unroll
-            for (int a = 0; a < 3; ++a) axis_map<float>(e, w[a], D[a]);
-            apply3_inc<float>(D[0], D[1], D[2], h, o);
+            for (int a = 0; a < 3; ++a) axis_map<R>(e, w[a], D[a]);
+            apply3_inc<R>(D[0], D[1], D[2], h, o);
+            load27<OFF, 27>(in, nbase, N, base);
 #pragma unroll
             for (int i = 0; i < 27; ++i) h[i] = (h[i] - base[i]) + o[i];
         } else {
 #pragma unroll
-            for (int a = 0; a < 3; ++a) axis_rows<float>(e, w[a], D[a]);
+            for (int a = 0; a < 3; ++a) axis_rows<R>(e, w[a], D[a]);
             apply_axis27<1>(D[0], h);
             apply_axis27<3>(D[1], h);
             apply_axis27<9>(D[2], h);
         }
-        float4 *dst = reinterpret_cast<float4 *>(slots + (size_t)k * DS);
+        R *dst = slots + (size_t)k * DS;
+        if constexpr (sizeof(R) == 4) {
 #pragma unroll
-        for (int c = 0; c < DS / 4; ++c)
-            dst[c] = make_float4(h[4 * c], h[4 * c + 1], h[4 * c + 2], 4 * c + 3 < 27 ? h[4 * c + 3 < 27 ? 4 * c + 3 : 0] : 0.0f);
-    }
-}
-template <int OFF>
-__device__ __forceinline__ void stage27(const DevParams &p, const Grid3 &g3, const double *__restrict__ in,
-                                        const Tile27 &t, size_t, const double (&gb)[4], bool, double *slots)
-{
-    const size_t N = (size_t)p.N;
-#pragma unroll 1
-    for (int k = threadIdx.x; k < SLOTS27; k += Q27_THREADS) {
-        const size_t nd = slot_node27(p, g3, t, k);
-        double gv[4], h[27];
-        load27<R_TH, 4>(in, nd, N, gv);
-        load27<OFF, 27>(in, nd, N, h);
-        const double w[3] = {gv[1] - gb[1], gv[2] - gb[2], gv[3] - gb[3]};
-        moments27(sqrt(gv[0]), w, h);
-        double *dst = slots + (size_t)k * Slot27<double>::stride;
+            for (int c = 0; c < DS / 4; ++c)
+                reinterpret_cast<float4 *>(dst)[c] =
+                    make_float4(h[4 * c], h[4 * c + 1], h[4 * c + 2], 4 * c + 3 < 27 ? h[4 * c + 3 < 27 ? 4 * c + 3 : 0] : 0.0f);
+        } else {
 #pragma unroll
-        for (int i = 0; i < 27; ++i) dst[i] = h[i];
+            for (int i = 0; i < 27; ++i) dst[i] = h[i];
+        }
     }
 }
 
@@ -1029,7 +948,7 @@ __device__ __forceinline__ void contract27(const float *own, const float (&a)[3]
         }
     }
 }
-// FP64 (slots of moments): each component's own four columns; acc = streamed populations.
+// FP64: each component's own four columns; acc = streamed populations.
 __device__ __forceinline__ void contract27(const double *own, const double (&a)[3][3][4], const bool (&near0)[3][3],
                                            const double (&L)[3][3][3], double (&acc)[27])
 {
@@ -1241,7 +1160,7 @@ __global__ void __launch_bounds__(Q27_THREADS, sizeof(R) == 4 ? 2 : 1)
     double *own_s = reinterpret_cast<double *>(q27_dyn_smem) + threadIdx.x;   // [OWN27][threads]
     R *slots = reinterpret_cast<R *>(q27_dyn_smem + (size_t)OWN27 * Q27_THREADS * 8);
     __shared__ StepCounts counts;
-    __shared__ uint4 best[Q27_THREADS / 32];   // per warp: largest theta (bits), its slot, smallest theta
+    __shared__ uint4 best[Q27_THREADS / 32];
     const int tid = threadIdx.x;
     const size_t N = (size_t)p.N;
     const Tile27 tl{(int)blockIdx.x * T27X, (int)blockIdx.y * T27Y, (int)blockIdx.z * T27Z};
@@ -1251,38 +1170,21 @@ __global__ void __launch_bounds__(Q27_THREADS, sizeof(R) == 4 ? 2 : 1)
     const size_t n = valid ? ((size_t)Z * p.ny + Y) * p.nx + X : 0;
     if (tid == 0) counts = StepCounts{};
 
-    // the tile's common gauge: FP32 the staged node of the largest theta, FP64 the velocity of
-    // the tile's middle node
-    size_t nbase;
-    bool smooth = false;
-    if constexpr (sizeof(R) == 4) {
-        unsigned top = 0, at = 0, low = 0xffffffffu;
-        for (int k = tid; k < SLOTS27; k += Q27_THREADS) {
-            const float th = __ldg(in + rec_at(in, slot_node27(p, g3, tl, k), R_TH, N));
-            const unsigned b = (th > 0.0f && th < 3.0e38f) ? __float_as_uint(th) : 0u;   // finite positive only
-            low = min(low, b);
-            if (b > top) { top = b; at = (unsigned)k; }
-        }
-        const unsigned m = __reduce_max_sync(0xffffffffu, top);
-        const unsigned w = __reduce_min_sync(0xffffffffu, top == m ? at : 0xffffffffu);
-        low = __reduce_min_sync(0xffffffffu, low);
-        if ((tid & 31) == 0) best[tid >> 5] = make_uint4(m, w, low, 0);
-        __syncthreads();
-        uint4 b = best[0];
-#pragma unroll
-        for (int k = 1; k < Q27_THREADS / 32; ++k) {
-            if (best[k].x > b.x || (best[k].x == b.x && best[k].y < b.y)) { b.x = best[k].x; b.y = best[k].y; }
-            b.z = min(b.z, best[k].z);
-        }
-        smooth = __uint_as_float(b.z) > SMOOTH_TILE * __uint_as_float(b.x);
-        nbase = slot_node27(p, g3, tl, (int)min(b.y, (unsigned)(SLOTS27 - 1)));
-    } else {
-        nbase = ((size_t)min(tl.Z0 + T27Z / 2, g3.nz - 1) * p.ny + min(tl.Y0 + T27Y / 2, p.ny - 1)) * p.nx +
-                min(tl.X0 + T27X / 2, p.nx - 1);
+    // the tile's common gauge
+    Extremes ex;
+    for (int k = tid; k < SLOTS27; k += Q27_THREADS)
+        ex.offer((float)__ldg(in + rec_at(in, slot_node27(p, g3, tl, k), R_TH, N)), k);
+    ex = tile_extremes(ex, best);
+    const bool inc = sizeof(R) == 4 && ex.smooth();
+    const size_t nbase = slot_node27(p, g3, tl, min((int)ex.at, SLOTS27 - 1));
+    R gb[4], thb;
+    {
+        R hot[4], cold[4];
+        load27<R_TH, 4>(in, nbase, N, hot);
+        load27<R_TH, 4>(in, slot_node27(p, g3, tl, min((int)ex.lat, SLOTS27 - 1)), N, cold);
+        common_gauge<R, 4>(inc, hot, cold, gb);
+        thb = inc ? hot[0] : gb[0] * gb[0];
     }
-    R gb[4];
-    load27<R_TH, 4>(in, nbase, N, gb);
-    gb[0] = sizeof(R) == 4 ? sqrt_(gb[0]) : R(1);
 
     R th = R(1), u[3] = {R(0), R(0), R(0)};
     if (valid) {
@@ -1323,11 +1225,7 @@ __global__ void __launch_bounds__(Q27_THREADS, sizeof(R) == 4 ? 2 : 1)
         for (int x = 0; x < 3; ++x) {
             const bool ok = axis_weights<R>(s, u[x], typed<R>(p).dt, a[x], near0[x]);
             fast = fast && ok;
-            if constexpr (sizeof(R) == 8) {
-                moment_rows(u[x] - gb[1 + x], inv_s, L[x]);
-            } else {
-                axis_rows<R>((gb[0] - s) * inv_s, (gb[1 + x] - u[x]) * inv_s, L[x]);
-            }
+            axis_rows<R>((gb[0] - s) * inv_s, (gb[1 + x] - u[x]) * inv_s, L[x]);
         }
         if (active) {
             its = it;
@@ -1351,8 +1249,8 @@ __global__ void __launch_bounds__(Q27_THREADS, sizeof(R) == 4 ? 2 : 1)
             const int fam = (it & 1) ? ps : 1 - ps;
             if (staged != fam) {
                 __syncthreads();
-                if (fam == 0) stage27<R_F>(p, g3, in, tl, nbase, gb, smooth, slots);
-                else stage27<R_G>(p, g3, in, tl, nbase, gb, smooth, slots);
+                if (fam == 0) stage27<R_F>(p, g3, in, tl, nbase, gb, thb, inc, slots);
+                else stage27<R_G>(p, g3, in, tl, nbase, gb, thb, inc, slots);
                 __syncthreads();
                 staged = fam;
             }

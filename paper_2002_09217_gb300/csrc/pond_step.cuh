@@ -33,15 +33,20 @@
 // by instruction issue (60 % active; FMA pipe 49 %, shared-memory pipe 41 %) in the mixed
 // form and by the FP64 pipe in the FP64 form; DRAM 6 % busy.
 //
-// FP32 accuracy.  The slots hold differences f^b - (populations of the tile's base node),
-// computed in increment form (the map as I + E with E = 0 for equal gauges), and the
-// stream accumulates differences to the node's own slot, so that equal gauges and
-// populations give exactly zero, and rounding is proportional to local differences and
-// not to the populations, and does not accumulate as a bias.  The base is the staged node
-// of the largest theta: across an interface rho theta (the second moment) varies little,
-// so that in the hottest gauge only the rest population differs much between the phases,
-// and carrying it into a colder gauge does not amplify its rounding.
-// In FP64 the slots hold the moments about the velocity of one node of the tile.
+// Accuracy.  A tile whose thetas differ holds the carried populations themselves in the
+// gauge of geometric-mean theta and mean velocity of its hottest and coldest nodes, by
+// product-form rows of the map.  Populations carried into a colder gauge are amplified (by
+// (theta_b / theta) per axis for the outermost of three velocities, more for four), those
+// carried into a hotter one cancel; the middle gauge splits that between the two maps.  On
+// a 0.8 T_cr interface the worst error of a single population in FP32 is 2e-7 (D3Q27) and
+// 7e-8 (D2Q16), no more than carrying each node straight into the arrival gauge; the
+// hottest gauge left 3e-5 on D2Q16, the coldest 1e-6.
+// The FP32 stream accumulates differences to the node's own slot, so that equal gauges and
+// populations give exactly zero, rounding is proportional to local differences and not to
+// the populations, and it does not accumulate as a bias.  FP32 tiles of nearly equal theta
+// hold, moreover, differences to the populations of the tile's hottest node in its gauge,
+// in increment form (the map as I + E with E = 0 for equal gauges), so that weak waves are
+// not rounded to the populations' ulp; across an interface that form would cancel.
 #pragma once
 
 #include "pond_kernels.cuh"
@@ -56,10 +61,10 @@ constexpr int HALO = 2;       // staged halo: stencil reach for |v| dt < 1, and 
 // that the general stream handles as a region; wider ones take the per-pair stream.
 constexpr int REGION_MAX = 8;
 // FP32: tiles whose smallest theta is above this share of the largest are staged in
-// increment form over the base node's populations, others as carried populations.  A
+// increment form over the hottest node's populations, others as carried populations.  A
 // weak wave (theta within 1e-3) needs the former; at a liquid-vapour interface (a factor of
 // 4 to 6) the increment form left 6e-6 on single populations in three dimensions, the
-// direct form 1.7e-7, as much as carrying each node straight into the arrival gauge.
+// direct form 1.7e-7.
 constexpr float SMOOTH_TILE = 0.9f;
 // Mixed form: a frame-search residual below this multiple of tol that no longer halves is
 // taken as the FP32 rounding floor (the EoS cancels up to ~200x inside interfaces).
@@ -510,6 +515,189 @@ __device__ __forceinline__ void eos_update(const DevParams &p, const float *bhi,
     o.dth = (ths.hi - lam[0]) + ths.lo;
     o.dux = dux.hi; o.duy = duy.hi;
 }
+// ---------------------------------------------------------------------------
+// Wide arithmetic of the D2Q16 and D3Q27 steps: FP64 in the FP64 form, float-float in the
+// FP32 form (GB300 runs an FP64 addition at the cost of 64 FP32 ones, a float-float addition
+// takes about 12).
+template <typename R> struct Wide;
+template <> struct Wide<float> { using type = ffv; };
+template <> struct Wide<double> { using type = double; };
+__device__ __forceinline__ ffv w_add(float a, float b) { return ff_pair(a, b); }
+__device__ __forceinline__ ffv w_add(ffv a, ffv b) { return ff_add(a, b); }
+__device__ __forceinline__ ffv w_add(ffv a, float b) { return ff_add(a, b); }
+__device__ __forceinline__ double w_add(double a, double b) { return a + b; }
+__device__ __forceinline__ ffv w_sub(float a, float b) { return ff_pair(a, -b); }
+__device__ __forceinline__ ffv w_sub(ffv a, ffv b) { return ff_add(a, ff_neg(b)); }
+__device__ __forceinline__ double w_sub(double a, double b) { return a - b; }
+__device__ __forceinline__ ffv w_mul(ffv a, ffv b) { return ff_mul(a, b); }
+__device__ __forceinline__ ffv w_mul(ffv a, float b) { return ff_mul(a, b); }
+__device__ __forceinline__ double w_mul(double a, double b) { return a * b; }
+__device__ __forceinline__ float w_x4(float a) { return 4.0f * a; }
+__device__ __forceinline__ ffv w_x4(ffv a) { return {4.0f * a.hi, 4.0f * a.lo}; }
+__device__ __forceinline__ double w_x4(double a) { return 4.0 * a; }
+__device__ __forceinline__ double w_double(ffv a) { return (double)a.hi + (double)a.lo; }
+__device__ __forceinline__ double w_double(double a) { return a; }
+__device__ __forceinline__ float w_round(ffv a) { return a.hi; }   // (hi, lo) are kept normalised
+__device__ __forceinline__ double w_round(double a) { return a; }
+__device__ __forceinline__ ffv w_wide(float a) { return {a, 0.0f}; }
+__device__ __forceinline__ double w_wide(double a) { return a; }
+// a FP64 constant in the wide type
+template <typename A> __device__ __forceinline__ A w_const(double x);
+template <> __device__ __forceinline__ double w_const<double>(double x) { return x; }
+template <> __device__ __forceinline__ ffv w_const<ffv>(double x)
+{
+    const float h = (float)x;
+    return {h, (float)(x - (double)h)};
+}
+__device__ __forceinline__ ffv w_rcp(ffv a) { return ff_rcp(a); }
+__device__ __forceinline__ double w_rcp(double a) { return rcp_d(a); }
+// square root of a value of type R in the wide type (FP32: one correction step)
+__device__ __forceinline__ ffv w_sqrt(float x)
+{
+    const float s = sqrtf(x);
+    return ff_norm(s, fmaf(-s, s, x) / (2.0f * s));
+}
+__device__ __forceinline__ double w_sqrt(double x) { return sqrt(x); }
+template <typename A> __device__ __forceinline__ A wide_dt(const DevParams &p);
+template <> __device__ __forceinline__ double wide_dt<double>(const DevParams &p) { return p.dt; }
+template <> __device__ __forceinline__ ffv wide_dt<ffv>(const DevParams &p) { return {p.ff_dt[0], p.ff_dt[1]}; }
+
+// p/rho of the run's equation of state; the exponential factor of the Dieterici form and
+// the double well's small polynomial in FP64 (rare forms, not worth a float-float one).
+__device__ __forceinline__ double w_p_over_rho(const DevParams &p, double r, double t)
+{
+    if (p.eos_kind != 0) return eos_pressure<double>(p.eos_kind, p.a, p.b, p.R, r, t, p.sp) / r;
+    return p.R * t * rcp_d(1.0 - p.b * r) - p.a * r;
+}
+__device__ __forceinline__ ffv w_p_over_rho(const DevParams &p, float r, float t)
+{
+    if (p.eos_kind != 0)
+        return w_const<ffv>(eos_pressure<double>(p.eos_kind, p.a, p.b, p.R, (double)r, (double)t, p.sp) / (double)r);
+    const ffv a = {p.ff_a[0], p.ff_a[1]}, b = {p.ff_b[0], p.ff_b[1]}, Rg = {p.ff_R[0], p.ff_R[1]};
+    const ffv den = ff_add(ff_neg(ff_mul(b, r)), 1.0f);
+    return w_sub(ff_mul(ff_mul(Rg, t), ff_rcp(den)), ff_mul(a, r));
+}
+// pressure p(rho, T) of wide rho, T
+__device__ __forceinline__ double w_pressure(const DevParams &p, double r, double t)
+{
+    if (p.eos_kind != 0) return eos_pressure<double>(p.eos_kind, p.a, p.b, p.R, r, t, p.sp);
+    return r * p.R * t * rcp_d(1.0 - p.b * r) - p.a * r * r;
+}
+__device__ __forceinline__ ffv w_pressure(const DevParams &p, ffv r, ffv t)
+{
+    if (p.eos_kind != 0)
+        return w_const<ffv>(eos_pressure<double>(p.eos_kind, p.a, p.b, p.R, w_double(r), w_double(t), p.sp));
+    const ffv a = {p.ff_a[0], p.ff_a[1]}, b = {p.ff_b[0], p.ff_b[1]}, Rg = {p.ff_R[0], p.ff_R[1]};
+    const ffv den = ff_add(ff_neg(ff_mul(r, b)), 1.0f);
+    return w_sub(ff_mul(ff_mul(ff_mul(r, Rg), t), ff_rcp(den)), ff_mul(ff_mul(r, r), a));
+}
+template <typename A> __device__ __forceinline__ A wide_p_floor(const DevParams &p);
+template <> __device__ __forceinline__ double wide_p_floor<double>(const DevParams &p) { return p.p_floor; }
+template <> __device__ __forceinline__ ffv wide_p_floor<ffv>(const DevParams &p) { return {p.ff_pfl[0], p.ff_pfl[1]}; }
+template <typename A> __device__ __forceinline__ A wide_T(const DevParams &p, A e, A rho);   // T of e (or T_iso)
+template <> __device__ __forceinline__ double wide_T<double>(const DevParams &p, double e, double rho)
+{
+    return p.isothermal ? p.T_iso : (e + p.a * rho) * p.pd.inv_cv;
+}
+template <> __device__ __forceinline__ ffv wide_T<ffv>(const DevParams &p, ffv e, ffv rho)
+{
+    if (p.isothermal) return {p.ff_Tiso[0], p.ff_Tiso[1]};
+    return ff_mul(ff_add(e, ff_mul(rho, ffv{p.ff_a[0], p.ff_a[1]})), ffv{p.ff_icv[0], p.ff_icv[1]});
+}
+__device__ __forceinline__ bool w_less(ffv a, ffv b) { return a.hi < b.hi || (a.hi == b.hi && a.lo < b.lo); }
+__device__ __forceinline__ bool w_less(double a, double b) { return a < b; }
+
+// Macroscopic fields of a node from the sums of its streamed populations in D dimensions
+// (moments Eq.), in the wide type.
+template <int D, typename R>
+struct Macro {
+    using A = typename Wide<R>::type;
+    A rho, gs, E, T, pr, P, ths;   // gs = sum of the streamed g; P = max(p, p_floor)
+    A uu[D], uh[D], du[D];         // streamed velocity u*, fluid velocity, u* - u
+    R dth;                         // theta* - theta
+    // own = stored sums {f, f c (D), g} and the momentum kept beside them (absolute, D);
+    // d = the stream's increments of the first D + 2; inv_TL = 1 / T_L
+    __device__ __forceinline__ void update(const DevParams &p, R th, const R (&u)[D], const A *own, const A *d,
+                                           const A (&F)[D], A rEl, double inv_TL)
+    {
+        const A s = w_sqrt(th);
+        rho = w_add(own[0], d[0]);
+        const A irho = w_rcp(rho);
+        const A hdt = w_mul(wide_dt<A>(p), R(0.5));
+        A kin;
+#pragma unroll
+        for (int a = 0; a < D; ++a) {
+            // sum f v = s sum f c + u sum f: the change of velocity alone
+            du[a] = w_mul(w_add(w_mul(s, w_add(own[1 + a], d[1 + a])), own[D + 2 + a]), irho);
+            uu[a] = w_add(du[a], w_wide(u[a]));
+            uh[a] = w_add(uu[a], w_mul(w_mul(F[a], hdt), irho));
+            const A k = w_mul(uh[a], uh[a]);
+            kin = a == 0 ? k : w_add(kin, k);
+        }
+        gs = w_add(own[D + 1], d[D + 1]);
+        E = w_mul(w_mul(gs, irho), R(0.5));
+        const A e = w_sub(w_sub(E, w_mul(kin, R(0.5))), w_mul(rEl, irho));
+        T = wide_T<A>(p, e, rho);
+        pr = w_pressure(p, rho, T);
+        const A fl = wide_p_floor<A>(p);
+        P = w_less(fl, pr) ? pr : fl;
+        ths = w_mul(w_mul(P, irho), R(inv_TL));
+        dth = w_round(w_sub(ths, w_wide(th)));
+    }
+    // relative change of the gauge
+    __device__ __forceinline__ float change(R th) const
+    {
+        const float sr = (float)sqrt_(th);
+        float r = fabsf((float)dth) / (float)th;
+#pragma unroll
+        for (int a = 0; a < D; ++a) r = fmaxf(r, fabsf((float)w_round(du[a])) / sr);
+        return !(dth == dth) || !(w_round(rho) == w_round(rho)) ? __int_as_float(0x7fc00000) : r;
+    }
+};
+
+// A tile's common gauge.  Each thread offers its staged nodes' thetas (finite positive
+// ones), then the block agrees on the nodes of the largest and the smallest (every thread
+// calls tile_extremes, which holds a barrier).
+struct Extremes {
+    unsigned top = 0, at = 0, low = 0xffffffffu, lat = 0;   // theta bits and slots
+    __device__ __forceinline__ void offer(float th, int slot)
+    {
+        if (!(th > 0.0f && th < 3.0e38f)) return;
+        const unsigned b = __float_as_uint(th);
+        if (b > top) { top = b; at = (unsigned)slot; }
+        if (b < low) { low = b; lat = (unsigned)slot; }
+    }
+    __device__ __forceinline__ float hottest() const { return __uint_as_float(top); }
+    // the tile's thetas lie within SMOOTH_TILE of each other
+    __device__ __forceinline__ bool smooth() const { return top != 0u && __uint_as_float(low) > SMOOTH_TILE * hottest(); }
+};
+__device__ __forceinline__ Extremes tile_extremes(Extremes t, uint4 *best)
+{
+    const unsigned m = __reduce_max_sync(0xffffffffu, t.top), w = __reduce_min_sync(0xffffffffu, t.top == m ? t.at : 0xffffffffu);
+    const unsigned n = __reduce_min_sync(0xffffffffu, t.low), v = __reduce_min_sync(0xffffffffu, t.low == n ? t.lat : 0xffffffffu);
+    if ((threadIdx.x & 31) == 0) best[threadIdx.x >> 5] = make_uint4(m, w, n, v);
+    __syncthreads();
+    uint4 b = best[0];
+#pragma unroll
+    for (int k = 1; k < STEP_THREADS / 32; ++k) {
+        const uint4 o = best[k];
+        if (o.x > b.x || (o.x == b.x && o.y < b.y)) { b.x = o.x; b.y = o.y; }
+        if (o.z < b.z || (o.z == b.z && o.w < b.w)) { b.z = o.z; b.w = o.w; }
+    }
+    t.top = b.x; t.at = b.y; t.low = b.z; t.lat = b.w;
+    return t;
+}
+// The gauge (sqrt theta, u) of a tile from the records' gauges at its hottest and coldest
+// nodes: the hottest node's own in increment form, else the geometric mean of the two
+// thetas and the mean velocity (half the amplification on the way in, half on the way out).
+template <typename R, int ND>
+__device__ __forceinline__ void common_gauge(bool inc, const R *hot, const R *cold, R (&gb)[ND])
+{
+    gb[0] = inc ? sqrt_(hot[0]) : sqrt_(sqrt_(hot[0]) * sqrt_(cold[0]));
+#pragma unroll
+    for (int k = 1; k < ND; ++k) gb[k] = inc ? hot[k] : R(0.5) * (hot[k] + cold[k]);
+}
+
 // Transfer increments along one axis, E[k][a] = l_k((a - 1) + e_a) - delta_ka with
 // e_a = q (a - 1) + w (q = (s_src - s)/s, w = (u_src - u)/s), from h = e/2 and
 // p = h (2 c_a + e): E_0 = p - h, E_1 = -2 p, E_2 = p + h.
@@ -552,37 +740,6 @@ __device__ __forceinline__ void map_inc(const R (&Ex)[3][3], const R (&Ey)[3][3]
 #pragma unroll
         for (int l = 0; l < 3; ++l) out[3 * l + k] = t[l] + (Ey[l][0] * u[0] + Ey[l][1] * u[1] + Ey[l][2] * u[2]);
     }
-}
-
-// Moments about (ux, uy) of nine populations at velocities s c + u_n along each axis
-// (wx, wy = u_n - u): M_mn at 3 n + m, m, n <= 2.
-__device__ __forceinline__ void moments9(const double *f, double s, double wx, double wy, double (&M)[9])
-{
-    const double s2 = s * s;
-    double r[9];
-#pragma unroll
-    for (int b = 0; b < 3; ++b) {
-        const double sum = f[3 * b] + f[3 * b + 2];
-        const double m0 = sum + f[3 * b + 1], A = s * (f[3 * b + 2] - f[3 * b]);
-        const double m1 = A + wx * m0;
-        r[3 * b] = m0; r[3 * b + 1] = m1; r[3 * b + 2] = s2 * sum + wx * (A + m1);
-    }
-#pragma unroll
-    for (int m = 0; m < 3; ++m) {
-        const double sum = r[m] + r[6 + m];
-        const double m0 = sum + r[3 + m], A = s * (r[6 + m] - r[m]);
-        const double m1 = A + wy * m0;
-        M[m] = m0; M[3 + m] = m1; M[6 + m] = s2 * sum + wy * (A + m1);
-    }
-}
-
-// Rows of the map from moments about u - t to populations of the gauge (s, u).
-__device__ __forceinline__ void moment_rows(double t, double inv_s, double (&L)[3][3])
-{
-    const double i2 = inv_s * inv_s, h2 = 0.5 * i2, ts = t * inv_s;
-    L[0][0] = 0.5 * ts * (ts + 1.0); L[0][1] = -(0.5 * inv_s + t * i2); L[0][2] = h2;
-    L[1][0] = 1.0 - ts * ts; L[1][1] = 2.0 * t * i2; L[1][2] = -i2;
-    L[2][0] = 0.5 * ts * (ts - 1.0); L[2][1] = 0.5 * inv_s - t * i2; L[2][2] = h2;
 }
 
 // Departure points of the three directions of an axis, x - (s (j - 1) + u) dt: their floors
@@ -776,7 +933,7 @@ __device__ __forceinline__ void contract(const float *own, int pitch, const floa
     }
 }
 
-// The same over the FP64 slots (moments): the x pass reads each direction's own four
+// The same over the FP64 slots: the x pass reads each direction's own four
 // columns (shared-memory reads are cheap beside the FP64 pipe, which runs at 1/64 of the
 // FP32 rate), and a row pass costs 36 multiply-adds instead of 45.  acc = the streamed
 // populations.
@@ -859,10 +1016,11 @@ __device__ __forceinline__ void stream_node(const DevParams &p, const R *__restr
     const int sx = (nx0[0] == nx0[1] && nx0[1] == nx0[2]) ? 4 : 5, sy = (ny0[0] == ny0[1] && ny0[1] == ny0[2]) ? 4 : 5;
     nreg += (unsigned)(sx * sy - (first ? 1 : 0));
     R Lx[3][3], Ly[3][3];
+    const R qb = (gauge_b[0] - s) * inv_s;
+    axis_rows<R>(qb, (gauge_b[1] - ux) * inv_s, Lx);
+    axis_rows<R>(qb, (gauge_b[2] - uy) * inv_s, Ly);
+    contract(slot, pitch, ax, nx0, ay, ny0, Lx, Ly, inc);
     if constexpr (sizeof(R) == 8) {
-        moment_rows(ux - gauge_b[1], inv_s, Lx);
-        moment_rows(uy - gauge_b[2], inv_s, Ly);
-        contract(slot, pitch, ax, nx0, ay, ny0, Lx, Ly, inc);
         R v[24];
         load_rec24(in, (size_t)Y * p.nx + X, (size_t)p.N, v);
 #pragma unroll
@@ -871,10 +1029,6 @@ __device__ __forceinline__ void stream_node(const DevParams &p, const R *__restr
             inc[1][i] -= v[P_G + i];
         }
     } else {
-        const R q = (gauge_b[0] - s) * inv_s;
-        axis_rows<R>(q, (gauge_b[1] - ux) * inv_s, Lx);
-        axis_rows<R>(q, (gauge_b[2] - uy) * inv_s, Ly);
-        contract(slot, pitch, ax, nx0, ay, ny0, Lx, Ly, inc);
         if (!first) {
             // the node's own populations carried from their stored gauge into this one
             R v[24], Ex[3][3], Ey[3][3], o[9];
@@ -1087,7 +1241,7 @@ __device__ __forceinline__ void stage_tile(const DevParams &p, const R *__restri
     const int tid = threadIdx.x;
     const int X0 = tl.X0, Y0 = tl.Y0, TX = tl.TX, TY = tl.TY, WT = tl.WT, nslots = tl.nslots;
     R *aux = tl.aux, *slots = tl.slots, *kq = tl.kq;
-    __shared__ uint4 best[ST_NT / 32];   // per warp: largest theta (bits), its slot, smallest theta
+    __shared__ uint4 best[ST_NT / 32];   // per warp: largest and smallest theta (bits) and their slots
     if (tid == 0) counts = StepCounts{};
     // k / WT through the float reciprocal: exact for k < 2^20 (the quotient's fraction
     // stays >= 0.5 / WT away from an integer)
@@ -1107,105 +1261,83 @@ __device__ __forceinline__ void stage_tile(const DevParams &p, const R *__restri
     };
 
     // ---------------- staging ------------------------------------------------------
-    if constexpr (sizeof(R) == 4) {
-        R va[24], vb[24];
-        const int ka = tid, kb = tid + ST_NT;
-        size_t na = 0, nb = 0;
-        unsigned top = 0, at = 0, low = 0xffffffffu;
-        auto offer = [&](R th, int k) {   // finite positive values only
-            const unsigned b = (th > R(0) && th < R(3.0e38)) ? __float_as_uint(th) : 0u;
-            low = min(low, b);
-            if (b > top) { top = b; at = (unsigned)k; }
-        };
-        if (ka < nslots) { na = node_of(ka); load_rec24(in, na, N, va); }
-        if (kb < nslots) { nb = node_of(kb); load_rec24(in, nb, N, vb); }
-        if (ka < nslots) offer(va[P_TH], ka);
-        if (kb < nslots) offer(vb[P_TH], kb);
-        for (int k = tid + 2 * ST_NT; k < nslots; k += ST_NT) offer(__ldg(in + rec_at(in, node_of(k), P_TH, N)), k);
-        {
-            const unsigned m = __reduce_max_sync(0xffffffffu, top);
-            const unsigned w = __reduce_min_sync(0xffffffffu, top == m ? at : 0xffffffffu);
-            low = __reduce_min_sync(0xffffffffu, low);
-            if ((tid & 31) == 0) best[tid >> 5] = make_uint4(m, w, low, 0);
+    R va[24], vb[24];
+    const int ka = tid, kb = tid + ST_NT;
+    size_t na = 0, nb = 0;
+    Extremes ex;
+    if (ka < nslots) { na = node_of(ka); load_rec24(in, na, N, va); }
+    if (kb < nslots) { nb = node_of(kb); load_rec24(in, nb, N, vb); }
+    if (ka < nslots) ex.offer((float)va[P_TH], ka);
+    if (kb < nslots) ex.offer((float)vb[P_TH], kb);
+    for (int k = tid + 2 * ST_NT; k < nslots; k += ST_NT) ex.offer((float)__ldg(in + rec_at(in, node_of(k), P_TH, N)), k);
+    ex = tile_extremes(ex, best);
+    const bool smooth = sizeof(R) == 4 && ex.smooth();
+    const size_t nhot = node_of(min((int)ex.at, nslots - 1)), ncold = node_of(min((int)ex.lat, nslots - 1));
+    R thb;
+    {
+        R hot[3], cold[3];
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            hot[k] = __ldg(in + rec_at(in, nhot, P_TH + k, N));
+            cold[k] = __ldg(in + rec_at(in, ncold, P_TH + k, N));
         }
-        __syncthreads();
-        uint4 b = best[0];
-#pragma unroll
-        for (int w = 1; w < ST_NT / 32; ++w) {
-            if (best[w].x > b.x || (best[w].x == b.x && best[w].y < b.y)) { b.x = best[w].x; b.y = best[w].y; }
-            b.z = min(b.z, best[w].z);
-        }
-        const bool smooth = __uint_as_float(b.z) > SMOOTH_TILE * __uint_as_float(b.x);
-        R base[24];
-        load_rec24(in, node_of((int)min(b.y, (unsigned)(nslots - 1))), N, base);
-        const R thb = base[P_TH];
-        gb[0] = sqrt_(thb); gb[1] = base[P_UX]; gb[2] = base[P_UY];
-        const R inv_sb = R(1) / gb[0];
-        auto carry = [&](int k, size_t nd, const R (&v)[24]) {
-            const R sn = sqrt_(v[P_TH]);
-            const R e = fdiv_(v[P_TH] - thb, (sn + gb[0]) * gb[0]);
-            const R wx = (v[P_UX] - gb[1]) * inv_sb, wy = (v[P_UY] - gb[2]) * inv_sb;
-            R Ex[3][3], Ey[3][3], d[DS];
-            if (smooth) {
-                R o[9];
-                axis_map<R>(e, wx, Ex);
-                axis_map<R>(e, wy, Ey);
-#pragma unroll
-                for (int fam = 0; fam < 2; ++fam) {
-                    map_inc<R>(Ex, Ey, v + 9 * fam, o);
-#pragma unroll
-                    for (int i = 0; i < 9; ++i) d[9 * fam + i] = (v[9 * fam + i] - base[9 * fam + i]) + o[i];
-                }
-            } else {
-                axis_rows<R>(e, wx, Ex);
-                axis_rows<R>(e, wy, Ey);
-#pragma unroll
-                for (int fam = 0; fam < 2; ++fam)
-#pragma unroll
-                    for (int k2 = 0; k2 < 3; ++k2) {
-                        R t[3];
-#pragma unroll
-                        for (int b2 = 0; b2 < 3; ++b2)
-                            t[b2] = Ex[k2][0] * v[9 * fam + 3 * b2] + Ex[k2][1] * v[9 * fam + 3 * b2 + 1] +
-                                    Ex[k2][2] * v[9 * fam + 3 * b2 + 2];
-#pragma unroll
-                        for (int l2 = 0; l2 < 3; ++l2)
-                            d[9 * fam + 3 * l2 + k2] = Ey[l2][0] * t[0] + Ey[l2][1] * t[1] + Ey[l2][2] * t[2];
-                    }
-            }
-            d[18] = d[19] = R(0);
-            float4 *dst = reinterpret_cast<float4 *>(slots + (size_t)k * DS);
-#pragma unroll
-            for (int c = 0; c < DS / 4; ++c) dst[c] = make_float4(d[4 * c], d[4 * c + 1], d[4 * c + 2], d[4 * c + 3]);
-            put_aux(k, nd, v[P_RHO], v[P_T]);
-        };
-        if (ka < nslots) carry(ka, na, va);
-        if (kb < nslots) carry(kb, nb, vb);
-        for (int k = tid + 2 * ST_NT; k < nslots; k += ST_NT) {
-            const size_t nd = node_of(k);
-            load_rec24(in, nd, N, va);
-            carry(k, nd, va);
-        }
-    } else {
-        // moments about the velocity of the tile's middle node
-        const size_t nc = (size_t)min(Y0 + TY / 2, p.ny - 1) * p.nx + min(X0 + TX / 2, p.nx - 1);
-        gb[0] = R(1);
-        gb[1] = __ldg(in + rec_at(in, nc, P_UX, N));
-        gb[2] = __ldg(in + rec_at(in, nc, P_UY, N));
-        for (int k = tid; k < nslots; k += ST_NT) {
-            const size_t nd = node_of(k);
-            R v[24], m[9];
-            load_rec24(in, nd, N, v);
-            const R sn = sqrt_(v[P_TH]), wx = v[P_UX] - gb[1], wy = v[P_UY] - gb[2];
-            R *dst = slots + (size_t)k * DS;
+        common_gauge<R, 3>(smooth, hot, cold, gb);
+        thb = smooth ? hot[0] : gb[0] * gb[0];
+    }
+    R base[24];
+    if (smooth) load_rec24(in, nhot, N, base);
+    const R inv_sb = R(1) / gb[0];
+    auto carry = [&](int k, size_t nd, const R (&v)[24]) {
+        const R sn = sqrt_(v[P_TH]);
+        const R e = fdiv_(v[P_TH] - thb, (sn + gb[0]) * gb[0]);
+        const R wx = (v[P_UX] - gb[1]) * inv_sb, wy = (v[P_UY] - gb[2]) * inv_sb;
+        R Ex[3][3], Ey[3][3], d[DS];
+        if (smooth) {
+            axis_map<R>(e, wx, Ex);
+            axis_map<R>(e, wy, Ey);
 #pragma unroll
             for (int fam = 0; fam < 2; ++fam) {
-                moments9(v + 9 * fam, sn, wx, wy, m);
+                R o[9];
+                map_inc<R>(Ex, Ey, v + 9 * fam, o);
 #pragma unroll
-                for (int i = 0; i < 9; ++i) dst[9 * fam + i] = m[i];
+                for (int i = 0; i < 9; ++i)
+                    d[9 * fam + i] = (v[9 * fam + i] - base[9 * fam + i]) + o[i];
             }
-            put_aux(k, nd, v[P_RHO], v[P_T]);
+        } else {
+            axis_rows<R>(e, wx, Ex);
+            axis_rows<R>(e, wy, Ey);
+#pragma unroll
+            for (int fam = 0; fam < 2; ++fam)
+#pragma unroll
+                for (int k2 = 0; k2 < 3; ++k2) {
+                    R t[3];
+#pragma unroll
+                    for (int b2 = 0; b2 < 3; ++b2)
+                        t[b2] = Ex[k2][0] * v[9 * fam + 3 * b2] + Ex[k2][1] * v[9 * fam + 3 * b2 + 1] +
+                                Ex[k2][2] * v[9 * fam + 3 * b2 + 2];
+#pragma unroll
+                    for (int l2 = 0; l2 < 3; ++l2)
+                        d[9 * fam + 3 * l2 + k2] = Ey[l2][0] * t[0] + Ey[l2][1] * t[1] + Ey[l2][2] * t[2];
+                }
         }
+        R *dst = slots + (size_t)k * DS;
+        if constexpr (sizeof(R) == 4) {
+            d[18] = d[19] = R(0);
+#pragma unroll
+            for (int c = 0; c < DS / 4; ++c)
+                reinterpret_cast<float4 *>(dst)[c] = make_float4(d[4 * c], d[4 * c + 1], d[4 * c + 2], d[4 * c + 3]);
+        } else {
+#pragma unroll
+            for (int i = 0; i < 18; ++i) dst[i] = d[i];
+        }
+        put_aux(k, nd, v[P_RHO], v[P_T]);
+    };
+    if (ka < nslots) carry(ka, na, va);
+    if (kb < nslots) carry(kb, nb, vb);
+    for (int k = tid + 2 * ST_NT; k < nslots; k += ST_NT) {
+        const size_t nd = node_of(k);
+        load_rec24(in, nd, N, va);
+        carry(k, nd, va);
     }
     __syncthreads();
 
@@ -1543,33 +1675,16 @@ __device__ __forceinline__ void step_tile_split(const DevParams &p, const R *__r
         R nf = 0, ng = 0;
         {
             // row k of the x map, column n (= l) of the y map
-            if constexpr (sizeof(R) == 8) {
-                const R i2 = inv_s * inv_s, c = R(k - 1);
-                const R t = ux - gb[1], ts = t * inv_s;
-                Lx[0] = k == 1 ? R(1) - ts * ts : R(0.5) * ts * (ts - c);
-                Lx[1] = k == 1 ? R(2) * t * i2 : R(0.5) * c * inv_s - t * i2;
-                Lx[2] = k == 1 ? -i2 : R(0.5) * i2;
-                const R ty_ = uy - gb[2], tsy = ty_ * inv_s;
+            const R qq = (gb[0] - s) * inv_s, w1 = (gb[1] - ux) * inv_s, w2 = (gb[2] - uy) * inv_s;
 #pragma unroll
-                for (int c2 = 0; c2 < 3; ++c2) {
-                    const R cc = R(c2 - 1);
-                    const R a0 = c2 == 1 ? R(1) - tsy * tsy : R(0.5) * tsy * (tsy - cc);
-                    const R a1 = c2 == 1 ? R(2) * ty_ * i2 : R(0.5) * cc * inv_s - ty_ * i2;
-                    const R a2 = c2 == 1 ? -i2 : R(0.5) * i2;
-                    Ly[c2] = l == 0 ? a0 : (l == 1 ? a1 : a2);
-                }
-            } else {
-                const R qq = (gb[0] - s) * inv_s, w1 = (gb[1] - ux) * inv_s, w2 = (gb[2] - uy) * inv_s;
-#pragma unroll
-                for (int m = 0; m < 3; ++m) {
-                    const R x = m == 1 ? w1 : (R(1) + qq) * R(m - 1) + w1;
-                    Lx[m] = k == 1 ? (R(1) - x) * (R(1) + x) : R(0.5) * x * (x + R(k - 1));
-                }
-                const R y = l == 1 ? w2 : (R(1) + qq) * R(l - 1) + w2;
-                Ly[0] = R(0.5) * y * (y - R(1));
-                Ly[1] = (R(1) - y) * (R(1) + y);
-                Ly[2] = R(0.5) * y * (y + R(1));
+            for (int m = 0; m < 3; ++m) {
+                const R x = m == 1 ? w1 : (R(1) + qq) * R(m - 1) + w1;
+                Lx[m] = k == 1 ? (R(1) - x) * (R(1) + x) : R(0.5) * x * (x + R(k - 1));
             }
+            const R y = l == 1 ? w2 : (R(1) + qq) * R(l - 1) + w2;
+            Ly[0] = R(0.5) * y * (y - R(1));
+            Ly[1] = (R(1) - y) * (R(1) + y);
+            Ly[2] = R(0.5) * y * (y + R(1));
             R wl[4][3];
 #pragma unroll
             for (int c = 0; c < 4; ++c)
