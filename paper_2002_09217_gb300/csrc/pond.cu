@@ -121,13 +121,8 @@ size_t step_smem(const pond_ctx *c)
 // Lets the step kernels of type R use more than the default 48 KB of dynamic shared
 // memory on the current device (idempotent; not a stream operation).
 template <typename R>
-cudaError_t allow_step_smem(int device)
+cudaError_t allow_step_smem()
 {
-    // set once per device (a context's creation need not pay for it again)
-    static std::mutex mutex;
-    static std::vector<bool> done;
-    std::lock_guard<std::mutex> lock(mutex);
-    if (device < (int)done.size() && done[device]) return cudaSuccess;
     size_t m = 0, ms = 0;
     for (int tx = 1; tx <= STEP_NB; tx *= 2)
         m = std::max(m, step_smem_bytes(tx, STEP_NB / tx, false, Slot<R>::stride, (int)sizeof(R)));
@@ -142,10 +137,6 @@ cudaError_t allow_step_smem(int device)
         e = cudaFuncSetAttribute(k_pond_step<R, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)m);
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(k_pond_step<R, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ms);
-    if (e == cudaSuccess) {
-        if (device >= (int)done.size()) done.resize(device + 1, false);
-        done[device] = true;
-    }
     return e;
 }
 
@@ -571,7 +562,7 @@ pond_status pond_create(const pond_grid *grid, const pond_lattice *lattice, cons
     }
     cudaError_t e = cudaGetDevice(&c->device);
     if (e == cudaSuccess)
-        e = opts->precision == POND_MIXED ? allow_step_smem<float>(c->device) : allow_step_smem<double>(c->device);
+        e = opts->precision == POND_MIXED ? allow_step_smem<float>() : allow_step_smem<double>();
     if (e != cudaSuccess) {
         delete c;
         return POND_ECUDA;
