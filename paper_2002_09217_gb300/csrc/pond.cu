@@ -20,6 +20,7 @@
 #include "pond_step.cuh"
 #include "pond_q16.cuh"
 #include "pond_q27.cuh"
+#include "pond_state.cuh"
 
 using namespace pond;
 
@@ -287,15 +288,6 @@ void launch_conserve(pond_ctx *c)
     k_conserve2<<<1, 32, 0, c->stream>>>(c->part, c->red_blocks, c->part + 8 * c->red_blocks);
 }
 
-// D2Q16 nodes and weights on the host (the same closed forms as the device's)
-void lattice16(double c[4], double w[4])
-{
-    const double s6 = std::sqrt(6.0), ci = std::sqrt(3.0 - s6), co = std::sqrt(3.0 + s6);
-    c[0] = -co; c[1] = -ci; c[2] = ci; c[3] = co;
-    w[0] = w[3] = (3.0 - s6) / 12.0;
-    w[1] = w[2] = (3.0 + s6) / 12.0;
-}
-
 pond_status check_ctx(pond_ctx *c)
 {
     if (!c) return POND_EINVAL;
@@ -342,6 +334,54 @@ pond_status report_flags(pond_ctx *c, const DevStats &hs)
 cudaError_t fetch_stats(pond_ctx *c, DevStats *hs)
 {
     return cudaMemcpyAsync(hs, c->dstats, sizeof(DevStats), cudaMemcpyDeviceToHost, c->stream);
+}
+
+// Calls f(R{}, lattice state description{}) for the context's precision and lattice.
+template <typename F>
+pond_status with_state(const pond_ctx *c, F f)
+{
+    if (c->lattice == POND_D3Q27) return mixed(c) ? f(0.0f, StateD3Q27{}) : f(0.0, StateD3Q27{});
+    if (c->lattice == POND_D2Q16) return mixed(c) ? f(0.0f, StateD2Q16{}) : f(0.0, StateD2Q16{});
+    return mixed(c) ? f(0.0f, StateD2Q9{}) : f(0.0, StateD2Q9{});
+}
+
+constexpr int STAGE_PLANES = 6;   // planes of the staging buffer
+
+// The state as host planes, a staging buffer's worth at a time.
+template <typename R, typename S>
+pond_status state_out(pond_ctx *c, double *state)
+{
+    const unsigned nb = blocks_for(c->N, 256);
+    for (int p = 0; p < S::planes; p += STAGE_PLANES) {
+        const int k = std::min(STAGE_PLANES, S::planes - p);
+        k_state_out<R, S><<<nb, 256, 0, c->stream>>>((const R *)c->state[c->cur], c->N, p, k, c->stage);
+        CK(cudaGetLastError(), "k_state_out launch");
+        CK(cudaMemcpyAsync(state + (size_t)p * c->N, c->stage, (size_t)k * c->N * sizeof(double),
+                           cudaMemcpyDeviceToHost, c->stream), "cudaMemcpyAsync D2H");
+    }
+    CK(cudaStreamSynchronize(c->stream), "cudaStreamSynchronize");
+    return POND_OK;
+}
+
+template <typename R, typename S>
+pond_status state_in(pond_ctx *c, const double *state)
+{
+    const unsigned nb = blocks_for(c->N, 256);
+    R *st = (R *)c->state[c->cur];
+    for (int p = 0; p < S::planes; p += STAGE_PLANES) {
+        const int k = std::min(STAGE_PLANES, S::planes - p);
+        CK(cudaMemcpyAsync(c->stage, state + (size_t)p * c->N, (size_t)k * c->N * sizeof(double),
+                           cudaMemcpyHostToDevice, c->stream), "cudaMemcpyAsync H2D");
+        // the non-local scratch (rewritten by every step) holds the remainders' sums
+        k_state_in<R, S><<<nb, 256, 0, c->stream>>>(c->stage, c->N, p, k, st, c->nlbuf);
+        CK(cudaGetLastError(), "k_state_in launch");
+    }
+    if constexpr (S::q != 9 && sizeof(R) == 4) {
+        k_state_finish<S><<<nb, 256, 0, c->stream>>>(c->N, st, c->nlbuf);
+        CK(cudaGetLastError(), "k_state_finish launch");
+    }
+    CK(cudaStreamSynchronize(c->stream), "cudaStreamSynchronize");
+    return POND_OK;
 }
 
 pond_status init_common(pond_ctx *c, const double *d_rho, const double *d_ux, const double *d_uy,
@@ -600,7 +640,7 @@ pond_status pond_create(const pond_grid *grid, const pond_lattice *lattice, cons
     size_t sb = (size_t)(c->lattice == POND_D2Q16 ? SLQ : (c->lattice == POND_D3Q27 ? SL27 : SL)) * c->N * c->esize;
     c->state[0] = dev_alloc(c, sb);
     c->state[1] = dev_alloc(c, sb);
-    c->stage = (double *)dev_alloc(c, 6 * c->N * sizeof(double));
+    c->stage = (double *)dev_alloc(c, STAGE_PLANES * c->N * sizeof(double));
     c->part = (double *)dev_alloc(c, (8 * (size_t)c->red_blocks + 8) * sizeof(double));
     c->dstats = (DevStats *)dev_alloc(c, sizeof(DevStats));
     if (c->lattice == POND_D2Q16) c->nlbuf = (double *)dev_alloc(c, (size_t)NL_PLANES * c->N * sizeof(double));
@@ -802,89 +842,7 @@ pond_status pond_get_state(pond_ctx *c, double *state)
     if (st) return st;
     if (!state) return fail(c, POND_EINVAL, "null output");
     if (!c->initialised) return fail(c, POND_EINVAL, "state not initialised");
-    if (c->lattice == POND_D3Q27) {
-        const size_t N = c->N, rec = (size_t)SL27 * N;
-        std::vector<double> d(mixed(c) ? 0 : rec);
-        std::vector<float> f(mixed(c) ? rec : 0);
-        void *dst = mixed(c) ? (void *)f.data() : (void *)d.data();
-        CK(cudaMemcpyAsync(dst, c->state[c->cur], rec * c->esize, cudaMemcpyDeviceToHost, c->stream),
-           "cudaMemcpyAsync D2H");
-        CK(cudaStreamSynchronize(c->stream), "cudaStreamSynchronize");
-        for (int p = 0; p < NP27; ++p) {
-            const int o = rec27_off(p);
-            for (size_t n = 0; n < N; ++n)
-                state[(size_t)p * N + n] = mixed(c) ? (double)f[rec_at(f.data(), n, o, N)] : d[rec_at(d.data(), n, o, N)];
-        }
-        if (mixed(c)) {
-            // kept remainders folded into the exchanged populations: W_i (m + c_i.J/(s T_L))
-            // on f, W_i G on g
-            const double w1[3] = {1.0 / 6.0, 2.0 / 3.0, 1.0 / 6.0};
-            for (size_t n = 0; n < N; ++n) {
-                auto r = [&](int o) -> double { return (double)f[rec_at(f.data(), n, o, N)]; };
-                const double sq = std::sqrt(r(R_TH));
-                const double m = r(R_MLO), gl = r(R_GLO);
-                const double J[3] = {r(R_JLO), r(R_JLO + 1), r(R_JLO + 2)};
-                for (int i = 0; i < Q27; ++i) {
-                    const int cx = i % 3 - 1, cy = (i / 3) % 3 - 1, cz = i / 9 - 1;
-                    const double w = w1[cx + 1] * w1[cy + 1] * w1[cz + 1];
-                    state[(size_t)i * N + n] += w * (m + (cx * J[0] + cy * J[1] + cz * J[2]) / (sq * (1.0 / 3.0)));
-                    state[(size_t)(Q27 + i) * N + n] += w * gl;
-                }
-            }
-        }
-        return POND_OK;
-    }
-    if (c->lattice == POND_D2Q16) {
-        // node records on the device, planes on the host
-        const size_t N = c->N, rec = (size_t)SLQ * N;
-        std::vector<double> d(mixed(c) ? 0 : rec);
-        std::vector<float> f(mixed(c) ? rec : 0);
-        void *dst = mixed(c) ? (void *)f.data() : (void *)d.data();
-        CK(cudaMemcpyAsync(dst, c->state[c->cur], rec * c->esize, cudaMemcpyDeviceToHost, c->stream),
-           "cudaMemcpyAsync D2H");
-        CK(cudaStreamSynchronize(c->stream), "cudaStreamSynchronize");
-        for (int p = 0; p < NP16; ++p)
-            for (size_t n = 0; n < N; ++n)
-                state[(size_t)p * N + n] = mixed(c) ? (double)f[rec_at(f.data(), n, p, N)] : d[rec_at(d.data(), n, p, N)];
-        if (mixed(c)) {
-            // the kept remainders go into the exchanged populations: mass and momentum as
-            // W_i (m + (c_ix J_x + c_iy J_y)/s) on f (its sum is m, its momentum m u + J),
-            // energy as W_i G on g
-            double cq[4], wq[4];
-            lattice16(cq, wq);
-            for (size_t n = 0; n < N; ++n) {
-                auto r = [&](int o) -> double { return (double)f[rec_at(f.data(), n, o, N)]; };
-                const double sq = std::sqrt(r(Q_TH));
-                const double m = r(Q_MLO), jx = r(Q_JXLO), jy = r(Q_JYLO), gl = r(Q_GLO);
-                for (int i = 0; i < Q16; ++i) {
-                    const double w = wq[i & 3] * wq[i >> 2];
-                    state[(size_t)(Q_F + i) * N + n] += w * (m + (cq[i & 3] * jx + cq[i >> 2] * jy) / sq);
-                    state[(size_t)(Q_G + i) * N + n] += w * gl;
-                }
-            }
-        }
-        return POND_OK;
-    }
-    const size_t N = c->N, rec = (size_t)SL * N;
-    std::vector<double> d(mixed(c) ? 0 : rec);
-    std::vector<float> f(mixed(c) ? rec : 0);
-    void *dst = mixed(c) ? (void *)f.data() : (void *)d.data();
-    CK(cudaMemcpyAsync(dst, c->state[c->cur], rec * c->esize, cudaMemcpyDeviceToHost, c->stream),
-       "cudaMemcpyAsync D2H");
-    CK(cudaStreamSynchronize(c->stream), "cudaStreamSynchronize");
-    for (int p = 0; p < NPL; ++p) {
-        const int o = rec_off(p);
-        for (size_t n = 0; n < N; ++n)
-            state[(size_t)p * N + n] = mixed(c) ? (double)f[rec_at(f.data(), n, o, N)] : d[rec_at(d.data(), n, o, N)];
-    }
-    // the rest populations with their kept low parts (the momentum low parts, below one
-    // ulp of the populations, are not part of the exchanged state)
-    for (int k = 0; k < 2; ++k) {
-        const int p = k == 0 ? P_F + 4 : P_G + 4, lo = k == 0 ? P_F4LO : P_G4LO;
-        for (size_t n = 0; n < N; ++n)
-            state[(size_t)p * N + n] += mixed(c) ? (double)f[rec_at(f.data(), n, lo, N)] : d[rec_at(d.data(), n, lo, N)];
-    }
-    return POND_OK;
+    return with_state(c, [&](auto r, auto lat) { return state_out<decltype(r), decltype(lat)>(c, state); });
 }
 
 pond_status pond_set_state(pond_ctx *c, const double *state)
@@ -892,99 +850,8 @@ pond_status pond_set_state(pond_ctx *c, const double *state)
     pond_status st = check_ctx(c);
     if (st) return st;
     if (!state) return fail(c, POND_EINVAL, "null input");
-    if (c->lattice == POND_D3Q27) {
-        const size_t N = c->N, rec = (size_t)SL27 * N;
-        std::vector<double> d(mixed(c) ? 0 : rec, 0.0);
-        std::vector<float> f(mixed(c) ? rec : 0, 0.0f);
-        for (int p = 0; p < NP27; ++p) {
-            const int o = rec27_off(p);
-            for (size_t n = 0; n < N; ++n) {
-                if (mixed(c)) f[rec_at(f.data(), n, o, N)] = (float)state[(size_t)p * N + n];
-                else d[rec_at(d.data(), n, o, N)] = state[(size_t)p * N + n];
-            }
-        }
-        if (mixed(c))
-            for (size_t n = 0; n < N; ++n) {
-                // what the FP32 populations leave out becomes the kept remainders again
-                auto r = [&](int o) -> float & { return f[rec_at(f.data(), n, o, N)]; };
-                const double sq = std::sqrt((double)r(R_TH));
-                double m = 0.0, S[3] = {0, 0, 0}, gl = 0.0;
-                for (int i = 0; i < Q27; ++i) {
-                    const double rf = state[(size_t)i * N + n] - (double)r(R_F + i);
-                    m += rf;
-                    S[0] += rf * (i % 3 - 1); S[1] += rf * ((i / 3) % 3 - 1); S[2] += rf * (i / 9 - 1);
-                    gl += state[(size_t)(Q27 + i) * N + n] - (double)r(R_G + i);
-                }
-                r(R_MLO) = (float)m;
-                for (int a = 0; a < 3; ++a) r(R_JLO + a) = (float)(sq * S[a]);
-                r(R_GLO) = (float)gl;
-            }
-        const void *src = mixed(c) ? (const void *)f.data() : (const void *)d.data();
-        CK(cudaMemcpyAsync(c->state[c->cur], src, rec * c->esize, cudaMemcpyHostToDevice, c->stream),
-           "cudaMemcpyAsync H2D");
-        CK(cudaStreamSynchronize(c->stream), "cudaStreamSynchronize");
-        c->initialised = true;
-        return POND_OK;
-    }
-    if (c->lattice == POND_D2Q16) {
-        const size_t N = c->N, rec = (size_t)SLQ * N;
-        std::vector<double> d(mixed(c) ? 0 : rec, 0.0);
-        std::vector<float> f(mixed(c) ? rec : 0, 0.0f);
-        for (int p = 0; p < NP16; ++p)
-            for (size_t n = 0; n < N; ++n) {
-                if (mixed(c)) f[rec_at(f.data(), n, p, N)] = (float)state[(size_t)p * N + n];
-                else d[rec_at(d.data(), n, p, N)] = state[(size_t)p * N + n];
-            }
-        if (mixed(c)) {
-            // what the FP32 populations leave out becomes the kept remainders again: mass
-            // sum r_i, momentum s sum r_i c_i (beyond the mass part's u m), energy sum r_gi
-            double cq[4], wq[4];
-            lattice16(cq, wq);
-            for (size_t n = 0; n < N; ++n) {
-                auto r = [&](int o) -> float & { return f[rec_at(f.data(), n, o, N)]; };
-                const double sq = std::sqrt((double)r(Q_TH));
-                double m = 0.0, sx = 0.0, sy = 0.0, gl = 0.0;
-                for (int i = 0; i < Q16; ++i) {
-                    const double rf = state[(size_t)(Q_F + i) * N + n] - (double)r(Q_F + i);
-                    m += rf;
-                    sx += rf * cq[i & 3];
-                    sy += rf * cq[i >> 2];
-                    gl += state[(size_t)(Q_G + i) * N + n] - (double)r(Q_G + i);
-                }
-                r(Q_MLO) = (float)m;
-                r(Q_JXLO) = (float)(sq * sx);
-                r(Q_JYLO) = (float)(sq * sy);
-                r(Q_GLO) = (float)gl;
-            }
-        }
-        const void *src = mixed(c) ? (const void *)f.data() : (const void *)d.data();
-        CK(cudaMemcpyAsync(c->state[c->cur], src, rec * c->esize, cudaMemcpyHostToDevice, c->stream),
-           "cudaMemcpyAsync H2D");
-        CK(cudaStreamSynchronize(c->stream), "cudaStreamSynchronize");
-        c->initialised = true;
-        return POND_OK;
-    }
-    const size_t N = c->N, rec = (size_t)SL * N;
-    std::vector<double> d(mixed(c) ? 0 : rec, 0.0);
-    std::vector<float> f(mixed(c) ? rec : 0, 0.0f);
-    for (int p = 0; p < NPL; ++p) {
-        const int o = rec_off(p);
-        for (size_t n = 0; n < N; ++n) {
-            if (mixed(c)) f[rec_at(f.data(), n, o, N)] = (float)state[(size_t)p * N + n];
-            else d[rec_at(d.data(), n, o, N)] = state[(size_t)p * N + n];
-        }
-    }
-    // FP32 form: the rest populations keep the part below their float as the low word
-    if (mixed(c))
-        for (int k = 0; k < 2; ++k) {
-            const int p = k == 0 ? P_F + 4 : P_G + 4, lo = k == 0 ? P_F4LO : P_G4LO;
-            for (size_t n = 0; n < N; ++n)
-                f[rec_at(f.data(), n, lo, N)] = (float)(state[(size_t)p * N + n] - (double)f[rec_at(f.data(), n, p, N)]);
-        }
-    const void *src = mixed(c) ? (const void *)f.data() : (const void *)d.data();
-    CK(cudaMemcpyAsync(c->state[c->cur], src, rec * c->esize, cudaMemcpyHostToDevice, c->stream),
-       "cudaMemcpyAsync H2D");
-    CK(cudaStreamSynchronize(c->stream), "cudaStreamSynchronize");
+    st = with_state(c, [&](auto r, auto lat) { return state_in<decltype(r), decltype(lat)>(c, state); });
+    if (st) return st;
     c->initialised = true;
     return POND_OK;
 }
