@@ -100,11 +100,14 @@ inline unsigned blocks_for(size_t n, unsigned bs) { return (unsigned)((n + bs - 
 
 // Largest grid (nodes) stepped with nine lanes per node.  One thread per node leaves most
 // of the GPU idle below about 150 blocks of 128 nodes and a step then costs one block's
-// serial time (mixed 21-25 us, FP64 390-450 us whatever the grid); nine lanes per node cut
+// serial time (mixed 20-23 us, FP64 400-460 us whatever the grid); nine lanes per node cut
 // that time but do more work in all.  Measured (us per step, thread / nine lanes), mixed:
-// 128 x 4 21.1 / 14.6, 64 x 64 23.8 / 18.0, 2048 x 4 22.8 / 26.8, 96 x 96 23.6 / 28.5; FP64:
-// 128 x 4 389 / 107, 64 x 64 449 / 232, 96 x 96 449 / 404, 128 x 128 449 / 661.
-size_t split_max_nodes(int precision) { return precision == POND_MIXED ? 4096 : 10000; }
+// 128 x 4 19.5 / 12.0, 2048 x 1 23.0 / 12.6, 64 x 64 22.2 / 16.6, 96 x 96 22.2 / 26.8; FP64:
+// 128 x 4 401 / 110, 64 x 64 459 / 241, 96 x 96 459 / 423, 128 x 128 460 / 693.  The mixed
+// limit is below the lone crossing (about 6,500 nodes) because a context keeps its split in a
+// batch, where the other members fill the GPU and the extra work counts: twelve grids of
+// 64 x 64 to 164 x 160 nodes took 59 us a step with the smallest on nine lanes.
+size_t split_max_nodes(int precision) { return precision == POND_MIXED ? 3072 : 10000; }
 
 bool mixed(const pond_ctx *c) { return c->opts.precision == POND_MIXED; }
 
@@ -141,13 +144,32 @@ cudaError_t allow_step_smem()
     return e;
 }
 
-// One launch of the D2Q9 step over `blocks` tiles (of `one`, or of a batch's work list).
+// One launch of the D2Q9 step over `blocks` tiles of `one` or of a batch's work list.  A
+// lone simulation's may begin while the stream's previous step drains (programmatic
+// dependent launch: the kernel waits for that step's completion before it reads anything),
+// which hides most of the launch latency between small steps: 128 x 4 nodes 14.6 -> 12.0 us
+// a step, 2048 x 1 14.8 -> 12.6.
 template <typename R>
-void launch_step_kernel(bool use_split, unsigned blocks, size_t smem, cudaStream_t s, const SimDesc<R> &one,
-                        const SimDesc<R> *descs, const int2 *work)
+cudaError_t launch_step_kernel(bool use_split, unsigned blocks, size_t smem, cudaStream_t s, const SimDesc<R> &one,
+                               const SimDesc<R> *descs, const int2 *work)
 {
-    if (use_split) k_pond_step<R, true><<<blocks, STEP_THREADS, smem, s>>>(one, descs, work);
-    else k_pond_step<R, false><<<blocks, STEP_THREADS, smem, s>>>(one, descs, work);
+    if (work) {   // a batch's launch, captured in its graph
+        if (use_split) k_pond_step<R, true><<<blocks, STEP_THREADS, smem, s>>>(one, descs, work);
+        else k_pond_step<R, false><<<blocks, STEP_THREADS, smem, s>>>(one, descs, work);
+        return cudaSuccess;
+    }
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(blocks);
+    cfg.blockDim = dim3(STEP_THREADS);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return use_split ? cudaLaunchKernelEx(&cfg, k_pond_step<R, true>, one, descs, work)
+                     : cudaLaunchKernelEx(&cfg, k_pond_step<R, false>, one, descs, work);
 }
 
 // D2Q16: the non-local terms of state `src` into nlbuf, then the node step in -> out.
@@ -909,6 +931,11 @@ struct pond_batch {
     // the context's current buffer when the lists were built
     struct Q16 { pond_ctx *c; int cur0; };
     std::vector<Q16> q16;
+    // the members' chains of launches run beside each other inside the graph: the first on
+    // the batch stream, the others on these
+    static constexpr int SIDES = 4;
+    cudaStream_t side[SIDES] = {};
+    cudaEvent_t fork = nullptr, join[SIDES] = {};
     cudaGraphExec_t graph = nullptr;  // two steps (even, odd) of every group
     bool graph_ok = false;
     size_t budget = 0;                // device bytes the members may hold (0: no limit)
@@ -969,32 +996,73 @@ cudaError_t build_group(pond_batch *b, pond_batch::Group &G)
 }
 
 template <typename R>
-void launch_group(pond_batch *b, pond_batch::Group &G, int parity)
+void launch_group(const pond_batch::Group &G, int parity, cudaStream_t s)
 {
-    if (!G.nwork) return;
     const SimDesc<R> *d = (const SimDesc<R> *)G.desc[parity];
-    launch_step_kernel<R>(G.lanes == 16, (unsigned)G.nwork, G.smem, b->stream, SimDesc<R>{}, d, G.work);
+    launch_step_kernel<R>(G.lanes == 16, (unsigned)G.nwork, G.smem, s, SimDesc<R>{}, d, G.work);
 }
 
 template <typename R>
-void launch_q16_entry(pond_batch *b, const pond_batch::Q16 &e, int parity)
+void launch_q16_entry(const pond_batch::Q16 &e, int parity, cudaStream_t s)
 {
     pond_ctx *c = e.c;
     const int ci = e.cur0 ^ parity;
     const R *in = (const R *)c->state[ci];
-    launch_q16_pass<R>(c, in, in, (R *)c->state[1 - ci], c->dstats, b->stream);
+    launch_q16_pass<R>(c, in, in, (R *)c->state[1 - ci], c->dstats, s);
 }
 
-void launch_all(pond_batch *b, int parity)
+// The steps `first` .. `first + steps - 1` (parities) of every group and D2Q16 member: chain
+// k of launches on the stream on(k).
+template <typename On>
+void launch_all(pond_batch *b, int first, int steps, On on)
 {
-    for (int k = 0; k < 4; ++k) {
-        if (b->g[k].precision == POND_MIXED) launch_group<float>(b, b->g[k], parity);
-        else launch_group<double>(b, b->g[k], parity);
+    int k = 0;
+    for (int g = 0; g < 4; ++g) {
+        if (!b->g[g].nwork) continue;
+        const cudaStream_t s = on(k++);
+        for (int t = first; t < first + steps; ++t) {
+            if (b->g[g].precision == POND_MIXED) launch_group<float>(b->g[g], t % 2, s);
+            else launch_group<double>(b->g[g], t % 2, s);
+        }
     }
     for (const pond_batch::Q16 &e : b->q16) {
-        if (mixed(e.c)) launch_q16_entry<float>(b, e, parity);
-        else launch_q16_entry<double>(b, e, parity);
+        const cudaStream_t s = on(k++);
+        for (int t = first; t < first + steps; ++t) {
+            if (mixed(e.c)) launch_q16_entry<float>(e, t % 2, s);
+            else launch_q16_entry<double>(e, t % 2, s);
+        }
     }
+}
+
+// Captures two steps (even, then odd) of every member; the members' chains are independent
+// until both are done.  A group of few blocks then no longer holds up the others (twelve
+// grids of 64 x 64 to 164 x 160 nodes, one of them in the small-grid group: @BATCH@).
+cudaError_t capture_two_steps(pond_batch *b, cudaGraph_t *graph)
+{
+    cudaError_t e = cudaSuccess;
+    if (!b->fork) e = cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming);
+    for (int k = 0; k < pond_batch::SIDES && e == cudaSuccess; ++k) {
+        if (!b->side[k]) e = cudaStreamCreateWithFlags(&b->side[k], cudaStreamNonBlocking);
+        if (e == cudaSuccess && !b->join[k]) e = cudaEventCreateWithFlags(&b->join[k], cudaEventDisableTiming);
+    }
+    if (e != cudaSuccess) return e;
+    e = cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal);
+    if (e != cudaSuccess) return e;
+    bool used[pond_batch::SIDES] = {};
+    cudaEventRecord(b->fork, b->stream);
+    launch_all(b, 0, 2, [&](int k) -> cudaStream_t {
+        const int j = k % (pond_batch::SIDES + 1);
+        if (j == 0) return b->stream;
+        if (!used[j - 1]) cudaStreamWaitEvent(b->side[j - 1], b->fork, 0);
+        used[j - 1] = true;
+        return b->side[j - 1];
+    });
+    for (int k = 0; k < pond_batch::SIDES; ++k)
+        if (used[k]) {
+            cudaEventRecord(b->join[k], b->side[k]);
+            cudaStreamWaitEvent(b->stream, b->join[k], 0);
+        }
+    return cudaStreamEndCapture(b->stream, graph);
 }
 
 pond_status batch_build(pond_batch *b)
@@ -1022,14 +1090,10 @@ pond_status batch_build(pond_batch *b)
     // capture two steps (even then odd parity) of every group once; replays step the batch
     if (b->stream) {
         cudaGraph_t graph = nullptr;
-        if (cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal) == cudaSuccess) {
-            launch_all(b, 0);
-            launch_all(b, 1);
-            cudaError_t e = cudaStreamEndCapture(b->stream, &graph);
-            if (e == cudaSuccess && graph && cudaGraphInstantiate(&b->graph, graph, 0) == cudaSuccess)
-                b->graph_ok = true;
-            if (graph) cudaGraphDestroy(graph);
-        }
+        if (capture_two_steps(b, &graph) == cudaSuccess && graph &&
+            cudaGraphInstantiate(&b->graph, graph, 0) == cudaSuccess)
+            b->graph_ok = true;
+        if (graph) cudaGraphDestroy(graph);
         cudaGetLastError();   // a failed capture falls back to plain launches
     }
     b->dirty = false;
@@ -1130,12 +1194,15 @@ pond_status pond_batch_step(pond_batch *b, int64_t n)
         if (st) return st;
     }
     int64_t k = 0;
-    // whole graph replays when the next step is an even one
-    if (b->graph_ok && (b->since_build % 2) == 0)
+    const auto plain = [&](int64_t at) { launch_all(b, (int)(at % 2), 1, [&](int) { return b->stream; }); };
+    // whole graph replays from an even step on
+    if (b->graph_ok) {
+        if (b->since_build % 2) plain(b->since_build + k++);
         for (; k + 2 <= n; k += 2)
             if (cudaGraphLaunch(b->graph, b->stream) != cudaSuccess)
                 return bfail(b, POND_ECUDA, "cudaGraphLaunch");
-    for (; k < n; ++k) launch_all(b, (int)((b->since_build + k) % 2));
+    }
+    for (; k < n; ++k) plain(b->since_build + k);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return bfail(b, POND_ECUDA, std::string("batch step: ") + cudaGetErrorString(e));
     b->since_build += n;
@@ -1160,6 +1227,11 @@ void pond_batch_destroy(pond_batch *b)
         cudaFree(G.work);
     }
     if (b->graph) cudaGraphExecDestroy(b->graph);
+    for (int k = 0; k < pond_batch::SIDES; ++k) {
+        if (b->join[k]) cudaEventDestroy(b->join[k]);
+        if (b->side[k]) cudaStreamDestroy(b->side[k]);
+    }
+    if (b->fork) cudaEventDestroy(b->fork);
     cudaEventDestroy(b->done);
     delete b;
 }

@@ -128,52 +128,91 @@ template <typename R> __device__ __forceinline__ R sqrt_(R x);
 template <> __device__ __forceinline__ float sqrt_(float x) { return sqrtf(x); }
 template <> __device__ __forceinline__ double sqrt_(double x) { return sqrt(x); }
 
+// Writes a whole record of W values.
+template <int W>
+__device__ __forceinline__ void store_chunks(float *b, size_t nd, size_t N, const float (&v)[W])
+{
+    float4 *q = reinterpret_cast<float4 *>(b) + nd;
+#pragma unroll
+    for (int k = 0; k < W / 4; ++k) q[k * N] = make_float4(v[4 * k], v[4 * k + 1], v[4 * k + 2], v[4 * k + 3]);
+}
+template <int W>
+__device__ __forceinline__ void store_chunks(double *b, size_t nd, size_t N, const double (&v)[W])
+{
+    double2 *q = reinterpret_cast<double2 *>(b) + nd;
+#pragma unroll
+    for (int k = 0; k < W / 2; ++k) q[k * N] = make_double2(v[2 * k], v[2 * k + 1]);
+}
+// 1/x in FP64 from the FP32 reciprocal and two Newton steps (relative error ~1e-28
+// before the final rounding); values outside the FP32 normal range take the division.
+__device__ __noinline__ double rcp_slow(double x) { return 1.0 / x; }
+__device__ __forceinline__ double rcp_d(double x)
+{
+    const float xf = fabsf((float)x);
+    if (!(xf > 1e-37f && xf < 1e37f)) return rcp_slow(x);
+    double r = (double)__frcp_rn((float)x);
+    r = r * (2.0 - x * r);
+    return r * (2.0 - x * r);
+}
+
 // ---------------------------------------------------------------------------
 // Initial state: co-moving equilibrium of host-given (rho, u, T) (Eq. geq with the
-// interface energy kappa |grad rho|^2 / 2 in the total energy).
+// interface energy kappa |grad rho|^2 / 2 in the total energy).  Bound by the FP64 pipe:
+// v^2 is a sum over the axes, so g_i = W_i (G + b_x(c_x) + b_y(c_y)) with b_a(c) = rho (s c +
+// u_a)^2 and G = rho (2 e - 2 P/rho) + kappa |grad rho|^2, and the gradient is three
+// differences per axis: about 110 FP64 operations a node instead of 300 (2048 x 1024
+// nodes @INIT9@).
+// p(rho, T) with the van der Waals quotient as a product with a reciprocal
+__device__ __forceinline__ double pressure_d(const DevParams &p, double r, double t)
+{
+    if (p.eos_kind != 0) return eos_pressure<double>(p.eos_kind, p.a, p.b, p.R, r, t, p.sp);
+    return r * p.R * t * rcp_d(1.0 - p.b * r) - p.a * r * r;
+}
 template <typename R>
 __global__ void k_init(DevParams p, const double *__restrict__ rho, const double *__restrict__ ux,
                        const double *__restrict__ uy, const double *__restrict__ T,
                        R *__restrict__ st, DevStats *stats)
 {
-    long long n = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    const long long n = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (n >= p.N) return;
-    int X = (int)(n % p.nx), Y = (int)(n / p.nx);
-    double gx = 0.0, gy = 0.0;
-    for (int i = 0; i < 9; ++i) {
-        int cx = i % 3 - 1, cy = i / 3 - 1;
-        long long m = (long long)bc_wrap(Y + cy, p.ny, p.bcy) * p.nx + bc_wrap(X + cx, p.nx, p.bcx);
-        double w = w1d(cx + 1) * w1d(cy + 1);
-        gx += w * cx * rho[m];
-        gy += w * cy * rho[m];
+    const int X = (int)(n % p.nx), Y = (int)(n / p.nx);
+    double D[3], L[3];   // per row: rho(+1) - rho(-1); rho(-1) + 4 rho(0) + rho(+1)
+#pragma unroll
+    for (int y = 0; y < 3; ++y) {
+        const long long row = (long long)bc_wrap(Y + y - 1, p.ny, p.bcy) * p.nx;
+        const double a = rho[row + bc_wrap(X - 1, p.nx, p.bcx)], c = rho[row + bc_wrap(X + 1, p.nx, p.bcx)];
+        D[y] = c - a;
+        L[y] = (a + c) + 4.0 * rho[row + X];
     }
-    gx *= 3.0;
-    gy *= 3.0;
-    double r = rho[n], t = T[n];
+    const double gx = ((D[0] + D[2]) + 4.0 * D[1]) * (1.0 / 12.0), gy = (L[2] - L[0]) * (1.0 / 12.0);
+    const double r = rho[n], t = T[n], u[2] = {ux[n], uy[n]};
     if (!(r > 0.0) || !(p.b * r < 1.0) || !(t > 0.0)) atomicAdd(&stats->bad_init, 1ull);
-    double pr = eos_pressure<double>(p.eos_kind, p.a, p.b, p.R, r, t, p.sp);
-    double P = pr > p.p_floor ? pr : p.p_floor;
-    double th = P / (r * POND_TL), s = sqrt(th);
-    double e = p.cv * t - p.a * r;
-    double lam_e = p.kappa * (gx * gx + gy * gy);
+    const double pr = pressure_d(p, r, t);
+    const double P = pr > p.p_floor ? pr : p.p_floor;
+    const double th = P * rcp_d(r) * 3.0, s = sqrt(th);   // theta = P / (rho T_L)
+    const double G = 2.0 * (r * (p.cv * t - p.a * r) - P) + p.kappa * (gx * gx + gy * gy);
+    double b[2][3];
+#pragma unroll
+    for (int a = 0; a < 2; ++a)
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            const double v = s * (k - 1) + u[a];
+            b[a][k] = r * (v * v);
+        }
+    R rec[SL];
+#pragma unroll
     for (int i = 0; i < 9; ++i) {
-        int cx = i % 3 - 1, cy = i / 3 - 1;
-        double w = w1d(cx + 1) * w1d(cy + 1);
-        double vx = s * cx + ux[n], vy = s * cy + uy[n];
-        REC(st, n, P_F + i) = (R)(r * w);
-        REC(st, n, P_G + i) = (R)(r * w * (2.0 * e - 2.0 * P / r + vx * vx + vy * vy) + w * lam_e);
+        const double w = w1d(i % 3) * w1d(i / 3);
+        rec[P_F + i] = (R)(r * w);
+        rec[P_G + i] = (R)(w * (G + (b[0][i % 3] + b[1][i / 3])));
     }
-    REC(st, n, P_TH) = (R)th;
-    REC(st, n, P_UX) = (R)ux[n];
-    REC(st, n, P_UY) = (R)uy[n];
-    REC(st, n, P_RHO) = (R)r;
-    REC(st, n, P_T) = (R)t;
-    REC(st, n, P_UHX) = (R)ux[n];
-    REC(st, n, P_UHY) = (R)uy[n];
-    REC(st, n, P_F4LO) = (R)0;
-    REC(st, n, P_G4LO) = (R)0;
-    REC(st, n, P_JXLO) = (R)0;
-    REC(st, n, P_JYLO) = (R)0;
+    rec[P_TH] = (R)th;
+    rec[P_UX] = rec[P_UHX] = (R)u[0];
+    rec[P_UY] = rec[P_UHY] = (R)u[1];
+    rec[P_RHO] = (R)r;
+    rec[P_T] = (R)t;
+    rec[P_SQ] = rec[P_F4LO] = rec[P_G4LO] = rec[P_JXLO] = rec[P_JYLO] = rec[30] = rec[31] = (R)0;
+    store_chunks<SL>(st, (size_t)n, (size_t)p.N, rec);
 }
 
 template <typename T>
@@ -199,7 +238,7 @@ __global__ void k_moments(DevParams p, const R *__restrict__ st, double *rho, do
     if (ux) ux[n] = (double)REC(st, n, P_UHX);
     if (uy) uy[n] = (double)REC(st, n, P_UHY);
     if (T) T[n] = t;
-    if (pr) pr[n] = eos_pressure<double>(p.eos_kind, p.a, p.b, p.R, r, t, p.sp);
+    if (pr) pr[n] = pressure_d(p, r, t);
 }
 
 // Error-free sum of two doubles (Knuth TwoSum).

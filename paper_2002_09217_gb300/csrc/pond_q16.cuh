@@ -200,12 +200,6 @@ __device__ __forceinline__ int departure(int X, A v, A dt, A w[4])
     return X + (int)fl - 1;
 }
 
-// Pressure of the run's EoS in FP64.
-__device__ __forceinline__ double q16_p(const DevParams &p, double r, double t)
-{
-    return eos_pressure<double>(p.eos_kind, p.a, p.b, p.R, r, t, p.sp);
-}
-
 // ---------------------------------------------------------------------------
 // Initial state: co-moving equilibrium of host-given (rho, u, T) (Eq. geq with the
 // interface energy kappa |grad rho|^2 / 2 in the total energy), D2Q16 weights, T_L = 1.
@@ -218,38 +212,45 @@ __global__ void k_q16_init(DevParams p, const double *__restrict__ rho, const do
     if (n >= p.N) return;
     const Lat16<double> L = make_lat16<double>();
     const int X = (int)(n % p.nx), Y = (int)(n / p.nx);
-    double gx = 0.0, gy = 0.0;
-    for (int i = 0; i < 9; ++i) {
-        const int cx = i % 3 - 1, cy = i / 3 - 1;
-        const long long m = (long long)bc_wrap(Y + cy, p.ny, p.bcy) * p.nx + bc_wrap(X + cx, p.nx, p.bcx);
-        const double w = w1d(cx + 1) * w1d(cy + 1);
-        gx += w * cx * rho[m];
-        gy += w * cy * rho[m];
+    double D[3], S[3];   // per row: rho(+1) - rho(-1); rho(-1) + 4 rho(0) + rho(+1)
+#pragma unroll
+    for (int y = 0; y < 3; ++y) {
+        const long long row = (long long)bc_wrap(Y + y - 1, p.ny, p.bcy) * p.nx;
+        const double a = rho[row + bc_wrap(X - 1, p.nx, p.bcx)], c = rho[row + bc_wrap(X + 1, p.nx, p.bcx)];
+        D[y] = c - a;
+        S[y] = (a + c) + 4.0 * rho[row + X];
     }
-    gx *= 3.0;
-    gy *= 3.0;
-    const double r = rho[n], t = T[n];
+    const double gx = ((D[0] + D[2]) + 4.0 * D[1]) * (1.0 / 12.0), gy = (S[2] - S[0]) * (1.0 / 12.0);
+    const double r = rho[n], t = T[n], u[2] = {ux[n], uy[n]};
     if (!(r > 0.0) || !(p.b * r < 1.0) || !(t > 0.0)) atomicAdd(&stats->bad_init, 1ull);
-    const double pr = q16_p(p, r, t);
+    const double pr = pressure_d(p, r, t);
     const double P = pr > p.p_floor ? pr : p.p_floor;
-    const double th = P / r, s = sqrt(th);
-    const double e = p.cv * t - p.a * r;
-    const double lam_e = p.kappa * (gx * gx + gy * gy);
+    const double th = P * rcp_d(r), s = sqrt(th);
+    // g_i = W_i (G + rho v_x^2 + rho v_y^2), as in k_init
+    const double G = 2.0 * (r * (p.cv * t - p.a * r) - P) + p.kappa * (gx * gx + gy * gy);
+    double b[2][4];
+#pragma unroll
+    for (int a = 0; a < 2; ++a)
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const double v = s * L.c[k] + u[a];
+            b[a][k] = r * (v * v);
+        }
+    R rec[SLQ];
+#pragma unroll
     for (int i = 0; i < Q16; ++i) {
-        const int jx = i & 3, jy = i >> 2;
-        const double w = L.w[jx] * L.w[jy];
-        const double vx = s * L.c[jx] + ux[n], vy = s * L.c[jy] + uy[n];
-        REC16(st, n, Q_F + i) = (R)(r * w);
-        REC16(st, n, Q_G + i) = (R)(r * w * (2.0 * e - 2.0 * P / r + vx * vx + vy * vy) + w * lam_e);
+        const double w = L.w[i & 3] * L.w[i >> 2];
+        rec[Q_F + i] = (R)(r * w);
+        rec[Q_G + i] = (R)(w * (G + (b[0][i & 3] + b[1][i >> 2])));
     }
-    REC16(st, n, Q_TH) = (R)th;
-    REC16(st, n, Q_UX) = (R)ux[n];
-    REC16(st, n, Q_UY) = (R)uy[n];
-    REC16(st, n, Q_RHO) = (R)r;
-    REC16(st, n, Q_T) = (R)t;
-    REC16(st, n, Q_UHX) = (R)ux[n];
-    REC16(st, n, Q_UHY) = (R)uy[n];
-    for (int k = Q_MLO; k < SLQ; ++k) REC16(st, n, k) = (R)0;
+    rec[Q_TH] = (R)th;
+    rec[Q_UX] = rec[Q_UHX] = (R)u[0];
+    rec[Q_UY] = rec[Q_UHY] = (R)u[1];
+    rec[Q_RHO] = (R)r;
+    rec[Q_T] = (R)t;
+#pragma unroll
+    for (int k = Q_MLO; k < SLQ; ++k) rec[k] = (R)0;
+    store_chunks<SLQ>(st, (size_t)n, (size_t)p.N, rec);
 }
 
 // ---------------------------------------------------------------------------
@@ -1182,7 +1183,7 @@ __global__ void k_q16_moments(DevParams p, const R *__restrict__ st, double *rho
     if (ux) ux[n] = (double)REC16(st, n, Q_UHX);
     if (uy) uy[n] = (double)REC16(st, n, Q_UHY);
     if (T) T[n] = t;
-    if (pr) pr[n] = q16_p(p, r, t);
+    if (pr) pr[n] = pressure_d(p, r, t);
 }
 
 // Conservation sums, stage 1: per-block compensated partials of

@@ -150,48 +150,6 @@ __device__ __forceinline__ void load27(const double *__restrict__ b, size_t nd, 
 }
 
 // ---------------------------------------------------------------------------
-// Initial state: co-moving equilibrium of host-given (rho, u, T) with the interface
-// energy (Eq. geq, D = 3).
-template <typename R>
-__global__ void k_q27_init(DevParams p, Grid3 g3, const double *__restrict__ rho, const double *__restrict__ ux,
-                           const double *__restrict__ uy, const double *__restrict__ uz,
-                           const double *__restrict__ T, R *__restrict__ st, DevStats *stats)
-{
-    const long long n = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (n >= p.N) return;
-    const int X = (int)(n % p.nx), Y = (int)((n / p.nx) % p.ny), Z = (int)(n / ((long long)p.nx * p.ny));
-    double gr[3] = {0.0, 0.0, 0.0};
-    for (int i = 0; i < Q27; ++i) {
-        const int cx = i % 3 - 1, cy = (i / 3) % 3 - 1, cz = i / 9 - 1;
-        const double v = rho[node27(p, g3, X + cx, Y + cy, Z + cz)], w = w27(i);
-        gr[0] += w * cx * v; gr[1] += w * cy * v; gr[2] += w * cz * v;
-    }
-    for (int k = 0; k < 3; ++k) gr[k] *= 3.0;
-    const double r = rho[n], t = T[n];
-    if (!(r > 0.0) || !(p.b * r < 1.0) || !(t > 0.0)) atomicAdd(&stats->bad_init, 1ull);
-    const double pr = eos_pressure<double>(p.eos_kind, p.a, p.b, p.R, r, t, p.sp);
-    const double P = pr > p.p_floor ? pr : p.p_floor;
-    const double th = P / (r * POND_TL), s = sqrt(th);
-    const double e = p.cv * t - p.a * r;
-    const double lam_e = p.kappa * (gr[0] * gr[0] + gr[1] * gr[1] + gr[2] * gr[2]);
-    const double u[3] = {ux[n], uy[n], uz[n]};
-    for (int i = 0; i < Q27; ++i) {
-        const double w = w27(i);
-        const double vx = s * (i % 3 - 1) + u[0], vy = s * ((i / 3) % 3 - 1) + u[1], vz = s * (i / 9 - 1) + u[2];
-        REC27(st, n, R_F + i) = (R)(r * w);
-        REC27(st, n, R_G + i) = (R)(r * w * (2.0 * e - 3.0 * P / r + vx * vx + vy * vy + vz * vz) + w * lam_e);
-    }
-    REC27(st, n, R_TH) = (R)th;
-    for (int a = 0; a < 3; ++a) {
-        REC27(st, n, R_UX + a) = (R)u[a];
-        REC27(st, n, R_UHX + a) = (R)u[a];
-    }
-    REC27(st, n, R_RHO) = (R)r;
-    REC27(st, n, R_T) = (R)t;
-    for (int k = R_MLO; k < SL27; ++k) REC27(st, n, k) = (R)0;
-}
-
-// ---------------------------------------------------------------------------
 // Non-local terms, stage 0: p/rho of every node of `src`.
 template <typename R>
 __global__ void k_q27_pi(DevParams p, const R *__restrict__ src, typename Wide<R>::type *__restrict__ nl)
@@ -249,6 +207,63 @@ struct Near27 {
     }
     __device__ __forceinline__ long long at(int z, int y, int k) const { return row[z][y] + x[k]; }
 };
+
+// ---------------------------------------------------------------------------
+// Initial state: co-moving equilibrium of host-given (rho, u, T) with the interface
+// energy (Eq. geq, D = 3).
+template <typename R>
+__global__ void k_q27_init(DevParams p, Grid3 g3, const double *__restrict__ rho, const double *__restrict__ ux,
+                           const double *__restrict__ uy, const double *__restrict__ uz,
+                           const double *__restrict__ T, R *__restrict__ st, DevStats *stats)
+{
+    const long long n = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (n >= p.N) return;
+    // the gradient by lines, planes and a column (the separable stencil, see diff3 below)
+    const Near27 nb(p, g3, n);
+    const Diff3<double> dr = diff3<double>([&](int z, int y, int k) { return rho[nb.at(z, y, k)]; });
+    double g2 = 0.0;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        const double g = dr.d[a] * (1.0 / 72.0);
+        g2 += g * g;
+    }
+    const double r = rho[n], t = T[n], u[3] = {ux[n], uy[n], uz[n]};
+    if (!(r > 0.0) || !(p.b * r < 1.0) || !(t > 0.0)) atomicAdd(&stats->bad_init, 1ull);
+    const double pr = pressure_d(p, r, t);
+    const double P = pr > p.p_floor ? pr : p.p_floor;
+    const double th = P * rcp_d(r) * 3.0, s = sqrt(th);   // theta = P / (rho T_L)
+    // g_i = W_i (G + rho v_x^2 + rho v_y^2 + rho v_z^2), as in k_init
+    const double G = r * (2.0 * (p.cv * t - p.a * r)) - 3.0 * P + p.kappa * g2;
+    double b[3][3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a)
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            const double v = s * (k - 1) + u[a];
+            b[a][k] = r * (v * v);
+        }
+    R rec[SL27];
+#pragma unroll
+    for (int z = 0; z < 3; ++z)
+#pragma unroll
+        for (int y = 0; y < 3; ++y) {
+            const double gyz = G + (b[1][y] + b[2][z]);
+#pragma unroll
+            for (int x = 0; x < 3; ++x) {
+                const int i = 9 * z + 3 * y + x;
+                rec[R_F + i] = (R)(r * w27(i));
+                rec[R_G + i] = (R)(w27(i) * (gyz + b[0][x]));
+            }
+        }
+    rec[R_TH] = (R)th;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) rec[R_UX + a] = rec[R_UHX + a] = (R)u[a];
+    rec[R_RHO] = (R)r;
+    rec[R_T] = (R)t;
+#pragma unroll
+    for (int k = R_MLO; k < SL27; ++k) rec[k] = (R)0;
+    store_chunks<SL27>(st, (size_t)n, (size_t)p.N, rec);
+}
 
 // Stage 1 (rho, T of `src`): K = -kappa (rho lap rho + |grad rho|^2/2) I + kappa grad rho
 // (x) grad rho, q = -mu grad h + k grad T (h = C_v T - a rho + p/rho), rho E_lambda = kappa
@@ -1339,7 +1354,7 @@ __global__ void k_q27_moments(DevParams p, const R *__restrict__ st, double *rho
     if (uy) uy[n] = (double)REC27(st, n, R_UHX + 1);
     if (uz) uz[n] = (double)REC27(st, n, R_UHX + 2);
     if (T) T[n] = t;
-    if (pr) pr[n] = eos_pressure<double>(p.eos_kind, p.a, p.b, p.R, r, t, p.sp);
+    if (pr) pr[n] = pressure_d(p, r, t);
 }
 
 // Conservation sums, stage 1: {rho, rho uhat_x, rho uhat_y, sum g / 2} per block.

@@ -180,15 +180,6 @@ __device__ __forceinline__ R pick(const R (&a)[K], int i)
     return r;
 }
 
-// 1/x in FP64 from the FP32 reciprocal and two Newton steps (relative error ~1e-28
-// before the final rounding); x must lie in the FP32 normal range.
-__device__ __forceinline__ double rcp_d(double x)
-{
-    double r = (double)__frcp_rn((float)x);
-    r = r * (2.0 - x * r);
-    return r * (2.0 - x * r);
-}
-
 // a / b for operands of moderate range (transfer-map offsets, collision coefficients):
 // the fast FP32 quotient, or a times the Newton reciprocal in FP64.
 template <typename R> __device__ __forceinline__ R fdiv_(R a, R b);
@@ -282,21 +273,6 @@ __device__ __forceinline__ void load_rec24(const double *__restrict__ b, size_t 
         const double2 t = __ldg(q + k * N);
         v[2 * k] = t.x; v[2 * k + 1] = t.y;
     }
-}
-// Writes a whole record of W values.
-template <int W>
-__device__ __forceinline__ void store_chunks(float *b, size_t nd, size_t N, const float (&v)[W])
-{
-    float4 *q = reinterpret_cast<float4 *>(b) + nd;
-#pragma unroll
-    for (int k = 0; k < W / 4; ++k) q[k * N] = make_float4(v[4 * k], v[4 * k + 1], v[4 * k + 2], v[4 * k + 3]);
-}
-template <int W>
-__device__ __forceinline__ void store_chunks(double *b, size_t nd, size_t N, const double (&v)[W])
-{
-    double2 *q = reinterpret_cast<double2 *>(b) + nd;
-#pragma unroll
-    for (int k = 0; k < W / 2; ++k) q[k * N] = make_double2(v[2 * k], v[2 * k + 1]);
 }
 // Four staged values from a 16-byte boundary.
 __device__ __forceinline__ void lds4(const float *s, float (&o)[4])
@@ -1930,6 +1906,11 @@ __global__ void __launch_bounds__(STEP_THREADS, SPLIT ? SPLIT_MIN_BLOCKS(R) : ST
     for (int k = threadIdx.x; k < (int)(sizeof(SimDesc<R>) / 8); k += STEP_THREADS)
         reinterpret_cast<unsigned long long *>(&d)[k] = src[k];
     __syncthreads();
+    // the launch may begin while the previous step still runs (its blocks, this far, only
+    // copy their descriptor): wait until that step is complete and its memory visible, then
+    // let the next one begin
+    asm volatile("griddepcontrol.wait;\n" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
     extern __shared__ __align__(128) unsigned char step_dyn_smem[];
     R *smem = reinterpret_cast<R *>(step_dyn_smem);
     if constexpr (SPLIT) step_tile_split<R>(d.p, d.in, d.out, d.stats, tile, d.nlsrc, smem);
