@@ -1035,8 +1035,7 @@ void launch_all(pond_batch *b, int first, int steps, On on)
 }
 
 // Captures two steps (even, then odd) of every member; the members' chains are independent
-// until both are done.  A group of few blocks then no longer holds up the others (twelve
-// grids of 64 x 64 to 164 x 160 nodes, one of them in the small-grid group: @BATCH@).
+// until both are done, so that a group of few blocks does not hold up the others.
 cudaError_t capture_two_steps(pond_batch *b, cudaGraph_t *graph)
 {
     cudaError_t e = cudaSuccess;

@@ -71,25 +71,34 @@ constexpr float SMOOTH_TILE = 0.9f;
 constexpr float STALL_TOL_FACTOR = 16.0f;
 // resident blocks per SM the register budget is sized for
 #define STEP_MIN_BLOCKS(R) (sizeof(R) == 8 ? 2 : 3)
-#define SPLIT_MIN_BLOCKS(R) (sizeof(R) == 8 ? 2 : 3)
+#define SPLIT_MIN_BLOCKS(R) 2
 
 // Values per staged slot: the 18 carried populations, padded so that slots start on
 // distinct banks (FP32: 16-byte loads, 20 words; FP64: 19 values).
 template <typename R> struct Slot;
 template <> struct Slot<float> { static constexpr int stride = 20; };
 template <> struct Slot<double> { static constexpr int stride = 19; };
+// place of population i of family fam (0 f, 1 g): side by side in FP32
+template <typename R> __host__ __device__ constexpr int slot_at(int fam, int i) { return sizeof(R) == 4 ? 2 * i + fam : 9 * fam + i; }
 constexpr int AUXW = 4;   // rho, T, p, p/rho of a staged node
 constexpr int SPLIT_WORDS = SL + 9 * 18;   // nine lanes per node: the own record, the lanes' partials
 constexpr int KQW = 5;    // K_xx, K_xy, K_yy, q_x, q_y of a node of the tile and its ring
 
 __host__ __device__ constexpr int step_slots(int tx, int ty) { return (tx + 2 * HALO) * (ty + 2 * HALO); }
 
+// What a thread of the one-thread-per-node form keeps in shared memory across the stream
+// instead of in registers (a column of KEEP values; the contraction's weights then fit 168
+// registers, three blocks per SM, without recomputing them): the node's own sums (hi, lo),
+// F, rho E_lambda, M_0, and the y weights and rows of the map.
+enum : int { K_HI = 0, K_LO = 4, K_F = 8, K_REL = 10, K_M0 = 11, K_WY = 12, K_LY = 27, KEEP = 36 };
+
 // Dynamic shared memory of one step block: slots' rho, T, p, p/rho; populations; K and q;
-// with nine lanes per node also the partials of the general stream and the own records.
+// then the threads' kept values, or with nine lanes per node the partials of the general
+// stream and the own records.
 __host__ __device__ constexpr size_t step_smem_bytes(int tx, int ty, bool split, int slot_values, int elem_bytes)
 {
     return ((size_t)step_slots(tx, ty) * (AUXW + slot_values) + (size_t)(tx + 2) * (ty + 2) * KQW +
-            (split ? (size_t)SPLIT_NB * SPLIT_WORDS : 0)) * elem_bytes;
+            (split ? (size_t)SPLIT_NB * SPLIT_WORDS : (size_t)STEP_THREADS * KEEP)) * elem_bytes;
 }
 
 // Counters of one block, summed into the context's by its last instructions.
@@ -832,81 +841,96 @@ __device__ __noinline__ void stream_general(const DevParams &p, const R *__restr
     }
 }
 
+// Pairs of FP32 values in one 64-bit register: one instruction multiplies and adds both
+// (fma.rn.f32x2: the rate of two FFMAs in one issue slot and one fetched instruction).
+using f32x2 = unsigned long long;
+__device__ __forceinline__ f32x2 pack2(float a, float b)
+{
+    f32x2 r;
+    asm("mov.b64 %0, {%1, %2};\n" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ void unpack2(f32x2 v, float &a, float &b) { asm("mov.b64 {%0, %1}, %2;\n" : "=f"(a), "=f"(b) : "l"(v)); }
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c)
+{
+    f32x2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;\n" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b)
+{
+    f32x2 r;
+    asm("add.rn.f32x2 %0, %1, %2;\n" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+
 // The stream as a contraction over the staged slots (see the head of this file), FP32:
 // own = the node's own slot, pitch = slots per staged row.  Five columns and rows with
-// zero weights outside a direction's four nodes, so that every offset is a constant.
-// acc = increments over the node's own populations (f, then g).
+// zero weights outside a direction's four nodes, so that every offset is a constant.  f and
+// g take the same weights, so a slot holds their values side by side and each instruction
+// works on both.  keep = the thread's kept values (y weights).  acc = increments over the
+// node's own populations (f, then g).
 __device__ __forceinline__ void contract(const float *own, int pitch, const float (&ax)[3][4],
-                                         const bool (&nx0)[3], const float (&ay)[3][4], const bool (&ny0)[3],
-                                         const float (&Lx)[3][3], const float (&Ly)[3][3], float (&acc)[2][9])
+                                         const bool (&nx0)[3], const float (&Lx)[3][3], const float *keep,
+                                         float (&acc)[2][9])
 {
     constexpr int DS = Slot<float>::stride;
-    float wl[3][5][3], wy[3][5], dx[DS];
+    f32x2 wl[3][5][3], a2[9], dx[DS / 2];
 #pragma unroll
     for (int k = 0; k < 3; ++k)
 #pragma unroll
         for (int c = 0; c < 5; ++c) {
             const float w = nx0[k] ? (c == 0 ? 0.0f : ax[k][c - 1 < 0 ? 0 : c - 1]) : (c == 4 ? 0.0f : ax[k][c > 3 ? 3 : c]);
-            wy[k][c] = ny0[k] ? (c == 0 ? 0.0f : ay[k][c - 1 < 0 ? 0 : c - 1]) : (c == 4 ? 0.0f : ay[k][c > 3 ? 3 : c]);
 #pragma unroll
-            for (int m = 0; m < 3; ++m) wl[k][c][m] = w * Lx[k][m];
+            for (int m = 0; m < 3; ++m) wl[k][c][m] = pack2(w * Lx[k][m], w * Lx[k][m]);
         }
 #pragma unroll
     for (int q = 0; q < DS / 4; ++q) {
         float t[4];
         lds4(own + 4 * q, t);
-#pragma unroll
-        for (int e = 0; e < 4; ++e) dx[4 * q + e] = t[e];
+        dx[2 * q] = pack2(-t[0], -t[1]);
+        dx[2 * q + 1] = pack2(-t[2], -t[3]);
     }
 #pragma unroll
-    for (int fam = 0; fam < 2; ++fam)
-#pragma unroll
-        for (int i = 0; i < 9; ++i) acc[fam][i] = 0.0f;
+    for (int i = 0; i < 9; ++i) a2[i] = 0ull;
     const float *row = own - (2 * pitch + 2) * DS;
 #pragma unroll 1
     for (int cy = 0; cy < 5; ++cy, row += pitch * DS) {
-        float t[2][3][3];   // family, n, k
+        f32x2 t[3][3];   // n, k
 #pragma unroll
-        for (int fam = 0; fam < 2; ++fam)
+        for (int n = 0; n < 3; ++n)
+#pragma unroll
+            for (int k = 0; k < 3; ++k) t[n][k] = 0ull;
+#pragma unroll
+        for (int cx = 0; cx < 5; ++cx) {
+            f32x2 v[DS / 2];
+#pragma unroll
+            for (int q = 0; q < DS / 4; ++q) {
+                const ulonglong2 x = reinterpret_cast<const ulonglong2 *>(row + cx * DS)[q];
+                v[2 * q] = add2(x.x, dx[2 * q]);
+                v[2 * q + 1] = add2(x.y, dx[2 * q + 1]);
+            }
 #pragma unroll
             for (int n = 0; n < 3; ++n)
 #pragma unroll
-                for (int k = 0; k < 3; ++k) t[fam][n][k] = 0.0f;
+                for (int m = 0; m < 3; ++m)
 #pragma unroll
-        for (int cx = 0; cx < 5; ++cx) {
-            float v[DS];
-#pragma unroll
-            for (int q = 0; q < DS / 4; ++q) {
-                float x[4];
-                lds4(row + cx * DS + 4 * q, x);
-#pragma unroll
-                for (int e = 0; e < 4; ++e) v[4 * q + e] = x[e] - dx[4 * q + e];
-            }
-#pragma unroll
-            for (int fam = 0; fam < 2; ++fam)
-#pragma unroll
-                for (int n = 0; n < 3; ++n)
-#pragma unroll
-                    for (int m = 0; m < 3; ++m)
-#pragma unroll
-                        for (int k = 0; k < 3; ++k)
-                            t[fam][n][k] = fmaf(wl[k][cx][m], v[9 * fam + 3 * n + m], t[fam][n][k]);
+                    for (int k = 0; k < 3; ++k) t[n][k] = fma2(wl[k][cx][m], v[3 * n + m], t[n][k]);
         }
 #pragma unroll
         for (int l = 0; l < 3; ++l) {
-            const float w = wy[l][0];
-#pragma unroll
-            for (int c = 0; c < 4; ++c) wy[l][c] = wy[l][c + 1];   // the next row's weight moves to the front
+            const float w = keep[(K_WY + 5 * l + cy) * STEP_THREADS];
 #pragma unroll
             for (int n = 0; n < 3; ++n) {
-                const float wn = w * Ly[l][n];
+                const float wl_n = w * keep[(K_LY + 3 * l + n) * STEP_THREADS];
+                const f32x2 wn = pack2(wl_n, wl_n);
 #pragma unroll
-                for (int fam = 0; fam < 2; ++fam)
-#pragma unroll
-                    for (int k = 0; k < 3; ++k) acc[fam][3 * l + k] = fmaf(wn, t[fam][n][k], acc[fam][3 * l + k]);
+                for (int k = 0; k < 3; ++k) a2[3 * l + k] = fma2(wn, t[n][k], a2[3 * l + k]);
             }
         }
     }
+#pragma unroll
+    for (int i = 0; i < 9; ++i) unpack2(a2[i], acc[0][i], acc[1][i]);
 }
 
 // The same over the FP64 slots: the x pass reads each direction's own four
@@ -914,11 +938,11 @@ __device__ __forceinline__ void contract(const float *own, int pitch, const floa
 // FP32 rate), and a row pass costs 36 multiply-adds instead of 45.  acc = the streamed
 // populations.
 __device__ __forceinline__ void contract(const double *own, int pitch, const double (&ax)[3][4],
-                                         const bool (&nx0)[3], const double (&ay)[3][4], const bool (&ny0)[3],
-                                         const double (&Lx)[3][3], const double (&Ly)[3][3], double (&acc)[2][9])
+                                         const bool (&nx0)[3], const double (&Lx)[3][3], const double *keep,
+                                         double (&acc)[2][9])
 {
     constexpr int DS = Slot<double>::stride;
-    double wl[3][4][3], wy[3][5];
+    double wl[3][4][3];
     int off[3];
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
@@ -927,9 +951,6 @@ __device__ __forceinline__ void contract(const double *own, int pitch, const dou
         for (int c = 0; c < 4; ++c)
 #pragma unroll
             for (int m = 0; m < 3; ++m) wl[k][c][m] = ax[k][c] * Lx[k][m];
-#pragma unroll
-        for (int c = 0; c < 5; ++c)
-            wy[k][c] = ny0[k] ? (c == 0 ? 0.0 : ay[k][c - 1 < 0 ? 0 : c - 1]) : (c == 4 ? 0.0 : ay[k][c > 3 ? 3 : c]);
     }
 #pragma unroll
     for (int fam = 0; fam < 2; ++fam)
@@ -941,11 +962,9 @@ __device__ __forceinline__ void contract(const double *own, int pitch, const dou
         double wn[3][3];
 #pragma unroll
         for (int l = 0; l < 3; ++l) {
-            const double w = wy[l][0];
+            const double w = keep[(K_WY + 5 * l + cy) * STEP_THREADS];
 #pragma unroll
-            for (int c = 0; c < 4; ++c) wy[l][c] = wy[l][c + 1];
-#pragma unroll
-            for (int n = 0; n < 3; ++n) wn[l][n] = w * Ly[l][n];
+            for (int n = 0; n < 3; ++n) wn[l][n] = w * keep[(K_LY + 3 * l + n) * STEP_THREADS];
         }
 #pragma unroll
         for (int fam = 0; fam < 2; ++fam)
@@ -968,11 +987,11 @@ __device__ __forceinline__ void contract(const double *own, int pitch, const dou
 
 // Streams node (X, Y) into the gauge (th, ux, uy): inc = the increments of the streamed
 // populations over the node's own (f, then g).  gauge_b: the tile's common gauge
-// (sqrt theta, u_x, u_y).
+// (sqrt theta, u_x, u_y); keep: the thread's column of kept values.
 template <typename R>
 __device__ __forceinline__ void stream_node(const DevParams &p, const R *__restrict__ in, int X, int Y, const R *slot,
                                             int pitch, const R (&gauge_b)[3], R th, R ux, R uy, bool first,
-                                            R (&inc)[2][9], unsigned &nreg, unsigned &npair)
+                                            R *keep, R (&inc)[2][9], unsigned &nreg, unsigned &npair)
 {
     const R dt = typed<R>(p).dt;
     const R s = sqrt_(th), inv_s = R(1) / s;
@@ -995,7 +1014,16 @@ __device__ __forceinline__ void stream_node(const DevParams &p, const R *__restr
     const R qb = (gauge_b[0] - s) * inv_s;
     axis_rows<R>(qb, (gauge_b[1] - ux) * inv_s, Lx);
     axis_rows<R>(qb, (gauge_b[2] - uy) * inv_s, Ly);
-    contract(slot, pitch, ax, nx0, ay, ny0, Lx, Ly, inc);
+#pragma unroll
+    for (int l = 0; l < 3; ++l) {
+#pragma unroll
+        for (int c = 0; c < 5; ++c)
+            keep[(K_WY + 5 * l + c) * STEP_THREADS] =
+                ny0[l] ? (c == 0 ? R(0) : ay[l][c - 1 < 0 ? 0 : c - 1]) : (c == 4 ? R(0) : ay[l][c > 3 ? 3 : c]);
+#pragma unroll
+        for (int n = 0; n < 3; ++n) keep[(K_LY + 3 * l + n) * STEP_THREADS] = Ly[l][n];
+    }
+    contract(slot, pitch, ax, nx0, Lx, keep, inc);
     if constexpr (sizeof(R) == 8) {
         R v[24];
         load_rec24(in, (size_t)Y * p.nx + X, (size_t)p.N, v);
@@ -1277,7 +1305,7 @@ __device__ __forceinline__ void stage_tile(const DevParams &p, const R *__restri
                 map_inc<R>(Ex, Ey, v + 9 * fam, o);
 #pragma unroll
                 for (int i = 0; i < 9; ++i)
-                    d[9 * fam + i] = (v[9 * fam + i] - base[9 * fam + i]) + o[i];
+                    d[slot_at<R>(fam, i)] = (v[9 * fam + i] - base[9 * fam + i]) + o[i];
             }
         } else {
             axis_rows<R>(e, wx, Ex);
@@ -1293,7 +1321,7 @@ __device__ __forceinline__ void stage_tile(const DevParams &p, const R *__restri
                                 Ex[k2][2] * v[9 * fam + 3 * b2 + 2];
 #pragma unroll
                     for (int l2 = 0; l2 < 3; ++l2)
-                        d[9 * fam + 3 * l2 + k2] = Ey[l2][0] * t[0] + Ey[l2][1] * t[1] + Ey[l2][2] * t[2];
+                        d[slot_at<R>(fam, 3 * l2 + k2)] = Ey[l2][0] * t[0] + Ey[l2][1] * t[1] + Ey[l2][2] * t[2];
                 }
         }
         R *dst = slots + (size_t)k * DS;
@@ -1308,12 +1336,18 @@ __device__ __forceinline__ void stage_tile(const DevParams &p, const R *__restri
         }
         put_aux(k, nd, v[P_RHO], v[P_T]);
     };
-    if (ka < nslots) carry(ka, na, va);
-    if (kb < nslots) carry(kb, nb, vb);
-    for (int k = tid + 2 * ST_NT; k < nslots; k += ST_NT) {
-        const size_t nd = node_of(k);
-        load_rec24(in, nd, N, va);
-        carry(k, nd, va);
+    // (one copy of the carrying code: it is fetched once and runs for every slot)
+#pragma unroll 1
+    for (int k = tid; k < nslots; k += ST_NT) {
+        if (k >= 2 * ST_NT) {
+            na = node_of(k);
+            load_rec24(in, na, N, va);
+        } else if (k >= ST_NT) {
+            na = nb;
+#pragma unroll
+            for (int i = 0; i < 24; ++i) va[i] = vb[i];
+        }
+        carry(k, na, va);
     }
     __syncthreads();
 
@@ -1433,6 +1467,7 @@ __device__ __forceinline__ void step_tile(const DevParams &p, const R *__restric
     const int tx = tid % tl.TX, ty = tid / tl.TX;
     const int X = tl.X0 + tx, Y = tl.Y0 + ty;
     const bool valid = X < p.nx && Y < p.ny;
+    R *keep = tl.kq + (size_t)(tl.TX + 2) * (tl.TY + 2) * KQW + tid;   // this thread's column
     const int slot = (ty + HALO) * tl.WT + tx + HALO;
     unsigned its = 0, nreg = 0, npair = 0;
     bool conv = true, stall = false, floored = false, bad = false;
@@ -1441,13 +1476,16 @@ __device__ __forceinline__ void step_tile(const DevParams &p, const R *__restric
 #pragma unroll
         for (int i = 0; i < 4; ++i)
             divergence_pair<R>(tl, tl.kq + ((ty + 1) * tl.RW + tx + 1) * KQW, tl.aux + slot * AUXW, i, Fx, Fy, M0, gxn, gyn);
-        const R nl[3] = {Fx, Fy, R(0.5) * q.kappa * (gxn * gxn + gyn * gyn)};
+        keep[K_F * STEP_THREADS] = Fx;
+        keep[(K_F + 1) * STEP_THREADS] = Fy;
+        keep[K_REL * STEP_THREADS] = R(0.5) * q.kappa * (gxn * gxn + gyn * gyn);
+        keep[K_M0 * STEP_THREADS] = M0;
         // exact sums of the node's stored populations (error-free in R: TwoSum cascades,
         // each sum an unevaluated (hi, lo) pair); the stored low parts start the error terms
         const size_t n = (size_t)Y * p.nx + X;
-        R hi[4] = {R(0), R(0), R(0), R(0)}, lo[4];
         R th, ux, uy;
         {
+            R hi[4] = {R(0), R(0), R(0), R(0)}, lo[4];
             R v[24];
             load_rec24(in, n, N, v);
             lo[0] = __ldg(in + rec_at(in, n, P_F4LO, N));
@@ -1468,6 +1506,11 @@ __device__ __forceinline__ void step_tile(const DevParams &p, const R *__restric
                     lo[k] += e;
                 }
             }
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                keep[(K_HI + k) * STEP_THREADS] = hi[k];
+                keep[(K_LO + k) * STEP_THREADS] = lo[k];
+            }
         }
 
         // ---------------- phase 1: frame search -------------------------------------
@@ -1476,7 +1519,8 @@ __device__ __forceinline__ void step_tile(const DevParams &p, const R *__restric
         float last = 3.0e38f;   // previous residual
         for (;;) {
             ++its;
-            stream_node<R>(p, in, X, Y, tl.slots + (size_t)slot * DS, tl.WT, gb, th, ux, uy, its == 1, inc, nreg, npair);
+            stream_node<R>(p, in, X, Y, tl.slots + (size_t)slot * DS, tl.WT, gb, th, ux, uy, its == 1, keep, inc,
+                           nreg, npair);
             R sum[4] = {R(0), R(0), R(0), R(0)};
 #pragma unroll
             for (int i = 0; i < 9; ++i) {
@@ -1489,6 +1533,14 @@ __device__ __forceinline__ void step_tile(const DevParams &p, const R *__restric
             }
             const R lam[3] = {th, ux, uy};
             const R sr = sqrt_(th);
+            R hi[4], lo[4], nl[3];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                hi[k] = keep[(K_HI + k) * STEP_THREADS];
+                lo[k] = keep[(K_LO + k) * STEP_THREADS];
+            }
+#pragma unroll
+            for (int k = 0; k < 3; ++k) nl[k] = keep[(K_F + k) * STEP_THREADS];
             eos_update(p, hi, lo, sum, nl, lam, sr, o);
             const float res = gauge_change<R>(o, th, sr);
             stop_rules<R>(p, res, last, its, conv, stall);
@@ -1508,7 +1560,8 @@ __device__ __forceinline__ void step_tile(const DevParams &p, const R *__restric
                 ft[i] = v[P_F + i] + inc[0][i];
                 gt[i] = v[P_G + i] + inc[1][i];
             }
-            collide<R>(q, o, th, ux, uy, Fx, Fy, M0, ft, gt, rec);
+            collide<R>(q, o, th, ux, uy, keep[K_F * STEP_THREADS], keep[(K_F + 1) * STEP_THREADS],
+                       keep[K_M0 * STEP_THREADS], ft, gt, rec);
         }
         store_chunks<SL>(out, n, N, rec);
         floored = o.pr < q.p_floor;
@@ -1605,8 +1658,8 @@ __device__ __forceinline__ void step_tile_split(const DevParams &p, const R *__r
     const R *sl = tl.slots + (size_t)slot * DS;
 #pragma unroll
     for (int m = 0; m < 3; ++m) {
-        dx[m] = sizeof(R) == 4 ? sl[3 * l + m] : R(0);
-        dx[3 + m] = sizeof(R) == 4 ? sl[9 + 3 * l + m] : R(0);
+        dx[m] = sizeof(R) == 4 ? sl[slot_at<R>(0, 3 * l + m)] : R(0);
+        dx[3 + m] = sizeof(R) == 4 ? sl[slot_at<R>(1, 3 * l + m)] : R(0);
     }
 
     // ---------------- phase 1: frame search (warp lockstep) ---------------------------
@@ -1667,22 +1720,49 @@ __device__ __forceinline__ void step_tile_split(const DevParams &p, const R *__r
 #pragma unroll
                 for (int m = 0; m < 3; ++m) wl[c][m] = wx[c] * Lx[m];
             R af[3] = {R(0), R(0), R(0)}, ag[3] = {R(0), R(0), R(0)};
-            const R *row = sl - (2 * tl.WT + (near_x ? 1 : 2)) * DS + 3 * l;
+            const R *row = sl - (2 * tl.WT + (near_x ? 1 : 2)) * DS + slot_at<R>(0, 3 * l);
+            if constexpr (sizeof(R) == 4) {
+                // f and g side by side (see contract)
+                f32x2 w2[4][3], d2[3], a2[3] = {0ull, 0ull, 0ull};
 #pragma unroll
-            for (int cy = 0; cy < 5; ++cy, row += tl.WT * DS) {
-                R tf = 0, tg = 0;
+                for (int m = 0; m < 3; ++m) {
+                    d2[m] = pack2(-dx[m], -dx[3 + m]);
 #pragma unroll
-                for (int c = 0; c < 4; ++c)
+                    for (int c = 0; c < 4; ++c) w2[c][m] = pack2(wl[c][m], wl[c][m]);
+                }
 #pragma unroll
-                    for (int m = 0; m < 3; ++m) {
-                        tf += wl[c][m] * (sizeof(R) == 4 ? row[c * DS + m] - dx[m] : row[c * DS + m]);
-                        tg += wl[c][m] * (sizeof(R) == 4 ? row[c * DS + 9 + m] - dx[3 + m] : row[c * DS + 9 + m]);
+                for (int cy = 0; cy < 5; ++cy, row += tl.WT * DS) {
+                    f32x2 t = 0ull;
+#pragma unroll
+                    for (int c = 0; c < 4; ++c)
+#pragma unroll
+                        for (int m = 0; m < 3; ++m)
+                            t = fma2(w2[c][m], add2(reinterpret_cast<const f32x2 *>(row + c * DS)[m], d2[m]), t);
+#pragma unroll
+                    for (int c = 0; c < 3; ++c) {
+                        const float w = wy[c][cy] * Ly[c];
+                        a2[c] = fma2(pack2(w, w), t, a2[c]);
                     }
+                }
 #pragma unroll
-                for (int c = 0; c < 3; ++c) {
-                    const R w = wy[c][cy] * Ly[c];
-                    af[c] += w * tf;
-                    ag[c] += w * tg;
+                for (int c = 0; c < 3; ++c) unpack2(a2[c], af[c], ag[c]);
+            } else {
+#pragma unroll
+                for (int cy = 0; cy < 5; ++cy, row += tl.WT * DS) {
+                    R tf = 0, tg = 0;
+#pragma unroll
+                    for (int c = 0; c < 4; ++c)
+#pragma unroll
+                        for (int m = 0; m < 3; ++m) {
+                            tf += wl[c][m] * row[c * DS + m];
+                            tg += wl[c][m] * row[c * DS + 9 + m];
+                        }
+#pragma unroll
+                    for (int c = 0; c < 3; ++c) {
+                        const R w = wy[c][cy] * Ly[c];
+                        af[c] += w * tf;
+                        ag[c] += w * tg;
+                    }
                 }
             }
             // lane (k, n) keeps its share of l = n and sends the others to their lanes
