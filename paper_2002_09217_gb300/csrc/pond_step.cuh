@@ -1271,25 +1271,48 @@ __device__ __forceinline__ void stage_tile(const DevParams &p, const R *__restri
     Extremes ex;
     if (ka < nslots) { na = node_of(ka); load_rec24(in, na, N, va); }
     if (kb < nslots) { nb = node_of(kb); load_rec24(in, nb, N, vb); }
-    if (ka < nslots) ex.offer((float)va[P_TH], ka);
-    if (kb < nslots) ex.offer((float)vb[P_TH], kb);
-    for (int k = tid + 2 * ST_NT; k < nslots; k += ST_NT) ex.offer((float)__ldg(in + rec_at(in, node_of(k), P_TH, N)), k);
+    // every slot's gauge goes to shared memory (where its rho, T will lie), so that the
+    // agreed nodes' gauges and populations need no further global loads
+    auto note = [&](int k, R th, R ux, R uy) {
+        ex.offer((float)th, k);
+        R *a = aux + (size_t)k * AUXW;
+        a[0] = th; a[1] = ux; a[2] = uy;
+    };
+    if (ka < nslots) note(ka, va[P_TH], va[P_UX], va[P_UY]);
+    if (kb < nslots) note(kb, vb[P_TH], vb[P_UX], vb[P_UY]);
+    for (int k = tid + 2 * ST_NT; k < nslots; k += ST_NT) {
+        const size_t nd = node_of(k);
+        note(k, __ldg(in + rec_at(in, nd, P_TH, N)), __ldg(in + rec_at(in, nd, P_UX, N)), __ldg(in + rec_at(in, nd, P_UY, N)));
+    }
     ex = tile_extremes(ex, best);
     const bool smooth = sizeof(R) == 4 && ex.smooth();
-    const size_t nhot = node_of(min((int)ex.at, nslots - 1)), ncold = node_of(min((int)ex.lat, nslots - 1));
+    const int khot = min((int)ex.at, nslots - 1), kcold = min((int)ex.lat, nslots - 1);
     R thb;
     {
         R hot[3], cold[3];
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
-            hot[k] = __ldg(in + rec_at(in, nhot, P_TH + k, N));
-            cold[k] = __ldg(in + rec_at(in, ncold, P_TH + k, N));
+            hot[k] = aux[khot * AUXW + k];
+            cold[k] = aux[kcold * AUXW + k];
         }
         common_gauge<R, 3>(smooth, hot, cold, gb);
         thb = smooth ? hot[0] : gb[0] * gb[0];
     }
-    R base[24];
-    if (smooth) load_rec24(in, nhot, N, base);
+    __shared__ R base[18];   // the hottest node's populations
+    if (smooth) {
+        if (khot == ka) {
+#pragma unroll
+            for (int i = 0; i < 18; ++i) base[i] = va[i];
+        } else if (khot == kb) {
+#pragma unroll
+            for (int i = 0; i < 18; ++i) base[i] = vb[i];
+        } else if (khot >= 2 * ST_NT && tid == 0) {
+            const size_t nd = node_of(khot);
+#pragma unroll
+            for (int i = 0; i < 18; ++i) base[i] = __ldg(in + rec_at(in, nd, i, N));
+        }
+    }
+    __syncthreads();   // base is there, and aux may be overwritten
     const R inv_sb = R(1) / gb[0];
     auto carry = [&](int k, size_t nd, const R (&v)[24]) {
         const R sn = sqrt_(v[P_TH]);
@@ -1670,7 +1693,8 @@ __device__ __forceinline__ void step_tile_split(const DevParams &p, const R *__r
     float last = 3.0e38f;
     for (unsigned it = 1; __any_sync(ALL, active); ++it) {
         const R s = sqrt_(th), inv_s = R(1) / s, dt = q.dt;
-        // departure along x of component k, along y of all three
+        // departure along x of component k, along y of component l; the other y components'
+        // weights come from the lanes that hold them
         R wx[4], wy[3][5], Lx[3], Ly[3];
         bool near_x, ok = true;
         {
@@ -1687,10 +1711,14 @@ __device__ __forceinline__ void step_tile_split(const DevParams &p, const R *__r
                 return f == R(0);
             };
             near_x = weights(s * R(k - 1) + ux, wx);
+            R ya[4];
+            const unsigned nym = __ballot_sync(ALL, weights(s * R(l - 1) + uy, ya));
 #pragma unroll
             for (int c = 0; c < 3; ++c) {
                 R a[4];
-                const bool near = weights(s * R(c - 1) + uy, a);
+#pragma unroll
+                for (int j2 = 0; j2 < 4; ++j2) a[j2] = grp(ya[j2], base, 3 * c);
+                const bool near = (nym >> (base + 3 * c)) & 1u;
                 wy[c][0] = near ? R(0) : a[0];
                 wy[c][1] = near ? a[0] : a[1];
                 wy[c][2] = near ? a[1] : a[2];
