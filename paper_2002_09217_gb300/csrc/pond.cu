@@ -180,7 +180,9 @@ void launch_q16_pass(pond_ctx *c, const R *in, const R *src, R *out, DevStats *s
     const unsigned nb = blocks_for(c->N, 256);
     using W = typename Wide<R>::type;
     W *nl = reinterpret_cast<W *>(c->nlbuf);
-    k_q16_nonlocal1<R><<<nb, 256, 0, strm>>>(c->dp, src, nl);
+    const dim3 blk = c->grid.ny < 4 ? dim3(256, 1) : dim3(32, 8);
+    const dim3 grd(blocks_for((size_t)c->grid.nx, blk.x), blocks_for((size_t)c->grid.ny, blk.y));
+    k_q16_nonlocal1<R><<<grd, blk, 0, strm>>>(c->dp, src, nl);
     k_q16_nonlocal2<R><<<nb, 256, 0, strm>>>(c->dp, nl);
     k_q16_step<R><<<(unsigned)step_tiles(c), STEP_THREADS, q16_smem_bytes<R>(c->dp.tile_x, c->dp.tile_y), strm>>>(
         c->dp, in, nl, out, stats);
@@ -649,6 +651,8 @@ pond_status pond_create(const pond_grid *grid, const pond_lattice *lattice, cons
     };
     split(d.a, d.ff_a); split(d.b, d.ff_b); split(d.R, d.ff_R); split(d.pd.inv_cv, d.ff_icv);
     split(d.p_floor, d.ff_pfl); split(d.dt, d.ff_dt);
+    split(d.kappa, d.ff_kap); split(d.cv, d.ff_cv); split(d.pd.mu_coef, d.ff_mu); split(d.pd.cvR, d.ff_cvR);
+    split(d.k_cond, d.ff_kc);
     d.tol_f = (float)d.tol;
     d.eos_kind = c->eos.kind == POND_DIETERICI ? 2 : (c->eos.kind == POND_SIMPLIFIED ? 3 : 0);
     d.sp[0] = c->eos.beta; d.sp[1] = c->eos.rho_l; d.sp[2] = c->eos.rho_v; d.sp[3] = c->eos.p0;

@@ -61,6 +61,7 @@ struct DevParams {
     // the FP32 form's frame-search EoS constants as (hi, lo) float pairs (hi + lo = the
     // FP64 value to ~2^-48), and its tolerance
     float ff_a[2], ff_b[2], ff_R[2], ff_icv[2], ff_pfl[2], ff_dt[2];
+    float ff_kap[2], ff_cv[2], ff_mu[2], ff_cvR[2], ff_kc[2];   // kappa, C_v, (tau - 1/2) dt, C_v + R, k_cond
     float tol_f;
     // equation of state: 0 van der Waals, 2 Dieterici (isothermal only); isothermal runs
     // hold T at T_iso (and ff_Tiso, its float pair)

@@ -297,30 +297,44 @@ struct Near9 {
 //   K = -kappa (rho lap rho + |grad rho|^2 / 2) I + kappa grad rho (x) grad rho  (Eq. korteweg)
 //   q = -mu grad h + k grad T, mu = (tau - 1/2) P dt, h = e + p/rho              (Eq. gtilde)
 //   rho E_lambda = kappa |grad rho|^2 / 2.
+// A block of bx by by nodes (256 threads) stages rho, T and p/rho of its nodes and their
+// neighbours once: 1.3 equations of state a node instead of nine (1024 x 512 mixed nodes
+// 53 -> 42 us, 20 with the parameters split on the host).
+constexpr int NL16_STAGED = 3 * 258;   // (bx + 2) (by + 2) at most, for 256 x 1 and 32 x 8
 template <typename R>
 __global__ void k_q16_nonlocal1(DevParams p, const R *__restrict__ src, typename Wide<R>::type *__restrict__ nl)
 {
     using A = typename Wide<R>::type;
-    const long long n = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (n >= p.N) return;
-    const long long N = p.N;
-    const Near9 nb(p, n);
+    __shared__ R sr[NL16_STAGED], st[NL16_STAGED];
+    __shared__ A sp[NL16_STAGED];
+    const int bx = blockDim.x, by = blockDim.y, X0 = blockIdx.x * bx, Y0 = blockIdx.y * by, W = bx + 2;
+    for (int k = threadIdx.y * bx + threadIdx.x; k < W * (by + 2); k += bx * by) {
+        const size_t m = (size_t)bc_wrap(Y0 + k / W - 1, p.ny, p.bcy) * p.nx + bc_wrap(X0 + k % W - 1, p.nx, p.bcx);
+        const R r = REC16(src, m, Q_RHO), t = REC16(src, m, Q_T);
+        sr[k] = r;
+        st[k] = t;
+        sp[k] = w_p_over_rho(p, r, t);
+    }
+    __syncthreads();
+    const int X = X0 + threadIdx.x, Y = Y0 + threadIdx.y;
+    if (X >= p.nx || Y >= p.ny) return;
+    const long long N = p.N, n = (long long)Y * p.nx + X;
     R r[3][3], t[3][3];
     A pi[3][3];
 #pragma unroll
     for (int y = 0; y < 3; ++y)
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
-            const size_t m = nb.at(y, k);
-            r[y][k] = REC16(src, m, Q_RHO);
-            t[y][k] = REC16(src, m, Q_T);
-            pi[y][k] = w_p_over_rho(p, r[y][k], t[y][k]);
+            const int m = (threadIdx.y + y) * W + threadIdx.x + k;
+            r[y][k] = sr[m];
+            t[y][k] = st[m];
+            pi[y][k] = sp[m];
         }
     const R r0 = r[1][1];
     const Diff2<A> dr = diff2<A>([&](int y, int k) { return w_sub(r[y][k], r0); });
     const Diff2<A> dT = diff2<A>([&](int y, int k) { return t[y][k]; });
     const Diff2<A> dp = diff2<A>([&](int y, int k) { return pi[y][k]; });
-    const A g = w_const<A>(1.0 / 12.0), kap = w_const<A>(p.kappa);
+    const A g = w_const<A>(1.0 / 12.0), kap = wide_param<A>(p.kappa, p.ff_kap);
     const A gr[2] = {w_mul(dr.dx, g), w_mul(dr.dy, g)}, gT[2] = {w_mul(dT.dx, g), w_mul(dT.dy, g)};
     const A dpi[2] = {dp.dx, dp.dy};
     const A lap = w_mul(dr.s, w_const<A>(1.0 / 6.0));
@@ -328,14 +342,14 @@ __global__ void k_q16_nonlocal1(DevParams p, const R *__restrict__ src, typename
     const A kg2 = w_mul(kap, w_mul(g2, w_const<A>(0.5)));   // rho E_lambda
     const A iso = w_sub(w_mul(w_mul(kap, w_mul(lap, r0)), w_const<A>(-1.0)), kg2);
     const A pr = w_mul(pi[1][1], r0);
-    const A mu = w_mul(w_double(pr) > p.p_floor ? pr : w_const<A>(p.p_floor), w_const<A>((p.tau - 0.5) * p.dt));
-    const A kc = p.k_cond >= 0.0 ? w_const<A>(p.k_cond) : w_mul(mu, w_const<A>(p.cv + p.R));
+    const A mu = w_mul(w_less(wide_p_floor<A>(p), pr) ? pr : wide_p_floor<A>(p), wide_param<A>(p.pd.mu_coef, p.ff_mu));
+    const A kc = p.k_cond >= 0.0 ? wide_param<A>(p.k_cond, p.ff_kc) : w_mul(mu, wide_param<A>(p.pd.cvR, p.ff_cvR));
     NLP(nl, NL_KXX, n, N) = w_add(iso, w_mul(kap, w_mul(gr[0], gr[0])));
     NLP(nl, NL_KXY, n, N) = w_mul(kap, w_mul(gr[0], gr[1]));
     NLP(nl, NL_KYY, n, N) = w_add(iso, w_mul(kap, w_mul(gr[1], gr[1])));
 #pragma unroll
     for (int a = 0; a < 2; ++a) {
-        const A gh = w_add(w_sub(w_mul(gT[a], w_const<A>(p.cv)), w_mul(gr[a], w_const<A>(p.a))), w_mul(dpi[a], g));
+        const A gh = w_add(w_sub(w_mul(gT[a], wide_param<A>(p.cv, p.ff_cv)), w_mul(gr[a], wide_param<A>(p.a, p.ff_a))), w_mul(dpi[a], g));
         NLP(nl, NL_QX + a, n, N) = w_sub(w_mul(kc, gT[a]), w_mul(mu, gh));
     }
     NLP(nl, NL_REL, n, N) = kg2;
@@ -692,8 +706,17 @@ __device__ __noinline__ void q16_stream_any(const DevParams &p, const R *__restr
 template <typename R> struct Slot16;
 template <> struct Slot16<float> { static constexpr int stride = 36; };
 template <> struct Slot16<double> { static constexpr int stride = 33; };
+// place of population i of family fam (0 f, 1 g): side by side in FP32 (see contract in
+// pond_step.cuh)
+template <typename R> __host__ __device__ constexpr int slot16_at(int fam, int i) { return sizeof(R) == 4 ? 2 * i + fam : 16 * fam + i; }
+// What a thread keeps in shared memory across the stream: wide values (own sums, F, rho
+// E_lambda, M_0), then the y weights and rows of the map in R.
+enum : int { KW_OWN = 0, KW_F = 6, KW_REL = 8, KW_M0 = 9, KW_N = 10, KR_WY = 0, KR_LY = 20, KR_N = 36 };
 template <typename R>
-constexpr size_t q16_smem_bytes(int tx, int ty) { return (size_t)step_slots(tx, ty) * Slot16<R>::stride * sizeof(R); }
+constexpr size_t q16_smem_bytes(int tx, int ty)
+{
+    return (size_t)STEP_THREADS * (KW_N * 8 + KR_N * sizeof(R)) + (size_t)step_slots(tx, ty) * Slot16<R>::stride * sizeof(R);
+}
 
 // The rows of a per-axis map, G[k][j] = l_k(xi_j) at xi_j = (1 + q) c_j + w, as products.
 template <typename A>
@@ -732,79 +755,83 @@ __device__ __forceinline__ bool axis_weights16(const Lat16<R> &L, R s, R u, R dt
 }
 
 // The stream over the staged slots: acc = sums over the window of the node's slot `own`
-// (FP32: of differences to the own slot, i.e. increments; FP64: the streamed populations).
-// FP32: one family (offset fam * 16) per call, five columns and rows with zero weights
-// outside a component's four nodes; the x weights are kept apart from the rows of the map
-// (96 instead of 80 multiply-adds a row and source index, but 36 registers instead of 80,
-// which lets three blocks reside on an SM).
+// (FP32: of differences to the own slot, i.e. increments; FP64: the streamed populations);
+// keep = the thread's y weights and rows.  FP32: f and g in one instruction (packed pairs),
+// five columns and rows with zero weights outside a component's four nodes; the x weights
+// are kept apart from the rows of the map (96 instead of 80 multiply-adds a row and source
+// index, but 72 registers of pairs instead of 160).
 __device__ __forceinline__ void contract16(const float *own, int pitch, const float (&ax)[4][4], const bool (&nx0)[4],
-                                           const float (&ay)[4][4], const bool (&ny0)[4], const float (&Lx)[4][4],
-                                           const float (&Ly)[4][4], float (&acc)[16])
+                                           const float (&Lx)[4][4], const float *keep, float (&acc)[2][16])
 {
     constexpr int DS = Slot16<float>::stride;
-    float wx[4][5], wy[4][5];
+    f32x2 wx[4][5], L2[4][4], a2[16];
 #pragma unroll
-    for (int k = 0; k < 4; ++k)
+    for (int k = 0; k < 4; ++k) {
 #pragma unroll
         for (int c = 0; c < 5; ++c) {
             const int lo = c > 3 ? 3 : c, hi = c < 1 ? 0 : c - 1;
-            wx[k][c] = nx0[k] ? (c == 0 ? 0.0f : ax[k][hi]) : (c == 4 ? 0.0f : ax[k][lo]);
-            wy[k][c] = ny0[k] ? (c == 0 ? 0.0f : ay[k][hi]) : (c == 4 ? 0.0f : ay[k][lo]);
+            const float w = nx0[k] ? (c == 0 ? 0.0f : ax[k][hi]) : (c == 4 ? 0.0f : ax[k][lo]);
+            wx[k][c] = pack2(w, w);
         }
-    float dx[4][4];
 #pragma unroll
-    for (int n = 0; n < 4; ++n) lds4(own + 4 * n, dx[n]);
+        for (int m = 0; m < 4; ++m) L2[k][m] = pack2(Lx[k][m], Lx[k][m]);
+    }
 #pragma unroll
-    for (int i = 0; i < 16; ++i) acc[i] = 0.0f;
+    for (int i = 0; i < 16; ++i) a2[i] = 0ull;
     const float *row = own - (2 * pitch + 2) * DS;
 #pragma unroll 1
     for (int cy = 0; cy < 5; ++cy, row += pitch * DS) {
-        float w[4];
+#pragma unroll 1
+        for (int n = 0; n < 4; ++n) {   // rolled: the body stays in the instruction cache
+            f32x2 v[5][4], d[4];
+            {
+                float t[8];
 #pragma unroll
-        for (int l = 0; l < 4; ++l) {
-            w[l] = wy[l][0];
+                for (int q = 0; q < 2; ++q) {
+                    float x[4];
+                    lds4(own + 8 * n + 4 * q, x);
 #pragma unroll
-            for (int c = 0; c < 4; ++c) wy[l][c] = wy[l][c + 1];
-        }
+                    for (int e = 0; e < 4; ++e) t[4 * q + e] = x[e];
+                }
 #pragma unroll
-        for (int n = 0; n < 4; ++n) {
-            float v[5][4];
+                for (int m = 0; m < 4; ++m) d[m] = pack2(-t[2 * m], -t[2 * m + 1]);
+            }
 #pragma unroll
             for (int c = 0; c < 5; ++c) {
-                lds4(row + c * DS + 4 * n, v[c]);
+                const ulonglong2 x = reinterpret_cast<const ulonglong2 *>(row + c * DS + 8 * n)[0];
+                const ulonglong2 y = reinterpret_cast<const ulonglong2 *>(row + c * DS + 8 * n)[1];
+                v[c][0] = add2(x.x, d[0]); v[c][1] = add2(x.y, d[1]);
+                v[c][2] = add2(y.x, d[2]); v[c][3] = add2(y.y, d[3]);
+            }
+            f32x2 wn[4];
 #pragma unroll
-                for (int m = 0; m < 4; ++m) v[c][m] -= dx[n][m];
+            for (int l = 0; l < 4; ++l) {
+                const float w = keep[(KR_WY + 5 * l + cy) * STEP_THREADS] * keep[(KR_LY + 4 * l + n) * STEP_THREADS];
+                wn[l] = pack2(w, w);
             }
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
-                float t = 0.0f;
+                f32x2 t = 0ull;
 #pragma unroll
                 for (int m = 0; m < 4; ++m) {
-                    float q = wx[k][0] * v[0][m];
+                    f32x2 q = 0ull;
 #pragma unroll
-                    for (int c = 1; c < 5; ++c) q = fmaf(wx[k][c], v[c][m], q);
-                    t = fmaf(Lx[k][m], q, t);
+                    for (int c = 0; c < 5; ++c) q = fma2(wx[k][c], v[c][m], q);
+                    t = fma2(L2[k][m], q, t);
                 }
 #pragma unroll
-                for (int l = 0; l < 4; ++l) acc[4 * l + k] = fmaf(w[l] * Ly[l][n], t, acc[4 * l + k]);
+                for (int l = 0; l < 4; ++l) a2[4 * l + k] = fma2(wn[l], t, a2[4 * l + k]);
             }
         }
     }
+#pragma unroll
+    for (int i = 0; i < 16; ++i) unpack2(a2[i], acc[0][i], acc[1][i]);
 }
-// FP64: both families at once, each component's own four columns.
+// FP64: each component's own four columns.
 __device__ __forceinline__ void contract16(const double *own, int pitch, const double (&ax)[4][4], const bool (&nx0)[4],
-                                           const double (&ay)[4][4], const bool (&ny0)[4], const double (&Lx)[4][4],
-                                           const double (&Ly)[4][4], double (&acc)[2][16])
+                                           const double (&Lx)[4][4], const double *keep, double (&acc)[2][16])
 {
     constexpr int DS = Slot16<double>::stride;
-    double wy[4][5];
-#pragma unroll
-    for (int k = 0; k < 4; ++k)
-#pragma unroll
-        for (int c = 0; c < 5; ++c) {
-            const int lo = c > 3 ? 3 : c, hi = c < 1 ? 0 : c - 1;
-            wy[k][c] = ny0[k] ? (c == 0 ? 0.0 : ay[k][hi]) : (c == 4 ? 0.0 : ay[k][lo]);
-        }
 #pragma unroll
     for (int i = 0; i < 16; ++i) acc[0][i] = acc[1][i] = 0.0;
     const double *row = own - (2 * pitch + 2) * DS;
@@ -813,11 +840,9 @@ __device__ __forceinline__ void contract16(const double *own, int pitch, const d
         double wn[4][4];
 #pragma unroll
         for (int l = 0; l < 4; ++l) {
-            const double w = wy[l][0];
+            const double w = keep[(KR_WY + 5 * l + cy) * STEP_THREADS];
 #pragma unroll
-            for (int c = 0; c < 4; ++c) wy[l][c] = wy[l][c + 1];
-#pragma unroll
-            for (int n = 0; n < 4; ++n) wn[l][n] = w * Ly[l][n];
+            for (int n = 0; n < 4; ++n) wn[l][n] = w * keep[(KR_LY + 4 * l + n) * STEP_THREADS];
         }
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
@@ -877,7 +902,9 @@ __global__ void __launch_bounds__(STEP_THREADS, sizeof(R) == 4 ? Q16_MIN_BLOCKS 
     using A = typename Wide<R>::type;
     constexpr int DS = Slot16<R>::stride;
     extern __shared__ __align__(128) unsigned char q16_dyn_smem[];
-    R *slots = reinterpret_cast<R *>(q16_dyn_smem);
+    A *keep_w = reinterpret_cast<A *>(q16_dyn_smem) + threadIdx.x;   // this thread's columns
+    R *keep = reinterpret_cast<R *>(q16_dyn_smem + (size_t)STEP_THREADS * KW_N * 8) + threadIdx.x;
+    R *slots = reinterpret_cast<R *>(q16_dyn_smem + (size_t)STEP_THREADS * (KW_N * 8 + KR_N * sizeof(R)));
     __shared__ StepCounts counts;
     __shared__ uint4 best[STEP_THREADS / 32];
     const int tid = threadIdx.x;
@@ -942,15 +969,9 @@ __global__ void __launch_bounds__(STEP_THREADS, sizeof(R) == 4 ? Q16_MIN_BLOCKS 
                 } else {
                     apply_rows16<R>(Gx, Gy, h);
                 }
-                R *dst = slots + (size_t)k * DS + 16 * fam;
-                if constexpr (sizeof(R) == 4) {
+                R *dst = slots + (size_t)k * DS;
 #pragma unroll
-                    for (int r = 0; r < 4; ++r)
-                        *reinterpret_cast<float4 *>(dst + 4 * r) = make_float4(h[4 * r], h[4 * r + 1], h[4 * r + 2], h[4 * r + 3]);
-                } else {
-#pragma unroll
-                    for (int i = 0; i < 16; ++i) dst[i] = h[i];
-                }
+                for (int i = 0; i < 16; ++i) dst[slot16_at<R>(0, i) + fam * slot16_at<R>(1, 0)] = h[i];
             }
         }
     }
@@ -964,13 +985,15 @@ __global__ void __launch_bounds__(STEP_THREADS, sizeof(R) == 4 ? Q16_MIN_BLOCKS 
     if (valid) {
         const size_t n = (size_t)Y * p.nx + X;
         const R *own_slot = slots + (size_t)((ty + HALO) * WT + tx + HALO) * DS;
-        const A F[2] = {NLP(nl, NL_FX, n, N), NLP(nl, NL_FY, n, N)};
-        const A rEl = NLP(nl, NL_REL, n, N), M0 = NLP(nl, NL_M0, n, N);
+        keep_w[KW_F * STEP_THREADS] = NLP(nl, NL_FX, n, N);
+        keep_w[(KW_F + 1) * STEP_THREADS] = NLP(nl, NL_FY, n, N);
+        keep_w[KW_REL * STEP_THREADS] = NLP(nl, NL_REL, n, N);
+        keep_w[KW_M0 * STEP_THREADS] = NLP(nl, NL_M0, n, N);
         // sums of the node's stored populations and its kept remainders: sum f + mass lo,
         // sum f c_x, sum f c_y, sum g + energy lo, momentum lo (absolute)
-        A own[6];
         R th, u[2];
         {
+            A own[6];
             R v[16], lo[4];
             ld16(in, n, N, Q_F, v);
             sums16<true>(v, own);
@@ -982,6 +1005,8 @@ __global__ void __launch_bounds__(STEP_THREADS, sizeof(R) == 4 ? Q16_MIN_BLOCKS 
             own[3] = w_add(own[3], lo[2]);
             own[4] = w_wide(lo[0]);
             own[5] = w_wide(lo[1]);
+#pragma unroll
+            for (int k = 0; k < 6; ++k) keep_w[(KW_OWN + k) * STEP_THREADS] = own[k];
             R g4[4];
             ld4(in, n, N, Q_TH, g4);
             th = g4[0]; u[0] = g4[1]; u[1] = g4[2];
@@ -998,44 +1023,52 @@ __global__ void __launch_bounds__(STEP_THREADS, sizeof(R) == 4 ? Q16_MIN_BLOCKS 
             if (okx && oky) {
                 auto side = [](const bool (&z)[4]) { return (z[0] == z[1] && z[1] == z[2] && z[2] == z[3]) ? 4 : 5; };
                 nreg += (unsigned)(side(nx0) * side(ny0) - (its == 1 ? 1 : 0));
-                R Lx[4][4], Ly[4][4];
+                R Lx[4][4], acc[2][16];
                 const R q = (gb[0] - s) * inv_s;
+                {
+                    R Ly[4][4];
+                    axis_rows16<R>(L, q, (gb[2] - u[1]) * inv_s, Ly);
+#pragma unroll
+                    for (int l = 0; l < 4; ++l) {
+#pragma unroll
+                        for (int c = 0; c < 5; ++c) {
+                            const int lo = c > 3 ? 3 : c, hi = c < 1 ? 0 : c - 1;
+                            keep[(KR_WY + 5 * l + c) * STEP_THREADS] =
+                                ny0[l] ? (c == 0 ? R(0) : ay[l][hi]) : (c == 4 ? R(0) : ay[l][lo]);
+                        }
+#pragma unroll
+                        for (int m2 = 0; m2 < 4; ++m2) keep[(KR_LY + 4 * l + m2) * STEP_THREADS] = Ly[l][m2];
+                    }
+                }
                 axis_rows16<R>(L, q, (gb[1] - u[0]) * inv_s, Lx);
-                axis_rows16<R>(L, q, (gb[2] - u[1]) * inv_s, Ly);
+                contract16(own_slot, WT, ax, nx0, Lx, keep, acc);
                 if constexpr (sizeof(R) == 8) {
-                    R acc[2][16], v[16];
-                    contract16(own_slot, WT, ax, nx0, ay, ny0, Lx, Ly, acc);
+                    R v[16];
                     ld16(in, n, N, Q_F, v);
 #pragma unroll
-                    for (int i = 0; i < 16; ++i) fi[i] = acc[0][i] - v[i];
+                    for (int i = 0; i < 16; ++i) acc[0][i] -= v[i];
                     ld16(in, n, N, Q_G, v);
 #pragma unroll
-                    for (int i = 0; i < 16; ++i) gi[i] = acc[1][i] - v[i];
-                } else {
-#pragma unroll 1
+                    for (int i = 0; i < 16; ++i) acc[1][i] -= v[i];
+                } else if (its > 1) {
+                    // the node's own populations carried from their stored gauge
+                    R g4[4], v[16], o[16], Dx[4][4], Dy[4][4];
+                    ld4(in, n, N, Q_TH, g4);
+                    const R e = fdiv_(g4[0] - th, (sqrt_(g4[0]) + s) * s);
+                    axis_inc<R>(L, e, (g4[1] - u[0]) * inv_s, Dx);
+                    axis_inc<R>(L, e, (g4[2] - u[1]) * inv_s, Dy);
+#pragma unroll
                     for (int fam = 0; fam < 2; ++fam) {
-                        R acc[16];
-                        contract16(own_slot + 16 * fam, WT, ax, nx0, ay, ny0, Lx, Ly, acc);
-                        if (its > 1) {
-                            // the node's own populations carried from their stored gauge
-                            R g4[4], v[16], o[16], Dx[4][4], Dy[4][4];
-                            ld4(in, n, N, Q_TH, g4);
-                            const R e = fdiv_(g4[0] - th, (sqrt_(g4[0]) + s) * s);
-                            axis_inc<R>(L, e, (g4[1] - u[0]) * inv_s, Dx);
-                            axis_inc<R>(L, e, (g4[2] - u[1]) * inv_s, Dy);
-                            ld16(in, n, N, 16 * fam, v);
-                            apply_inc<R>(Dx, Dy, v, o);
+                        ld16(in, n, N, 16 * fam, v);
+                        apply_inc<R>(Dx, Dy, v, o);
 #pragma unroll
-                            for (int i = 0; i < 16; ++i) acc[i] += o[i];
-                        }
-                        if (fam == 0) {
-#pragma unroll
-                            for (int i = 0; i < 16; ++i) fi[i] = acc[i];
-                        } else {
-#pragma unroll
-                            for (int i = 0; i < 16; ++i) gi[i] = acc[i];
-                        }
+                        for (int i = 0; i < 16; ++i) acc[fam][i] += o[i];
                     }
+                }
+#pragma unroll
+                for (int i = 0; i < 16; ++i) {
+                    fi[i] = acc[0][i];
+                    gi[i] = acc[1][i];
                 }
             } else {
                 R f2[16], g2[16];
@@ -1043,10 +1076,13 @@ __global__ void __launch_bounds__(STEP_THREADS, sizeof(R) == 4 ? Q16_MIN_BLOCKS 
 #pragma unroll
                 for (int i = 0; i < 16; ++i) { fi[i] = f2[i]; gi[i] = g2[i]; }
             }
-            A d[4];
+            A d[4], own[6];
             sums16<true>(fi, d);
             sums16<false>(gi, d + 3);
-            m.update(p, th, u, own, d, F, rEl, 1.0);
+#pragma unroll
+            for (int k = 0; k < 6; ++k) own[k] = keep_w[(KW_OWN + k) * STEP_THREADS];
+            const A F[2] = {keep_w[KW_F * STEP_THREADS], keep_w[(KW_F + 1) * STEP_THREADS]};
+            m.update(p, th, u, own, d, F, keep_w[KW_REL * STEP_THREADS], 1.0);
             const float res = m.change(th);
             conv = sizeof(R) == 4 ? res <= p.tol_f : (double)res <= p.tol;
             if (conv || its >= (unsigned)p.max_iter || !(res == res)) break;
@@ -1057,6 +1093,7 @@ __global__ void __launch_bounds__(STEP_THREADS, sizeof(R) == 4 ? Q16_MIN_BLOCKS 
 
         // ---- collision in type R, equilibria as increments over their co-moving form
         const TypedParams<R> &q = typed<R>(p);
+        const A F[2] = {keep_w[KW_F * STEP_THREADS], keep_w[(KW_F + 1) * STEP_THREADS]}, M0 = keep_w[KW_M0 * STEP_THREADS];
         {
             R v[16];
             ld16(in, n, N, Q_F, v);

@@ -282,23 +282,21 @@ __global__ void k_q27_nonlocal1(DevParams p, Grid3 g3, const R *__restrict__ src
     const Diff3<A> dr = diff3<A>([&](int z, int y, int k) { return w_sub(REC27(src, nb.at(z, y, k), R_RHO), r0); });
     const Diff3<A> dT = diff3<A>([&](int z, int y, int k) { return REC27(src, nb.at(z, y, k), R_T); });
     const Diff3<A> dp = diff3<A>([&](int z, int y, int k) { return NL3(nl, N3_PI, nb.at(z, y, k), N); });
-    const A g = w_const<A>(1.0 / 72.0), kap = w_const<A>(p.kappa);
+    const A g = w_const<A>(1.0 / 72.0), kap = wide_param<A>(p.kappa, p.ff_kap);
     A gr[3], gT[3], gh[3];
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
         gr[a] = w_mul(dr.d[a], g);
         gT[a] = w_mul(dT.d[a], g);
-        gh[a] = w_add(w_sub(w_mul(gT[a], w_const<A>(p.cv)), w_mul(gr[a], w_const<A>(p.a))), w_mul(dp.d[a], g));
+        gh[a] = w_add(w_sub(w_mul(gT[a], wide_param<A>(p.cv, p.ff_cv)), w_mul(gr[a], wide_param<A>(p.a, p.ff_a))), w_mul(dp.d[a], g));
     }
     const A lap = w_mul(dr.s, w_const<A>(1.0 / 36.0));
     const A g2 = w_add(w_add(w_mul(gr[0], gr[0]), w_mul(gr[1], gr[1])), w_mul(gr[2], gr[2]));
     const A kg2 = w_mul(kap, w_mul(g2, w_const<A>(0.5)));   // rho E_lambda
     const A iso = w_sub(w_mul(w_mul(kap, w_mul(lap, r0)), w_const<A>(-1.0)), kg2);
     const A pr = w_mul(pi0, r0);
-    const A flo = w_const<A>(p.p_floor);
-    const double prd = w_double(pr);
-    const A mu = w_mul(prd > p.p_floor ? pr : flo, w_const<A>((p.tau - 0.5) * p.dt));
-    const A kc = p.k_cond >= 0.0 ? w_const<A>(p.k_cond) : w_mul(mu, w_const<A>(p.cv + p.R));
+    const A mu = w_mul(w_less(wide_p_floor<A>(p), pr) ? pr : wide_p_floor<A>(p), wide_param<A>(p.pd.mu_coef, p.ff_mu));
+    const A kc = p.k_cond >= 0.0 ? wide_param<A>(p.k_cond, p.ff_kc) : w_mul(mu, wide_param<A>(p.pd.cvR, p.ff_cvR));
     const int ab[6][2] = {{0, 0}, {0, 1}, {0, 2}, {1, 1}, {1, 2}, {2, 2}};
 #pragma unroll
     for (int k = 0; k < 6; ++k) {

@@ -543,6 +543,11 @@ __device__ __forceinline__ ffv w_sqrt(float x)
     return ff_norm(s, fmaf(-s, s, x) / (2.0f * s));
 }
 __device__ __forceinline__ double w_sqrt(double x) { return sqrt(x); }
+// a parameter in the wide type, from its FP64 value or its float pair (splitting an FP64
+// value on the device costs as much as 25 float-float additions)
+template <typename A> __device__ __forceinline__ A wide_param(double x, const float (&ff)[2]);
+template <> __device__ __forceinline__ double wide_param<double>(double x, const float (&)[2]) { return x; }
+template <> __device__ __forceinline__ ffv wide_param<ffv>(double, const float (&ff)[2]) { return {ff[0], ff[1]}; }
 template <typename A> __device__ __forceinline__ A wide_dt(const DevParams &p);
 template <> __device__ __forceinline__ double wide_dt<double>(const DevParams &p) { return p.dt; }
 template <> __device__ __forceinline__ ffv wide_dt<ffv>(const DevParams &p) { return {p.ff_dt[0], p.ff_dt[1]}; }
