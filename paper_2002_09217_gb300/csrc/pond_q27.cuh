@@ -27,18 +27,17 @@
 // combine the cubic Lagrange weights and the rows of the map into the arrival gauge: 12,500
 // multiply-adds a population family, where carrying each of 125 nodes into the arrival
 // gauge and spreading it over 27 directions took about 45,000.  One family at a time is
-// staged (86 KB in FP32, two blocks per SM; 166 KB in FP64, one block); a further stream
-// of the frame search starts with the family that is already staged.  The sums of
-// populations and the non-local terms are float-float in the FP32 form, and products of
-// one reciprocal replace quotients.
-// Measured: two mixed steps of a 96 x 96 x 64 droplet (with init and read-out) 29.3 -> 8.2
-// ms; two FP64 steps of 33 x 29 x 21 nodes 152 -> 21 ms; ten mixed steps of 9 x 8 x 7 nodes
-// 36.9 -> 11.5 ms.  The mixed step issues on 45 % of its cycles (FMA pipe 39 %): with two
-// warps per scheduler, the shared-memory reads' latency shows.
+// staged (two blocks per SM in FP32, one in FP64, by shared memory); a further stream of
+// the frame search starts with the family that is already staged.  The sums of populations,
+// the moments, the EoS and the non-local terms are float-float in the FP32 form.
+// Measured: two mixed steps of a 96 x 96 x 64 droplet (with init and read-out) 29.3 -> 6.1
+// ms, two FP64 steps of 33 x 29 x 21 nodes 152 -> 21 ms.  With two warps per scheduler the
+// shared-memory latency decides: a row's slots are replaced by the next row's as they are
+// used (3.78 -> 2.88 ms a step; issue 41 -> 53 %, FMA pipe 53 % busy).
 #pragma once
 
 #include "pond_kernels.cuh"
-#include "pond_step.cuh"   // float-float values, map helpers
+#include "pond_step.cuh"   // float-float and wide values, map helpers
 
 namespace pond {
 
@@ -448,31 +447,6 @@ __device__ __forceinline__ void axis3(A ds, A du, A D[3][3])
     }
 }
 
-// increment of (I + Dz)(I + Dy)(I + Dx) applied to h (27 values)
-template <typename A>
-__device__ __forceinline__ void apply3_inc(const A Dx[3][3], const A Dy[3][3], const A Dz[3][3], const A *h,
-                                           A *out)
-{
-    A t1[27], t2[27];
-#pragma unroll
-    for (int i = 0; i < 27; ++i) {
-        const int ix = i % 3, r = i - ix;
-        t1[i] = Dx[ix][0] * h[r] + Dx[ix][1] * h[r + 1] + Dx[ix][2] * h[r + 2];
-    }
-#pragma unroll
-    for (int i = 0; i < 27; ++i) {
-        const int iy = (i / 3) % 3, r = i - 3 * iy;
-        t2[i] = Dy[iy][0] * (h[r] + t1[r]) + Dy[iy][1] * (h[r + 3] + t1[r + 3]) + Dy[iy][2] * (h[r + 6] + t1[r + 6]);
-    }
-#pragma unroll
-    for (int i = 0; i < 27; ++i) {
-        const int iz = i / 9, r = i - 9 * iz;
-        const A z = Dz[iz][0] * (h[r] + t1[r] + t2[r]) + Dz[iz][1] * (h[r + 9] + t1[r + 9] + t2[r + 9]) +
-                    Dz[iz][2] * (h[r + 18] + t1[r + 18] + t2[r + 18]);
-        out[i] = t1[i] + t2[i] + z;
-    }
-}
-
 // ---------------------------------------------------------------------------
 // General stream, for departure points beyond the staged halo (|v| dt >= 1) and non-finite
 // gauges: reads the stencil nodes' records from global memory.  On the tensor lattice the union of a node's 27 departure stencils
@@ -663,9 +637,9 @@ __device__ __noinline__ void q27_stream_any(const DevParams &p, const Grid3 &g3,
 // ---------------------------------------------------------------------------
 // Sums of 27 values v and their first moments: out = sum v, sum v c_x, sum v c_y, sum v c_z
 // (the last three with MOM).  Lines, planes, then the column; FP32 values in float-float
-// (exact up to ~2^-48), returned as doubles.
+// (exact up to ~2^-48).
 template <bool MOM>
-__device__ __forceinline__ void sums27(const float *v, double *out)
+__device__ __forceinline__ void sums27(const float *v, ffv *out)
 {
     ffv S = {0.f, 0.f}, D = S, Y = S, S0 = S, S2 = S;
 #pragma unroll
@@ -692,11 +666,11 @@ __device__ __forceinline__ void sums27(const float *v, double *out)
             if (z == 2) S2 = pS;
         }
     }
-    out[0] = w_double(S);
+    out[0] = S;
     if (MOM) {
-        out[1] = w_double(D);
-        out[2] = w_double(Y);
-        out[3] = w_double(ff_add(S2, ff_neg(S0)));
+        out[1] = D;
+        out[2] = Y;
+        out[3] = ff_add(S2, ff_neg(S0));
     }
 }
 template <bool MOM>
@@ -732,31 +706,6 @@ __device__ __forceinline__ void sums27(const double *v, double *out)
     }
 }
 
-// Macroscopic fields from the sums of the streamed populations (own + increments, momentum
-// in gauge units), FP64: out = rho, u (3), uhat (3), E, e, T, p, P, theta* (13 values).
-__device__ __forceinline__ void q27_macro(const DevParams &p, double s, const double (&u)[3], const double (&own)[8],
-                                          const double (&d)[5], const double (&F)[3], double rEl, double out[13])
-{
-    const double rho = own[0] + d[0], irho = rcp_d(rho);
-    double uu[3], uh[3];
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        const double j = s * (own[1 + a] + d[1 + a]) + u[a] * rho + own[5 + a];
-        uu[a] = j * irho;
-        uh[a] = uu[a] + (0.5 * p.dt) * F[a] * irho;
-    }
-    const double E = 0.5 * (own[4] + d[4]) * irho;
-    const double e = E - 0.5 * (uh[0] * uh[0] + uh[1] * uh[1] + uh[2] * uh[2]) - rEl * irho;
-    const double T = p.isothermal ? p.T_iso : (e + p.a * rho) * p.pd.inv_cv;
-    const double pr = p.eos_kind == 0 ? rho * p.R * T * rcp_d(1.0 - p.b * rho) - p.a * rho * rho
-                                      : eos_pressure<double>(p.eos_kind, p.a, p.b, p.R, rho, T, p.sp);
-    const double P = pr > p.p_floor ? pr : p.p_floor;
-    out[0] = rho;
-#pragma unroll
-    for (int a = 0; a < 3; ++a) { out[1 + a] = uu[a]; out[4 + a] = uh[a]; }
-    out[7] = E; out[8] = e; out[9] = T; out[10] = pr; out[11] = P; out[12] = P * irho * 3.0;
-}
-
 // increment of (I + Dz)(I + Dy)(I + Dx) applied to h (27 values)
 template <typename A>
 __device__ __forceinline__ void apply3_inc(const A (&Dx)[3][3], const A (&Dy)[3][3], const A (&Dz)[3][3], const A *h,
@@ -787,23 +736,28 @@ __device__ __forceinline__ void apply3_inc(const A (&Dx)[3][3], const A (&Dy)[3]
 constexpr int Q27_THREADS = STEP_THREADS, T27X = 8, T27Y = 4, T27Z = 4, HALO27 = 2;
 constexpr int S27X = T27X + 2 * HALO27, S27Y = T27Y + 2 * HALO27, S27Z = T27Z + 2 * HALO27;
 constexpr int SLOTS27 = S27X * S27Y * S27Z;
-constexpr int PY27 = S27X, PZ27 = S27X * S27Y;   // slots per row, per plane
-// values per slot: 27, padded to 28 words for 16-byte loads in FP32 (eight consecutive
-// slots then start on distinct groups of four banks)
+constexpr int PY27 = S27X, PZ27 = S27X * S27Y + 8;   // slots per row, per plane (padded: the two planes
+                                                     // a half warp reads start 16 banks apart)
+constexpr int SLOT_SPACE27 = PZ27 * S27Z;
+__host__ __device__ constexpr int slot27(int k) { return k + 8 * (k / (S27X * S27Y)); }   // place of staged node k
+// Values per slot.  FP32: ten words for each source plane p: the pairs (n = 0, 1) of m = 0,
+// 1, 2, then the three values of n = 2, then a pad (8-byte loads; sixteen consecutive slots
+// fall on distinct pairs of banks).  FP64: 27 values.
 template <typename R> struct Slot27;
-template <> struct Slot27<float> { static constexpr int stride = 28; };
+template <> struct Slot27<float> { static constexpr int stride = 30; };
 template <> struct Slot27<double> { static constexpr int stride = 27; };
-constexpr int OWN27 = 13;   // FP64 values kept per node: own sums (8), F (3), rho E_lambda, M_0
+// What a thread keeps in shared memory across the FP32 stream: y weights and rows.
+enum : int { K27_WY = 0, K27_LY = 15, K27_N = 24 };
 template <typename R>
 constexpr size_t q27_smem_bytes()
 {
-    return (size_t)OWN27 * Q27_THREADS * 8 + (size_t)SLOTS27 * Slot27<R>::stride * sizeof(R);
+    return (size_t)SLOT_SPACE27 * Slot27<R>::stride * sizeof(R) + (sizeof(R) == 4 ? (size_t)K27_N * Q27_THREADS * sizeof(R) : 0);
 }
 
 struct Tile27 { int X0, Y0, Z0; };
 __device__ __forceinline__ size_t slot_node27(const DevParams &p, const Grid3 &g3, const Tile27 &t, int k)
 {
-    const int x = k % S27X, y = (k / S27X) % S27Y, z = k / PZ27;
+    const int x = k % S27X, y = (k / S27X) % S27Y, z = k / (S27X * S27Y);
     return (size_t)node27(p, g3, t.X0 - HALO27 + x, t.Y0 - HALO27 + y, t.Z0 - HALO27 + z);
 }
 
@@ -854,12 +808,17 @@ __device__ __forceinline__ void stage27(const DevParams &p, const Grid3 &g3, con
             apply_axis27<3>(D[1], h);
             apply_axis27<9>(D[2], h);
         }
-        R *dst = slots + (size_t)k * DS;
+        R *dst = slots + (size_t)slot27(k) * DS;
         if constexpr (sizeof(R) == 4) {
+            f32x2 *d2 = reinterpret_cast<f32x2 *>(dst);
 #pragma unroll
-            for (int c = 0; c < DS / 4; ++c)
-                reinterpret_cast<float4 *>(dst)[c] =
-                    make_float4(h[4 * c], h[4 * c + 1], h[4 * c + 2], 4 * c + 3 < 27 ? h[4 * c + 3 < 27 ? 4 * c + 3 : 0] : 0.0f);
+            for (int q = 0; q < 3; ++q) {
+                const R *hp = h + 9 * q;
+#pragma unroll
+                for (int m = 0; m < 3; ++m) d2[5 * q + m] = pack2(hp[m], hp[3 + m]);
+                d2[5 * q + 3] = pack2(hp[6], hp[7]);
+                d2[5 * q + 4] = pack2(hp[8], 0.0f);
+            }
         } else {
 #pragma unroll
             for (int i = 0; i < 27; ++i) dst[i] = h[i];
@@ -872,98 +831,114 @@ __device__ __forceinline__ void stage27(const DevParams &p, const Grid3 &g3, con
 // L = the rows of the map from the tile's gauge.  FP32: five columns, rows and planes with
 // zero weights outside a component's four nodes, and differences to the node's own slot
 // (see the head of pond_step.cuh).
+// One source plane p at a time, so that the accumulators and a row's five slots fit the
+// registers and the loads of a row go out together; n = 0 and 1 share packed instructions.
 __device__ __forceinline__ void contract27(const float *own, const float (&a)[3][3][4], const bool (&near0)[3][3],
-                                           const float (&L)[3][3][3], float (&acc)[27])
+                                           const float (&L)[3][3][3], float *keep, float (&acc)[27])
 {
     constexpr int DS = Slot27<float>::stride;
-    float wl[3][5][3], wy[3][5], wz[3][5];
+    f32x2 wl[3][5][3];
+    float wz[3][5];
 #pragma unroll
     for (int k = 0; k < 3; ++k)
 #pragma unroll
         for (int c = 0; c < 5; ++c) {
             const int lo = c > 3 ? 3 : c, hi = c < 1 ? 0 : c - 1;
             const float w = near0[0][k] ? (c == 0 ? 0.0f : a[0][k][hi]) : (c == 4 ? 0.0f : a[0][k][lo]);
-            wy[k][c] = near0[1][k] ? (c == 0 ? 0.0f : a[1][k][hi]) : (c == 4 ? 0.0f : a[1][k][lo]);
+            keep[(K27_WY + 5 * k + c) * Q27_THREADS] = near0[1][k] ? (c == 0 ? 0.0f : a[1][k][hi]) : (c == 4 ? 0.0f : a[1][k][lo]);
             wz[k][c] = near0[2][k] ? (c == 0 ? 0.0f : a[2][k][hi]) : (c == 4 ? 0.0f : a[2][k][lo]);
 #pragma unroll
-            for (int m = 0; m < 3; ++m) wl[k][c][m] = w * L[0][k][m];
+            for (int m = 0; m < 3; ++m) wl[k][c][m] = pack2(w * L[0][k][m], w * L[0][k][m]);
         }
-    float dx[DS];
 #pragma unroll
-    for (int c = 0; c < DS / 4; ++c) {
-        float x[4];
-        lds4(own + 4 * c, x);
-#pragma unroll
-        for (int e = 0; e < 4; ++e) dx[4 * c + e] = x[e];
-    }
+    for (int i = 0; i < 9; ++i) keep[(K27_LY + i) * Q27_THREADS] = L[1][i / 3][i % 3];
 #pragma unroll
     for (int i = 0; i < 27; ++i) acc[i] = 0.0f;
     const float *plane = own - (2 * PZ27 + 2 * PY27 + 2) * DS;
 #pragma unroll 1
     for (int cz = 0; cz < 5; ++cz, plane += PZ27 * DS) {
-        float b[3][9];   // p; 3 l + k
-#pragma unroll
-        for (int q = 0; q < 3; ++q)
-#pragma unroll
-            for (int i = 0; i < 9; ++i) b[q][i] = 0.0f;
-        const float *row = plane;
 #pragma unroll 1
-        for (int cy = 0; cy < 5; ++cy, row += PY27 * DS) {
-            float t[9][3];   // 3 p + n; k
+        for (int q = 0; q < 3; ++q) {
+            const f32x2 *op = reinterpret_cast<const f32x2 *>(own) + 5 * q;
+            f32x2 dp[3], b2[9];   // b: 3 l + k, the shares of n = 0, 1 apart
+            float ds[3], b1[9];   // n = 2
+            {
+                float x, y;
 #pragma unroll
-            for (int q = 0; q < 9; ++q)
-#pragma unroll
-                for (int k = 0; k < 3; ++k) t[q][k] = 0.0f;
-#pragma unroll
-            for (int cx = 0; cx < 5; ++cx) {
-                float v[DS];
-#pragma unroll
-                for (int c = 0; c < DS / 4; ++c) {
-                    float x[4];
-                    lds4(row + cx * DS + 4 * c, x);
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) v[4 * c + e] = x[e] - dx[4 * c + e];
+                for (int m = 0; m < 3; ++m) {
+                    unpack2(op[m], x, y);
+                    dp[m] = pack2(-x, -y);
                 }
-#pragma unroll
-                for (int q = 0; q < 9; ++q)
-#pragma unroll
-                    for (int m = 0; m < 3; ++m)
-#pragma unroll
-                        for (int k = 0; k < 3; ++k) t[q][k] = fmaf(wl[k][cx][m], v[3 * q + m], t[q][k]);
+                unpack2(op[3], ds[0], ds[1]);
+                unpack2(op[4], ds[2], y);
             }
 #pragma unroll
-            for (int l = 0; l < 3; ++l) {
-                const float w = wy[l][0];
+            for (int i = 0; i < 9; ++i) { b2[i] = 0ull; b1[i] = 0.0f; }
+            const f32x2 *row = reinterpret_cast<const f32x2 *>(plane) + 5 * q;
+            f32x2 v[5][5];   // the row's slots; each is replaced by the next row's once it is used
 #pragma unroll
-                for (int c = 0; c < 4; ++c) wy[l][c] = wy[l][c + 1];
-                wy[l][4] = w;   // rotate: the weights are needed again in the next plane
+            for (int cx = 0; cx < 5; ++cx)
 #pragma unroll
-                for (int n = 0; n < 3; ++n) {
-                    const float wn = w * L[1][l][n];
+                for (int e = 0; e < 5; ++e) v[cx][e] = row[cx * (DS / 2) + e];
+#pragma unroll 1
+            for (int cy = 0; cy < 5; ++cy) {
+                f32x2 tp[3] = {0ull, 0ull, 0ull};
+                float ts[3] = {0.0f, 0.0f, 0.0f};
+                if (cy < 4) row += PY27 * (DS / 2);   // (the last row loads itself again)
 #pragma unroll
-                    for (int q = 0; q < 3; ++q)
+                for (int cx = 0; cx < 5; ++cx) {
+                    float x[3], pad;
+                    unpack2(v[cx][3], x[0], x[1]);
+                    unpack2(v[cx][4], x[2], pad);
 #pragma unroll
-                        for (int k = 0; k < 3; ++k) b[q][3 * l + k] = fmaf(wn, t[3 * q + n][k], b[q][3 * l + k]);
+                    for (int m = 0; m < 3; ++m) {
+                        const f32x2 vp = add2(v[cx][m], dp[m]);
+                        const float vs = x[m] - ds[m];
+#pragma unroll
+                        for (int k = 0; k < 3; ++k) {
+                            float w, w_;
+                            unpack2(wl[k][cx][m], w, w_);
+                            tp[k] = fma2(wl[k][cx][m], vp, tp[k]);
+                            ts[k] = fmaf(w, vs, ts[k]);
+                        }
+                    }
+#pragma unroll
+                    for (int e = 0; e < 5; ++e) v[cx][e] = row[cx * (DS / 2) + e];
                 }
+#pragma unroll
+                for (int l = 0; l < 3; ++l) {
+                    const float w = keep[(K27_WY + 5 * l + cy) * Q27_THREADS];
+                    const f32x2 wp = pack2(w * keep[(K27_LY + 3 * l) * Q27_THREADS], w * keep[(K27_LY + 3 * l + 1) * Q27_THREADS]);
+                    const float ws = w * keep[(K27_LY + 3 * l + 2) * Q27_THREADS];
+#pragma unroll
+                    for (int k = 0; k < 3; ++k) {
+                        b2[3 * l + k] = fma2(wp, tp[k], b2[3 * l + k]);
+                        b1[3 * l + k] = fmaf(ws, ts[k], b1[3 * l + k]);
+                    }
+                }
+            }
+#pragma unroll
+            for (int i = 0; i < 9; ++i) {
+                float x, y;
+                unpack2(b2[i], x, y);
+                b1[i] += x + y;
+            }
+#pragma unroll
+            for (int r = 0; r < 3; ++r) {
+                const float w = wz[r][0] * sel3(q, L[2][r][0], L[2][r][1], L[2][r][2]);
+#pragma unroll
+                for (int i = 0; i < 9; ++i) acc[9 * r + i] = fmaf(w, b1[i], acc[9 * r + i]);
             }
         }
 #pragma unroll
-        for (int r = 0; r < 3; ++r) {
-            const float w = wz[r][0];
+        for (int r = 0; r < 3; ++r)
 #pragma unroll
-            for (int c = 0; c < 4; ++c) wz[r][c] = wz[r][c + 1];
-#pragma unroll
-            for (int q = 0; q < 3; ++q) {
-                const float wn = w * L[2][r][q];
-#pragma unroll
-                for (int i = 0; i < 9; ++i) acc[9 * r + i] = fmaf(wn, b[q][i], acc[9 * r + i]);
-            }
-        }
+            for (int c = 0; c < 4; ++c) wz[r][c] = wz[r][c + 1];   // the next plane's weight moves to the front
     }
 }
 // FP64: each component's own four columns; acc = streamed populations.
 __device__ __forceinline__ void contract27(const double *own, const double (&a)[3][3][4], const bool (&near0)[3][3],
-                                           const double (&L)[3][3][3], double (&acc)[27])
+                                           const double (&L)[3][3][3], double *, double (&acc)[27])
 {
     constexpr int DS = Slot27<double>::stride;
     double wl[3][4][3], wy[3][5], wz[3][5];
@@ -1036,28 +1011,30 @@ __device__ __forceinline__ void contract27(const double *own, const double (&a)[
 
 // ---------------------------------------------------------------------------
 // Collision of one node in type R, equilibria as increments over their co-moving form
-// (ft, gt = streamed populations, mac = the last corrector's fields, th, u = the streaming
+// (ft, gt = streamed populations, mc = the last corrector's fields, th, u = the streaming
 // gauge); writes the record.  Returns whether the results are finite.
 template <typename R>
 __device__ __forceinline__ bool q27_collide(const DevParams &p, R *__restrict__ out, size_t n, R th, const R (&u)[3],
-                                            const double (&mac)[13], const double (&F)[3], double M0, R (&ft)[27],
-                                            R (&gt)[27])
+                                            const Macro<3, R> &mc, const typename Wide<R>::type (&F)[3],
+                                            typename Wide<R>::type M0, R (&ft)[27], R (&gt)[27])
 {
+    using A = typename Wide<R>::type;
     const size_t N = (size_t)p.N;
     const TypedParams<R> &q = typed<R>(p);
-    const R rho = (R)mac[0], E = (R)mac[7], Pg = (R)mac[11];
-    const R uu[3] = {(R)mac[1], (R)mac[2], (R)mac[3]}, uh[3] = {(R)mac[4], (R)mac[5], (R)mac[6]};
-    const R f3[3] = {(R)F[0], (R)F[1], (R)F[2]}, m0 = (R)M0, dt = q.dt, om = q.omega;
-    const double sd = sqrt((double)th), ssd = sqrt(mac[12]), isd = rcp_d(sd);
-    const R is = (R)isd, sst = (R)ssd;
-    const R ds = (R)((mac[12] - (double)th) * rcp_d(ssd + sd) * isd);
+    const R rho = w_round(mc.rho), E = w_round(mc.E), Pg = w_round(mc.P);
+    const R uu[3] = {w_round(mc.uu[0]), w_round(mc.uu[1]), w_round(mc.uu[2])};
+    const R uh[3] = {w_round(mc.uh[0]), w_round(mc.uh[1]), w_round(mc.uh[2])};
+    const R f3[3] = {w_round(F[0]), w_round(F[1]), w_round(F[2])}, m0 = w_round(M0), dt = q.dt, om = q.omega;
+    const A sA = w_sqrt(th);
+    const R s = w_round(sA), is = R(1) / s, sst = sqrt_(w_round(mc.ths));
+    const R ds = fdiv_(mc.dth, (sst + s) * s);             // (s* - s)/s
     const R irho = R(1) / rho, ihP = R(1) / (R(2) * Pg);   // 1/rho, 1/(2P)
     R D[3][3][3], h[Q27], inc[Q27], fo[Q27];
     {
         R Es[3][3][3], shi[Q27];
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
-            const R du = (R)(mac[1 + a] - (double)u[a]) * is;
+            const R du = w_round(mc.du[a]) * is;
             axis3<R>(ds, du, D[a]);
             axis3<R>(ds, du + f3[a] * dt * irho * is, Es[a]);
         }
@@ -1069,29 +1046,27 @@ __device__ __forceinline__ bool q27_collide(const DevParams &p, R *__restrict__ 
         for (int i = 0; i < Q27; ++i) fo[i] = ft[i] + om * ((h[i] - ft[i]) + inc[i]) + (shi[i] - inc[i]);
     }
     bool finite = inc[0] - inc[0] == R(0);
-    double sm[4];
+    A sm[4];
     sums27<true>(fo, sm);
-    // mass and momentum defects (sum f = rho, sum f v = rho u + F dt exactly), spread by
-    // W_i and W_i c_i / (s T_L)
-    const double mdef = mac[0] - sm[0];
-    double jex[3];   // the exact momentum rho u + F dt
+    // mass and momentum defects (sum f = rho, sum f (v - u) = rho (u* - u) + F dt exactly),
+    // spread by W_i and W_i c_i / (s T_L)
+    const R mdef = w_round(w_sub(mc.rho, sm[0]));
+    A jex[3];
     R jd[3];
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-        jex[a] = mac[0] * mac[1 + a] + F[a] * p.dt;
-        const double jst = sd * sm[1 + a] + (double)u[a] * sm[0];
-        jd[a] = (R)((jex[a] - jst - mdef * (double)u[a]) * (isd * 3.0));
+        jex[a] = w_add(w_mul(mc.rho, mc.du[a]), w_mul(F[a], wide_dt<A>(p)));
+        jd[a] = w_round(w_sub(jex[a], w_mul(sA, sm[1 + a]))) * (is * R(3));
     }
 #pragma unroll
     for (int i = 0; i < Q27; ++i)
-        fo[i] += (R)w27(i) * ((R)mdef + jd[0] * R(i % 3 - 1) + jd[1] * R((i / 3) % 3 - 1) + jd[2] * R(i / 9 - 1));
-    double mlo = 0.0, jlo[3] = {0, 0, 0};
-    if (sizeof(R) == 4) {
+        fo[i] += (R)w27(i) * (mdef + jd[0] * R(i % 3 - 1) + jd[1] * R((i / 3) % 3 - 1) + jd[2] * R(i / 9 - 1));
+    R mlo = R(0), jlo[3] = {R(0), R(0), R(0)};
+    if constexpr (sizeof(R) == 4) {
         sums27<true>(fo, sm);
-        mlo = mac[0] - sm[0];
+        mlo = w_round(w_sub(mc.rho, sm[0]));
 #pragma unroll
-        for (int a = 0; a < 3; ++a)
-            jlo[a] = jex[a] - (sd * sm[1 + a] + (double)u[a] * sm[0]) - mlo * (double)u[a];
+        for (int a = 0; a < 3; ++a) jlo[a] = w_round(w_sub(jex[a], w_mul(sA, sm[1 + a])));
     }
 
     const R Prh = Pg * irho, H = E + Prh;
@@ -1129,16 +1104,18 @@ __device__ __forceinline__ bool q27_collide(const DevParams &p, R *__restrict__ 
     finite = finite && inc[0] - inc[0] == R(0);
 #pragma unroll
     for (int i = 0; i < Q27; ++i) gt[i] = gt[i] - om * gt[i] + (h[i] + inc[i]);
-    double sg;
-    sums27<false>(gt, &sg);
-    const double g_tot = 2.0 * mac[0] * mac[7] + p.dt * (M0 + 2.0 * (mac[4] * F[0] + mac[5] * F[1] + mac[6] * F[2]));
-    const R gdef = (R)(g_tot - sg);
+    // energy: sum g_out = sum g~ + dt (M_0 + 2 uhat . F) exactly; the same defect spreading
+    A wk = w_mul(mc.uh[0], F[0]);
+    wk = w_add(w_add(wk, w_mul(mc.uh[1], F[1])), w_mul(mc.uh[2], F[2]));
+    const A g_tot = w_add(mc.gs, w_mul(w_add(M0, w_mul(wk, R(2))), wide_dt<A>(p)));
+    sums27<false>(gt, sm);
+    const R gdef = w_round(w_sub(g_tot, sm[0]));
 #pragma unroll
     for (int i = 0; i < Q27; ++i) gt[i] += gdef * (R)w27(i);
-    double glo = 0.0;
-    if (sizeof(R) == 4) {
-        sums27<false>(gt, &sg);
-        glo = g_tot - sg;
+    R glo = R(0);
+    if constexpr (sizeof(R) == 4) {
+        sums27<false>(gt, sm);
+        glo = w_round(w_sub(g_tot, sm[0]));
     }
     R rec[SL27];
     rec[R_TH] = th;
@@ -1146,7 +1123,7 @@ __device__ __forceinline__ bool q27_collide(const DevParams &p, R *__restrict__ 
     for (int a = 0; a < 3; ++a) {
         rec[R_UX + a] = u[a];
         rec[R_UHX + a] = uh[a];
-        rec[R_JLO + a] = (R)jlo[a];
+        rec[R_JLO + a] = jlo[a];
     }
 #pragma unroll
     for (int i = 0; i < Q27; ++i) {
@@ -1154,30 +1131,32 @@ __device__ __forceinline__ bool q27_collide(const DevParams &p, R *__restrict__ 
         rec[R_G + i] = gt[i];
     }
     rec[R_RHO] = rho;
-    rec[R_T] = (R)mac[9];
-    rec[R_MLO] = (R)mlo;
-    rec[R_GLO] = (R)glo;
+    const R T = w_round(mc.T);
+    rec[R_T] = T;
+    rec[R_MLO] = mlo;
+    rec[R_GLO] = glo;
     store_chunks<SL27>(out, n, N, rec);
-    const double chk = mac[0] + mac[9];
-    return finite && chk - chk == 0.0;
+    return finite && rho - rho == R(0) && T - T == R(0);
 }
 
 // The node step, one thread per node of the block's tile.  Registers for two resident
 // blocks per SM in FP32 (255, its two staged families' worth of shared memory), one in FP64.
 template <typename R>
 __global__ void __launch_bounds__(Q27_THREADS, sizeof(R) == 4 ? 2 : 1)
-    k_q27_step(DevParams p, Grid3 g3, const R *__restrict__ in, const typename Wide<R>::type *__restrict__ nl,
-               R *__restrict__ out, DevStats *stats)
+    k_q27_step(DevParams p, Grid3 g3, const R *__restrict__ in, typename Wide<R>::type *nl, R *__restrict__ out,
+               DevStats *stats)
 {
+    using A = typename Wide<R>::type;
     extern __shared__ __align__(128) unsigned char q27_dyn_smem[];
-    double *own_s = reinterpret_cast<double *>(q27_dyn_smem) + threadIdx.x;   // [OWN27][threads]
-    R *slots = reinterpret_cast<R *>(q27_dyn_smem + (size_t)OWN27 * Q27_THREADS * 8);
+    R *slots = reinterpret_cast<R *>(q27_dyn_smem);
+    R *keep = slots + (size_t)SLOT_SPACE27 * Slot27<R>::stride + threadIdx.x;   // this thread's column (FP32)
     __shared__ StepCounts counts;
     __shared__ uint4 best[Q27_THREADS / 32];
     const int tid = threadIdx.x;
     const size_t N = (size_t)p.N;
     const Tile27 tl{(int)blockIdx.x * T27X, (int)blockIdx.y * T27Y, (int)blockIdx.z * T27Z};
-    const int tx = tid % T27X, ty = (tid / T27X) % T27Y, tz = tid / (T27X * T27Y);
+    // a warp takes 8 x 1 x 4 nodes: the half warps' slots then fall on distinct banks
+    const int tx = tid % T27X, tz = (tid / T27X) % T27Z, ty = tid / (T27X * T27Z);
     const int X = tl.X0 + tx, Y = tl.Y0 + ty, Z = tl.Z0 + tz;
     const bool valid = X < p.nx && Y < p.ny && Z < g3.nz;
     const size_t n = valid ? ((size_t)Z * p.ny + Y) * p.nx + X : 0;
@@ -1204,32 +1183,29 @@ __global__ void __launch_bounds__(Q27_THREADS, sizeof(R) == 4 ? 2 : 1)
         R gv[4], v[27];
         load27<R_TH, 4>(in, n, N, gv);
         th = gv[0]; u[0] = gv[1]; u[1] = gv[2]; u[2] = gv[3];
-        // sums of the node's own stored populations and kept remainders; the non-local terms
-        double s4[4], sg;
-        load27<R_F, 27>(in, n, N, v);
-        sums27<true>(v, s4);
-        load27<R_G, 27>(in, n, N, v);
-        sums27<false>(v, &sg);
+        // sums of the node's own stored populations and kept remainders {f, f c, g, momentum
+        // lo}: they wait in the stress and flux planes, which the divergences are done with
+        A own[5];
         R lo[5];
+        load27<R_F, 27>(in, n, N, v);
+        sums27<true>(v, own);
+        load27<R_G, 27>(in, n, N, v);
+        sums27<false>(v, own + 4);
         load27<R_MLO, 5>(in, n, N, lo);
-        own_s[0] = s4[0] + (double)lo[0];
-        own_s[Q27_THREADS] = s4[1]; own_s[2 * Q27_THREADS] = s4[2]; own_s[3 * Q27_THREADS] = s4[3];
-        own_s[4 * Q27_THREADS] = sg + (double)lo[4];
+        own[0] = w_add(own[0], lo[0]);
+        own[4] = w_add(own[4], lo[4]);
 #pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            own_s[(5 + a) * Q27_THREADS] = (double)lo[1 + a];
-            own_s[(8 + a) * Q27_THREADS] = w_double(NL3(nl, N3_F + a, n, N));
-        }
-        own_s[11 * Q27_THREADS] = w_double(NL3(nl, N3_REL, n, N));
-        own_s[12 * Q27_THREADS] = w_double(NL3(nl, N3_M0, n, N));
+        for (int k = 0; k < 5; ++k) NL3(nl, N3_K + k, n, N) = own[k];
+#pragma unroll
+        for (int a = 0; a < 3; ++a) NL3(nl, N3_K + 5 + a, n, N) = w_wide(lo[1 + a]);
     }
 
     unsigned its = 0, nreg = 0, npair = 0;
     bool active = valid, conv = true, floored = false, bad = false;
     R fi[27], gi[27];   // increments of the streamed populations
-    double mac[13];
+    Macro<3, R> m;
     int staged = -1;    // family in the slots
-    const R *own_slot = slots + (size_t)(((tz + HALO27) * S27Y + ty + HALO27) * S27X + tx + HALO27) * Slot27<R>::stride;
+    const R *own_slot = slots + (size_t)((tz + HALO27) * PZ27 + (ty + HALO27) * PY27 + tx + HALO27) * Slot27<R>::stride;
     for (unsigned it = 1; __syncthreads_or(active); ++it) {
         const R s = sqrt_(th), inv_s = R(1) / s;
         R a[3][3][4], L[3][3][3];
@@ -1269,7 +1245,7 @@ __global__ void __launch_bounds__(Q27_THREADS, sizeof(R) == 4 ? 2 : 1)
             }
             if (!active || !fast) continue;
             R acc[27];
-            contract27(own_slot, a, near0, L, acc);
+            contract27(own_slot, a, near0, L, keep, acc);
             if (sizeof(R) == 8 || it > 1) {
                 R v[27];
                 if (fam == 0) load27<R_F, 27>(in, n, N, v);
@@ -1299,28 +1275,22 @@ __global__ void __launch_bounds__(Q27_THREADS, sizeof(R) == 4 ? 2 : 1)
             }
         }
         if (active) {
-            double d5[5], d4[4], own[8], F[3];
-            sums27<true>(fi, d4);
-            sums27<false>(gi, &d5[4]);
+            A d[5], own[8], F[3];
+            sums27<true>(fi, d);
+            sums27<false>(gi, d + 4);
 #pragma unroll
-            for (int k = 0; k < 4; ++k) d5[k] = d4[k];
+            for (int k = 0; k < 8; ++k) own[k] = NL3(nl, N3_K + k, n, N);
 #pragma unroll
-            for (int k = 0; k < 8; ++k) own[k] = own_s[k * Q27_THREADS];
-#pragma unroll
-            for (int k = 0; k < 3; ++k) F[k] = own_s[(8 + k) * Q27_THREADS];
-            const double t0 = (double)th, st0 = sqrt(t0), ist = rcp_d(st0);
-            const double ud[3] = {(double)u[0], (double)u[1], (double)u[2]};
-            q27_macro(p, st0, ud, own, d5, F, own_s[11 * Q27_THREADS], mac);
-            double r = fabs(mac[12] - t0) * (ist * ist);
-#pragma unroll
-            for (int x = 0; x < 3; ++x) r = fmax(r, fabs(mac[1 + x] - ud[x]) * ist);
-            conv = r <= p.tol;
-            if (conv || it >= (unsigned)p.max_iter || !(r == r)) {
+            for (int k = 0; k < 3; ++k) F[k] = NL3(nl, N3_F + k, n, N);
+            m.update(p, th, u, own, d, F, NL3(nl, N3_REL, n, N), 3.0);
+            const float res = m.change(th);
+            conv = sizeof(R) == 4 ? res <= p.tol_f : (double)res <= p.tol;
+            if (conv || it >= (unsigned)p.max_iter || !(res == res)) {
                 active = false;
             } else {
-                th = (R)mac[12];
+                th = w_round(m.ths);
 #pragma unroll
-                for (int x = 0; x < 3; ++x) u[x] = (R)mac[1 + x];
+                for (int x = 0; x < 3; ++x) u[x] = w_round(m.uu[x]);
             }
         }
     }
@@ -1332,9 +1302,9 @@ __global__ void __launch_bounds__(Q27_THREADS, sizeof(R) == 4 ? 2 : 1)
         load27<R_G, 27>(in, n, N, v);
 #pragma unroll
         for (int i = 0; i < 27; ++i) gi[i] += v[i];
-        const double F[3] = {own_s[8 * Q27_THREADS], own_s[9 * Q27_THREADS], own_s[10 * Q27_THREADS]};
-        bad = !q27_collide<R>(p, out, n, th, u, mac, F, own_s[12 * Q27_THREADS], fi, gi);
-        floored = mac[10] < p.p_floor;
+        const A F[3] = {NL3(nl, N3_F, n, N), NL3(nl, N3_F + 1, n, N), NL3(nl, N3_F + 2, n, N)};
+        bad = !q27_collide<R>(p, out, n, th, u, m, F, NL3(nl, N3_M0, n, N), fi, gi);
+        floored = w_double(m.pr) < p.p_floor;
     }
     add_counts(counts, stats, its, nreg, npair, valid && !conv, false, floored, bad);
 }
