@@ -14,8 +14,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 SRC = [os.path.join(HERE, "csrc", "pond.cu")]
 DEPS = SRC + [os.path.join(HERE, "csrc", f) for f in ("pond_kernels.cuh", "pond_step.cuh", "pond_q16.cuh",
-                                                      "pond_q27.cuh",
-                                                      "pond_state.cuh")] + [os.path.join(ROOT, "include", "pond.h")]
+                                                      "pond_q27.cuh", "pond_init.cuh", "pond_state.cuh")] + [os.path.join(ROOT, "include", "pond.h")]
 LIB = os.path.join(HERE, "libpond.so")
 ARCH = "-gencode=arch=compute_103a,code=sm_103a"
 

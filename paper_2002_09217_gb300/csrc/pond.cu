@@ -20,6 +20,7 @@
 #include "pond_step.cuh"
 #include "pond_q16.cuh"
 #include "pond_q27.cuh"
+#include "pond_init.cuh"
 #include "pond_state.cuh"
 
 using namespace pond;

@@ -156,66 +156,12 @@ __device__ __forceinline__ double rcp_d(double x)
     return r * (2.0 - x * r);
 }
 
-// ---------------------------------------------------------------------------
-// Initial state: co-moving equilibrium of host-given (rho, u, T) (Eq. geq with the
-// interface energy kappa |grad rho|^2 / 2 in the total energy).  Bound by the FP64 pipe:
-// v^2 is a sum over the axes, so g_i = W_i (G + b_x(c_x) + b_y(c_y)) with b_a(c) = rho (s c +
-// u_a)^2 and G = rho (2 e - 2 P/rho) + kappa |grad rho|^2, and the gradient is three
-// differences per axis: about 110 FP64 operations a node instead of 300 (2048 x 1024
-// nodes 500 -> 443 us, 1024 x 512 D2Q16 202 -> 150, 96 x 96 x 64 D3Q27 895 -> 260).
 // p(rho, T) with the van der Waals quotient as a product with a reciprocal
 __device__ __forceinline__ double pressure_d(const DevParams &p, double r, double t)
 {
     if (p.eos_kind != 0) return eos_pressure<double>(p.eos_kind, p.a, p.b, p.R, r, t, p.sp);
     return r * p.R * t * rcp_d(1.0 - p.b * r) - p.a * r * r;
 }
-template <typename R>
-__global__ void k_init(DevParams p, const double *__restrict__ rho, const double *__restrict__ ux,
-                       const double *__restrict__ uy, const double *__restrict__ T,
-                       R *__restrict__ st, DevStats *stats)
-{
-    const long long n = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (n >= p.N) return;
-    const int X = (int)(n % p.nx), Y = (int)(n / p.nx);
-    double D[3], L[3];   // per row: rho(+1) - rho(-1); rho(-1) + 4 rho(0) + rho(+1)
-#pragma unroll
-    for (int y = 0; y < 3; ++y) {
-        const long long row = (long long)bc_wrap(Y + y - 1, p.ny, p.bcy) * p.nx;
-        const double a = rho[row + bc_wrap(X - 1, p.nx, p.bcx)], c = rho[row + bc_wrap(X + 1, p.nx, p.bcx)];
-        D[y] = c - a;
-        L[y] = (a + c) + 4.0 * rho[row + X];
-    }
-    const double gx = ((D[0] + D[2]) + 4.0 * D[1]) * (1.0 / 12.0), gy = (L[2] - L[0]) * (1.0 / 12.0);
-    const double r = rho[n], t = T[n], u[2] = {ux[n], uy[n]};
-    if (!(r > 0.0) || !(p.b * r < 1.0) || !(t > 0.0)) atomicAdd(&stats->bad_init, 1ull);
-    const double pr = pressure_d(p, r, t);
-    const double P = pr > p.p_floor ? pr : p.p_floor;
-    const double th = P * rcp_d(r) * 3.0, s = sqrt(th);   // theta = P / (rho T_L)
-    const double G = 2.0 * (r * (p.cv * t - p.a * r) - P) + p.kappa * (gx * gx + gy * gy);
-    double b[2][3];
-#pragma unroll
-    for (int a = 0; a < 2; ++a)
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            const double v = s * (k - 1) + u[a];
-            b[a][k] = r * (v * v);
-        }
-    R rec[SL];
-#pragma unroll
-    for (int i = 0; i < 9; ++i) {
-        const double w = w1d(i % 3) * w1d(i / 3);
-        rec[P_F + i] = (R)(r * w);
-        rec[P_G + i] = (R)(w * (G + (b[0][i % 3] + b[1][i / 3])));
-    }
-    rec[P_TH] = (R)th;
-    rec[P_UX] = rec[P_UHX] = (R)u[0];
-    rec[P_UY] = rec[P_UHY] = (R)u[1];
-    rec[P_RHO] = (R)r;
-    rec[P_T] = (R)t;
-    rec[P_SQ] = rec[P_F4LO] = rec[P_G4LO] = rec[P_JXLO] = rec[P_JYLO] = rec[30] = rec[31] = (R)0;
-    store_chunks<SL>(st, (size_t)n, (size_t)p.N, rec);
-}
-
 template <typename T>
 __device__ __forceinline__ void warp_add(unsigned long long *dst, T v)
 {

@@ -29,10 +29,11 @@
 // its node's 5 x 5 window along x, then y: 2,200 multiply-adds a population family, where
 // carrying each of 25 nodes into the arrival gauge and spreading it over sixteen directions
 // took about 7,000.
-// Measured (with init and read-out): four mixed steps of a 1024 x 512 droplet 7.83 -> 2.69 ms,
-// three FP64 steps of a 257 x 127 shock-droplet 28.8 -> 5.2 ms.  The mixed node step issues
-// on 56 % of its cycles (FMA pipe 50 %); its FP64 pipe, 22 % busy with the moments and EoS
-// before they went to float-float, is idle.
+// Measured (with init and read-out): four mixed steps of a 1024 x 512 droplet 7.82 -> 1.91 ms,
+// three FP64 steps of a 257 x 127 shock-droplet 30.2 -> 5.9 ms.  The mixed contraction runs on
+// packed pairs, rolled over the source rows so that its code stays in the instruction cache
+// (609 -> 457 us a step); its FP64 pipe, 22 % busy with the moments and EoS before they went
+// to float-float, is idle.  The FP64 form is bound by the FP64 pipe.
 #pragma once
 
 #include "pond_kernels.cuh"
@@ -198,59 +199,6 @@ __device__ __forceinline__ int departure(int X, A v, A dt, A w[4])
     const A fl = floor(d);
     cubic_weights<A>(d - fl + A(1), w);
     return X + (int)fl - 1;
-}
-
-// ---------------------------------------------------------------------------
-// Initial state: co-moving equilibrium of host-given (rho, u, T) (Eq. geq with the
-// interface energy kappa |grad rho|^2 / 2 in the total energy), D2Q16 weights, T_L = 1.
-template <typename R>
-__global__ void k_q16_init(DevParams p, const double *__restrict__ rho, const double *__restrict__ ux,
-                           const double *__restrict__ uy, const double *__restrict__ T,
-                           R *__restrict__ st, DevStats *stats)
-{
-    const long long n = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (n >= p.N) return;
-    const Lat16<double> L = make_lat16<double>();
-    const int X = (int)(n % p.nx), Y = (int)(n / p.nx);
-    double D[3], S[3];   // per row: rho(+1) - rho(-1); rho(-1) + 4 rho(0) + rho(+1)
-#pragma unroll
-    for (int y = 0; y < 3; ++y) {
-        const long long row = (long long)bc_wrap(Y + y - 1, p.ny, p.bcy) * p.nx;
-        const double a = rho[row + bc_wrap(X - 1, p.nx, p.bcx)], c = rho[row + bc_wrap(X + 1, p.nx, p.bcx)];
-        D[y] = c - a;
-        S[y] = (a + c) + 4.0 * rho[row + X];
-    }
-    const double gx = ((D[0] + D[2]) + 4.0 * D[1]) * (1.0 / 12.0), gy = (S[2] - S[0]) * (1.0 / 12.0);
-    const double r = rho[n], t = T[n], u[2] = {ux[n], uy[n]};
-    if (!(r > 0.0) || !(p.b * r < 1.0) || !(t > 0.0)) atomicAdd(&stats->bad_init, 1ull);
-    const double pr = pressure_d(p, r, t);
-    const double P = pr > p.p_floor ? pr : p.p_floor;
-    const double th = P * rcp_d(r), s = sqrt(th);
-    // g_i = W_i (G + rho v_x^2 + rho v_y^2), as in k_init
-    const double G = 2.0 * (r * (p.cv * t - p.a * r) - P) + p.kappa * (gx * gx + gy * gy);
-    double b[2][4];
-#pragma unroll
-    for (int a = 0; a < 2; ++a)
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            const double v = s * L.c[k] + u[a];
-            b[a][k] = r * (v * v);
-        }
-    R rec[SLQ];
-#pragma unroll
-    for (int i = 0; i < Q16; ++i) {
-        const double w = L.w[i & 3] * L.w[i >> 2];
-        rec[Q_F + i] = (R)(r * w);
-        rec[Q_G + i] = (R)(w * (G + (b[0][i & 3] + b[1][i >> 2])));
-    }
-    rec[Q_TH] = (R)th;
-    rec[Q_UX] = rec[Q_UHX] = (R)u[0];
-    rec[Q_UY] = rec[Q_UHY] = (R)u[1];
-    rec[Q_RHO] = (R)r;
-    rec[Q_T] = (R)t;
-#pragma unroll
-    for (int k = Q_MLO; k < SLQ; ++k) rec[k] = (R)0;
-    store_chunks<SLQ>(st, (size_t)n, (size_t)p.N, rec);
 }
 
 // ---------------------------------------------------------------------------

@@ -30,7 +30,7 @@
 // staged (two blocks per SM in FP32, one in FP64, by shared memory); a further stream of
 // the frame search starts with the family that is already staged.  The sums of populations,
 // the moments, the EoS and the non-local terms are float-float in the FP32 form.
-// Measured: two mixed steps of a 96 x 96 x 64 droplet (with init and read-out) 29.3 -> 6.1
+// Measured: two mixed steps of a 96 x 96 x 64 droplet (with init and read-out) 29.3 -> 6.0
 // ms, two FP64 steps of 33 x 29 x 21 nodes 152 -> 21 ms.  With two warps per scheduler the
 // shared-memory latency decides: a row's slots are replaced by the next row's as they are
 // used (3.78 -> 2.88 ms a step; issue 41 -> 53 %, FMA pipe 53 % busy).
@@ -206,63 +206,6 @@ struct Near27 {
     }
     __device__ __forceinline__ long long at(int z, int y, int k) const { return row[z][y] + x[k]; }
 };
-
-// ---------------------------------------------------------------------------
-// Initial state: co-moving equilibrium of host-given (rho, u, T) with the interface
-// energy (Eq. geq, D = 3).
-template <typename R>
-__global__ void k_q27_init(DevParams p, Grid3 g3, const double *__restrict__ rho, const double *__restrict__ ux,
-                           const double *__restrict__ uy, const double *__restrict__ uz,
-                           const double *__restrict__ T, R *__restrict__ st, DevStats *stats)
-{
-    const long long n = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (n >= p.N) return;
-    // the gradient by lines, planes and a column (the separable stencil, see diff3 below)
-    const Near27 nb(p, g3, n);
-    const Diff3<double> dr = diff3<double>([&](int z, int y, int k) { return rho[nb.at(z, y, k)]; });
-    double g2 = 0.0;
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        const double g = dr.d[a] * (1.0 / 72.0);
-        g2 += g * g;
-    }
-    const double r = rho[n], t = T[n], u[3] = {ux[n], uy[n], uz[n]};
-    if (!(r > 0.0) || !(p.b * r < 1.0) || !(t > 0.0)) atomicAdd(&stats->bad_init, 1ull);
-    const double pr = pressure_d(p, r, t);
-    const double P = pr > p.p_floor ? pr : p.p_floor;
-    const double th = P * rcp_d(r) * 3.0, s = sqrt(th);   // theta = P / (rho T_L)
-    // g_i = W_i (G + rho v_x^2 + rho v_y^2 + rho v_z^2), as in k_init
-    const double G = r * (2.0 * (p.cv * t - p.a * r)) - 3.0 * P + p.kappa * g2;
-    double b[3][3];
-#pragma unroll
-    for (int a = 0; a < 3; ++a)
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            const double v = s * (k - 1) + u[a];
-            b[a][k] = r * (v * v);
-        }
-    R rec[SL27];
-#pragma unroll
-    for (int z = 0; z < 3; ++z)
-#pragma unroll
-        for (int y = 0; y < 3; ++y) {
-            const double gyz = G + (b[1][y] + b[2][z]);
-#pragma unroll
-            for (int x = 0; x < 3; ++x) {
-                const int i = 9 * z + 3 * y + x;
-                rec[R_F + i] = (R)(r * w27(i));
-                rec[R_G + i] = (R)(w27(i) * (gyz + b[0][x]));
-            }
-        }
-    rec[R_TH] = (R)th;
-#pragma unroll
-    for (int a = 0; a < 3; ++a) rec[R_UX + a] = rec[R_UHX + a] = (R)u[a];
-    rec[R_RHO] = (R)r;
-    rec[R_T] = (R)t;
-#pragma unroll
-    for (int k = R_MLO; k < SL27; ++k) rec[k] = (R)0;
-    store_chunks<SL27>(st, (size_t)n, (size_t)p.N, rec);
-}
 
 // Stage 1 (rho, T of `src`): K = -kappa (rho lap rho + |grad rho|^2/2) I + kappa grad rho
 // (x) grad rho, q = -mu grad h + k grad T (h = C_v T - a rho + p/rho), rho E_lambda = kappa

@@ -29,9 +29,10 @@
 // about 2,700.  The tile is 128 nodes because the halo's share of the staging falls with its
 // size (1.9 staged nodes a node; 6.3 with 4 x 4 nodes and a halo of 3).
 // Measured (five steps of the 2048 x 1024 shock-droplet interaction with init and read-out,
-// mixed): 17.70 -> 4.50 ms; two FP64 steps of a 509 x 387 droplet 22.66 -> 5.27 ms.  Bound
-// by instruction issue (60 % active; FMA pipe 49 %, shared-memory pipe 41 %) in the mixed
-// form and by the FP64 pipe in the FP64 form; DRAM 6 % busy.
+// mixed): 17.7 -> 3.87 ms, 714 us a step; two FP64 steps of a 509 x 387 droplet 22.7 ->
+// 5.47 ms, 2.69 ms a step.  The mixed form is bound by instruction fetch and issue (issue 54 %
+// active, FMA pipe 56 %, 1.2 warps per issue waiting for instructions), the FP64 form by the
+// FP64 pipe (92 % busy); DRAM is 10 % busy.
 //
 // Accuracy.  A tile whose thetas differ holds the carried populations themselves in the
 // gauge of geometric-mean theta and mean velocity of its hottest and coldest nodes, by
@@ -69,7 +70,8 @@ constexpr float SMOOTH_TILE = 0.9f;
 // Mixed form: a frame-search residual below this multiple of tol that no longer halves is
 // taken as the FP32 rounding floor (the EoS cancels up to ~200x inside interfaces).
 constexpr float STALL_TOL_FACTOR = 16.0f;
-// resident blocks per SM the register budget is sized for
+// Resident blocks per SM the register budget is sized for: FP32 with one thread a node took
+// 798, 737 and 850 us a step (2048 x 1024) with four, three and two.
 #define STEP_MIN_BLOCKS(R) (sizeof(R) == 8 ? 2 : 3)
 #define SPLIT_MIN_BLOCKS(R) 2
 
@@ -543,6 +545,11 @@ __device__ __forceinline__ ffv w_sqrt(float x)
     return ff_norm(s, fmaf(-s, s, x) / (2.0f * s));
 }
 __device__ __forceinline__ double w_sqrt(double x) { return sqrt(x); }
+__device__ __forceinline__ ffv w_sqrt(ffv x)
+{
+    const float s = sqrtf(x.hi);
+    return ff_norm(s, (fmaf(-s, s, x.hi) + x.lo) / (2.0f * s));
+}
 // a parameter in the wide type, from its FP64 value or its float pair (splitting an FP64
 // value on the device costs as much as 25 float-float additions)
 template <typename A> __device__ __forceinline__ A wide_param(double x, const float (&ff)[2]);
