@@ -110,6 +110,15 @@ inline unsigned blocks_for(size_t n, unsigned bs) { return (unsigned)((n + bs - 
 // 64 x 64 to 164 x 160 nodes took 59 us a step with the smallest on nine lanes.
 size_t split_max_nodes(int precision) { return precision == POND_MIXED ? 3072 : 10000; }
 
+// Strips of up to four rows stepped with one thread per node take tiles of 64 nodes while
+// that is at most one block per SM (152 x 64 nodes): with 128 fewer than half of the SMs
+// would work, and a step costs one block's serial time, which falls with the slots it stages.
+// Measured (mixed, us per step, 128 / 64 / 32 nodes): 2048 x 4 15.0 / 13.6 / 14.2, 4096 x 2
+// 16.0 / 13.7 / 13.4, 8192 x 1 17.6 / 14.9 / 14.2, 1600 x 3 14.4 / 13.3 / 13.7.  Grids of more
+// rows keep 128: they are what batches hold, where the wider halo share counts.
+constexpr int STRIP_NB = 64;
+constexpr size_t STRIP_MAX_NODES = 152 * STRIP_NB;
+
 bool mixed(const pond_ctx *c) { return c->opts.precision == POND_MIXED; }
 
 // Tiles of the D2Q9 step kernel over the grid.
@@ -612,8 +621,8 @@ pond_status pond_create(const pond_grid *grid, const pond_lattice *lattice, cons
     // (The other lattices' kernels have one split and share the tile rule.)
     c->lanes = opts->lanes_per_node ? opts->lanes_per_node : (c->N <= split_max_nodes(opts->precision) ? 16 : 8);
     if (c->lattice != POND_D2Q9) c->lanes = 8;
-    // Its tile: TX x TY nodes of STEP_NB (SPLIT_NB) nodes, by default no taller than the grid
-    // and otherwise 16 x 8 (4 x 3)
+    // Its tile: TX x TY nodes of STEP_NB (SPLIT_NB; STRIP_NB) nodes, by default no taller than
+    // the grid and otherwise 16 x 8 (4 x 3)
     int tile_x = opts->tile_x, tile_y;
     if (c->lanes == 16) {
         if (!tile_x) tile_x = grid->ny == 1 ? 12 : (grid->ny == 2 || grid->ny == 4 ? 6 : 4);
@@ -621,9 +630,11 @@ pond_status pond_create(const pond_grid *grid, const pond_lattice *lattice, cons
         else if (tile_x == 16) tile_x = 12;
         tile_y = SPLIT_NB / tile_x;
     } else {
+        const bool strip = !tile_x && c->lattice == POND_D2Q9 && grid->ny <= 4 && c->N <= STRIP_MAX_NODES;
+        const int nodes = strip ? STRIP_NB : STEP_NB;
         if (!tile_x)
-            for (tile_x = 16; tile_x < STEP_NB && STEP_NB / (2 * tile_x) >= grid->ny; tile_x *= 2) {}
-        tile_y = STEP_NB / tile_x;
+            for (tile_x = 16; tile_x < nodes && nodes / (2 * tile_x) >= grid->ny; tile_x *= 2) {}
+        tile_y = nodes / tile_x;
     }
     cudaError_t e = cudaGetDevice(&c->device);
     if (e == cudaSuccess)

@@ -1501,7 +1501,7 @@ __device__ __forceinline__ void step_tile(const DevParams &p, const R *__restric
     stage_tile<R>(p, in, nlsrc, tl, counts, gb);
     const int tx = tid % tl.TX, ty = tid / tl.TX;
     const int X = tl.X0 + tx, Y = tl.Y0 + ty;
-    const bool valid = X < p.nx && Y < p.ny;
+    const bool valid = ty < tl.TY && X < p.nx && Y < p.ny;   // (a tile may have fewer nodes than threads)
     R *keep = tl.kq + (size_t)(tl.TX + 2) * (tl.TY + 2) * KQW + tid;   // this thread's column
     const int slot = (ty + HALO) * tl.WT + tx + HALO;
     unsigned its = 0, nreg = 0, npair = 0;

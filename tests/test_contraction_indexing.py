@@ -11,7 +11,7 @@ HALO, NB, SPLIT = 2, 128, 12
 AUX, KQ, KEEP, SL = 4, 5, 36, 32
 MAX_SMEM = 227 * 1024            # a block's shared memory on this part
 TILES = [(tx, NB // tx, False) for tx in (1, 2, 4, 8, 16, 32, 64, 128)] + [
-    (tx, SPLIT // tx, True) for tx in (1, 2, 4, 6, 12)]
+    (tx, 64 // tx, False) for tx in (16, 32, 64)] + [(tx, SPLIT // tx, True) for tx in (1, 2, 4, 6, 12)]
 GAUGES = [0.0, 1e-30, 0.05, 0.5, 0.9999999, 1.0, 1.7, 3.0, 1e4, 1e38, np.inf, np.nan]
 C16 = np.sqrt(3 - np.sqrt(6.0)), np.sqrt(3 + np.sqrt(6.0))
 

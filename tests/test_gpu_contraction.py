@@ -87,6 +87,20 @@ def test_2d_matches_oracle(pond, case, lattice, lanes, precision):
         assert abs(gstats["streams"] - ostats["streams"]) <= 0.01 * ostats["streams"] + 2
 
 
+@pytest.mark.parametrize("nx,ny,bc", [(3073, 1, 0), (1601, 2, ZG), (1025, 3, 0), (2432, 4, ZG), (9728, 1, 0), (9729, 1, ZG)])
+def test_strips_match_oracle(pond, nx, ny, bc):
+    """Strips in the default shape: tiles of 64 nodes up to 9,728 nodes, of 128 beyond."""
+    w = droplet(nx, ny, bc=bc, steps=4)
+    P, st, _ = oracle_run(w)
+    with pond.from_workload(w) as sim:
+        sim.init_fields(*w.fields())
+        sim.step(w.steps)
+        got = sim.moments()
+        assert sim.stats()["nonfinite"] == 0
+    err = rel_linf(got, oracle.moments(P, st))
+    assert max(err.values()) <= TOL["mixed"], err
+
+
 def cases3d():
     yield "one_node_more_9x5x5", dict(n=9, ny=5, nz=5)
     yield "one_node_less_7x3x3_zerograd", dict(n=7, ny=3, nz=3, bc=ZG)
