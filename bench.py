@@ -131,102 +131,42 @@ def bytes_per_update(precision: str, lattice: str = "d2q9") -> int:
     return 48 * e
 
 
-# Algorithmic FLOPs of the D2Q9 step kernel's formula (an FMA counts 2).  A stream of a
-# node transforms each node of its stencil region (the union of its nine directions'
-# 4x4 stencils, counted by the kernel: pond_stats region_nodes) once for all directions:
-#  per region node: gauge offsets (9), the per-axis transfer increments from h = e/2 and
-#  p = h (2c + e) (42), the nine weight products (9), and per population family the
-#  x-transform of the three source rows (45), the sums for the y-transform (9), the
-#  increment-form outputs (72) and the weighted accumulation (18) => 348;
-#  per stream: departure points, Lagrange weight tables and moment sums of the nine
-#  directions (9 x 20) and the moments, EoS and residual (60) => 240;
-#  streams of regions wider than 8 nodes take the per-direction path: per stencil pair
-#  (9 directions x 16 stencil nodes) gauge offsets (8), six transfer increments (24), the
-#  x-increments of three source rows for f and g (30), the f and g components (22),
-#  weight and accumulation (7) => 91, plus the same 240 per stream;
-#  per node update: the Korteweg tensor, heat flux and their divergences counted once per
-#  node (200; the kernel recomputes them at each neighbour) and the collision (1300:
-#  transfer rows of both axes ~230, forced g equilibrium ~410, BGK updates ~150, carrying
-#  X* into the streaming gauge ~390, exact rest-population remainders ~100).
-FLOPS_REGION_NODE = 348
-FLOPS_PAIR = 91
-FLOPS_DIR = 20
-FLOPS_STREAM_EXTRA = 60
-FLOPS_NONLOCAL = 200
-FLOPS_COLLIDE = 1300
+# Algorithmic FLOPs of the step kernels, per node update (an FMA counts 2), from the kernels'
+# counters (pond_stats).  A node's populations are carried into its tile's gauge once (counted
+# once per node; the kernels also carry each tile's halo), and a stream contracts the node's
+# window axis by axis, each component over its own four columns and over five rows (and
+# planes), f and g (the FP32 forms run five columns with zero weights and take differences to
+# the own slot besides: not counted):
+#  D2Q9    x 5 rows x 3 n x 3 k x 12, y 5 x 27 => 675 FMAs a family, 2,700 flops; products of
+#          the weights (81), cubic weights (96), rows of the map (60) => 240; moments, EoS and
+#          residual 110; carry: gauge and rows 64, two applications 216 => 280;
+#  D2Q16   x 5 x 4 x 4 x 16, y 5 x 64 => 1,600 FMAs, 6,400; weights 144 + 128 + 160 => 430;
+#          moments and residual 130; carry 170 + 512 => 680;
+#  D3Q27   x 25 rows x 9 x 3 x 12, y 25 x 81, z 5 x 81 => 10,530 FMAs, 42,120; weights 530;
+#          moments and residual 260; carry 92 + 972 => 1,064.
+# Streams whose departure points lie beyond the window carry each node of their stencil region
+# instead (counted like the others), or, where the region is wider than the kernels' tables
+# (pair_streams), each direction's stencil nodes one by one: 9 x 16 x 91 + 180, 16 x (40 + 16 x
+# 206), 27 x (60 + 64 x 289) flops.  Per node update the non-local terms (200, 200, 600: counted
+# once per node) and the collision (1,300, 2,300, 7,000).
+FLOPS = {   # contraction and weights per stream, per-pair stream, moments, and per node update
+    "d2q9": (2700 + 240, 9 * 16 * 91 + 180, 110, 280 + 200 + 1300),
+    "d2q16": (6400 + 430, 16 * (40 + 16 * 206), 130, 680 + 200 + 2300),
+    "d3q27": (42120 + 530, 27 * (60 + 64 * 289), 260, 1064 + 600 + 7000),
+}
 
 
-def flops_d2q9(st: dict, updates: int) -> float:
-    """FLOPs per node update of the D2Q9 step from its counters (pond_stats)."""
-    per_stream = 9 * FLOPS_DIR + FLOPS_STREAM_EXTRA
-    pair_streams = st.get("pair_streams", 0)
-    total = (st["region_nodes"] * FLOPS_REGION_NODE + st["streams"] * per_stream
-             + pair_streams * 9 * 16 * FLOPS_PAIR + updates * (FLOPS_NONLOCAL + FLOPS_COLLIDE))
-    return total / max(1, updates)
-
-# The same count for the D2Q16 step (k_q16_step), per node update.  Region stream, per
-# region node (the union of the sixteen 4 x 4 departure stencils, 5 x 5 for |v| dt < 1):
-# gauge offsets (9), both per-axis increment maps (eight rows of 31 and their offsets 16:
-# 264), for f and g the x-increments (128), the y-increments (144) and the weighted
-# accumulation (80), the weight products (16) => 990; per region stream: departure floors,
-# cubic weights and tables of both axes (220).  Per-pair fallback stream (regions wider
-# than 6): per stencil pair (16 directions x 16 stencil nodes) gauge offsets (9), the eight
-# increments of the pair's row per axis (16 for their offsets, 82 for the entries), the
-# x-increments of the four source rows for f and g (64), the y-increment (24), weight and
-# accumulation (11) => 206, per direction departure points and cubic weights (40).  Per
-# stream: moments and residual (FP64, 130); per node update: non-local terms (200) and the
-# collision (2300: four per-axis increment maps ~700, three tensor-product applications
-# ~900, forced g equilibrium ~640, mass and energy defect sums ~70).
-FLOPS_Q16_REGION_NODE = 990
-FLOPS_Q16_REGION_STREAM = 220
-FLOPS_Q16_PAIR = 206
-FLOPS_Q16_DIR = 40
-FLOPS_Q16_STREAM_EXTRA = 130
-FLOPS_Q16_COLLIDE = 2300
-
-
-def flops_q16(st: dict, updates: int) -> float:
-    """FLOPs per node update of the D2Q16 step from its counters (pond_stats)."""
+def flops_per_update(lattice: str, st: dict, updates: int) -> float:
+    """FLOPs per node update of a lattice's step from its counters (pond_stats)."""
+    contract, per_pair, moments, node = FLOPS[lattice]
     pair = st.get("pair_streams", 0)
-    total = (st["region_nodes"] * FLOPS_Q16_REGION_NODE + (st["streams"] - pair) * FLOPS_Q16_REGION_STREAM
-             + st["streams"] * FLOPS_Q16_STREAM_EXTRA + pair * 16 * (FLOPS_Q16_DIR + 16 * FLOPS_Q16_PAIR)
-             + updates * (FLOPS_NONLOCAL + FLOPS_Q16_COLLIDE))
-    return total / max(1, updates)
-
-
-# The D3Q27 step (k_q27_step), per node update.  Region stream, per region node (the
-# union of the 27 departure stencils of 4 x 4 x 4, 5 x 5 x 5 for |v| dt < 1), for each of the
-# two population passes: gauge offsets (11), the three per-axis increment maps (123), the
-# weight products (27), x-, y- and z-increments (3 x 135), the running sums of the
-# increments (135) and the accumulation (81) => 782, 1564 per node; per region stream:
-# departure floors, cubic weights and tables of the three axes (175).  Per-pair fallback
-# stream (regions wider than 6): per stencil pair (27 directions x 64 stencil nodes) gauge
-# offsets (29), the three per-axis increment rows (60), the x-, y- and z-increments and
-# accumulation for f and g (198), weight (2) => 289, per direction three departure points
-# and cubic weights (60).  Per stream: moments and residual (FP64, 260); per node update:
-# non-local terms (600) and the collision (7000: six per-axis increment maps ~360, three
-# three-axis applications ~4800, forced g equilibrium ~1620, defect sums ~300).
-FLOPS_Q27_REGION_NODE = 1564
-FLOPS_Q27_REGION_STREAM = 175
-FLOPS_Q27_PAIR = 289
-FLOPS_Q27_DIR = 60
-FLOPS_Q27_STREAM_EXTRA = 260
-FLOPS_Q27_NONLOCAL = 600
-FLOPS_Q27_COLLIDE = 7000
-
-
-def flops_q27(st: dict, updates: int) -> float:
-    """FLOPs per node update of the D3Q27 step from its counters (pond_stats)."""
-    pair = st.get("pair_streams", 0)
-    total = (st["region_nodes"] * FLOPS_Q27_REGION_NODE + (st["streams"] - pair) * FLOPS_Q27_REGION_STREAM
-             + st["streams"] * FLOPS_Q27_STREAM_EXTRA + pair * 27 * (FLOPS_Q27_DIR + 64 * FLOPS_Q27_PAIR)
-             + updates * (FLOPS_Q27_NONLOCAL + FLOPS_Q27_COLLIDE))
+    total = (st["streams"] - pair) * contract + pair * per_pair + st["streams"] * moments + updates * node
     return total / max(1, updates)
 
 
 def d3q27_run(pond, torch, stream, precision, steps, warmup, nx=96, ny=96, nz=64, sm_mhz=2070.0) -> dict:
-    """MLUPS of the D3Q27 step on a liquid sphere in its vapour (96 x 96 x 64 nodes, 72-value
-    records; 0.6 M nodes x 288 B = 170 MB per FP32 state buffer, larger than L2), with its
+    """MLUPS of the D3Q27 step on a liquid sphere in its vapour (96 x 96 x 64 nodes, 68-value
+    records; 0.6 M nodes x 272 B = 160 MB per FP32 state buffer, larger than L2), with its
     ALU roofline and an end-to-end figure (host fields in, steps, host fields out)."""
     import numpy as np
     from paper_2002_09217_gb300 import inputs
@@ -250,12 +190,12 @@ def d3q27_run(pond, torch, stream, precision, steps, warmup, nx=96, ny=96, nz=64
     sim.moments()
     e2e = w.nodes * steps / (time.perf_counter() - t0) / 1e6
     sim.close()
-    fl = flops_q27(st, st["node_updates"])
+    fl = flops_per_update("d3q27", st, st["node_updates"])
     achieved = w.nodes * fl / (ms * 1e-3) / 1e12
     peak = alu_peak_tflops(precision, sm_mhz)
     return {"workload": w.name, "mlups": w.nodes / ms / 1e3, "ms_per_step": ms, "streams_per_node": its,
             "e2e_mlups": e2e,
-            "roofline": {"bound": "alu", "kernel": "k_q27_step (+ two non-local kernels, timed together)",
+            "roofline": {"bound": "alu", "kernel": "k_q27_step (+ three non-local kernels, timed together)",
                          "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
                          "flops_per_update": fl}}
 
@@ -263,9 +203,9 @@ def d3q27_run(pond, torch, stream, precision, steps, warmup, nx=96, ny=96, nz=64
 # DRAM bytes per launch of k_pond_step (dram__bytes_read.sum + dram__bytes_write.sum) from
 # one ncu capture of the bench workload; they hold only for the kernel source they were
 # taken on (sha256 over the two kernel headers), any other source reports null.
-NCU_TRAFFIC = {"kernel_sha256": "804944b3cf14dfdb4985ac6b9233784f0279b3f7c34f8b526fea166cf068bb7f",
-               "bytes": {"dropletshock2048x1024/mixed": 637875968.0,
-                         "dropletshock2048x1024/fp64": 1170719488.0}}
+NCU_TRAFFIC = {"kernel_sha256": "88e894a2f614c0ebf0c223f987bacb220bc5a0f6d56fe1a6f59b03db0b9ae876",
+               "bytes": {"dropletshock2048x1024/mixed": 496968192.0,
+                         "dropletshock2048x1024/fp64": 968942336.0}}
 
 
 def kernel_sha256() -> str:
@@ -342,10 +282,10 @@ def run_form(w, pond, torch, stream, flush, precision, steps, warmup, shape, ws)
 
 def roofline(w, precision, its, kernel_ms, pk, lattice="d2q9", st=None, updates=0):
     if lattice == "d2q16":
-        fl = flops_q16(st, updates)
+        fl = flops_per_update("d2q16", st, updates)
         kernel, traffic = "k_q16_step (+ two non-local kernels, timed together)", None
     else:
-        fl = flops_d2q9(st, updates)
+        fl = flops_per_update("d2q9", st, updates)
         kernel, traffic = "k_pond_step", ncu_traffic(w, precision)
     achieved = w.nodes * fl / (kernel_ms * 1e-3) / 1e12
     peak = alu_peak_tflops(precision, pk["sm_max_mhz"])
@@ -530,7 +470,7 @@ def other_configs(pond, torch, stream, sm_mhz: float = 2070.0, skip: str = "") -
         st = sim.stats()
         sim.close()
         its = st["streams"] / max(1, st["node_updates"])
-        fl = flops_q16(st, st["node_updates"])
+        fl = flops_per_update("d2q16", st, st["node_updates"])
         achieved = w.nodes * fl / (ms * 1e-3) / 1e12
         peak = alu_peak_tflops(prec, sm_mhz)
         out["%s/d2q16/%s" % (w.name, prec)] = {
@@ -740,8 +680,8 @@ def main():
                 "scaling": "weak", "vs_baseline": None,
                 "dtype": "f32" if args.precision == "mixed" else "f64", "data": "synthetic",
                 "config": {"workload": r["workload"], "nx": 96, "ny": 96, "nz": 64, "lattice": "d3q27",
-                           "precision": args.precision, "l2": "inputs larger than L2 (170 MB per FP32 buffer)"},
-                "frame_search_streams_per_node": r["streams_per_node"], "gpu_launches": 3 * steps,
+                           "precision": args.precision, "l2": "inputs larger than L2 (160 MB per FP32 buffer)"},
+                "frame_search_streams_per_node": r["streams_per_node"], "gpu_launches": 4 * steps,
                 "roofline": r["roofline"], "clocks": clocks.summary(),
                 "e2e": {"value": ws * r["e2e_mlups"], "unit": "MLUPS", "h2d_bytes_per_step": 5 * nodes * 8 / steps,
                         "d2h_bytes_per_step": 6 * nodes * 8 / steps}}
@@ -791,8 +731,9 @@ def main():
         "gpu_launches": args.steps * (3 if args.lattice == "d2q16" else 1),
         "roofline": roofline(w, args.precision, its, kms, pk, args.lattice, st, w.nodes * args.steps),
         "region_nodes_per_stream": st["region_nodes"] / max(1, st["streams"] - st["pair_streams"]),
-        # streams a block runs (its nodes search in lockstep) per node's own streams
-        "block_stream_ratio": st["block_streams"] * 16 / max(1, st["streams"]),
+        # streams a warp runs (its nodes search in lockstep) per node's own streams, with one
+        # thread per node (nine lanes per node: three nodes a warp)
+        "block_stream_ratio": st["block_streams"] * 32 / max(1, st["streams"]),
         "hbm": {"bytes_per_update": bytes_per_update(args.precision, args.lattice),
                 "achieved_gbs": value / ws * 1e6 * bytes_per_update(args.precision, args.lattice) / 1e9,
                 "peak_gbs": pk["hbm_gbs"], "peak_src": pk["src"]},

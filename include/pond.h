@@ -126,9 +126,9 @@ typedef struct {
  * size.  tile_x: width of a block's tile of nodes, 1, 2, 4, 8 or 16 (its height is the
  * block's nodes divided by it; with nine lanes per node 8 and 16 mean 6 and 12), 0 = by the
  * grid's rows.  Both are performance knobs (autotuning); results are the same to rounding.
- * The D2Q16 and D3Q27 kernels ignore them.
- * In the mixed form on D2Q16 the moments, e->T, EoS and frame-search residual are FP64;
- * the storage-rounding remainders of mass, momentum and energy are kept beside each
+ * The D2Q16 kernel takes tile_x (of 128 nodes); the D3Q27 kernel ignores both.
+ * In the mixed form the moments, e->T, EoS and frame-search residual are float-float; the
+ * storage-rounding remainders of mass, momentum and energy are kept beside each
  * node as on D2Q9.
  * nonlocal: time level of the Korteweg force, interface energy and heat-flux source,
  * which the paper leaves open.  POND_NONLOCAL_LAGGED (0): from rho, T at t - dt (one
@@ -167,8 +167,8 @@ typedef struct {
     int64_t max_streams;   /* largest streaming-pass count of any node         */
     int64_t timeouts;      /* tiles skipped because a bounded device wait ran
                               out (reported as POND_ETIMEOUT)                  */
-    int64_t region_nodes;  /* stencil-region nodes carried into the arrival gauge,
-                              summed over streams (the union of a node's 4x4
+    int64_t region_nodes;  /* stencil nodes contracted or carried into the arrival
+                              gauge, summed over streams (the union of a node's 4x4
                               (4x4x4) departure stencils: 16..64 per stream on
                               D2Q9, 16..36 on D2Q16, 64..216 on D3Q27, less the
                               node's own entry in a first stream)              */
@@ -178,9 +178,10 @@ typedef struct {
 } pond_stats_t;
 
 /* Create a context and allocate its device state (two state buffers holding one record
- * per node, 32 values on D2Q9 and 44 on D2Q16, in FP32 or FP64; a 5-plane FP64 staging
- * buffer and reduction partials; on D2Q16 also 9 FP64 planes of non-local terms).
- * lattice: POND_D2Q9 or POND_D2Q16 (else POND_EINVAL).  kappa >= 0: Korteweg coefficient
+ * per node, 32 values on D2Q9, 44 on D2Q16 and 68 on D3Q27, in FP32 or FP64; a 6-plane FP64
+ * staging buffer and reduction partials; on D2Q16 (D3Q27) also 9 (15) 8-byte planes of
+ * non-local terms).
+ * lattice: POND_D2Q9, POND_D2Q16 or POND_D3Q27 (else POND_EINVAL).  kappa >= 0: Korteweg coefficient
  * (Eq. korteweg); tau > 1/2: BGK relaxation time, omega = 1/tau.  On success *out owns
  * the context. */
 pond_status pond_create(const pond_grid *grid, const pond_lattice *lattice, const pond_eos *eos,
@@ -247,7 +248,7 @@ pond_status pond_get_state(pond_ctx *ctx, double *state);
 pond_status pond_set_state(pond_ctx *ctx, const double *state);
 
 /* One time step (its launches: the fused step kernel on D2Q9; the two non-local kernels
- * and the node step on D2Q16) bracketed by CUDA events on the
+ * and the node step on D2Q16, with one more for p/rho on D3Q27) bracketed by CUDA events on the
  * context stream; *ms_out = its duration in milliseconds.  Synchronises (a tracing
  * aid; pond_step is the fast path). */
 pond_status pond_step_timed(pond_ctx *ctx, double *ms_out);

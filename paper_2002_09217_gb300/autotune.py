@@ -3,8 +3,9 @@
 For a grid (nx, ny, boundaries) and precision it times a few steps of every valid
 (lanes_per_node, tile_x) pair on the current GPU with CUDA events and returns the fastest;
 results are cached per device name in ``autotune_cache.json`` next to this file (created
-on first use, not part of the sources).  Results do not depend on the choice (the step is
-the same arithmetic for every shape), only the speed does.
+on first use, not part of the sources), keyed by the kernels' revision so that a choice
+saved for older ones is measured again.  The choice decides the speed only: results agree
+to rounding.
 """
 from __future__ import annotations
 
@@ -18,12 +19,13 @@ _HERE = os.path.dirname(os.path.abspath(__file__))
 CACHE = os.path.join(_HERE, "autotune_cache.json")
 _lock = threading.Lock()
 
+REVISION = 2   # of the step kernel's work splits (what a saved choice was measured on)
 LANES = (8, 16)
 TILES = (1, 2, 4, 8, 16)
 
 
 def _key(w, precision: str, device: str) -> str:
-    return "%s|%dx%d|bc%d%d|%s" % (device, w.nx, w.ny, w.bc_x, w.bc_y, precision)
+    return "r%d|%s|%dx%d|bc%d%d|%s" % (REVISION, device, w.nx, w.ny, w.bc_x, w.bc_y, precision)
 
 
 def _load() -> dict:
