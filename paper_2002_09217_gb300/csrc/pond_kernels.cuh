@@ -113,7 +113,7 @@ struct DevStats {
 __device__ __forceinline__ double w1d(int a) { return a == 1 ? 2.0 / 3.0 : 1.0 / 6.0; }
 
 // Index of a node after the boundary rule: periodic wrap or zero-gradient clamp.
-__device__ __forceinline__ int bc_wrap(int i, int n, int bc)
+__host__ __device__ __forceinline__ int bc_wrap(int i, int n, int bc)
 {
     if (bc == 0) {
         if (i >= 0 && i < n) return i;
@@ -123,6 +123,17 @@ __device__ __forceinline__ int bc_wrap(int i, int n, int bc)
         return i < 0 ? i + n : i;
     }
     return i < 0 ? 0 : (i >= n ? n - 1 : i);
+}
+
+// First stencil node of a departure point whose displacement from node X has the floor fl:
+// X + fl - 1, with fl limited to +-2^30 (NaN to the lower bound) before it becomes an int,
+// so that the sum, and the stencil's three further nodes, stay in int range whatever the
+// gauge (a diverging run's is infinite or NaN; bc_wrap of a sum past the int range is not a
+// node of the grid).  A grid has fewer than 2^30 nodes (304 bytes a node at the least).
+template <typename A>
+__host__ __device__ __forceinline__ int stencil_start(int X, A fl)
+{
+    return X + (int)fmin(fmax(fl, A(-1073741824)), A(1073741824)) - 1;
 }
 
 template <typename R> __device__ __forceinline__ R sqrt_(R x);

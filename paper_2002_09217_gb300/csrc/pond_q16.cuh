@@ -179,7 +179,7 @@ __device__ __forceinline__ IncRow<A> inc_row(const Lat16<A> &L, int k)
 
 // Cubic Lagrange weights on the nodes 0, 1, 2, 3 at xi (SM "Reconstruction").
 template <typename A>
-__device__ __forceinline__ void cubic_weights(A xi, A a[4])
+__host__ __device__ __forceinline__ void cubic_weights(A xi, A a[4])
 {
     const A x0 = xi, x1 = xi - A(1), x2 = xi - A(2), x3 = xi - A(3);
     a[0] = -(x1 * x2 * x3) / A(6);
@@ -193,12 +193,12 @@ __device__ __forceinline__ void cubic_weights(A xi, A a[4])
 // x0 .. x0 + 3 (x0 = floor(X - v dt) - 1); computed from the displacement so that FP32
 // keeps full precision on large grids.
 template <typename A>
-__device__ __forceinline__ int departure(int X, A v, A dt, A w[4])
+__host__ __device__ __forceinline__ int departure(int X, A v, A dt, A w[4])
 {
     const A d = -v * dt;
     const A fl = floor(d);
     cubic_weights<A>(d - fl + A(1), w);
-    return X + (int)fl - 1;
+    return stencil_start(X, fl);
 }
 
 // ---------------------------------------------------------------------------

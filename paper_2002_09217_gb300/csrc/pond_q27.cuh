@@ -96,7 +96,7 @@ __device__ __forceinline__ void inc_row3(int k, const A (&eps)[3], A (&out)[3])
 }
 
 template <typename A>
-__device__ __forceinline__ void cubic_w(A xi, A a[4])
+__host__ __device__ __forceinline__ void cubic_w(A xi, A a[4])
 {
     const A x0 = xi, x1 = xi - A(1), x2 = xi - A(2), x3 = xi - A(3);
     a[0] = -(x1 * x2 * x3) / A(6);
@@ -106,12 +106,12 @@ __device__ __forceinline__ void cubic_w(A xi, A a[4])
 }
 
 template <typename A>
-__device__ __forceinline__ int depart(int X, A v, A dt, A w[4])
+__host__ __device__ __forceinline__ int depart(int X, A v, A dt, A w[4])
 {
     const A d = -v * dt;
     const A fl = floor(d);
     cubic_w<A>(d - fl + A(1), w);
-    return X + (int)fl - 1;
+    return stencil_start(X, fl);
 }
 
 __device__ __forceinline__ double w27(int i) { return w1d(i % 3) * w1d((i / 3) % 3) * w1d(i / 9); }
