@@ -498,10 +498,11 @@ __device__ __forceinline__ void apply_inc(const A Dx[4][4], const A Dy[4][4], co
 }
 
 // ---------------------------------------------------------------------------
-// General stream, for departure points beyond the staged halo (|v| dt >= 1) and non-finite
-// gauges: reads the stencil nodes' records from global memory.  On a tensor lattice the union of a node's sixteen 4 x 4 departure
-// stencils is the product of the per-axis unions: W x H nodes with W (H) = 4 + the spread
-// of the four departure floors along the axis, 5 x 5 while |v| dt < 1 in every direction.
+// General stream, for departure points beyond the staged halo (|v| dt >= 1), tiles whose
+// velocities spread too far (FAR_SPEED) and non-finite gauges: reads the stencil nodes'
+// records from global memory.  On a tensor lattice the union of a node's sixteen 4 x 4
+// departure stencils is the product of the per-axis unions: W x H nodes with W (H) = 4 + the
+// spread of the four departure floors along the axis, 5 x 5 while |v| dt < 1 in every direction.
 // Each region node is carried into the arrival gauge once for all sixteen directions
 // (G f = f + [(I + Dy) (x) (I + Dx) - I] f), and direction i takes its Lagrange-weighted
 // share of component i.  The arithmetic per (direction, stencil node) pair is that of
@@ -854,7 +855,7 @@ __global__ void __launch_bounds__(STEP_THREADS, sizeof(R) == 4 ? Q16_MIN_BLOCKS 
     R *keep = reinterpret_cast<R *>(q16_dyn_smem + (size_t)STEP_THREADS * KW_N * 8) + threadIdx.x;
     R *slots = reinterpret_cast<R *>(q16_dyn_smem + (size_t)STEP_THREADS * (KW_N * 8 + KR_N * sizeof(R)));
     __shared__ StepCounts counts;
-    __shared__ uint4 best[STEP_THREADS / 32];
+    __shared__ uint4 best[BEST];
     const int tid = threadIdx.x;
     const size_t N = (size_t)p.N;
     const int TX = p.tile_x, TY = p.tile_y, WT = TX + 2 * HALO, nslots = step_slots(TX, TY);
@@ -868,17 +869,26 @@ __global__ void __launch_bounds__(STEP_THREADS, sizeof(R) == 4 ? Q16_MIN_BLOCKS 
     };
 
     // ---- staging: every record of the tile and its halo carried into the common gauge
-    Extremes ex;
-    for (int k = tid; k < nslots; k += STEP_THREADS) ex.offer((float)__ldg(in + rec_at(in, node_of(k), Q_TH, N)), k);
+    Extremes<2> ex;
+    for (int k = tid; k < nslots; k += STEP_THREADS) {
+        R g4[4];
+        ld4(in, node_of(k), N, Q_TH, g4);
+        ex.offer(g4[0], g4 + 1, k);
+    }
     ex = tile_extremes(ex, best);
-    const bool inc = sizeof(R) == 4 && ex.smooth();
+    bool inc = sizeof(R) == 4 && ex.smooth();
     const size_t nbase = node_of(min((int)ex.at, nslots - 1));
-    R gb[3];   // sqrt(theta), u_x, u_y of the tile's gauge
+    R gb[3];     // sqrt(theta), u_x, u_y of the tile's gauge
+    R dt_b = typed<R>(p).dt;   // infinite in a tile whose velocities spread too far (no contraction)
     {
         R g4[4], cold[4];
         ld4(in, nbase, N, Q_TH, g4);
         ld4(in, node_of(min((int)ex.lat, nslots - 1)), N, Q_TH, cold);
         common_gauge<R, 3>(inc, g4, cold, gb);
+        if (__syncthreads_or(ex.spread(gb))) {
+            inc = false;
+            if (!middle_gauge<R, 2>(ex, best, gb)) dt_b = R(1) / R(0);
+        }
         const R thb = inc ? g4[0] : gb[0] * gb[0], inv_sb = R(1) / gb[0];
 #pragma unroll 1
         for (int k = tid; k < nslots; k += STEP_THREADS) {
@@ -966,8 +976,7 @@ __global__ void __launch_bounds__(STEP_THREADS, sizeof(R) == 4 ? Q16_MIN_BLOCKS 
             const R s = sqrt_(th), inv_s = R(1) / s;
             R ax[4][4], ay[4][4];
             bool nx0[4], ny0[4];
-            const R dt = typed<R>(p).dt;
-            const bool okx = axis_weights16<R>(L, s, u[0], dt, ax, nx0), oky = axis_weights16<R>(L, s, u[1], dt, ay, ny0);
+            const bool okx = axis_weights16<R>(L, s, u[0], dt_b, ax, nx0), oky = axis_weights16<R>(L, s, u[1], dt_b, ay, ny0);
             if (okx && oky) {
                 auto side = [](const bool (&z)[4]) { return (z[0] == z[1] && z[1] == z[2] && z[2] == z[3]) ? 4 : 5; };
                 nreg += (unsigned)(side(nx0) * side(ny0) - (its == 1 ? 1 : 0));

@@ -391,10 +391,11 @@ __device__ __forceinline__ void axis3(A ds, A du, A D[3][3])
 }
 
 // ---------------------------------------------------------------------------
-// General stream, for departure points beyond the staged halo (|v| dt >= 1) and non-finite
-// gauges: reads the stencil nodes' records from global memory.  On the tensor lattice the union of a node's 27 departure stencils
-// (4 x 4 x 4 each) is the product of the per-axis unions: W x H x D nodes, each side 4 +
-// the spread of its axis's three departure floors (5 x 5 x 5 while |v| dt < 1).  Each
+// General stream, for departure points beyond the staged halo (|v| dt >= 1), tiles whose
+// velocities spread too far (FAR_SPEED) and non-finite gauges: reads the stencil nodes'
+// records from global memory.  On the tensor lattice the union of a node's 27 departure
+// stencils (4 x 4 x 4 each) is the product of the per-axis unions: W x H x D nodes, each side
+// 4 + the spread of its axis's three departure floors (5 x 5 x 5 while |v| dt < 1).  Each
 // region node is carried into the arrival gauge once for all 27 directions and every
 // direction adds its Lagrange-weighted share, with the per-(direction, node) arithmetic of
 // q27_stream: the region form transforms about 125 nodes per stream against 1,728 pairs.
@@ -1094,7 +1095,7 @@ __global__ void __launch_bounds__(Q27_THREADS, sizeof(R) == 4 ? 2 : 1)
     R *slots = reinterpret_cast<R *>(q27_dyn_smem);
     R *keep = slots + (size_t)SLOT_SPACE27 * Slot27<R>::stride + threadIdx.x;   // this thread's column (FP32)
     __shared__ StepCounts counts;
-    __shared__ uint4 best[Q27_THREADS / 32];
+    __shared__ uint4 best[BEST];
     const int tid = threadIdx.x;
     const size_t N = (size_t)p.N;
     const Tile27 tl{(int)blockIdx.x * T27X, (int)blockIdx.y * T27Y, (int)blockIdx.z * T27Z};
@@ -1106,11 +1107,14 @@ __global__ void __launch_bounds__(Q27_THREADS, sizeof(R) == 4 ? 2 : 1)
     if (tid == 0) counts = StepCounts{};
 
     // the tile's common gauge
-    Extremes ex;
-    for (int k = tid; k < SLOTS27; k += Q27_THREADS)
-        ex.offer((float)__ldg(in + rec_at(in, slot_node27(p, g3, tl, k), R_TH, N)), k);
+    Extremes<3> ex;
+    for (int k = tid; k < SLOTS27; k += Q27_THREADS) {
+        R gv[4];
+        load27<R_TH, 4>(in, slot_node27(p, g3, tl, k), N, gv);
+        ex.offer(gv[0], gv + 1, k);
+    }
     ex = tile_extremes(ex, best);
-    const bool inc = sizeof(R) == 4 && ex.smooth();
+    bool inc = sizeof(R) == 4 && ex.smooth();
     const size_t nbase = slot_node27(p, g3, tl, min((int)ex.at, SLOTS27 - 1));
     R gb[4], thb;
     {
@@ -1119,6 +1123,12 @@ __global__ void __launch_bounds__(Q27_THREADS, sizeof(R) == 4 ? 2 : 1)
         load27<R_TH, 4>(in, slot_node27(p, g3, tl, min((int)ex.lat, SLOTS27 - 1)), N, cold);
         common_gauge<R, 4>(inc, hot, cold, gb);
         thb = inc ? hot[0] : gb[0] * gb[0];
+    }
+    R dt_b = typed<R>(p).dt;   // infinite in a tile whose velocities spread too far (no contraction)
+    if (__syncthreads_or(ex.spread(gb))) {
+        inc = false;
+        if (!middle_gauge<R, 3>(ex, best, gb)) dt_b = R(1) / R(0);
+        thb = gb[0] * gb[0];
     }
 
     R th = R(1), u[3] = {R(0), R(0), R(0)};
@@ -1155,7 +1165,7 @@ __global__ void __launch_bounds__(Q27_THREADS, sizeof(R) == 4 ? 2 : 1)
         bool near0[3][3], fast = true;
 #pragma unroll
         for (int x = 0; x < 3; ++x) {
-            const bool ok = axis_weights<R>(s, u[x], typed<R>(p).dt, a[x], near0[x]);
+            const bool ok = axis_weights<R>(s, u[x], dt_b, a[x], near0[x]);
             fast = fast && ok;
             axis_rows<R>((gb[0] - s) * inv_s, (gb[1 + x] - u[x]) * inv_s, L[x]);
         }

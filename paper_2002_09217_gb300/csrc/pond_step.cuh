@@ -47,7 +47,8 @@
 // the populations, and it does not accumulate as a bias.  FP32 tiles of nearly equal theta
 // hold, moreover, differences to the populations of the tile's hottest node in its gauge,
 // in increment form (the map as I + E with E = 0 for equal gauges), so that weak waves are
-// not rounded to the populations' ulp; across an interface that form would cancel.
+// not rounded to the populations' ulp; across an interface that form would cancel, as it
+// would across a velocity jump (SMOOTH_SPREAD).
 #pragma once
 
 #include "pond_kernels.cuh"
@@ -67,6 +68,18 @@ constexpr int REGION_MAX = 8;
 // 4 to 6) the increment form left 6e-6 on single populations in three dimensions, the
 // direct form 1.7e-7.
 constexpr float SMOOTH_TILE = 0.9f;
+// Velocities.  Carried populations are amplified by the velocity between a node's gauge and
+// the tile's, in the increment form more than in the other.  Emulated in FP32 at uniform
+// theta, a node U sqrt(theta) from the tile's gauge gets back single populations with an error
+// of (D2Q9, D3Q27) 9e-8, 1e-7 in increment form at U = 0.4 and 7e-5, 3e-3 at 2; of 1.5e-7,
+// 2e-7 in direct form at 0.5, 4e-7, 9e-7 at 1 and 5e-6, 3e-5 at 1.5.  So a tile in which a
+// node moves faster than SMOOTH_SPREAD sqrt(theta_b) in the tile's gauge is staged in direct
+// form around the middle of its velocities, and one in which a node then still moves faster
+// than FAR_SPEED sqrt(theta_b) takes the general stream, which carries each node straight
+// into the arrival gauge.
+constexpr float SMOOTH_SPREAD = 0.4f;
+constexpr float FAR_SPEED = 1.0f;
+constexpr int BEST = 8;   // uint4 of shared memory in which a block agrees on its gauge
 // Mixed form: a frame-search residual below this multiple of tol that no longer halves is
 // taken as the FP32 rounding floor (the EoS cancels up to ~200x inside interfaces).
 constexpr float STALL_TOL_FACTOR = 16.0f;
@@ -652,23 +665,52 @@ struct Macro {
     }
 };
 
-// A tile's common gauge.  Each thread offers its staged nodes' thetas (finite positive
-// ones), then the block agrees on the nodes of the largest and the smallest (every thread
-// calls tile_extremes, which holds a barrier).
+// A tile's common gauge.  Each thread offers its staged nodes' gauges (those of finite
+// positive theta), then the block agrees on the nodes of the largest and the smallest theta
+// (every thread calls tile_extremes, which holds a barrier).  lo, hi: the velocity components
+// of the thread's own nodes.
+template <int D>
 struct Extremes {
     unsigned top = 0, at = 0, low = 0xffffffffu, lat = 0;   // theta bits and slots
-    __device__ __forceinline__ void offer(float th, int slot)
+    float lo[D], hi[D];
+    __device__ __forceinline__ Extremes()
     {
+#pragma unroll
+        for (int a = 0; a < D; ++a) { lo[a] = 1.0e38f; hi[a] = -1.0e38f; }
+    }
+    // u[0 .. D-1]: the velocity
+    template <typename R>
+    __device__ __forceinline__ void offer(R theta, const R *u, int slot)
+    {
+        const float th = (float)theta;
         if (!(th > 0.0f && th < 3.0e38f)) return;
         const unsigned b = __float_as_uint(th);
         if (b > top) { top = b; at = (unsigned)slot; }
         if (b < low) { low = b; lat = (unsigned)slot; }
+#pragma unroll
+        for (int a = 0; a < D; ++a) {
+            lo[a] = fminf(lo[a], (float)u[a]);
+            hi[a] = fmaxf(hi[a], (float)u[a]);
+        }
     }
     __device__ __forceinline__ float hottest() const { return __uint_as_float(top); }
     // the tile's thetas lie within SMOOTH_TILE of each other
     __device__ __forceinline__ bool smooth() const { return top != 0u && __uint_as_float(low) > SMOOTH_TILE * hottest(); }
+    // a node of this thread moves faster than SMOOTH_SPREAD in the gauge (sqrt theta, u)
+    template <typename R>
+    __device__ __forceinline__ bool spread(const R (&gb)[D + 1]) const
+    {
+        bool far = false;
+#pragma unroll
+        for (int a = 0; a < D; ++a) {
+            const float u = (float)gb[1 + a], lim = SMOOTH_SPREAD * (float)gb[0];
+            far = far || hi[a] - u > lim || u - lo[a] > lim;
+        }
+        return far;
+    }
 };
-__device__ __forceinline__ Extremes tile_extremes(Extremes t, uint4 *best)
+template <int D>
+__device__ __forceinline__ Extremes<D> tile_extremes(Extremes<D> t, uint4 *best)
 {
     const unsigned m = __reduce_max_sync(0xffffffffu, t.top), w = __reduce_min_sync(0xffffffffu, t.top == m ? t.at : 0xffffffffu);
     const unsigned n = __reduce_min_sync(0xffffffffu, t.low), v = __reduce_min_sync(0xffffffffu, t.low == n ? t.lat : 0xffffffffu);
@@ -693,6 +735,46 @@ __device__ __forceinline__ void common_gauge(bool inc, const R *hot, const R *co
     gb[0] = inc ? sqrt_(hot[0]) : sqrt_(sqrt_(hot[0]) * sqrt_(cold[0]));
 #pragma unroll
     for (int k = 1; k < ND; ++k) gb[k] = inc ? hot[k] : R(0.5) * (hot[k] + cold[k]);
+}
+// The gauge of a tile whose velocities spread: its extreme thetas' geometric mean and, along
+// each axis, the middle of the tile's velocities.  Returns whether all of them lie within
+// FAR_SPEED of it.  Every thread calls it, between barriers of its own use of `best`; it
+// holds one.
+__device__ __forceinline__ int ordered(float v)   // keeps the order of floats
+{
+    const int b = __float_as_int(v);
+    return b ^ ((b >> 31) & 0x7fffffff);
+}
+__device__ __forceinline__ float unordered(int b) { return __int_as_float(b ^ ((b >> 31) & 0x7fffffff)); }
+template <typename R, int D>
+__device__ __forceinline__ bool middle_gauge(const Extremes<D> &t, uint4 *best, R (&gb)[D + 1])
+{
+    static_assert(STEP_THREADS / 32 * 2 * D * 4 <= BEST * (int)sizeof(uint4), "best holds the warps' velocities");
+    int *w = reinterpret_cast<int *>(best);
+#pragma unroll
+    for (int a = 0; a < D; ++a) {
+        const int l = __reduce_min_sync(0xffffffffu, ordered(t.lo[a])), h = __reduce_max_sync(0xffffffffu, ordered(t.hi[a]));
+        if ((threadIdx.x & 31) == 0) {
+            w[(threadIdx.x >> 5) * 2 * D + a] = l;
+            w[(threadIdx.x >> 5) * 2 * D + D + a] = h;
+        }
+    }
+    __syncthreads();
+    gb[0] = sqrt_(sqrt_((R)t.hottest()) * sqrt_((R)__uint_as_float(t.low)));
+    bool near = true;
+#pragma unroll
+    for (int a = 0; a < D; ++a) {
+        int l = w[a], h = w[D + a];
+#pragma unroll 1
+        for (int k = 1; k < STEP_THREADS / 32; ++k) {
+            l = min(l, w[k * 2 * D + a]);
+            h = max(h, w[k * 2 * D + D + a]);
+        }
+        const R u = R(0.5) * (R)unordered(l), v = R(0.5) * (R)unordered(h);
+        gb[1 + a] = u + v;
+        near = near && v - u <= R(FAR_SPEED) * gb[0];
+    }
+    return near;
 }
 
 // Transfer increments along one axis, E[k][a] = l_k((a - 1) + e_a) - delta_ka with
@@ -764,13 +846,13 @@ __device__ __forceinline__ bool axis_weights(R s, R u, R dt, R (&a)[3][4], bool 
 }
 
 // General stream of node (X, Y) into the gauge (th, ux, uy), for departure points farther
-// than the staged halo (|v| dt >= 1) and non-finite gauges: reads the stencil nodes'
-// records from global memory.  Offsets are clamped to +-2^20 nodes first (a NaN offset
-// goes to the bound), so that the floors and their spread stay in int range.  Regions of
-// up to REGION_MAX nodes a side carry each node once for all nine directions; wider ones
-// take each direction's 16 stencil nodes in turn.  inc = the increments of the streamed
-// populations over the node's own (f, then g); of `lanes` callers, caller `lane` adds
-// every lanes-th stencil node only.
+// than the staged halo (|v| dt >= 1), tiles whose velocities spread too far (FAR_SPEED) and
+// non-finite gauges: reads the stencil nodes' records from global memory.  Offsets are
+// clamped to +-2^20 nodes first (a NaN offset goes to the bound), so that the floors and
+// their spread stay in int range.  Regions of up to REGION_MAX nodes a side carry each node
+// once for all nine directions; wider ones take each direction's 16 stencil nodes in turn.
+// inc = the increments of the streamed populations over the node's own (f, then g); of
+// `lanes` callers, caller `lane` adds every lanes-th stencil node only.
 template <typename R>
 __device__ __noinline__ void stream_general(const DevParams &p, const R *__restrict__ in, int X, int Y, R th, R ux,
                                             R uy, bool first, int lane, int lanes, R *inc, unsigned &nreg,
@@ -999,13 +1081,12 @@ __device__ __forceinline__ void contract(const double *own, int pitch, const dou
 
 // Streams node (X, Y) into the gauge (th, ux, uy): inc = the increments of the streamed
 // populations over the node's own (f, then g).  gauge_b: the tile's common gauge
-// (sqrt theta, u_x, u_y); keep: the thread's column of kept values.
+// (sqrt theta, u_x, u_y); dt: of stage_tile; keep: the thread's column of kept values.
 template <typename R>
 __device__ __forceinline__ void stream_node(const DevParams &p, const R *__restrict__ in, int X, int Y, const R *slot,
-                                            int pitch, const R (&gauge_b)[3], R th, R ux, R uy, bool first,
+                                            int pitch, const R (&gauge_b)[3], R dt, R th, R ux, R uy, bool first,
                                             R *keep, R (&inc)[2][9], unsigned &nreg, unsigned &npair)
 {
-    const R dt = typed<R>(p).dt;
     const R s = sqrt_(th), inv_s = R(1) / s;
     R ax[3][4], ay[3][4];
     bool nx0[3], ny0[3];
@@ -1245,10 +1326,12 @@ __device__ __forceinline__ Tile<R> make_tile(const DevParams &p, int idx, R *sme
 }
 
 // Stages a tile and its halo (see the head of this file) and computes K and q on the tile
-// and its ring; gb = the tile's common gauge: sqrt(theta), u_x, u_y.  Every thread of the
-// block calls it; it ends with a barrier.
+// and its ring; gb = the tile's common gauge: sqrt(theta), u_x, u_y.  Returns the time step
+// of the contraction's departure points: dt, or infinity, which no contraction takes, in a
+// tile whose velocities spread too far for it.  Every thread of the block calls it; it ends
+// with a barrier.
 template <typename R>
-__device__ __forceinline__ void stage_tile(const DevParams &p, const R *__restrict__ in, const R *nlsrc,
+__device__ __forceinline__ R stage_tile(const DevParams &p, const R *__restrict__ in, const R *nlsrc,
                                            const Tile<R> &tl, StepCounts &counts, R (&gb)[3])
 {
     constexpr int DS = Slot<R>::stride, ST_NT = STEP_THREADS;
@@ -1257,7 +1340,7 @@ __device__ __forceinline__ void stage_tile(const DevParams &p, const R *__restri
     const int tid = threadIdx.x;
     const int X0 = tl.X0, Y0 = tl.Y0, TX = tl.TX, TY = tl.TY, WT = tl.WT, nslots = tl.nslots;
     R *aux = tl.aux, *slots = tl.slots, *kq = tl.kq;
-    __shared__ uint4 best[ST_NT / 32];   // per warp: largest and smallest theta (bits) and their slots
+    __shared__ uint4 best[BEST];   // per warp: largest and smallest theta (bits) and their slots; velocities
     if (tid == 0) counts = StepCounts{};
     // k / WT through the float reciprocal: exact for k < 2^20 (the quotient's fraction
     // stays >= 0.5 / WT away from an integer)
@@ -1280,13 +1363,14 @@ __device__ __forceinline__ void stage_tile(const DevParams &p, const R *__restri
     R va[24], vb[24];
     const int ka = tid, kb = tid + ST_NT;
     size_t na = 0, nb = 0;
-    Extremes ex;
+    Extremes<2> ex;
     if (ka < nslots) { na = node_of(ka); load_rec24(in, na, N, va); }
     if (kb < nslots) { nb = node_of(kb); load_rec24(in, nb, N, vb); }
     // every slot's gauge goes to shared memory (where its rho, T will lie), so that the
     // agreed nodes' gauges and populations need no further global loads
     auto note = [&](int k, R th, R ux, R uy) {
-        ex.offer((float)th, k);
+        const R u[2] = {ux, uy};
+        ex.offer(th, u, k);
         R *a = aux + (size_t)k * AUXW;
         a[0] = th; a[1] = ux; a[2] = uy;
     };
@@ -1297,7 +1381,7 @@ __device__ __forceinline__ void stage_tile(const DevParams &p, const R *__restri
         note(k, __ldg(in + rec_at(in, nd, P_TH, N)), __ldg(in + rec_at(in, nd, P_UX, N)), __ldg(in + rec_at(in, nd, P_UY, N)));
     }
     ex = tile_extremes(ex, best);
-    const bool smooth = sizeof(R) == 4 && ex.smooth();
+    bool smooth = sizeof(R) == 4 && ex.smooth();
     const int khot = min((int)ex.at, nslots - 1), kcold = min((int)ex.lat, nslots - 1);
     R thb;
     {
@@ -1324,7 +1408,13 @@ __device__ __forceinline__ void stage_tile(const DevParams &p, const R *__restri
             for (int i = 0; i < 18; ++i) base[i] = __ldg(in + rec_at(in, nd, i, N));
         }
     }
-    __syncthreads();   // base is there, and aux may be overwritten
+    // (the barrier: base is there, and aux may be overwritten)
+    R dt = q.dt;
+    if (__syncthreads_or(ex.spread(gb))) {
+        smooth = false;
+        if (!middle_gauge<R, 2>(ex, best, gb)) dt = R(1) / R(0);
+        thb = gb[0] * gb[0];
+    }
     const R inv_sb = R(1) / gb[0];
     auto carry = [&](int k, size_t nd, const R (&v)[24]) {
         const R sn = sqrt_(v[P_TH]);
@@ -1403,6 +1493,7 @@ __device__ __forceinline__ void stage_tile(const DevParams &p, const R *__restri
         }
     }
     __syncthreads();
+    return dt;
 }
 
 // Adds a block's counters (its warps' values) to the context's.  Every thread calls it.
@@ -1498,7 +1589,7 @@ __device__ __forceinline__ void step_tile(const DevParams &p, const R *__restric
     __shared__ StepCounts counts;
     const Tile<R> tl = make_tile<R>(p, tile_idx, smem);
     R gb[3];
-    stage_tile<R>(p, in, nlsrc, tl, counts, gb);
+    const R dt = stage_tile<R>(p, in, nlsrc, tl, counts, gb);
     const int tx = tid % tl.TX, ty = tid / tl.TX;
     const int X = tl.X0 + tx, Y = tl.Y0 + ty;
     const bool valid = ty < tl.TY && X < p.nx && Y < p.ny;   // (a tile may have fewer nodes than threads)
@@ -1554,7 +1645,7 @@ __device__ __forceinline__ void step_tile(const DevParams &p, const R *__restric
         float last = 3.0e38f;   // previous residual
         for (;;) {
             ++its;
-            stream_node<R>(p, in, X, Y, tl.slots + (size_t)slot * DS, tl.WT, gb, th, ux, uy, its == 1, keep, inc,
+            stream_node<R>(p, in, X, Y, tl.slots + (size_t)slot * DS, tl.WT, gb, dt, th, ux, uy, its == 1, keep, inc,
                            nreg, npair);
             R sum[4] = {R(0), R(0), R(0), R(0)};
 #pragma unroll
@@ -1657,7 +1748,7 @@ __device__ __forceinline__ void step_tile_split(const DevParams &p, const R *__r
     __shared__ StepCounts counts;
     const Tile<R> tl = make_tile<R>(p, tile_idx, smem);
     R gb[3];
-    stage_tile<R>(p, in, nlsrc, tl, counts, gb);
+    const R dt = stage_tile<R>(p, in, nlsrc, tl, counts, gb);
 
     const int ln = threadIdx.x & 31, lq = ln < 27 ? ln : ln - 9;
     const int base = lq < 9 ? 0 : (lq < 18 ? 9 : 18);
@@ -1704,7 +1795,7 @@ __device__ __forceinline__ void step_tile_split(const DevParams &p, const R *__r
     EosOut<R> o{};
     float last = 3.0e38f;
     for (unsigned it = 1; __any_sync(ALL, active); ++it) {
-        const R s = sqrt_(th), inv_s = R(1) / s, dt = q.dt;
+        const R s = sqrt_(th), inv_s = R(1) / s;
         // departure along x of component k, along y of component l; the other y components'
         // weights come from the lanes that hold them
         R wx[4], wy[3][5], Lx[3], Ly[3];
