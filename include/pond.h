@@ -122,10 +122,10 @@ typedef struct {
  * stream: a cudaStream_t (NULL = default stream).
  * dalloc/dfree/alloc_ctx: optional device allocator (both or neither).
  * lanes_per_node: work split of the D2Q9 step kernel: 8 = one thread per node (blocks of
- * 128 nodes), 16 = nine lanes per node (blocks of 12 nodes, for small grids), 0 = by grid
- * size.  tile_x: width of a block's tile of nodes, 1, 2, 4, 8 or 16 (its height is the
- * block's nodes divided by it; with nine lanes per node 8 and 16 mean 6 and 12), 0 = by the
- * grid's rows.  Both are performance knobs (autotuning); results are the same to rounding.
+ * 128 nodes; in FP64 as 0, since small grids take up to 3.8 times as long with it), 16 = nine
+ * lanes per node (blocks of 12 nodes, for small grids), 0 = by grid size.  tile_x: width of a
+ * block's tile of nodes, 1, 2, 4, 8 or 16 (its height is the block's nodes divided by it;
+ * with nine lanes per node 8 and 16 mean 6 and 12), 0 = by the grid's shape.  Both are performance knobs (autotuning); results are the same to rounding.
  * The D2Q16 kernel takes tile_x (of 128 nodes); the D3Q27 kernel ignores both.
  * In the mixed form the moments, e->T, EoS and frame-search residual are float-float; the
  * storage-rounding remainders of mass, momentum and energy are kept beside each

@@ -19,7 +19,7 @@ _HERE = os.path.dirname(os.path.abspath(__file__))
 CACHE = os.path.join(_HERE, "autotune_cache.json")
 _lock = threading.Lock()
 
-REVISION = 2   # of the step kernel's work splits (what a saved choice was measured on)
+REVISION = 3   # of the step kernel's work splits (what a saved choice was measured on)
 LANES = (8, 16)
 TILES = (1, 2, 4, 8, 16)
 

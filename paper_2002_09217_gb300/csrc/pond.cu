@@ -99,26 +99,6 @@ void dev_free(pond_ctx *c, void *p)
 
 inline unsigned blocks_for(size_t n, unsigned bs) { return (unsigned)((n + bs - 1) / bs); }
 
-// Largest grid (nodes) stepped with nine lanes per node.  One thread per node leaves most
-// of the GPU idle below about 150 blocks of 128 nodes and a step then costs one block's
-// serial time (mixed 20-23 us, FP64 400-460 us whatever the grid); nine lanes per node cut
-// that time but do more work in all.  Measured (us per step, thread / nine lanes), mixed:
-// 128 x 4 19.5 / 12.0, 2048 x 1 23.0 / 12.6, 64 x 64 22.2 / 16.6, 96 x 96 22.2 / 26.8; FP64:
-// 128 x 4 401 / 110, 64 x 64 459 / 241, 96 x 96 459 / 423, 128 x 128 460 / 693.  The mixed
-// limit is below the lone crossing (about 6,500 nodes) because a context keeps its split in a
-// batch, where the other members fill the GPU and the extra work counts: twelve grids of
-// 64 x 64 to 164 x 160 nodes took 59 us a step with the smallest on nine lanes.
-size_t split_max_nodes(int precision) { return precision == POND_MIXED ? 3072 : 10000; }
-
-// Strips of up to four rows stepped with one thread per node take tiles of 64 nodes while
-// that is at most one block per SM (152 x 64 nodes): with 128 fewer than half of the SMs
-// would work, and a step costs one block's serial time, which falls with the slots it stages.
-// Measured (mixed, us per step, 128 / 64 / 32 nodes): 2048 x 4 15.0 / 13.6 / 14.2, 4096 x 2
-// 16.0 / 13.7 / 13.4, 8192 x 1 17.6 / 14.9 / 14.2, 1600 x 3 14.4 / 13.3 / 13.7.  Grids of more
-// rows keep 128: they are what batches hold, where the wider halo share counts.
-constexpr int STRIP_NB = 64;
-constexpr size_t STRIP_MAX_NODES = 152 * STRIP_NB;
-
 bool mixed(const pond_ctx *c) { return c->opts.precision == POND_MIXED; }
 
 // Tiles of the D2Q9 step kernel over the grid.
@@ -617,39 +597,25 @@ pond_status pond_create(const pond_grid *grid, const pond_lattice *lattice, cons
     c->N = (size_t)grid->nx * (size_t)grid->ny * (size_t)(grid->nz > 1 ? grid->nz : 1);
     if (c->lattice == POND_D3Q27) c->g3 = Grid3{grid->nz, grid->bc_z};
     c->esize = opts->precision == POND_MIXED ? sizeof(float) : sizeof(double);
-    // Work split of the D2Q9 step: one thread per node (8) or nine lanes per node (16).
-    // (The other lattices' kernels have one split and share the tile rule.)
-    c->lanes = opts->lanes_per_node ? opts->lanes_per_node : (c->N <= split_max_nodes(opts->precision) ? 16 : 8);
-    if (c->lattice != POND_D2Q9) c->lanes = 8;
-    // Its tile: TX x TY nodes of STEP_NB (SPLIT_NB; STRIP_NB) nodes, by default no taller than
-    // the grid and otherwise 16 x 8 (4 x 3)
-    int tile_x = opts->tile_x, tile_y;
-    if (c->lanes == 16) {
-        if (!tile_x) tile_x = grid->ny == 1 ? 12 : (grid->ny == 2 || grid->ny == 4 ? 6 : 4);
-        else if (tile_x == 8) tile_x = 6;
-        else if (tile_x == 16) tile_x = 12;
-        tile_y = SPLIT_NB / tile_x;
-    } else {
-        const bool strip = !tile_x && c->lattice == POND_D2Q9 && grid->ny <= 4 && c->N <= STRIP_MAX_NODES;
-        const int nodes = strip ? STRIP_NB : STEP_NB;
-        if (!tile_x)
-            for (tile_x = 16; tile_x < nodes && nodes / (2 * tile_x) >= grid->ny; tile_x *= 2) {}
-        tile_y = nodes / tile_x;
-    }
     cudaError_t e = cudaGetDevice(&c->device);
+    int sms = 0;
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
     if (e == cudaSuccess)
         e = opts->precision == POND_MIXED ? allow_step_smem<float>() : allow_step_smem<double>();
     if (e != cudaSuccess) {
         delete c;
         return POND_ECUDA;
     }
+    const StepShape shape = step_shape(c->lattice == POND_D2Q9, opts->precision == POND_MIXED, grid->nx, grid->ny,
+                                       opts->lanes_per_node, opts->tile_x, sms);
+    c->lanes = shape.lanes;
     DevParams &d = c->dp;
     d.nx = grid->nx; d.ny = grid->ny; d.bcx = grid->bc_x; d.bcy = grid->bc_y;
     d.N = (long long)c->N;
     d.a = c->eos.a; d.b = c->eos.b; d.R = c->eos.R; d.delta = c->eos.delta; d.cv = c->eos.R / c->eos.delta;
     d.kappa = kappa; d.tau = tau; d.omega = 1.0 / tau; d.dt = opts->dt; d.k_cond = opts->k_cond;
     d.p_floor = opts->p_floor; d.tol = opts->tol; d.max_iter = opts->max_iter;
-    d.tile_x = tile_x; d.tile_y = tile_y; d.tiles_x = (grid->nx + tile_x - 1) / tile_x;
+    d.tile_x = shape.tx; d.tile_y = shape.ty; d.tiles_x = (grid->nx + shape.tx - 1) / shape.tx;
     d.pd.a = d.a; d.pd.b = d.b; d.pd.R = d.R; d.pd.cv = d.cv; d.pd.inv_cv = 1.0 / d.cv;
     d.pd.kappa = d.kappa; d.pd.p_floor = d.p_floor; d.pd.dt = d.dt; d.pd.omega = d.omega;
     d.pd.mu_coef = (d.tau - 0.5) * d.dt; d.pd.cvR = d.cv + d.R; d.pd.k_cond = d.k_cond;

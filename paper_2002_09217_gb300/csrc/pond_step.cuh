@@ -116,6 +116,61 @@ __host__ __device__ constexpr size_t step_smem_bytes(int tx, int ty, bool split,
             (split ? (size_t)SPLIT_NB * SPLIT_WORDS : (size_t)STEP_THREADS * KEEP)) * elem_bytes;
 }
 
+// Work split (8: one thread per node, 16: nine lanes per node) and tile of the D2Q9 step on an
+// nx x ny grid; D2Q16 has one split and shares the tile rule.  lanes, tile_x: the caller's
+// choice, 0 = by size.
+//
+// Nine lanes.  A step of a small grid costs one block's serial time: one thread per node
+// 14.4 us (mixed) and 395 us (FP64), whatever the grid; nine lanes per node less, until their
+// blocks of 12 nodes need further turns on the SMs.  Mixed: while all of them are resident at
+// once, two on each SM (us a step, thread / nine lanes: 128 x 4 13.9 / 10.9, 64 x 48 14.4 /
+// 13.0, 64 x 64 14.5 / 20.1).  FP64: up to five an SM (128 x 4 377 / 105, 64 x 64 395 / 265,
+// 90 x 90 396 / 376, 96 x 96 395 / 424).  FP64 grids take them also where the caller asks for
+// 8: the eight lanes a node of earlier kernels took 242 us on small grids, a thread 396.
+//
+// Tile.  One thread per node: 16 x 8, no taller than the grid for grids of few rows, and no
+// wider than the grid for those of few columns once there is more than one block an SM (us a
+// step in 16 x 8 / narrower tiles: 4 x 20000 mixed 118 / 46; D2Q16 mixed 1 x 4096 78.7 / 50.7,
+// 2 x 2048 51.0 / 44.8, but 4 x 1024, one turn in either, 44.6 / 47.7: a narrow tile stages
+// more slots).  Nine lanes: 4 x 3 and alike (1 x 2048 mixed: 29.9 in 4 x 3, 12.1 in 1 x 12).
+// Strips of up to four rows or columns take tiles of 32 or 64 nodes while that is at most one
+// block an SM, because the serial time falls with the slots a block stages (mixed, tiles of
+// 128 / 64 / 32 nodes: 1024 x 4 15.2 / 13.9 / 13.6, 4096 x 1 17.6 / 14.9 / 13.8, 4096 x 2 16.0
+// / 13.8 / 13.6, 8192 x 1 17.7 / 14.7 / 14.3, 1600 x 3 14.7 / 13.6 / 13.7, 2400 x 4 15.0 / 13.9
+// / 13.9, 2048 x 4 15.5 / 13.9 / 13.9 and as a shock tube 64 nodes 3 % ahead of 32; beyond
+// one block an SM, 5000 x 4 16.0 / 18.1 / 22.5).  Grids of more rows and columns gain 1 to 4 %
+// from small tiles (1024 x 8 14.6 / 14.0 / 14.1, 90 x 90 14.8 / 14.6 / 14.3) and keep 128:
+// they are what batches hold, where the other members fill the GPU and the wider share of the
+// halo counts (128 x 128, which nearly fills it by itself, 15.3 / 19.2 / 21.1).
+struct StepShape {
+    int lanes, tx, ty;
+    long long blocks(int nx, int ny) const { return (long long)((nx + tx - 1) / tx) * ((ny + ty - 1) / ty); }
+};
+inline StepShape step_shape(bool d2q9, bool mixed, int nx, int ny, int lanes, int tile_x, int sms)
+{
+    if (d2q9 && (lanes != 8 || !mixed)) {
+        StepShape s{16, tile_x, 0};
+        if (!s.tx) s.tx = nx < 4 ? nx : (ny == 1 ? 12 : (ny == 2 || ny == 4 ? 6 : 4));
+        else if (s.tx == 8) s.tx = 6;
+        else if (s.tx == 16) s.tx = 12;
+        s.ty = SPLIT_NB / s.tx;
+        if (lanes == 16 || s.blocks(nx, ny) <= (long long)(mixed ? SPLIT_MIN_BLOCKS(float) : 5) * sms) return s;
+    }
+    if (tile_x) return {8, tile_x, STEP_NB / tile_x};
+    auto fit = [&](int nodes, int tx, bool narrow) {
+        while (tx < nodes && nodes / (2 * tx) >= ny) tx *= 2;
+        StepShape s{8, tx, nodes / tx};
+        while (s.tx > 1 && s.tx / 2 >= nx && (narrow || s.blocks(nx, ny) > sms)) s = {8, s.tx / 2, 2 * s.ty};
+        return s;
+    };
+    if (d2q9 && (nx <= 4 || ny <= 4))
+        for (int nodes = 32; nodes < STEP_NB; nodes *= 2) {
+            const StepShape s = fit(nodes, 8, true);
+            if (s.blocks(nx, ny) <= sms) return s;
+        }
+    return fit(STEP_NB, 16, false);
+}
+
 // Counters of one block, summed into the context's by its last instructions.
 struct StepCounts {
     unsigned streams, region_nodes, pair_streams, nonconv, stalled, clamped, nonfinite, warp_streams, max_streams;
