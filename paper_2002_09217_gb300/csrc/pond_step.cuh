@@ -59,6 +59,7 @@ constexpr int STEP_THREADS = 128;   // threads per block
 constexpr int STEP_NB = 128;        // nodes per block, one thread per node
 constexpr int SPLIT_NB = 12;        // nodes per block, nine lanes per node (three nodes per warp)
 constexpr int HALO = 2;       // staged halo: stencil reach for |v| dt < 1, and of the non-local terms
+constexpr int HALO_FAR = 3;   // and for |v| dt < 2 (D2Q9, FP64)
 // Largest side of a node's stencil region (the union of its 9 directions' 4x4 stencils)
 // that the general stream handles as a region; wider ones take the per-pair stream.
 constexpr int REGION_MAX = 8;
@@ -99,7 +100,7 @@ constexpr int AUXW = 4;   // rho, T, p, p/rho of a staged node
 constexpr int SPLIT_WORDS = SL + 9 * 18;   // nine lanes per node: the own record, the lanes' partials
 constexpr int KQW = 5;    // K_xx, K_xy, K_yy, q_x, q_y of a node of the tile and its ring
 
-__host__ __device__ constexpr int step_slots(int tx, int ty) { return (tx + 2 * HALO) * (ty + 2 * HALO); }
+__host__ __device__ constexpr int step_slots(int tx, int ty, int halo = HALO) { return (tx + 2 * halo) * (ty + 2 * halo); }
 
 // What a thread of the one-thread-per-node form keeps in shared memory across the stream
 // instead of in registers (a column of KEEP values; the contraction's weights then fit 168
@@ -107,12 +108,22 @@ __host__ __device__ constexpr int step_slots(int tx, int ty) { return (tx + 2 * 
 // F, rho E_lambda, M_0, and the y weights and rows of the map.
 enum : int { K_HI = 0, K_LO = 4, K_F = 8, K_REL = 10, K_M0 = 11, K_WY = 12, K_LY = 27, KEEP = 36 };
 
+// Halo that a tile's shared memory holds.  FP64: the wider one where it costs no resident
+// block (16 x 8 nodes: 205 instead of 179 KB of an SM's memory for two blocks; long tiles of
+// 128 nodes would lose one).  FP32 tiles do without: carrying the populations into the tile's
+// gauge rounds them once more, which at the velocities of such flows doubles the error of p
+// (u = 2.6, -1.9 in a droplet: 1.9e-5 -> 3.5e-5), and asking every tile cost 2 % of a step.
+__host__ __device__ constexpr int widest_halo(int tx, int ty, int elem_bytes)
+{
+    return elem_bytes == 8 && (tx * ty < STEP_NB || (tx >= 8 && ty >= 8)) ? HALO_FAR : HALO;
+}
+
 // Dynamic shared memory of one step block: slots' rho, T, p, p/rho; populations; K and q;
 // then the threads' kept values, or with nine lanes per node the partials of the general
 // stream and the own records.
 __host__ __device__ constexpr size_t step_smem_bytes(int tx, int ty, bool split, int slot_values, int elem_bytes)
 {
-    return ((size_t)step_slots(tx, ty) * (AUXW + slot_values) + (size_t)(tx + 2) * (ty + 2) * KQW +
+    return ((size_t)step_slots(tx, ty, widest_halo(tx, ty, elem_bytes)) * (AUXW + slot_values) + (size_t)(tx + 2) * (ty + 2) * KQW +
             (split ? (size_t)SPLIT_NB * SPLIT_WORDS : (size_t)STEP_THREADS * KEEP)) * elem_bytes;
 }
 
@@ -763,6 +774,14 @@ struct Extremes {
         }
         return far;
     }
+    // with sqrt theta = s, a node of this thread moves |v| dt >= 1 along an axis
+    __device__ __forceinline__ bool reach(float s, float dt) const
+    {
+        float m = s;
+#pragma unroll
+        for (int a = 0; a < D; ++a) m = fmaxf(m, fmaxf(s + hi[a], s - lo[a]));
+        return m * dt >= 1.0f;
+    }
 };
 template <int D>
 __device__ __forceinline__ Extremes<D> tile_extremes(Extremes<D> t, uint4 *best)
@@ -908,6 +927,12 @@ __device__ __forceinline__ bool axis_weights(R s, R u, R dt, R (&a)[3][4], bool 
 // once for all nine directions; wider ones take each direction's 16 stencil nodes in turn.
 // inc = the increments of the streamed populations over the node's own (f, then g); of
 // `lanes` callers, caller `lane` adds every lanes-th stencil node only.
+// One thread per node is bound by its serial chain of region nodes where few blocks fill an
+// SM.  Measured (mixed, us a step, eight lanes a node over a staged halo of three, as in
+// earlier kernels / this): a droplet at 1.4 T_cr and dt = 1, 256 x 256 nodes 133 / 148, 40 x 28
+// 26 / 34; at 2.7 T_cr, 128 x 128 nodes 75 / 362; a flow at |v| dt = 1.3, 512 x 256 nodes 243 /
+// 233, 128 x 128 51 / 98, 30 x 9 25 / 32.  (The next record's loads sent ahead: slower, 406
+// instead of 362, and 7 % on a step that never comes here, by the registers.)
 template <typename R>
 __device__ __noinline__ void stream_general(const DevParams &p, const R *__restrict__ in, int X, int Y, R th, R ux,
                                             R uy, bool first, int lane, int lanes, R *inc, unsigned &nreg,
@@ -1134,10 +1159,151 @@ __device__ __forceinline__ void contract(const double *own, int pitch, const dou
     }
 }
 
+// The streamed populations of one direction (k, l) as a contraction over the direction's own
+// 4 x 4 staged slots: first the nodes by their Lagrange weights, then the rows of the map.  For
+// departure floors other than -1 and 0 (fx, fy), which the window of `contract` does not hold.
+__device__ __forceinline__ void contract_one(const double *own, int pitch, const double (&ax)[4], int fx,
+                                             const double (&ay)[4], int fy, const double (&Lx)[3], const double (&Ly)[3],
+                                             double &of, double &og)
+{
+    constexpr int DS = Slot<double>::stride;
+    double a[18];
+#pragma unroll
+    for (int i = 0; i < 18; ++i) a[i] = 0.0;
+    const double *row = own + ((fy - 1) * pitch + fx - 1) * DS;
+#pragma unroll 1
+    for (int r = 0; r < 4; ++r, row += pitch * DS) {
+        const double wr = r < 2 ? (r == 0 ? ay[0] : ay[1]) : (r == 2 ? ay[2] : ay[3]);
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            const double w = ax[c] * wr;
+#pragma unroll
+            for (int i = 0; i < 18; ++i) a[i] = fma(w, row[c * DS + i], a[i]);
+        }
+    }
+    of = og = 0.0;
+#pragma unroll
+    for (int n = 0; n < 3; ++n) {
+        of = fma(Ly[n], Lx[0] * a[3 * n] + Lx[1] * a[3 * n + 1] + Lx[2] * a[3 * n + 2], of);
+        og = fma(Ly[n], Lx[0] * a[9 + 3 * n] + Lx[1] * a[9 + 3 * n + 1] + Lx[2] * a[9 + 3 * n + 2], og);
+    }
+}
+
+// Weights and floor of the departure point x - v dt; whether its stencil lies within HALO_FAR
+// nodes of the arrival node (false for NaN).
+template <typename R>
+__device__ __forceinline__ bool far_departure(R v, R dt, R (&a)[4], int &floor_)
+{
+    const R d = -v * dt;
+    const R f = floor(d);
+    const bool ok = f >= R(1 - HALO_FAR) && f <= R(HALO_FAR - 2);
+    floor_ = ok ? (int)f : 0;
+    const R t0 = d - f + R(1), t1 = t0 - R(1), t2 = t0 - R(2), t3 = t0 - R(3);
+    const R p12 = t1 * t2, p03 = t0 * t3;
+    a[0] = p12 * t3 * R(-1.0 / 6.0);
+    a[1] = p03 * t2 * R(0.5);
+    a[2] = p03 * t1 * R(-0.5);
+    a[3] = p12 * t0 * R(1.0 / 6.0);
+    return ok;
+}
+// Row k (run time) of the map: l_k at (1 + q) (m - 1) + w.
+template <typename R>
+__device__ __forceinline__ void map_row(int k, R q, R w, R (&L)[3])
+{
+#pragma unroll
+    for (int m = 0; m < 3; ++m) {
+        const R x = m == 1 ? w : (R(1) + q) * R(m - 1) + w;
+        L[m] = k == 1 ? (R(1) - x) * (R(1) + x) : R(0.5) * x * (x + R(k - 1));
+    }
+}
+
+// The streamed populations of direction (k, l) where the wider halo holds its stencil (ok).
+struct FarOne { double f, g; int fx, fy; bool ok; };
+__device__ __noinline__ FarOne far_one(const double *own, int pitch, int k, int l, double sb, double ubx, double uby,
+                                       double s, double inv_s, double dt, double ux, double uy)
+{
+    FarOne o{0.0, 0.0, 0, 0, false};
+    double ax[4], ay[4], Lx[3], Ly[3];
+    const bool okx = far_departure<double>(s * (k - 1) + ux, dt, ax, o.fx), oky = far_departure<double>(s * (l - 1) + uy, dt, ay, o.fy);
+    o.ok = okx && oky;
+    map_row<double>(k, (sb - s) * inv_s, (ubx - ux) * inv_s, Lx);
+    map_row<double>(l, (sb - s) * inv_s, (uby - uy) * inv_s, Ly);
+    if (o.ok) contract_one(own, pitch, ax, o.fx, ay, o.fy, Lx, Ly, o.f, o.g);
+    return o;
+}
+
+// FP64, over slots with the wider halo: streams a node whose departure points leave the window
+// of `contract`, where that halo holds them as a contraction over 7 rows, of each x
+// component's own four columns, else in general.  buf = the increments of the streamed
+// populations over the node's own.  Measured (us a step, the eight-lane kernels / the general
+// stream / this): a droplet at 1.4 T_cr, dt = 1, 256 x 256 nodes 4498 / 4607 / 2202; at 2.7
+// T_cr, 128 x 128 nodes 1973 / 4145 / 1050; a flow at |v| dt = 1.3, 128 x 128 nodes 1194 / 1139
+// / 580, with nine lanes 30 x 9 nodes 208 / 281 / 197.
+__device__ __noinline__ void stream_far(const DevParams &p, const double *__restrict__ in, int X, int Y,
+                                        const double *own, int pitch, double sb, double ubx, double uby,
+                                        double dt, double th, double ux, double uy, bool first, double *buf,
+                                        unsigned &nreg, unsigned &npair)
+{
+    constexpr int DS = Slot<double>::stride;
+    const double s = sqrt_(th), inv_s = 1.0 / s;
+    double wx[3][4], wy[3][4];
+    int fx[3], fy[3];
+    bool far = true;
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+        far = far_departure<double>(s * (j - 1) + ux, dt, wx[j], fx[j]) && far;
+        far = far_departure<double>(s * (j - 1) + uy, dt, wy[j], fy[j]) && far;
+    }
+    if (!far) {
+        stream_general<double>(p, in, X, Y, th, ux, uy, first, 0, 1, buf, nreg, npair);
+        return;
+    }
+    nreg += (unsigned)((4 + max(fx[0], max(fx[1], fx[2])) - min(fx[0], min(fx[1], fx[2]))) *
+                           (4 + max(fy[0], max(fy[1], fy[2])) - min(fy[0], min(fy[1], fy[2]))) - (first ? 1 : 0));
+    double Lx[3][3], Ly[3][3], acc[2][9];
+    const double qb = (sb - s) * inv_s;
+    axis_rows<double>(qb, (ubx - ux) * inv_s, Lx);
+    axis_rows<double>(qb, (uby - uy) * inv_s, Ly);
+#pragma unroll
+    for (int i = 0; i < 9; ++i) acc[0][i] = acc[1][i] = 0.0;
+#pragma unroll 1
+    for (int r = -HALO_FAR; r <= HALO_FAR; ++r) {
+        double wr[3];
+#pragma unroll
+        for (int l = 0; l < 3; ++l) {
+            const int j = r - fy[l] + 1;   // the row's place in the stencil of component l
+            wr[l] = (j >= 0 && j < 4) ? pick(wy[l], j) : 0.0;
+        }
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            const double *c0 = own + (r * pitch + fx[k] - 1) * DS;
+#pragma unroll
+            for (int fam = 0; fam < 2; ++fam)
+#pragma unroll
+                for (int n = 0; n < 3; ++n) {
+                    double t = 0.0;
+#pragma unroll
+                    for (int m = 0; m < 3; ++m) {
+                        double v = 0.0;
+#pragma unroll
+                        for (int c = 0; c < 4; ++c) v = fma(wx[k][c], c0[c * DS + 9 * fam + 3 * n + m], v);
+                        t = fma(Lx[k][m], v, t);
+                    }
+#pragma unroll
+                    for (int l = 0; l < 3; ++l) acc[fam][3 * l + k] = fma(wr[l] * Ly[l][n], t, acc[fam][3 * l + k]);
+                }
+        }
+    }
+    double v[24];
+    load_rec24(in, (size_t)Y * p.nx + X, (size_t)p.N, v);
+#pragma unroll
+    for (int i = 0; i < 18; ++i) buf[i] = acc[i / 9][i % 9] - v[i];
+}
+
 // Streams node (X, Y) into the gauge (th, ux, uy): inc = the increments of the streamed
 // populations over the node's own (f, then g).  gauge_b: the tile's common gauge
-// (sqrt theta, u_x, u_y); dt: of stage_tile; keep: the thread's column of kept values.
-template <typename R>
+// (sqrt theta, u_x, u_y); dt: of stage_tile; FAR: the slots have a halo of HALO_FAR; keep: the thread's column of kept values.
+template <typename R, bool FAR>
 __device__ __forceinline__ void stream_node(const DevParams &p, const R *__restrict__ in, int X, int Y, const R *slot,
                                             int pitch, const R (&gauge_b)[3], R dt, R th, R ux, R uy, bool first,
                                             R *keep, R (&inc)[2][9], unsigned &nreg, unsigned &npair)
@@ -1148,7 +1314,10 @@ __device__ __forceinline__ void stream_node(const DevParams &p, const R *__restr
     const bool okx = axis_weights<R>(s, ux, dt, ax, nx0), oky = axis_weights<R>(s, uy, dt, ay, ny0);
     if (!(okx && oky)) {
         R buf[18];
-        stream_general<R>(p, in, X, Y, th, ux, uy, first, 0, 1, buf, nreg, npair);
+        if constexpr (FAR)
+            stream_far(p, in, X, Y, slot, pitch, gauge_b[0], gauge_b[1], gauge_b[2], dt, th, ux, uy, first, buf, nreg, npair);
+        else
+            stream_general<R>(p, in, X, Y, th, ux, uy, first, 0, 1, buf, nreg, npair);
 #pragma unroll
         for (int i = 0; i < 9; ++i) {
             inc[0][i] = buf[i];
@@ -1355,36 +1524,37 @@ __device__ __forceinline__ void collide(const TypedParams<R> &q, const EosOut<R>
     rec[30] = rec[31] = 0;
 }
 
-// A tile of a step kernel's block: NB = TX x TY nodes from (X0, Y0), WT staged slots and RW
-// ring nodes per row, and its shared memory.
+// A tile of a step kernel's block: TX x TY nodes from (X0, Y0) staged with a halo of `halo`
+// nodes, WT staged slots and RW ring nodes per row, and its shared memory.
 template <typename R>
 struct Tile {
-    int X0, Y0, TX, TY, WT, RW, nslots;
-    R *aux, *slots, *kq;
+    int X0, Y0, TX, TY, halo, WT, RW, nslots;
+    R *aux, *slots, *kq, *rest;   // rest: after the others, whatever the halo
+    __device__ __forceinline__ Tile(const DevParams &p, int idx, R *smem) : TX(p.tile_x), TY(p.tile_y), RW(TX + 2)
+    {
+        X0 = (idx % p.tiles_x) * TX;
+        Y0 = (idx / p.tiles_x) * TY;
+        aux = smem;
+        rest = aux + (size_t)step_slots(TX, TY, widest_halo(TX, TY, sizeof(R))) * (AUXW + Slot<R>::stride) + (size_t)RW * (TY + 2) * KQW;
+        set_halo(HALO);
+    }
+    __device__ __forceinline__ void set_halo(int h)
+    {
+        halo = h;
+        WT = TX + 2 * h;
+        nslots = step_slots(TX, TY, h);
+        slots = aux + (size_t)nslots * AUXW;
+        kq = slots + (size_t)nslots * Slot<R>::stride;
+    }
+    __device__ __forceinline__ int slot(int tx, int ty) const { return (ty + halo) * WT + tx + halo; }
 };
-
-template <typename R>
-__device__ __forceinline__ Tile<R> make_tile(const DevParams &p, int idx, R *smem)
-{
-    Tile<R> t;
-    t.TX = p.tile_x;
-    t.TY = p.tile_y;
-    t.X0 = (idx % p.tiles_x) * t.TX;
-    t.Y0 = (idx / p.tiles_x) * t.TY;
-    t.WT = t.TX + 2 * HALO;
-    t.RW = t.TX + 2;
-    t.nslots = t.WT * (t.TY + 2 * HALO);
-    t.aux = smem;
-    t.slots = t.aux + (size_t)t.nslots * AUXW;
-    t.kq = t.slots + (size_t)t.nslots * Slot<R>::stride;
-    return t;
-}
 
 // Stages a tile and its halo (see the head of this file) and computes K and q on the tile
 // and its ring; gb = the tile's common gauge: sqrt(theta), u_x, u_y.  Returns the time step
 // of the contraction's departure points: dt, or infinity, which no contraction takes, in a
-// tile whose velocities spread too far for it.  Every thread of the block calls it; it ends
-// with a barrier.
+// tile whose velocities spread too far for it; or 0, with nothing staged, where a node moves
+// |v| dt >= 1 and the tile can hold a wider halo than tl's.  Every thread of the block calls
+// it; it ends with a barrier.
 template <typename R>
 __device__ __forceinline__ R stage_tile(const DevParams &p, const R *__restrict__ in, const R *nlsrc,
                                            const Tile<R> &tl, StepCounts &counts, R (&gb)[3])
@@ -1402,7 +1572,7 @@ __device__ __forceinline__ R stage_tile(const DevParams &p, const R *__restrict_
     const float iwt = 1.0f / (float)WT;
     auto node_of = [&](int k) -> size_t {
         const int cv = (int)(((float)k + 0.5f) * iwt), cu = k - cv * WT;
-        return (size_t)bc_wrap(Y0 - HALO + cv, p.ny, p.bcy) * p.nx + bc_wrap(X0 - HALO + cu, p.nx, p.bcx);
+        return (size_t)bc_wrap(Y0 - tl.halo + cv, p.ny, p.bcy) * p.nx + bc_wrap(X0 - tl.halo + cu, p.nx, p.bcx);
     };
     auto put_aux = [&](int k, size_t nd, R r, R t) {
         if (nlsrc != in) {   // current-time non-local terms: rho, T of the first pass's prediction
@@ -1438,7 +1608,7 @@ __device__ __forceinline__ R stage_tile(const DevParams &p, const R *__restrict_
     ex = tile_extremes(ex, best);
     bool smooth = sizeof(R) == 4 && ex.smooth();
     const int khot = min((int)ex.at, nslots - 1), kcold = min((int)ex.lat, nslots - 1);
-    R thb;
+    R thb, shot;   // theta of the gauge; sqrt theta of the hottest node
     {
         R hot[3], cold[3];
 #pragma unroll
@@ -1447,6 +1617,7 @@ __device__ __forceinline__ R stage_tile(const DevParams &p, const R *__restrict_
             cold[k] = aux[kcold * AUXW + k];
         }
         common_gauge<R, 3>(smooth, hot, cold, gb);
+        shot = sqrt_(hot[0]);
         thb = smooth ? hot[0] : gb[0] * gb[0];
     }
     __shared__ R base[18];   // the hottest node's populations
@@ -1465,10 +1636,14 @@ __device__ __forceinline__ R stage_tile(const DevParams &p, const R *__restrict_
     }
     // (the barrier: base is there, and aux may be overwritten)
     R dt = q.dt;
-    if (__syncthreads_or(ex.spread(gb))) {
-        smooth = false;
-        if (!middle_gauge<R, 2>(ex, best, gb)) dt = R(1) / R(0);
-        thb = gb[0] * gb[0];
+    const bool spread = ex.spread(gb), reach = ex.reach((float)shot, p.pf.dt) && tl.halo < widest_halo(TX, TY, sizeof(R));
+    if (__syncthreads_or(spread || reach)) {
+        if (__syncthreads_or(spread)) {
+            smooth = false;
+            if (!middle_gauge<R, 2>(ex, best, gb)) dt = R(1) / R(0);
+            thb = gb[0] * gb[0];
+        }
+        if (sizeof(R) == 8 && __syncthreads_or(reach) && dt == q.dt) return R(0);
     }
     const R inv_sb = R(1) / gb[0];
     auto carry = [&](int k, size_t nd, const R (&v)[24]) {
@@ -1542,7 +1717,7 @@ __device__ __forceinline__ R stage_tile(const DevParams &p, const R *__restrict_
             const int mx = p.bcx == 0 ? X0 + i - 1 : bc_wrap(X0 + i - 1, p.nx, 1);
             const int my = p.bcy == 0 ? Y0 + j - 1 : bc_wrap(Y0 + j - 1, p.ny, 1);
             R o[KQW];
-            stress_and_flux<R>(q, aux, (my - (Y0 - HALO)) * WT + (mx - (X0 - HALO)), WT, o);
+            stress_and_flux<R>(q, aux, (my - (Y0 - tl.halo)) * WT + (mx - (X0 - tl.halo)), WT, o);
 #pragma unroll
             for (int c = 0; c < KQW; ++c) kq[k * KQW + c] = o[c];
         }
@@ -1632,8 +1807,11 @@ __device__ __forceinline__ void stop_rules(const DevParams &p, float res, float 
     stall = sizeof(R) == 4 && its >= 2 && !conv && res > 0.5f * last && res < STALL_TOL_FACTOR * p.tol_f;
 }
 
-// One time step of one tile, one thread per node.
-template <typename R>
+// One time step of one tile, one thread per node.  FAR (FP64): with the wider halo, apart
+// from the common form, whose registers and code it would burden.
+__device__ __noinline__ void step_tile_far(const DevParams &p, const double *__restrict__ in, double *__restrict__ out,
+                                           DevStats *stats, int tile_idx, const double *nlsrc, double *smem);
+template <typename R, bool FAR>
 __device__ __forceinline__ void step_tile(const DevParams &p, const R *__restrict__ in, R *__restrict__ out,
                                           DevStats *stats, int tile_idx, const R *nlsrc, R *smem)
 {
@@ -1642,14 +1820,20 @@ __device__ __forceinline__ void step_tile(const DevParams &p, const R *__restric
     const size_t N = (size_t)p.N;
     const int tid = threadIdx.x;
     __shared__ StepCounts counts;
-    const Tile<R> tl = make_tile<R>(p, tile_idx, smem);
+    Tile<R> tl(p, tile_idx, smem);
+    if constexpr (FAR) tl.set_halo(HALO_FAR);
     R gb[3];
     const R dt = stage_tile<R>(p, in, nlsrc, tl, counts, gb);
+    if constexpr (sizeof(R) == 8 && !FAR)
+        if (dt == R(0)) {
+            step_tile_far(p, in, out, stats, tile_idx, nlsrc, smem);
+            return;
+        }
     const int tx = tid % tl.TX, ty = tid / tl.TX;
     const int X = tl.X0 + tx, Y = tl.Y0 + ty;
     const bool valid = ty < tl.TY && X < p.nx && Y < p.ny;   // (a tile may have fewer nodes than threads)
-    R *keep = tl.kq + (size_t)(tl.TX + 2) * (tl.TY + 2) * KQW + tid;   // this thread's column
-    const int slot = (ty + HALO) * tl.WT + tx + HALO;
+    R *keep = tl.rest + tid;   // this thread's column
+    const int slot = tl.slot(tx, ty);
     unsigned its = 0, nreg = 0, npair = 0;
     bool conv = true, stall = false, floored = false, bad = false;
     if (valid) {
@@ -1700,8 +1884,8 @@ __device__ __forceinline__ void step_tile(const DevParams &p, const R *__restric
         float last = 3.0e38f;   // previous residual
         for (;;) {
             ++its;
-            stream_node<R>(p, in, X, Y, tl.slots + (size_t)slot * DS, tl.WT, gb, dt, th, ux, uy, its == 1, keep, inc,
-                           nreg, npair);
+            stream_node<R, FAR>(p, in, X, Y, tl.slots + (size_t)slot * DS, tl.WT, gb, dt, th, ux, uy, its == 1, keep, inc,
+                                nreg, npair);
             R sum[4] = {R(0), R(0), R(0), R(0)};
 #pragma unroll
             for (int i = 0; i < 9; ++i) {
@@ -1792,7 +1976,10 @@ __device__ __forceinline__ void lane_sums(R f, R g, int base, int l, R (&hi)[4],
     lo[2] = e + (s2l - s0l);
 }
 
-template <typename R>
+__device__ __noinline__ void step_tile_split_far(const DevParams &p, const double *__restrict__ in,
+                                                 double *__restrict__ out, DevStats *stats, int tile_idx,
+                                                 const double *nlsrc, double *smem);
+template <typename R, bool FAR>
 __device__ __forceinline__ void step_tile_split(const DevParams &p, const R *__restrict__ in, R *__restrict__ out,
                                                 DevStats *stats, int tile_idx, const R *nlsrc, R *smem)
 {
@@ -1801,9 +1988,15 @@ __device__ __forceinline__ void step_tile_split(const DevParams &p, const R *__r
     const TypedParams<R> &q = typed<R>(p);
     const size_t N = (size_t)p.N;
     __shared__ StepCounts counts;
-    const Tile<R> tl = make_tile<R>(p, tile_idx, smem);
+    Tile<R> tl(p, tile_idx, smem);
+    if constexpr (FAR) tl.set_halo(HALO_FAR);
     R gb[3];
     const R dt = stage_tile<R>(p, in, nlsrc, tl, counts, gb);
+    if constexpr (sizeof(R) == 8 && !FAR)
+        if (dt == R(0)) {
+            step_tile_split_far(p, in, out, stats, tile_idx, nlsrc, smem);
+            return;
+        }
 
     const int ln = threadIdx.x & 31, lq = ln < 27 ? ln : ln - 9;
     const int base = lq < 9 ? 0 : (lq < 18 ? 9 : 18);
@@ -1813,10 +2006,10 @@ __device__ __forceinline__ void step_tile_split(const DevParams &p, const R *__r
     const bool valid = tl.X0 + tx < p.nx && tl.Y0 + ty < p.ny;
     const int X = min(tl.X0 + tx, p.nx - 1), Y = min(tl.Y0 + ty, p.ny - 1);
     const size_t n = (size_t)Y * p.nx + X;
-    const int slot = (ty + HALO) * tl.WT + tx + HALO;
+    const int slot = tl.slot(tx, ty);
     const bool writer = ln < 27;
     // the node's own record and the general stream's partials
-    R *own = tl.kq + (size_t)(tl.TX + 2) * (tl.TY + 2) * KQW + (size_t)j * SPLIT_WORDS, *part = own + SL;
+    R *own = tl.rest + (size_t)j * SPLIT_WORDS, *part = own + SL;
     for (int v = e; v < 30; v += 9)
         if (writer) own[v] = __ldg(in + rec_at(in, n, v, N));
     R Fx = 0, Fy = 0, M0 = 0, rEl;
@@ -1886,7 +2079,7 @@ __device__ __forceinline__ void step_tile_split(const DevParams &p, const R *__r
         }
         const unsigned okm = __ballot_sync(ALL, ok), nxm = __ballot_sync(ALL, near_x);
         const unsigned gm = 0x1ffu << base;
-        const bool fast = (okm & gm) == gm;
+        bool fast = (okm & gm) == gm;
         R nf = 0, ng = 0;
         {
             // row k of the x map, column n (= l) of the y map
@@ -1996,6 +2189,20 @@ __device__ __forceinline__ void step_tile_split(const DevParams &p, const R *__r
             add_reg = (unsigned)(sx * (dy0 == dy2 ? 4 : 5) - (it == 1 ? 1 : 0));
         }
         if (__any_sync(ALL, active && !fast)) {
+            if constexpr (FAR) {
+                // departure points within the wider halo: each lane streams its direction
+                const FarOne o1 = far_one(sl, tl.WT, k, l, gb[0], gb[1], gb[2], s, inv_s, dt, ux, uy);
+                const unsigned rm = __ballot_sync(ALL, o1.ok);
+                const int x0 = grp(o1.fx, base, 0), x1 = grp(o1.fx, base, 1), x2 = grp(o1.fx, base, 2);
+                const int y0 = grp(o1.fy, base, 0), y1 = grp(o1.fy, base, 3), y2 = grp(o1.fy, base, 6);
+                if (!fast && (rm & gm) == gm) {
+                    fast = true;
+                    nf = o1.f - fe;
+                    ng = o1.g - ge;
+                    add_reg = (unsigned)((4 + max(x0, max(x1, x2)) - min(x0, min(x1, x2))) *
+                                             (4 + max(y0, max(y1, y2)) - min(y0, min(y1, y2))) - (it == 1 ? 1 : 0));
+                }
+            }
             // departure points beyond the halo: the node's lanes share its stencil nodes
             if (!fast) {
                 R buf[18];
@@ -2140,6 +2347,18 @@ __device__ __forceinline__ void step_tile_split(const DevParams &p, const R *__r
                one && o.pr < q.p_floor, one && bad);
 }
 
+__device__ __noinline__ void step_tile_far(const DevParams &p, const double *__restrict__ in, double *__restrict__ out,
+                                           DevStats *stats, int tile_idx, const double *nlsrc, double *smem)
+{
+    step_tile<double, true>(p, in, out, stats, tile_idx, nlsrc, smem);
+}
+__device__ __noinline__ void step_tile_split_far(const DevParams &p, const double *__restrict__ in,
+                                                 double *__restrict__ out, DevStats *stats, int tile_idx,
+                                                 const double *nlsrc, double *smem)
+{
+    step_tile_split<double, true>(p, in, out, stats, tile_idx, nlsrc, smem);
+}
+
 // A simulation as one launch sees it: parameters, the buffers this step reads and writes
 // (nlsrc: the state the non-local terms come from) and its counters.
 template <typename R>
@@ -2179,8 +2398,8 @@ __global__ void __launch_bounds__(STEP_THREADS, SPLIT ? SPLIT_MIN_BLOCKS(R) : ST
     asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
     extern __shared__ __align__(128) unsigned char step_dyn_smem[];
     R *smem = reinterpret_cast<R *>(step_dyn_smem);
-    if constexpr (SPLIT) step_tile_split<R>(d.p, d.in, d.out, d.stats, tile, d.nlsrc, smem);
-    else step_tile<R>(d.p, d.in, d.out, d.stats, tile, d.nlsrc, smem);
+    if constexpr (SPLIT) step_tile_split<R, false>(d.p, d.in, d.out, d.stats, tile, d.nlsrc, smem);
+    else step_tile<R, false>(d.p, d.in, d.out, d.stats, tile, d.nlsrc, smem);
 }
 
 }  // namespace pond

@@ -26,6 +26,20 @@ int main(int argc, char **argv)
                                        : step_smem_bytes(s.tx, s.ty, split, Slot<double>::stride, 8));
         std::printf("%d %d %d %lld %zu\n", s.lanes, s.tx, s.ty, s.blocks(a[2], a[3]), m);
     }
+    // the wider halo (FP64): every stencil it serves (floors -2 .. 1, four nodes from the floor
+    // less one) lies within the staged rows and columns, and the slots within a block's memory
+    for (int nodes = 12; nodes <= STEP_NB; nodes += nodes == 12 ? 20 : nodes)
+        for (int tx = 1; tx <= nodes; ++tx) {
+            const int ty = nodes / tx, h = widest_halo(tx, ty, 8), wt = tx + 2 * h, n = step_slots(tx, ty, h);
+            const int first = h * wt + h, last = (ty - 1 + h) * wt + tx - 1 + h;
+            if (tx * ty != nodes) continue;
+            if ((nodes < STEP_NB || tx == 16) != (h == HALO_FAR) && tx != 8) return 1;
+            if (widest_halo(tx, ty, 4) != HALO) return 1;
+            if (first + (1 - h - 1) * (wt + 1) < 0 || last + (h - 2 + 2) * (wt + 1) >= n) return 2;
+            const size_t m = step_smem_bytes(tx, ty, nodes == 12, Slot<double>::stride, 8);
+            // two resident blocks on the tiles of large grids
+            if (m + 2048 > 227 * 1024 || (tx == 16 && 2 * (m + 2048) > 228 * 1024)) return 3;
+        }
     std::printf("%d %d\n", STEP_THREADS, SPLIT_NB);
 }
 """
