@@ -171,8 +171,8 @@ void launch_q16_pass(pond_ctx *c, const R *in, const R *src, R *out, DevStats *s
     using W = typename Wide<R>::type;
     W *nl = reinterpret_cast<W *>(c->nlbuf);
     const dim3 blk = c->grid.ny < 4 ? dim3(256, 1) : dim3(32, 8);
-    const dim3 grd(blocks_for((size_t)c->grid.nx, blk.x), blocks_for((size_t)c->grid.ny, blk.y));
-    k_q16_nonlocal1<R><<<grd, blk, 0, strm>>>(c->dp, src, nl);
+    const unsigned across = blocks_for((size_t)c->grid.nx, blk.x);   // (along y a launch holds 65,535 blocks only)
+    k_q16_nonlocal1<R><<<across * blocks_for((size_t)c->grid.ny, blk.y), blk, 0, strm>>>(c->dp, src, nl, (int)across);
     k_q16_nonlocal2<R><<<nb, 256, 0, strm>>>(c->dp, nl);
     k_q16_step<R><<<(unsigned)step_tiles(c), STEP_THREADS, q16_smem_bytes<R>(c->dp.tile_x, c->dp.tile_y), strm>>>(
         c->dp, in, nl, out, stats);
@@ -207,9 +207,9 @@ void launch_q27_pass(pond_ctx *c, const R *in, const R *src, R *out, DevStats *s
     k_q27_pi<R><<<nb, 256, 0, c->stream>>>(c->dp, src, nl);
     k_q27_nonlocal1<R><<<nb, 256, 0, c->stream>>>(c->dp, c->g3, src, nl);
     k_q27_nonlocal2<R><<<nb, 256, 0, c->stream>>>(c->dp, c->g3, nl);
-    const dim3 grd(blocks_for((size_t)c->grid.nx, T27X), blocks_for((size_t)c->grid.ny, T27Y),
-                   blocks_for((size_t)c->g3.nz, T27Z));
-    k_q27_step<R><<<grd, Q27_THREADS, q27_smem_bytes<R>(), c->stream>>>(c->dp, c->g3, in, nl, out, stats);
+    const unsigned nx = blocks_for((size_t)c->grid.nx, T27X), ny = blocks_for((size_t)c->grid.ny, T27Y);
+    k_q27_step<R><<<nx * ny * blocks_for((size_t)c->g3.nz, T27Z), Q27_THREADS, q27_smem_bytes<R>(), c->stream>>>(
+        c->dp, c->g3, (int)nx, (int)ny, in, nl, out, stats);
 }
 
 template <typename R>

@@ -247,15 +247,15 @@ struct Near9 {
 //   rho E_lambda = kappa |grad rho|^2 / 2.
 // A block of bx by by nodes (256 threads) stages rho, T and p/rho of its nodes and their
 // neighbours once: 1.3 equations of state a node instead of nine (1024 x 512 mixed nodes
-// 53 -> 42 us, 20 with the parameters split on the host).
+// 53 -> 42 us, 20 with the parameters split on the host).  across: blocks along x.
 constexpr int NL16_STAGED = 3 * 258;   // (bx + 2) (by + 2) at most, for 256 x 1 and 32 x 8
 template <typename R>
-__global__ void k_q16_nonlocal1(DevParams p, const R *__restrict__ src, typename Wide<R>::type *__restrict__ nl)
+__global__ void k_q16_nonlocal1(DevParams p, const R *__restrict__ src, typename Wide<R>::type *__restrict__ nl, int across)
 {
     using A = typename Wide<R>::type;
     __shared__ R sr[NL16_STAGED], st[NL16_STAGED];
     __shared__ A sp[NL16_STAGED];
-    const int bx = blockDim.x, by = blockDim.y, X0 = blockIdx.x * bx, Y0 = blockIdx.y * by, W = bx + 2;
+    const int bx = blockDim.x, by = blockDim.y, X0 = (int)(blockIdx.x % across) * bx, Y0 = (int)(blockIdx.x / across) * by, W = bx + 2;
     for (int k = threadIdx.y * bx + threadIdx.x; k < W * (by + 2); k += bx * by) {
         const size_t m = (size_t)bc_wrap(Y0 + k / W - 1, p.ny, p.bcy) * p.nx + bc_wrap(X0 + k % W - 1, p.nx, p.bcx);
         const R r = REC16(src, m, Q_RHO), t = REC16(src, m, Q_T);

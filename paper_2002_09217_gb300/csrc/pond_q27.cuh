@@ -1083,12 +1083,13 @@ __device__ __forceinline__ bool q27_collide(const DevParams &p, R *__restrict__ 
     return finite && rho - rho == R(0) && T - T == R(0);
 }
 
-// The node step, one thread per node of the block's tile.  Registers for two resident
-// blocks per SM in FP32 (255, its two staged families' worth of shared memory), one in FP64.
+// The node step, one thread per node of the block's tile; bx, by: blocks along x and y (in
+// one launch dimension, since the others hold 65,535 blocks only).  Two resident blocks per SM
+// in FP32 (255 registers; the shared memory of one staged family each), one in FP64.
 template <typename R>
 __global__ void __launch_bounds__(Q27_THREADS, sizeof(R) == 4 ? 2 : 1)
-    k_q27_step(DevParams p, Grid3 g3, const R *__restrict__ in, typename Wide<R>::type *nl, R *__restrict__ out,
-               DevStats *stats)
+    k_q27_step(DevParams p, Grid3 g3, int bx, int by, const R *__restrict__ in, typename Wide<R>::type *nl,
+               R *__restrict__ out, DevStats *stats)
 {
     using A = typename Wide<R>::type;
     extern __shared__ __align__(128) unsigned char q27_dyn_smem[];
@@ -1098,7 +1099,8 @@ __global__ void __launch_bounds__(Q27_THREADS, sizeof(R) == 4 ? 2 : 1)
     __shared__ uint4 best[BEST];
     const int tid = threadIdx.x;
     const size_t N = (size_t)p.N;
-    const Tile27 tl{(int)blockIdx.x * T27X, (int)blockIdx.y * T27Y, (int)blockIdx.z * T27Z};
+    const int b = (int)blockIdx.x;
+    const Tile27 tl{b % bx * T27X, b / bx % by * T27Y, b / bx / by * T27Z};
     // a warp takes 8 x 1 x 4 nodes: the half warps' slots then fall on distinct banks
     const int tx = tid % T27X, tz = (tid / T27X) % T27Z, ty = tid / (T27X * T27Z);
     const int X = tl.X0 + tx, Y = tl.Y0 + ty, Z = tl.Z0 + tz;
