@@ -162,6 +162,15 @@ cudaError_t launch_step_kernel(bool use_split, unsigned blocks, size_t smem, cud
                      : cudaLaunchKernelEx(&cfg, k_pond_step<R, false>, one, descs, work);
 }
 
+// After a step's launches: the state is the buffer they write, unless one of them failed.
+pond_status step_launched(pond_ctx *c)
+{
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return cuda_fail(c, e, "step launch");
+    c->cur = 1 - c->cur;
+    return POND_OK;
+}
+
 // D2Q16: the non-local terms of state `src` into nlbuf, then the node step in -> out.
 template <typename R>
 void launch_q16_pass(pond_ctx *c, const R *in, const R *src, R *out, DevStats *stats,
@@ -193,8 +202,7 @@ pond_status launch_step_q16(pond_ctx *c, cudaEvent_t *ev)
     }
     launch_q16_pass<R>(c, in, nl, out, c->dstats, c->stream);
     if (ev) cudaEventRecord(ev[1], c->stream);
-    c->cur = 1 - c->cur;
-    return POND_OK;
+    return step_launched(c);
 }
 
 // D3Q27: the non-local terms of state `src`, then the node step in -> out.
@@ -225,8 +233,7 @@ pond_status launch_step_q27(pond_ctx *c, cudaEvent_t *ev)
     }
     launch_q27_pass<R>(c, in, nl, out, c->dstats);
     if (ev) cudaEventRecord(ev[1], c->stream);
-    c->cur = 1 - c->cur;
-    return POND_OK;
+    return step_launched(c);
 }
 
 template <typename R>
@@ -251,8 +258,7 @@ pond_status launch_step(pond_ctx *c, cudaEvent_t *ev = nullptr)
     const SimDesc<R> one{c->dp, in, out, c->dstats, nl};
     launch_step_kernel<R>(split(c), nb, smem, c->stream, one, nullptr, nullptr);
     if (ev) cudaEventRecord(ev[1], c->stream);
-    c->cur = 1 - c->cur;
-    return POND_OK;
+    return step_launched(c);
 }
 
 template <typename R>
@@ -734,11 +740,10 @@ pond_status pond_step(pond_ctx *c, int64_t n)
     if (!c->initialised) return fail(c, POND_EINVAL, "state not initialised");
     if (c->batch) return fail(c, POND_EINVAL, "context belongs to a batch: step it with pond_batch_step");
     for (int64_t k = 0; k < n; ++k) {
-        if (mixed(c)) launch_step<float>(c);
-        else launch_step<double>(c);
+        st = mixed(c) ? launch_step<float>(c) : launch_step<double>(c);
+        if (st) return st;
+        ++c->steps;
     }
-    CK(cudaGetLastError(), "step launch");
-    c->steps += n;
     return POND_OK;
 }
 
@@ -750,14 +755,13 @@ pond_status pond_step_timed(pond_ctx *c, double *ms_out)
     if (!c->initialised) return fail(c, POND_EINVAL, "state not initialised");
     cudaEvent_t ev[2];
     for (int k = 0; k < 2; ++k) CK(cudaEventCreate(&ev[k]), "cudaEventCreate");
-    if (mixed(c)) launch_step<float>(c, ev);
-    else launch_step<double>(c, ev);
-    cudaError_t e = cudaGetLastError();
-    if (e == cudaSuccess) e = cudaEventSynchronize(ev[1]);
+    st = mixed(c) ? launch_step<float>(c, ev) : launch_step<double>(c, ev);
+    cudaError_t e = st ? cudaSuccess : cudaEventSynchronize(ev[1]);
     float ms = 0.f;
-    if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, ev[0], ev[1]);
+    if (!st && e == cudaSuccess) e = cudaEventElapsedTime(&ms, ev[0], ev[1]);
     *ms_out = ms;
     for (int k = 0; k < 2; ++k) cudaEventDestroy(ev[k]);
+    if (st) return st;
     if (e != cudaSuccess) return cuda_fail(c, e, "pond_step_timed");
     c->steps += 1;
     return POND_OK;
