@@ -45,11 +45,11 @@
  *     conditions (non-converged frame search, pressure floor hit, NaN) are counted on
  *     the device (pond_stats() reads the counts) and raised as sticky flags that the
  *     synchronising calls pond_moments, pond_moments3 and pond_conservation return as
- *     their status: POND_ETIMEOUT if a bounded device wait ran out, else
- *     POND_ENAN while the state holds non-finite values, else POND_ENONCONV, else
- *     POND_ETHETA for conditions that occurred since the previous report.  ENONCONV and ETHETA are warnings: the call has completed and its
- *     outputs are written; the report clears both flags.  There is no CPU fallback: a
- *     missing or unusable GPU is POND_ECUDA.
+ *     their status: POND_ENAN while the state holds non-finite values, else
+ *     POND_ENONCONV, else POND_ETHETA for conditions that occurred since the previous
+ *     report.  ENONCONV and ETHETA are warnings: the call has completed and its outputs
+ *     are written; the report clears both flags.  There is no CPU fallback: a missing or
+ *     unusable GPU is POND_ECUDA.
  *   - A context is not thread safe; distinct contexts may be used concurrently.
  */
 #ifndef POND_H
@@ -166,7 +166,7 @@ typedef struct {
                               streams until all its nodes stop)                */
     int64_t max_streams;   /* largest streaming-pass count of any node         */
     int64_t timeouts;      /* tiles skipped because a bounded device wait ran
-                              out (reported as POND_ETIMEOUT)                  */
+                              out: 0, since no kernel of this version waits    */
     int64_t region_nodes;  /* stencil nodes contracted or carried into the arrival
                               gauge, summed over streams (the union of a node's 4x4
                               (4x4x4) departure stencils: 16..64 per stream on

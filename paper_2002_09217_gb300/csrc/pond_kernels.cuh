@@ -103,9 +103,8 @@ template <> __device__ __forceinline__ const TypedParams<double> &typed<double>(
 
 struct DevStats {
     unsigned long long streams, nonconv, clamped, nonfinite, bad_init, stalled, block_streams, max_streams;
-    unsigned long long timeouts;   // tiles skipped because a bounded wait for their copies ran out
-    unsigned long long region_nodes;   // D2Q9 step: stencil-region nodes transformed, summed over streams
-    unsigned long long pair_streams;   // D2Q9 step: streams that took the per-pair path (wide regions)
+    unsigned long long region_nodes;   // stencil nodes contracted or carried, summed over streams
+    unsigned long long pair_streams;   // streams that took the per-pair path (wide regions)
 };
 
 // lattice temperature T_L = 1/3 and 1-D weights W_-1, W_0, W_+1 (SM "Equilibrium")
@@ -173,16 +172,6 @@ __device__ __forceinline__ double pressure_d(const DevParams &p, double r, doubl
     if (p.eos_kind != 0) return eos_pressure<double>(p.eos_kind, p.a, p.b, p.R, r, t, p.sp);
     return r * p.R * t * rcp_d(1.0 - p.b * r) - p.a * r * r;
 }
-template <typename T>
-__device__ __forceinline__ void warp_add(unsigned long long *dst, T v)
-{
-    unsigned mask = __activemask();
-    unsigned long long x = (unsigned long long)v;
-    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(mask, x, o);
-    if ((threadIdx.x & 31) == (__ffs(mask) - 1) && x) atomicAdd(dst, x);
-}
-
-
 // ---------------------------------------------------------------------------
 // Output fields: rho, uhat, T, p (vdW EoS) in FP64.
 template <typename R>

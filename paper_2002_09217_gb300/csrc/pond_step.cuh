@@ -228,17 +228,6 @@ __device__ __forceinline__ R wst(int ex, int ey)
     return (ex == 0 ? R(2.0 / 3.0) : R(1.0 / 6.0)) * (ey == 0 ? R(2.0 / 3.0) : R(1.0 / 6.0));
 }
 
-// One cubic Lagrange basis function a_j(xi) on nodes 0..3 (SM "Reconstruction").
-template <typename R>
-__device__ __forceinline__ R lag1(int j, R xi)
-{
-    R t0 = xi, t1 = xi - R(1), t2 = xi - R(2), t3 = xi - R(3);
-    if (j == 0) return -(t1 * t2 * t3) * R(1.0 / 6.0);
-    if (j == 1) return t0 * t2 * t3 * R(0.5);
-    if (j == 2) return -(t0 * t1 * t3) * R(0.5);
-    return t0 * t1 * t2 * R(1.0 / 6.0);
-}
-
 // A departure offset (in nodes) limited to +-2^20, NaN mapped to the lower bound: keeps
 // stencil indices derived from it in int range whatever the gauge (fmax returns the
 // non-NaN operand).
@@ -248,7 +237,8 @@ __device__ __forceinline__ R clamp_offset(R d)
     return fmin(fmax(d, R(-1048576)), R(1048576));
 }
 
-// a_j(xi) for a run-time j: the three factors (xi - m), m != j, picked by selects.
+// The cubic Lagrange basis function a_j(xi) on nodes 0..3 (SM "Reconstruction") for a
+// run-time j: the three factors (xi - m), m != j, picked by selects.
 template <typename R>
 __device__ __forceinline__ R lag1_rt(int j, R xi)
 {
