@@ -684,7 +684,7 @@ __device__ __forceinline__ void axis_rows16(const Lat16<A> &L, A q, A w, A (&G)[
 // Departure points of the four components of an axis and their cubic weights; true when
 // every floor is -1 or 0 (the stencils then lie within two nodes of the arrival node).
 template <typename R>
-__device__ __forceinline__ bool axis_weights16(const Lat16<R> &L, R s, R u, R dt, R (&a)[4][4], bool (&near0)[4])
+__host__ __device__ __forceinline__ bool axis_weights16(const Lat16<R> &L, R s, R u, R dt, R (&a)[4][4], bool (&near0)[4])
 {
     bool ok = true;
 #pragma unroll

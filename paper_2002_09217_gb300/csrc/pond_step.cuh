@@ -890,7 +890,7 @@ __device__ __forceinline__ void map_inc(const R (&Ex)[3][3], const R (&Ey)[3][3]
 // 0 (|v| dt < 1 in general), so that the stencils lie within two nodes of the arrival node;
 // false also for NaN.
 template <typename R>
-__device__ __forceinline__ bool axis_weights(R s, R u, R dt, R (&a)[3][4], bool (&near0)[3])
+__host__ __device__ __forceinline__ bool axis_weights(R s, R u, R dt, R (&a)[3][4], bool (&near0)[3])
 {
     bool ok = true;
 #pragma unroll
