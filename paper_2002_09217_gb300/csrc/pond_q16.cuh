@@ -26,11 +26,11 @@
 //
 // The node step streams as the D2Q9 step does (pond_step.cuh): the block's tile with a halo
 // of two is carried once into a common gauge in shared memory and each thread contracts
-// its node's 5 x 5 window along x, then y: 2,200 multiply-adds a population family, where
-// carrying each of 25 nodes into the arrival gauge and spreading it over sixteen directions
-// took about 7,000.
-// Measured (with init and read-out): four mixed steps of a 1024 x 512 droplet 7.82 -> 1.91 ms,
-// three FP64 steps of a 257 x 127 shock-droplet 30.2 -> 5.9 ms.  The mixed contraction runs on
+// its node's 5 x 5 window along x, then y: 2,240 (FP32) or 1,600 (FP64) multiply-adds a
+// population family, where carrying each of 25 nodes into the arrival gauge and spreading it
+// over sixteen directions took about 7,000.
+// Measured (with init and read-out): four mixed steps of a 1024 x 512 droplet 7.94 -> 1.90 ms,
+// three FP64 steps of a 257 x 127 shock-droplet 29 -> 5.5 ms.  The mixed contraction runs on
 // packed pairs, rolled over the source rows so that its code stays in the instruction cache
 // (609 -> 457 us a step); its FP64 pipe, 22 % busy with the moments and EoS before they went
 // to float-float, is idle.  The FP64 form is bound by the FP64 pipe.
@@ -509,7 +509,13 @@ __device__ __forceinline__ void apply_inc(const A Dx[4][4], const A Dy[4][4], co
 // q16_stream, so the two agree up to the rounding of zero-weight terms; the region form
 // transforms about 25 nodes per stream against 256 pairs.
 
-// Largest region side the region stream takes; wider regions take q16_stream.
+// Largest region side the region stream takes; wider regions take q16_stream.  Departures
+// beyond the halo are the one thing that earlier kernels, which streamed every node this way,
+// did faster (us a step of 128 x 128 nodes at dt = 1, earlier / this, mixed: a droplet at 1.4
+// T_cr 174 / 192, at 1.9 T_cr, a seventh of the streams per pair, 629 / 838; a flow at |v| dt = 1.3
+// 183 / 204; FP64 within 4 %): f and g take two passes, and the weight tables lie in local
+// memory.  One pass over both gave 168 and 175 us but cost every other step 3.7 %, by the
+// registers of the calling kernel.
 constexpr int Q16_REGION_MAX = 6;
 // Entries of a thread's Lagrange weight tables: (axis * 4 + k) * Q16_REGION_MAX + c is the
 // weight of region column (row) c in the stencil of axis component k, zero outside it.

@@ -24,9 +24,9 @@
 // The node step streams as the D2Q9 step does (pond_step.cuh): a block's tile of 8 x 4 x 4
 // nodes with a halo of two is carried once into a common gauge in shared memory, and each
 // thread contracts its node's 5 x 5 x 5 window axis by axis (x, y, z) with weights that
-// combine the cubic Lagrange weights and the rows of the map into the arrival gauge: 12,500
-// multiply-adds a population family, where carrying each of 125 nodes into the arrival
-// gauge and spreading it over 27 directions took about 45,000.  One family at a time is
+// combine the cubic Lagrange weights and the rows of the map into the arrival gauge: 12,560
+// (FP32) or 10,530 (FP64) multiply-adds a population family, where carrying each of 125
+// nodes into the arrival gauge and spreading it over 27 directions took about 45,000.  One family at a time is
 // staged (two blocks per SM in FP32, one in FP64, by shared memory); a further stream of
 // the frame search starts with the family that is already staged.  The sums of populations,
 // the moments, the EoS and the non-local terms are float-float in the FP32 form.
@@ -400,7 +400,10 @@ __device__ __forceinline__ void axis3(A ds, A du, A D[3][3])
 // direction adds its Lagrange-weighted share, with the per-(direction, node) arithmetic of
 // q27_stream: the region form transforms about 125 nodes per stream against 1,728 pairs.
 
-// Largest region side the region stream takes; wider regions take q27_stream.
+// Largest region side the region stream takes; wider regions take q27_stream, which earlier
+// kernels did faster (us a step of 32 x 32 x 16 nodes at 2.7 T_cr and dt = 1, three quarters of
+// the streams per pair, earlier / this: mixed 13,550 / 17,600, FP64 247,000 / 263,000; at 1.6 T_cr,
+// none of them, 1,320 / 274 and 45,800 / 8,500).
 constexpr int Q27_REGION_MAX = 6;
 
 // A thread's Lagrange weight tables.  Entries 0..17: x, (k * Q27_REGION_MAX + c) = weight

@@ -1,7 +1,7 @@
 // pond_step.cuh -- the fused time-step kernel of the PonD van der Waals model (sm_103a).
 //
-// One launch per time step, one thread per node, a block owns a tile of STEP_NB nodes
-// (tile_x columns).  Per block:
+// One launch per time step, one thread per node (nine lanes on small grids), a block owns a
+// tile of nodes (step_shape).  Per block:
 //   staging  every record of the tile and a halo of HALO = 2 nodes is read once from
 //            global memory, its populations are carried into one gauge common to the tile
 //            (SM "Transfer matrix": G = M_lambda'^-1 M_lambda) and left in shared memory,
@@ -24,13 +24,13 @@
 // tile's common gauge b, the streamed population of direction (k, l) is
 //   f~_(k,l) = sum_cy sum_n (wy[l][cy] Ly[l][n]) sum_cx sum_m (wx[k][cx] Lx[k][m]) f^b_(m,n)(cx, cy)
 // (L = row of G_(b->lambda) along one axis, w = Lagrange weights): an x pass of 5 rows x 3 n
-// x 3 k and a y pass, about 650 multiply-adds a population family, where carrying each of
-// the 25 stencil nodes into the arrival gauge and spreading it over nine directions took
-// about 2,700.  The tile is 128 nodes because the halo's share of the staging falls with its
+// x 3 k and a y pass, 675 multiply-adds a population family over each component's own four
+// columns (FP64) and 810 over five (FP32), where carrying each of the 25 stencil nodes into
+// the arrival gauge and spreading it over nine directions took about 2,700.  The tile is 128 nodes because the halo's share of the staging falls with its
 // size (1.9 staged nodes a node; 6.3 with 4 x 4 nodes and a halo of 3).
 // Measured (five steps of the 2048 x 1024 shock-droplet interaction with init and read-out,
-// mixed): 17.7 -> 3.87 ms, 714 us a step; two FP64 steps of a 509 x 387 droplet 22.7 ->
-// 5.47 ms, 2.69 ms a step.  The mixed form is bound by instruction fetch and issue (issue 54 %
+// mixed): 17.7 -> 3.90 ms, 720 us a step; two FP64 steps of a 509 x 387 droplet 22.8 ->
+// 5.49 ms, 2.69 ms a step.  The mixed form is bound by instruction fetch and issue (issue 54 %
 // active, FMA pipe 56 %, 1.2 warps per issue waiting for instructions), the FP64 form by the
 // FP64 pipe (92 % busy); DRAM is 10 % busy.
 //
@@ -38,7 +38,8 @@
 // gauge of geometric-mean theta and mean velocity of its hottest and coldest nodes, by
 // product-form rows of the map.  Populations carried into a colder gauge are amplified (by
 // (theta_b / theta) per axis for the outermost of three velocities, more for four), those
-// carried into a hotter one cancel; the middle gauge splits that between the two maps.  On
+// carried into a hotter one cancel; the middle gauge splits that between the two maps.  (In
+// a tile whose velocities spread it is the middle of those, see SMOOTH_SPREAD.)  On
 // a 0.8 T_cr interface the worst error of a single population in FP32 is 2e-7 (D3Q27) and
 // 7e-8 (D2Q16), no more than carrying each node straight into the arrival gauge; the
 // hottest gauge left 3e-5 on D2Q16, the coldest 1e-6.
