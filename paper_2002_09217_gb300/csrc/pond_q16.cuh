@@ -891,7 +891,7 @@ __global__ void __launch_bounds__(STEP_THREADS, sizeof(R) == 4 ? Q16_MIN_BLOCKS 
         ld4(in, nbase, N, Q_TH, g4);
         ld4(in, node_of(min((int)ex.lat, nslots - 1)), N, Q_TH, cold);
         common_gauge<R, 3>(inc, g4, cold, gb);
-        if (__syncthreads_or(ex.spread(gb))) {
+        if (__syncthreads_or(ex.spread(gb, sqrtf(ex.hottest())))) {
             inc = false;
             if (!middle_gauge<R, 2>(ex, best, gb)) dt_b = R(1) / R(0);
         }

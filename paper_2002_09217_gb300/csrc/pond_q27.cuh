@@ -1130,7 +1130,7 @@ __global__ void __launch_bounds__(Q27_THREADS, sizeof(R) == 4 ? 2 : 1)
         thb = inc ? hot[0] : gb[0] * gb[0];
     }
     R dt_b = typed<R>(p).dt;   // infinite in a tile whose velocities spread too far (no contraction)
-    if (__syncthreads_or(ex.spread(gb))) {
+    if (__syncthreads_or(ex.spread(gb, sqrtf(ex.hottest())))) {
         inc = false;
         if (!middle_gauge<R, 3>(ex, best, gb)) dt_b = R(1) / R(0);
         thb = gb[0] * gb[0];

@@ -26,8 +26,9 @@
 // (L = row of G_(b->lambda) along one axis, w = Lagrange weights): an x pass of 5 rows x 3 n
 // x 3 k and a y pass, 675 multiply-adds a population family over each component's own four
 // columns (FP64) and 810 over five (FP32), where carrying each of the 25 stencil nodes into
-// the arrival gauge and spreading it over nine directions took about 2,700.  The tile is 128 nodes because the halo's share of the staging falls with its
-// size (1.9 staged nodes a node; 6.3 with 4 x 4 nodes and a halo of 3).
+// the arrival gauge and spreading it over nine directions took about 2,700.  The tile is 128
+// nodes because the halo's share of the staging falls with its size (1.9 staged nodes a
+// node; 6.3 with 4 x 4 nodes and a halo of 3).
 // Measured (five steps of the 2048 x 1024 shock-droplet interaction with init and read-out,
 // mixed): 17.7 -> 3.90 ms, 720 us a step; two FP64 steps of a 509 x 387 droplet 22.8 ->
 // 5.49 ms, 2.69 ms a step.  The mixed form is bound by instruction fetch and issue (issue 54 %
@@ -75,10 +76,13 @@ constexpr float SMOOTH_TILE = 0.9f;
 // theta, a node U sqrt(theta) from the tile's gauge gets back single populations with an error
 // of (D2Q9, D3Q27) 9e-8, 1e-7 in increment form at U = 0.4 and 7e-5, 3e-3 at 2; of 1.5e-7,
 // 2e-7 in direct form at 0.5, 4e-7, 9e-7 at 1 and 5e-6, 3e-5 at 1.5.  So a tile in which a
-// node moves faster than SMOOTH_SPREAD sqrt(theta_b) in the tile's gauge is staged in direct
+// node moves faster than SMOOTH_SPREAD sqrt(theta) in the tile's gauge is staged in direct
 // form around the middle of its velocities, and one in which a node then still moves faster
-// than FAR_SPEED sqrt(theta_b) takes the general stream, which carries each node straight
-// into the arrival gauge.
+// than FAR_SPEED sqrt(theta) takes the general stream, which carries each node straight into
+// the arrival gauge.  theta is the tile's hottest: at interfaces whose coldest nodes are at
+// the pressure floor, the gauge's own theta_b is a small part of it, and asking for
+// velocities against theta_b sent tiles of quiet droplets to the general stream (D3Q27, 96 x 96
+// x 64 sphere: 3.07 against 2.78 ms a step).
 constexpr float SMOOTH_SPREAD = 0.4f;
 constexpr float FAR_SPEED = 1.0f;
 constexpr int BEST = 8;   // uint4 of shared memory in which a block agrees on its gauge
@@ -753,14 +757,16 @@ struct Extremes {
     __device__ __forceinline__ float hottest() const { return __uint_as_float(top); }
     // the tile's thetas lie within SMOOTH_TILE of each other
     __device__ __forceinline__ bool smooth() const { return top != 0u && __uint_as_float(low) > SMOOTH_TILE * hottest(); }
-    // a node of this thread moves faster than SMOOTH_SPREAD in the gauge (sqrt theta, u)
+    // a node of this thread moves faster than SMOOTH_SPREAD s in the gauge gb, s = sqrt of the
+    // tile's hottest theta
     template <typename R>
-    __device__ __forceinline__ bool spread(const R (&gb)[D + 1]) const
+    __device__ __forceinline__ bool spread(const R (&gb)[D + 1], float s) const
     {
         bool far = false;
+        const float lim = SMOOTH_SPREAD * s;
 #pragma unroll
         for (int a = 0; a < D; ++a) {
-            const float u = (float)gb[1 + a], lim = SMOOTH_SPREAD * (float)gb[0];
+            const float u = (float)gb[1 + a];
             far = far || hi[a] - u > lim || u - lo[a] > lim;
         }
         return far;
@@ -801,32 +807,40 @@ __device__ __forceinline__ void common_gauge(bool inc, const R *hot, const R *co
 #pragma unroll
     for (int k = 1; k < ND; ++k) gb[k] = inc ? hot[k] : R(0.5) * (hot[k] + cold[k]);
 }
-// The gauge of a tile whose velocities spread: its extreme thetas' geometric mean and, along
-// each axis, the middle of the tile's velocities.  Returns whether all of them lie within
-// FAR_SPEED of it.  Every thread calls it, between barriers of its own use of `best`; it
-// holds one.
 __device__ __forceinline__ int ordered(float v)   // keeps the order of floats
 {
     const int b = __float_as_int(v);
     return b ^ ((b >> 31) & 0x7fffffff);
 }
 __device__ __forceinline__ float unordered(int b) { return __int_as_float(b ^ ((b >> 31) & 0x7fffffff)); }
+// The gauge of a tile whose velocities spread: its extreme thetas' geometric mean and, along
+// each axis, the middle of the tile's velocities (near: all of them lie within FAR_SPEED
+// sqrt(hottest theta) of it).  Every thread calls it, between barriers of its own use of
+// `best`; it holds one.  Apart from the step, whose code it would spread (2048 x 1024 nodes,
+// us a step: 520 inline, 517 as a function).
 template <typename R, int D>
-__device__ __forceinline__ bool middle_gauge(const Extremes<D> &t, uint4 *best, R (&gb)[D + 1])
+struct MiddleGauge { R g[D + 1]; bool near; };
+template <typename R, int D>
+__device__ __noinline__ MiddleGauge<R, D> middle_gauge_of(unsigned top, unsigned low, float l0, float h0, float l1, float h1,
+                                                          float l2, float h2, uint4 *best)
 {
+    const float lo[3] = {l0, l1, l2}, hi[3] = {h0, h1, h2};
     static_assert(STEP_THREADS / 32 * 2 * D * 4 <= BEST * (int)sizeof(uint4), "best holds the warps' velocities");
     int *w = reinterpret_cast<int *>(best);
 #pragma unroll
     for (int a = 0; a < D; ++a) {
-        const int l = __reduce_min_sync(0xffffffffu, ordered(t.lo[a])), h = __reduce_max_sync(0xffffffffu, ordered(t.hi[a]));
+        const int l = __reduce_min_sync(0xffffffffu, ordered(lo[a])), h = __reduce_max_sync(0xffffffffu, ordered(hi[a]));
         if ((threadIdx.x & 31) == 0) {
             w[(threadIdx.x >> 5) * 2 * D + a] = l;
             w[(threadIdx.x >> 5) * 2 * D + D + a] = h;
         }
     }
     __syncthreads();
-    gb[0] = sqrt_(sqrt_((R)t.hottest()) * sqrt_((R)__uint_as_float(t.low)));
-    bool near = true;
+    MiddleGauge<R, D> o;
+    const R hot = (R)__uint_as_float(top);
+    o.g[0] = sqrt_(sqrt_(hot) * sqrt_((R)__uint_as_float(low)));
+    const R lim = R(FAR_SPEED) * sqrt_(hot);
+    o.near = true;
 #pragma unroll
     for (int a = 0; a < D; ++a) {
         int l = w[a], h = w[D + a];
@@ -836,10 +850,18 @@ __device__ __forceinline__ bool middle_gauge(const Extremes<D> &t, uint4 *best, 
             h = max(h, w[k * 2 * D + D + a]);
         }
         const R u = R(0.5) * (R)unordered(l), v = R(0.5) * (R)unordered(h);
-        gb[1 + a] = u + v;
-        near = near && v - u <= R(FAR_SPEED) * gb[0];
+        o.g[1 + a] = u + v;
+        o.near = o.near && v - u <= lim;
     }
-    return near;
+    return o;
+}
+template <typename R, int D>
+__device__ __forceinline__ bool middle_gauge(const Extremes<D> &t, uint4 *best, R (&gb)[D + 1])
+{
+    const MiddleGauge<R, D> m = middle_gauge_of<R, D>(t.top, t.low, t.lo[0], t.hi[0], t.lo[1], t.hi[1], t.lo[D - 1], t.hi[D - 1], best);
+#pragma unroll
+    for (int a = 0; a <= D; ++a) gb[a] = m.g[a];
+    return m.near;
 }
 
 // Transfer increments along one axis, E[k][a] = l_k((a - 1) + e_a) - delta_ka with
@@ -1293,7 +1315,8 @@ __device__ __noinline__ void stream_far(const DevParams &p, const double *__rest
 
 // Streams node (X, Y) into the gauge (th, ux, uy): inc = the increments of the streamed
 // populations over the node's own (f, then g).  gauge_b: the tile's common gauge
-// (sqrt theta, u_x, u_y); dt: of stage_tile; FAR: the slots have a halo of HALO_FAR; keep: the thread's column of kept values.
+// (sqrt theta, u_x, u_y); dt: of stage_tile; FAR: the slots have a halo of HALO_FAR; keep:
+// the thread's column of kept values.
 template <typename R, bool FAR>
 __device__ __forceinline__ void stream_node(const DevParams &p, const R *__restrict__ in, int X, int Y, const R *slot,
                                             int pitch, const R (&gauge_b)[3], R dt, R th, R ux, R uy, bool first,
@@ -1627,8 +1650,8 @@ __device__ __forceinline__ R stage_tile(const DevParams &p, const R *__restrict_
     }
     // (the barrier: base is there, and aux may be overwritten)
     R dt = q.dt;
-    const bool spread = ex.spread(gb), reach = ex.reach((float)shot, p.pf.dt) && tl.halo < widest_halo(TX, TY, sizeof(R));
-    if (__syncthreads_or(spread || reach)) {
+    const bool spread = ex.spread(gb, (float)shot), reach = ex.reach((float)shot, p.pf.dt) && tl.halo < widest_halo(TX, TY, sizeof(R));
+    if (__builtin_expect(__syncthreads_or(spread || reach), 0)) {   // (rare: out of the way)
         if (__syncthreads_or(spread)) {
             smooth = false;
             if (!middle_gauge<R, 2>(ex, best, gb)) dt = R(1) / R(0);
