@@ -31,9 +31,9 @@
 // node; 6.3 with 4 x 4 nodes and a halo of 3).
 // Measured (five steps of the 2048 x 1024 shock-droplet interaction with init and read-out,
 // mixed): 17.7 -> 3.90 ms, 720 us a step; two FP64 steps of a 509 x 387 droplet 22.8 ->
-// 5.49 ms, 2.69 ms a step.  The mixed form is bound by instruction fetch and issue (issue 54 %
-// active, FMA pipe 56 %, 1.2 warps per issue waiting for instructions), the FP64 form by the
-// FP64 pipe (92 % busy); DRAM is 10 % busy.
+// 5.49 ms, 2.69 ms a step.  The mixed form is bound by instruction fetch and issue (issue 52 %
+// active, FMA pipe 48 %, 1.1 warps per issue waiting for instructions), the FP64 form by the
+// FP64 pipe (90 % busy); DRAM is 14 % busy.
 //
 // Accuracy.  A tile whose thetas differ holds the carried populations themselves in the
 // gauge of geometric-mean theta and mean velocity of its hottest and coldest nodes, by
@@ -80,9 +80,9 @@ constexpr float SMOOTH_TILE = 0.9f;
 // form around the middle of its velocities, and one in which a node then still moves faster
 // than FAR_SPEED sqrt(theta) takes the general stream, which carries each node straight into
 // the arrival gauge.  theta is the tile's hottest: at interfaces whose coldest nodes are at
-// the pressure floor, the gauge's own theta_b is a small part of it, and asking for
-// velocities against theta_b sent tiles of quiet droplets to the general stream (D3Q27, 96 x 96
-// x 64 sphere: 3.07 against 2.78 ms a step).
+// the pressure floor, the gauge's own theta_b is a small part of it, and tiles of ordinary
+// shocks and droplets would change their gauge for nothing (their times are the same either
+// way: 96 x 96 x 64 sphere 2829 us a step against theta_b, 2826 against the hottest).
 constexpr float SMOOTH_SPREAD = 0.4f;
 constexpr float FAR_SPEED = 1.0f;
 constexpr int BEST = 8;   // uint4 of shared memory in which a block agrees on its gauge
